@@ -133,10 +133,9 @@ typedef struct {
  * m = row_ptr[n] < 2^32 and d_out(v) >= 1 for every v (FORA_ERR_DANGLING: a walk of
  * Section 2.1 needs an out-neighbour at every node).  Edges are taken with
  * multiplicity; self-loops are allowed.  flags: 0.  Device memory: about
- * 4 (n + 1) + 4 m + 20 n bytes, plus a bit-packed copy of col for the walks when
- * ceil(log2 n) <= 24, plus 4 m bytes of target codes for the push when some node has
- * in-degree >= 64 (the up to 128 nodes of highest in-degree are marked in them, see
- * "spread_hot").  Errors: FORA_ERR_BAD_ARG, FORA_ERR_DANGLING, FORA_ERR_OOM,
+ * 4 (n + 1) + 8 m + 16 n bytes (4 m of them the walks' edge records), plus 4 m bytes of
+ * target codes for the push when some node has in-degree >= 64 (the up to 128 nodes of
+ * highest in-degree are marked in them, see "spread_hot").  Errors: FORA_ERR_BAD_ARG, FORA_ERR_DANGLING, FORA_ERR_OOM,
  * FORA_ERR_CUDA (no device); *out is NULL on any error.
  */
 int fora_graph_create(int64_t n, const int64_t *row_ptr, const int32_t *col, uint32_t flags,
@@ -439,7 +438,8 @@ int fora_threshold_debug(const double *r, const double *rmax, const uint32_t *d,
  * residue with one atomic; 0 adds every push with its own atomic (results differ only by
  * the order of FP64 additions).  The tuning read-back also answers "hot_nodes", the
  * number of hot nodes of the graph (0: spread_hot has no effect).  "walk_blocks" (3, 4
- * or 5, default 4): resident walk blocks per SM, traded against registers per thread.
+ * or 5, default 4): resident walk blocks (of 384 threads) per SM, traded against registers
+ * per thread.
  * "push_host_loop" (0 or 1, default 0): 1 launches the push rounds from a host loop with
  * one device-to-host read per round, instead of the CUDA graph whose conditional while-node
  * runs them on the device; the kernels are the same (a profiler that cannot look inside
@@ -464,7 +464,7 @@ int fora_graph_tuning(fora_graph *g, const char *key, int64_t *value);
  * given sources (HOST array, a representative batch) once to warm up, then with
  * spread_width 1, 2, 4, 8, 16 keeping the fastest push phase, then (when the graph
  * has hot nodes) with "spread_hot" 0 and 1 at that width keeping the faster push, then
- * with walk_blocks 3, 4, 5 ("walk_blocks": resident 256-thread walk blocks per SM, i.e.
+ * with walk_blocks 3, 4, 5 ("walk_blocks": resident walk blocks per SM, i.e.
  * the register budget of the walk kernel) keeping the fastest walk phase (all with
  * "pipeline" 1), then, for nsrc >= 64, "pipeline" 1 or 2 by the whole batch's time (the faster of two
  * runs each).  The choices stay set on the graph; spread_width and walk_blocks are

@@ -102,7 +102,7 @@ fora::WorkspaceSizes fora::workspace_sizes(int64_t n, uint64_t hub_chunks, int n
   const size_t H = S * hub_chunks + 1;
   z.r = z.N * sizeof(double);
   z.res = z.N * sizeof(double);
-  z.tally = z.N * sizeof(Tally);
+  z.tally = 2 * z.N * sizeof(unsigned long long);
   z.q = (z.N + 1) * sizeof(unsigned long long);
   z.fa = (z.N + 1) * sizeof(double);
   z.hub = H * sizeof(unsigned long long);
@@ -390,7 +390,12 @@ int fora::run_batch_ws(fora_graph* g, Workspace* w, const fora_params* p,
     CUDA_TRY(cudaMemcpyAsync(w->rmax, rsrc.device, nsrc * sizeof(double), cudaMemcpyDeviceToDevice, stream));
   else
     CUDA_TRY(cudaMemcpyAsync(w->rmax, w->h_rmax, nsrc * sizeof(double), cudaMemcpyHostToDevice, stream));
-  CUDA_TRY(cudaMemsetAsync(w->tally, 0, N * sizeof(Tally), stream));
+  const bool want_count = dbg && dbg->count;
+  const size_t ends = (size_t)end_places(g->n, g->wbits);
+  uint32_t* wcount = reinterpret_cast<uint32_t*>(w->tally + (size_t)nsrc * ends);
+  CUDA_TRY(cudaMemsetAsync(w->tally, 0, (size_t)nsrc * ends * sizeof(unsigned long long), stream));
+  if (want_count)
+    CUDA_TRY(cudaMemsetAsync(wcount, 0, (size_t)nsrc * ends * sizeof(uint32_t), stream));
   CUDA_TRY(cudaMemsetAsync(w->small, 0, 8 * sizeof(unsigned long long), stream));
   CUDA_TRY(cudaMemsetAsync(w->err, 0, sizeof(uint32_t), stream));
   CUDA_TRY(cudaMemsetAsync(w->stats, 0, nsrc * sizeof(SlotStats), stream));
@@ -405,8 +410,8 @@ int fora::run_batch_ws(fora_graph* g, Workspace* w, const fora_params* p,
   b.seed = p->seed;
   set_round_keys(&b, p->seed);
   b.zero_hop = (p->flags & FORA_ZERO_HOP) != 0;
-  b.want_count = dbg && dbg->count;
-  b.r = w->r; b.res = w->res; b.tally = w->tally;
+  b.want_count = want_count;
+  b.r = w->r; b.res = w->res; b.acc = w->tally; b.wcount = wcount; b.ends = ends;
   b.q[0] = w->q[0]; b.q[1] = w->q[1]; b.fa = w->fa;
   b.hub[0] = w->hub[0]; b.hub[1] = w->hub[1];
   b.hub_stride = g->hub_chunks;
@@ -418,6 +423,7 @@ int fora::run_batch_ws(fora_graph* g, Workspace* w, const fora_params* p,
   b.work = w->work;
   b.ps = w->ps;
   b.totals = w->small + 4;
+  b.walk_next = w->small + 6;
   b.sources = w->sources; b.rmax = w->rmax; b.stats = w->stats; b.err = w->err;
   b.wr_entry = w->q[0];
   b.wr_offset = w->q[1];
@@ -491,7 +497,8 @@ int fora::run_batch_ws(fora_graph* g, Workspace* w, const fora_params* p,
         const size_t off = (size_t)first * n64, len = (size_t)k * n64;
         CUDA_TRY(cudaMemsetAsync(w->r + off, 0, len * sizeof(double), stream));
         CUDA_TRY(cudaMemsetAsync(w->res + off, 0, len * sizeof(double), stream));
-        CUDA_TRY(cudaMemsetAsync(w->tally + off, 0, len * sizeof(Tally), stream));
+        CUDA_TRY(cudaMemsetAsync(w->tally + (size_t)first * ends, 0,
+                                 (size_t)k * ends * sizeof(unsigned long long), stream));
         CUDA_TRY(cudaMemsetAsync(w->stats + first, 0, k * sizeof(SlotStats), stream));
         b.nsrc = first + k;
         CUDA_TRY(launch_push_join(gd, b, first, k, stream));
@@ -538,12 +545,12 @@ int fora::run_batch_ws(fora_graph* g, Workspace* w, const fora_params* p,
     CUDA_TRY(launch_walks(gd, b, g->num_sms, stream));
   if (timed) CUDA_TRY(cudaEventRecord(w->ev[3], stream));
   if (dbg && (dbg->count || dbg->acc))
-    CUDA_TRY(launch_unpack_tally(w->tally, dbg->count, reinterpret_cast<unsigned long long*>(dbg->acc), N,
-                                 g->num_sms, stream));
+    CUDA_TRY(launch_unpack_ends(gd, b, dbg->count, reinterpret_cast<unsigned long long*>(dbg->acc),
+                                g->num_sms, stream));
 
   // ---- estimate and top-k (the residue array becomes the estimate) ----
   nvtx_phase.next("fora: estimate and top-k");
-  CUDA_TRY(launch_estimate(w->res, w->tally, w->r, w->r, rp.alpha, b.zero_hop, N, g->num_sms, stream));
+  CUDA_TRY(launch_estimate(gd, b, w->r, stream));
   if (dbg && dbg->estimate)
     CUDA_TRY(cudaMemcpyAsync(dbg->estimate, w->r, N * sizeof(double), cudaMemcpyDeviceToDevice, stream));
   int32_t* ids_dev = out_dev ? out_ids : w->out_ids;
@@ -689,6 +696,88 @@ std::vector<uint32_t> hot_nodes_of(int64_t n, const int32_t* col, int64_t m) {
   return hot;
 }
 
+// The walks' numbering of the nodes of a CSR graph (GraphDev::wcol): records per node, the
+// {first edge - id * d, d} of every degree class and the {first edge, d} of the other nodes.
+struct WalkNumbering {
+  int bits = 1;
+  std::vector<uint32_t> id;
+  std::vector<uint2> cls, esc;
+};
+
+WalkNumbering walk_numbering(int64_t n, const uint32_t* row) {
+  WalkNumbering w;
+  while (w.bits < 31 && (1ll << w.bits) < n) ++w.bits;
+  // nodes per distinct degree; only m / 2^16 nodes can have a degree outside the array
+  constexpr uint32_t kDirect = 1u << 16;
+  std::vector<uint32_t> count(kDirect, 0u);
+  std::map<uint32_t, uint32_t> large;
+  for (int64_t v = 0; v < n; ++v) {
+    const uint32_t d = row[v + 1] - row[v];
+    if (d < kDirect) ++count[d]; else ++large[d];
+  }
+  for (const auto& x : large) count.push_back(x.second);
+  // the lowest degrees get a class each, as many as a record's upper bits and the walk
+  // kernel's table can tell apart; the classes of the others are all ncls
+  const size_t limit = std::min<size_t>((1ull << (32 - w.bits)) - 1, kMaxWalkClasses);
+  std::vector<uint32_t> of(count.size(), 0u), next(1, 0u);  // next[c + 1]: next id of class c
+  uint64_t coded = 0;
+  std::vector<uint32_t> members;
+  {
+    auto it = large.begin();
+    for (size_t k = 0; k < count.size(); ++k) {
+      const uint32_t d = k < kDirect ? (uint32_t)k : (it++)->first;
+      if (count[k] == 0) continue;
+      if (w.cls.size() < limit) {
+        of[k] = (uint32_t)w.cls.size();
+        w.cls.push_back(make_uint2(0u, d));
+        members.push_back(count[k]);
+        coded += count[k];
+      } else {
+        of[k] = 0xFFFFFFFFu;
+      }
+    }
+    uint32_t k = kDirect;
+    for (auto& x : large) x.second = k++;  // the degree's place in `of`
+  }
+  const uint32_t ncls = (uint32_t)w.cls.size(), nesc = (uint32_t)(n - (int64_t)coded);
+  w.esc.reserve(nesc);
+  w.id.resize((size_t)n);
+  // ids: the nodes without a class first, then class after class; rows in the order of ids
+  next.assign(ncls, 0u);
+  uint32_t first = nesc;
+  for (uint32_t c = 0; c < ncls; ++c) {
+    next[c] = first;
+    first += members[c];
+  }
+  uint32_t edge = 0;  // rows of the nodes without a class
+  for (int64_t v = 0; v < n; ++v) {
+    const uint32_t d = row[v + 1] - row[v];
+    const uint32_t c = of[d < kDirect ? d : large[d]];
+    if (c == 0xFFFFFFFFu) {
+      w.id[v] = (uint32_t)((uint64_t)ncls << w.bits) | (uint32_t)w.esc.size();
+      w.esc.push_back(make_uint2(edge, d));
+      edge += d;
+    } else {
+      w.id[v] = (uint32_t)((uint64_t)c << w.bits) | next[c]++;
+    }
+  }
+  for (uint32_t c = 0; c < ncls; ++c) {
+    const uint32_t d = w.cls[c].y, id0 = next[c] - members[c];
+    w.cls[c].x = edge - id0 * d;  // first edge of walk id x: w.cls[c].x + x * d, mod 2^32
+    edge += members[c] * d;
+  }
+  return w;
+}
+
+// A device copy of a host vector (of at least one element's room).
+template <typename T>
+cudaError_t upload(T** p, const std::vector<T>& v) {
+  cudaError_t e = dalloc(p, std::max<size_t>(v.size(), 1) * sizeof(T));
+  if (e == cudaSuccess && !v.empty())
+    e = cudaMemcpy(*p, v.data(), v.size() * sizeof(T), cudaMemcpyHostToDevice);
+  return e;
+}
+
 int run_batch(fora_graph* g, const fora_params* p, const int32_t* sources, int nsrc,
               int32_t* out_ids, double* out_vals, fora_stats* st, const fora_debug_io* dbg,
               uint32_t dbg_flags, cudaStream_t stream, RmaxSource rsrc = RmaxSource(),
@@ -750,25 +839,6 @@ int fora_graph_create(int64_t n, const int64_t* row_ptr, const int32_t* col, uin
   if (e == cudaSuccess) e = dalloc(&g->col, (size_t)m * sizeof(int32_t));
   if (e == cudaSuccess) e = cudaMemcpy(g->row, row.data(), ((size_t)n + 1) * sizeof(uint32_t), cudaMemcpyHostToDevice);
   if (e == cudaSuccess) e = cudaMemcpy(g->col, col, (size_t)m * sizeof(int32_t), cudaMemcpyHostToDevice);
-  // walk copy of col: ceil(log2 n) bits per target when that saves at least a quarter
-  int bits = 1;
-  while (bits < 31 && (1ll << bits) < n) ++bits;
-  if (e == cudaSuccess && bits <= 24) {
-    const size_t words = ((size_t)m * bits + 31) / 32 + 2;
-    std::vector<uint32_t> packed(words, 0u);
-    for (int64_t k = 0; k < m; ++k) {
-      const uint64_t bit = (uint64_t)k * bits;
-      const uint64_t w = bit >> 5;
-      const uint32_t off = (uint32_t)(bit & 31);
-      const uint64_t v = (uint64_t)(uint32_t)col[k] << off;
-      packed[w] |= (uint32_t)v;
-      packed[w + 1] |= (uint32_t)(v >> 32);
-    }
-    e = dalloc(&g->colp, words * sizeof(uint32_t));
-    if (e == cudaSuccess)
-      e = cudaMemcpy(g->colp, packed.data(), words * sizeof(uint32_t), cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) g->colbits = bits;
-  }
   if (e == cudaSuccess) {  // reciprocal out-degrees (every d >= 1 here)
     std::vector<double> invd((size_t)n);
     for (int64_t v = 0; v < n; ++v) invd[v] = 1.0 / (double)(row[v + 1] - row[v]);
@@ -776,12 +846,15 @@ int fora_graph_create(int64_t n, const int64_t* row_ptr, const int32_t* col, uin
     if (e == cudaSuccess)
       e = cudaMemcpy(g->invd, invd.data(), (size_t)n * sizeof(double), cudaMemcpyHostToDevice);
   }
-  if (e == cudaSuccess) {  // the walks' node records {first edge, out-degree}
-    std::vector<uint2> rd((size_t)n);
-    for (int64_t v = 0; v < n; ++v) rd[v] = make_uint2(row[v], row[v + 1] - row[v]);
-    e = dalloc(&g->rd, (size_t)n * sizeof(uint2));
-    if (e == cudaSuccess)
-      e = cudaMemcpy(g->rd, rd.data(), (size_t)n * sizeof(uint2), cudaMemcpyHostToDevice);
+  if (e == cudaSuccess) {  // the walks' numbering and edge records
+    const WalkNumbering wn = walk_numbering(n, row.data());
+    g->ncls = (int)wn.cls.size();
+    g->wbits = wn.bits;
+    e = upload(&g->wid, wn.id);
+    if (e == cudaSuccess) e = upload(&g->wcls, wn.cls);
+    if (e == cudaSuccess) e = upload(&g->wesc, wn.esc);
+    if (e == cudaSuccess) e = dalloc(&g->wcol, (size_t)m * sizeof(uint32_t));
+    if (e == cudaSuccess) e = launch_walk_records(g->dev(), g->wcol, g->num_sms, 0);
   }
   if (e == cudaSuccess) {
     // hot targets of the spread, and the target codes that mark them
@@ -843,10 +916,12 @@ void fora_graph_destroy(fora_graph* g) {
     }
     dfree(g->row);
     dfree(g->col);
-    dfree(g->colp);
     dfree(g->indeg);
     dfree(g->invd);
-    dfree(g->rd);
+    dfree(g->wcol);
+    dfree(g->wid);
+    dfree(g->wcls);
+    dfree(g->wesc);
     dfree(g->scol);
     dfree(g->hot_node);
     dfree(g->idx_off);
@@ -886,7 +961,7 @@ int fora_index_build(fora_graph* g, const fora_params* params, void* stream_) {
   set_round_keys(&b, params->seed);
   // zero-hop: omega_max from (1 - alpha) RN(r_max d(v)) and walks with a forced first move
   b.zero_hop = zero_hop ? 1 : 0;
-  b.r = w->r; b.res = w->res; b.tally = w->tally;
+  b.r = w->r; b.res = w->res; b.acc = w->tally;
   b.q[0] = w->q[0]; b.q[1] = w->q[1]; b.fa = w->fa;
   b.hub[0] = w->hub[0]; b.hub[1] = w->hub[1];
   b.hub_stride = g->hub_chunks;
@@ -898,6 +973,7 @@ int fora_index_build(fora_graph* g, const fora_params* params, void* stream_) {
   b.work = w->work;
   b.ps = w->ps;
   b.totals = w->small + 4;
+  b.walk_next = w->small + 6;
   b.sources = w->sources; b.rmax = w->rmax; b.stats = w->stats; b.err = w->err;
   b.wr_entry = w->q[0];
   b.wr_offset = w->q[1];
@@ -963,9 +1039,16 @@ int fora_index_export(const fora_graph* g, int64_t* off, uint32_t* dest) {
   if (!g->idx_dest) return fail(FORA_ERR_BAD_ARG, "the graph has no walk index");
   CUDA_TRY(cudaSetDevice(g->device));
   CUDA_TRY(cudaMemcpy(off, g->idx_off, ((size_t)g->n + 1) * sizeof(int64_t), cudaMemcpyDeviceToHost));
-  if (g->idx_entries > 0)
+  if (g->idx_entries > 0) {
     CUDA_TRY(cudaMemcpy(dest, g->idx_dest, (size_t)g->idx_entries * sizeof(uint32_t),
                         cudaMemcpyDeviceToHost));
+    // the device keeps walk ids: back to node ids
+    std::vector<uint32_t> rec((size_t)g->n), node((size_t)g->n);
+    CUDA_TRY(cudaMemcpy(rec.data(), g->wid, (size_t)g->n * sizeof(uint32_t), cudaMemcpyDeviceToHost));
+    const uint32_t mask = (1u << g->wbits) - 1u;
+    for (int64_t v = 0; v < g->n; ++v) node[rec[v] & mask] = (uint32_t)v;
+    for (int64_t i = 0; i < g->idx_entries; ++i) dest[i] = node[dest[i]];
+  }
   return FORA_OK;
 }
 

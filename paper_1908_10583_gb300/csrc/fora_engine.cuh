@@ -63,12 +63,22 @@ struct GraphDev {
   int64_t m;
   const uint32_t* row;  // [n+1] edge offsets (m < 2^32)
   const int32_t* col;   // [m]
-  // The same targets bit-packed, colbits bits each (0 = not packed), for the walks: a
-  // smaller footprint keeps more of the graph in L2 beside the walk tallies.
-  const uint32_t* colp;
-  int colbits;
   const double* invd;   // [n] RN(1 / d(v)): the push increment is a product, not a quotient
-  const uint2* rd;      // [n] {row[v], d(v)}: a walk's move reads one aligned 8-byte record
+  // The walks' own numbering and adjacency.  Nodes of equal out-degree have consecutive walk
+  // ids and consecutive rows of wcol, so a node's first edge is wcls[c].x + id * d with its
+  // degree class c (d = wcls[c].y), and an edge record {class : 32 - wbits bits, walk id :
+  // wbits bits} holds all that the next move needs: one 4-byte gather per move.  (A gather
+  // of a node record and one of a packed target, 2.8 sectors per move, kept the walks at the
+  // SMs' limit of one gathered sector per clock.)  The lowest ncls degrees have classes; the
+  // other nodes have the class ncls and the lowest walk ids, their {first edge, degree} in
+  // wesc[id].
+  const uint32_t* wcol;  // [m] edge records
+  const uint32_t* wid;   // [n] record of node v
+  const uint2* wcls;     // [ncls]
+  const uint2* wesc;     // [nodes of class ncls]
+  int ncls;
+  int wbits;
+  uint32_t ecols;        // end_cols(n, wbits)
   // The spread's copy of the targets (null when the graph has no hot nodes): the target
   // id, or kHotBit | h for the h-th hot node (a node of high in-degree, hot_node[h]), whose
   // increments a block sums in shared memory before one reduction reaches L2.
@@ -89,21 +99,34 @@ constexpr int kHotSlots = FORA_HOT_SLOTS;
 constexpr uint32_t kHotMinIndeg = 64;
 constexpr uint32_t kHotBit = 0x80000000u;
 
-// Target e of a bit-packed column array (two 32-bit words always readable).
-__device__ __forceinline__ uint32_t packed_target(const uint32_t* colp, int bits, uint32_t e) {
-  const unsigned long long bit = (unsigned long long)e * (unsigned long long)bits;
-  const unsigned long long w = bit >> 5;
-  const unsigned long long two = (unsigned long long)colp[w] | ((unsigned long long)colp[w + 1] << 32);
-  return (uint32_t)(two >> (bit & 31)) & ((1u << bits) - 1u);
+// Degree classes of the walk records: their table (8 bytes each) sits in shared memory of
+// the walk kernel.  The 2^20-node R-MAT graph has 743 distinct degrees.
+constexpr uint32_t kMaxWalkClasses = 1023;
+
+// Walk id of a record.
+__device__ __forceinline__ uint32_t walk_id(const GraphDev& g, uint32_t rec) {
+  return rec & ((1u << g.wbits) - 1u);
 }
 
-// Walk end tally of one (source, node): fixed-point weight and count share one
-// 16-byte record, so a walk's end touches a single L2 sector.
-struct __align__(16) Tally {
-  unsigned long long acc;  // sum of walk weights, 2^-63 units
-  uint32_t cnt;            // number of walks
-  uint32_t pad;
-};
+// Where a node's walk ends are summed, by walk id: neighbouring ids lie 32 sums (256 bytes)
+// apart.  Walk ids follow the out-degree, so the nodes where most walks end have neighbouring
+// ids, and sums of theirs in one sector would queue at one L2 slice.
+// end_rows = 2^(wbits - 5), end_cols = ceil(n / end_rows); a source has end_rows * end_cols
+// places, fewer than n + end_rows.
+__host__ __device__ __forceinline__ uint32_t end_shift(int wbits) {
+  return wbits > 5 ? (uint32_t)(wbits - 5) : 0u;
+}
+__host__ __device__ __forceinline__ uint32_t end_cols(int64_t n, int wbits) {
+  const uint32_t k = end_shift(wbits);
+  return (uint32_t)(((uint64_t)n + (1ull << k) - 1) >> k);
+}
+__host__ __device__ __forceinline__ unsigned long long end_places(int64_t n, int wbits) {
+  return (unsigned long long)end_cols(n, wbits) << end_shift(wbits);
+}
+__device__ __forceinline__ uint32_t end_place(const GraphDev& g, uint32_t id) {
+  const uint32_t k = end_shift(g.wbits);
+  return (id & ((1u << k) - 1u)) * g.ecols + (id >> k);
+}
 
 // Per-source counters kept on the device during a call.
 struct SlotStats {
@@ -139,11 +162,15 @@ struct BatchDev {
   uint2 round_key[10];       // Philox round keys of `seed` (key + i * (0x9E3779B9, 0xBB67AE85))
   int zero_hop;              // walk phase with zero-hop pruning (Section 4.1)
   int want_count;            // tally walk counts too (only a debug output reads them)
-  uint32_t* walk_dest;       // non-null: k_walks stores walk g's end in walk_dest[g]
-                             // (building a walk index) instead of tallying it
+  uint32_t* walk_dest;       // non-null: k_walks stores walk g's end (a walk id) in
+                             // walk_dest[g] (building a walk index) instead of tallying it
   double* r;                 // residue, later the estimate
   double* res;               // reserve
-  Tally* tally;              // walk ends per (source, node)
+  // Walk ends: the sum of walk weights (2^-63 units) at [slot * ends + end_place(walk id)],
+  // and, when want_count, the number of walks.
+  unsigned long long* acc;
+  uint32_t* wcount;
+  unsigned long long ends;  // end_places of the graph
   // Frontier of source `slot`: entries (slot << 32) | v at q[par][slot * n + j],
   // j < slot_cnt[par][slot], with increments fa[slot * n + j]; its hub items at
   // hub[par][slot * hub_stride + j], j < slot_cnt[2 + par][slot].
@@ -169,6 +196,7 @@ struct BatchDev {
   unsigned long long* blk_cnt;    // [grid] per-block counts, then block offsets
   unsigned long long* blk_walks;  // [grid] per-block counts, then block offsets
   unsigned long long* totals;     // [2]: |R|, W
+  unsigned long long* walk_next;  // shares of the walk range taken beyond the first (zeroed)
   int residual_grid;
   int spread_width;  // interleaved segments of the frontier the spread visits at once
   int spread_hot;    // the spread sums hot targets per block (GraphDev::scol is set)
@@ -236,8 +264,11 @@ cudaError_t launch_index_residue(const GraphDev& g, double* r, double rmax, cuda
 cudaError_t launch_walks_indexed(const GraphDev& g, const BatchDev& b, int num_sms,
                                  const unsigned long long* idx_off, const uint32_t* idx_dest,
                                  cudaStream_t st);
-cudaError_t launch_unpack_tally(const Tally* t, uint32_t* cnt, unsigned long long* acc,
-                                uint64_t count, int num_sms, cudaStream_t st);
+// The walk ends of a batch as [nsrc][n] arrays over node ids (either output may be null).
+cudaError_t launch_unpack_ends(const GraphDev& g, const BatchDev& b, uint32_t* cnt,
+                               unsigned long long* acc, int num_sms, cudaStream_t st);
+// wcol of a graph whose other walk arrays are in place.
+cudaError_t launch_walk_records(const GraphDev& g, uint32_t* wcol, int num_sms, cudaStream_t st);
 cudaError_t launch_philox_table(const uint32_t* ctr_key, uint32_t* out, int count,
                                 cudaStream_t st);
 
@@ -257,11 +288,9 @@ cudaError_t launch_pred_to_rmax(const float* pred, int n, double rmax_rule, floa
 int mlp_tile();
 
 // topk.cu
-// est may alias r (the residue array becomes the estimate); with zero_hop the estimate
-// also takes alpha * r.
-cudaError_t launch_estimate(const double* res, const Tally* tally, double* est, const double* r,
-                            double alpha, int zero_hop, uint64_t count, int num_sms,
-                            cudaStream_t st);
+// est may alias b.r (the residue array becomes the estimate); with zero-hop pruning the
+// estimate also takes alpha * r.
+cudaError_t launch_estimate(const GraphDev& g, const BatchDev& b, double* est, cudaStream_t st);
 // Scratch of the top-k select: hist [nrows][kBins], slots [nrows], cand [nrows][kSortCap].
 struct TopkScratch {
   uint32_t* hist;

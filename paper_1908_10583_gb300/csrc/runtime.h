@@ -62,7 +62,8 @@ struct Workspace {
   int cap = 0;
   double* r = nullptr;
   double* res = nullptr;
-  Tally* tally = nullptr;
+  // walk ends of every source (BatchDev::acc), then the walk counts of a debug call
+  unsigned long long* tally = nullptr;
   unsigned long long* q[2] = {nullptr, nullptr};
   unsigned long long* hub[2] = {nullptr, nullptr};
   double* fa = nullptr;
@@ -184,17 +185,20 @@ struct fora_graph {
   uint64_t hub_chunks = 0;  // sum over nodes with d > kHubChunk of ceil(d / kHubChunk)
   uint32_t* row = nullptr;
   int32_t* col = nullptr;
-  uint32_t* colp = nullptr;   // col bit-packed to colbits bits per target (0: not packed)
-  int colbits = 0;
   uint32_t* indeg = nullptr;  // in-degrees (features of the learned r_max)
   double* invd = nullptr;     // RN(1 / d(v)) per node
-  uint2* rd = nullptr;        // {row[v], d(v)} per node (the walks' node record)
+  // the walks' numbering and adjacency (GraphDev::wcol and the following)
+  uint32_t* wcol = nullptr;
+  uint32_t* wid = nullptr;
+  uint2* wcls = nullptr;
+  uint2* wesc = nullptr;
+  int ncls = 0, wbits = 1;
   uint32_t* scol = nullptr;   // the spread's target codes (GraphDev::scol), or null
   uint32_t* hot_node = nullptr;
   int nhot = 0;
   // FORA+ walk index (Section 3.3): ends of omega_max(v) walks from every v
   unsigned long long* idx_off = nullptr;  // [n + 1] exclusive prefix of omega_max
-  uint32_t* idx_dest = nullptr;           // [idx_entries] walk ends
+  uint32_t* idx_dest = nullptr;           // [idx_entries] walk ends (walk ids)
   int64_t idx_entries = 0;
   double idx_rmax = 0.0, idx_scale = 0.0, idx_alpha = 0.0;
   uint64_t idx_seed = 0;
@@ -208,7 +212,8 @@ struct fora_graph {
   fora::Workspace pipe_ws[fora::kMaxPipeline];
   cudaStream_t pipe_stream[fora::kMaxPipeline] = {};
   fora::GraphDev dev() const {
-    return fora::GraphDev{n, m, row, col, colp, colbits, invd, rd, scol, hot_node, nhot};
+    return fora::GraphDev{n,    m,    row,  col,   invd, wcol,     wid,
+                          wcls, wesc, ncls, wbits, fora::end_cols(n, wbits), scol, hot_node, nhot};
   }
 };
 

@@ -249,10 +249,9 @@ __global__ void __launch_bounds__(kResidualThreads) k_residual_weight(BatchDev b
   }
 }
 
-constexpr int kWalkThreads = 256;
+constexpr int kWalkThreads = 384;
 constexpr int kWalkWarps = kWalkThreads / 32;
-constexpr int kWalksPerLane = 32;
-constexpr int kChunk = 32 * kWalksPerLane;  // walks per warp chunk
+constexpr int kIndexedThreads = 256;
 constexpr uint32_t kMaxSteps = 16384u;
 
 // Largest i in [0, nR) with off[i] <= g (off non-decreasing, off[0] = 0 <= g);
@@ -274,48 +273,45 @@ __device__ __forceinline__ unsigned long long warp_find_entry(const unsigned lon
   return lo + (unsigned long long)(31 - __clz(bal));
 }
 
-// Map walk cbeg + i (i < cnt) to its residual entry idx0 + smap[i], 32 walks at a time
-// (the entries' walk offsets are read coalesced, a 5-step search per walk in registers).
-__device__ __forceinline__ void map_chunk(const unsigned long long* off, unsigned long long nR,
-                                          unsigned long long cbeg, uint32_t cnt,
-                                          unsigned long long idx0, uint16_t* smap) {
-  const uint32_t lane = threadIdx.x & 31;
-  unsigned long long idxw = idx0;
-  for (uint32_t rb = 0; rb < cnt; rb += 32) {
-    const unsigned long long gw = cbeg + rb + lane;
-    const unsigned long long o = idxw + lane < nR ? off[idxw + lane] : ~0ull;
-    int lo = 0, hi = 31;  // largest j with off[idxw + j] <= gw
-#pragma unroll
-    for (int s = 0; s < 5; ++s) {
-      const int mid = (lo + hi + 1) >> 1;
-      if (__shfl_sync(kFull, o, mid) <= gw) lo = mid; else hi = mid - 1;
-    }
-    const unsigned long long mine = idxw + (unsigned long long)lo;
-    smap[rb + lane] = (uint16_t)(mine - idx0);
-    idxw = __shfl_sync(kFull, mine, 31);
-  }
-  __syncwarp();
+// Walks a warp takes from the flat walk range at a time: fewer when the walks would not
+// give every warp several such shares, so that a small query still uses every warp.
+__device__ __forceinline__ uint32_t share_walks(unsigned long long W, unsigned long long nwarps,
+                                                uint32_t most) {
+  const unsigned long long share = (W + nwarps - 1) / nwarps / 6;
+  return share >= most ? most : (uint32_t)((share + 32) / 32 * 32);
 }
 
-// Target e of the walk copy of the adjacency (bit-packed when colbits > 0).
-__device__ __forceinline__ uint32_t walk_target(const GraphDev& g, uint32_t e) {
-  return g.colbits ? packed_target(g.colp, g.colbits, e) : (uint32_t)g.col[e];
+// The walk kernels' copy of the degree classes (GraphDev::wcls) in shared memory.
+__device__ __forceinline__ void load_classes(const GraphDev& g, uint2* cls) {
+  for (int c = threadIdx.x; c < g.ncls; c += blockDim.x) cls[c] = g.wcls[c];
 }
 
-constexpr uint32_t kCapped = 0xFFFFFFFFu;
+// {first edge, out-degree} of the node of a record: from its class, without a load from
+// global memory, or (when `need`) from the list of the nodes without a class.  cls has an
+// entry at ncls too.
+__device__ __forceinline__ uint2 node_row(const GraphDev& g, const uint2* cls, uint32_t rec,
+                                          bool need) {
+  const uint32_t c = rec >> g.wbits, id = walk_id(g, rec);
+  const uint2 k = cls[c];
+  uint2 r = make_uint2(k.x + id * k.y, k.y);
+  if (c >= (uint32_t)g.ncls && need) r = g.wesc[id];
+  return r;
+}
 
-// The rest of a walk whose neighbour draw at x (row offset rb, degree d) came out with
-// low word below d on its first try, m0 (Lemire's method then rejects the try when the low
-// word is below 2^32 mod d, probability below d / 2^32): the try is accepted or retried,
-// then the walk goes on with the words taken one at a time from word `pos` of the block
-// `blk` (the next block to generate is `cb`), stop tests and moves in stream order.
-// Returns the end node, or kCapped when the walk reaches the step cap (or, never in
-// practice, 64 rejected tries in a row).
-__device__ __forceinline__ uint32_t walk_rest(const GraphDev& g, uint4 blk, int pos, uint32_t cb,
-                                              uint32_t j, uint32_t v, uint32_t s, uint2 key,
-                                              uint32_t t_alpha, uint32_t x, uint32_t rb,
-                                              uint32_t d, unsigned long long m0,
-                                              uint32_t* steps) {
+constexpr uint32_t kCapped = 0x80000000u;
+
+// The rest of a walk whose neighbour draw at x came out with a low word below d on its first
+// try, word `pos - 1` of its Philox block cb - 1 (Lemire's method rejects the try when the
+// low word is below 2^32 mod d, probability below d / 2^32): the words are taken one at a
+// time from there, tries, stop tests and moves in stream order.  It evaluates the block again
+// rather than keep its words alive.  Returns the record of the end node (low word) and the walk's moves (high word), with kCapped set in the latter when
+// the walk reaches the step cap (or, never in practice, 64 rejected tries in a row).
+__device__ __forceinline__ unsigned long long walk_rest(const uint32_t* wcol, const uint2* wesc,
+                                                     const uint2* cls, uint32_t ncls,
+                                                     uint32_t wbits, int pos, uint32_t cb,
+                                                     uint32_t j, uint32_t v, uint32_t s, uint2 key,
+                                                     uint32_t t_alpha, uint32_t x, uint32_t steps) {
+  uint4 blk = philox4x32_10(make_uint4(cb - 1, j, v, s), key);
   auto next = [&]() -> uint32_t {
     if (pos == 4) {
       blk = philox4x32_10(make_uint4(cb, j, v, s), key);
@@ -326,246 +322,271 @@ __device__ __forceinline__ uint32_t walk_rest(const GraphDev& g, uint4 blk, int 
     ++pos;
     return w;
   };
-  unsigned long long m = m0;
-  bool first = true;  // the move at x has its first try in m0
-  for (;;) {
+  --pos;  // the move at x takes its first try again
+  for (bool first = true;; first = false) {
     if (!first) {
-      if (next() < t_alpha) return x;
-      if (*steps >= kMaxSteps) return kCapped;
-      const uint2 r = g.rd[x];
-      rb = r.x;
-      d = r.y;
-      m = (unsigned long long)next() * d;
+      if (next() < t_alpha) break;
+      if (steps >= kMaxSteps) { steps |= kCapped; break; }
     }
-    first = false;
-    uint32_t low = (uint32_t)m;
-    if (low < d) {
-      const uint32_t reject_below = (0u - d) % d;
-      int tries = 0;
-      while (low < reject_below) {
-        if (++tries > 64) return kCapped;
-        m = (unsigned long long)next() * d;
-        low = (uint32_t)m;
-      }
+    const uint32_t c = x >> wbits, id = x & ((1u << wbits) - 1u);
+    uint2 r;
+    if (c >= ncls) {
+      r = wesc[id];
+    } else {
+      const uint2 k = cls[c];
+      r = make_uint2(k.x + id * k.y, k.y);
     }
-    x = walk_target(g, rb + (uint32_t)(m >> 32));
-    ++*steps;
+    const uint32_t reject_below = (0u - r.y) % r.y;
+    unsigned long long m = (unsigned long long)next() * r.y;
+    int tries = 0;
+    while ((uint32_t)m < reject_below && ++tries <= 64) m = (unsigned long long)next() * r.y;
+    if (tries > 64) { steps |= kCapped; break; }
+    x = wcol[r.x + (uint32_t)(m >> 32)];
+    ++steps;
   }
+  return ((unsigned long long)steps << 32) | x;
 }
 
-// One move of a walk at x with the word u, on the fast path: false when the low word of
-// the product is below d (a try Lemire's method may reject; walk_rest decides it, with
-// rb, d and m left for it), else x becomes the chosen out-neighbour.
-__device__ __forceinline__ bool fast_move(const GraphDev& g, uint32_t u, uint32_t& x,
-                                          uint32_t& rb, uint32_t& d, unsigned long long& m,
-                                          uint32_t* err, bool& bad) {
-  if (!FORA_IN_RANGE(err, x, g.n)) { bad = true; return false; }
-  const uint2 r = g.rd[x];
-  rb = r.x;
-  d = r.y;
-  m = (unsigned long long)u * d;
-  if ((uint32_t)m < d) return false;
-  const uint32_t e = rb + (uint32_t)(m >> 32);
-  if (!FORA_IN_RANGE(err, e, g.m)) { bad = true; return false; }
-  x = walk_target(g, e);
-  return true;
-}
-
-// The first kStartCache residual entries of a warp's chunk, staged in shared memory when
-// the chunk starts (one coalesced load per lane), so that a lane starting a walk of one of
-// them reads its data there instead of making two dependent global loads.
-constexpr int kStartCache = 32;
-struct StartCache {
-  unsigned long long off[kStartCache];
-  unsigned long long wgt[kStartCache];
-  uint32_t v[kStartCache];
-  uint32_t s[kStartCache];
-  uint32_t slot[kStartCache];
+// A warp's window on the residual entries: the data of up to 32 consecutive entries, twice
+// (walks of the window before are still running while the next one's are started), and the
+// entry of each of the window's walks.
+constexpr uint32_t kWindowWalks = 512;
+constexpr uint32_t kWalkShare = 4096;
+struct WalkWindow {
+  uint4 walk[64];  // node v, source, record of v, low word of the entry's walk offset
+  uint4 end[64];   // weight (low, high), slot
+  unsigned long long pos, stop;  // the warp's share of the walk range that is still to start
+  unsigned long long entry;      // the entry of walk pos
+  unsigned long long next;       // the warp's next share
+  uint8_t map[kWindowWalks];
 };
 
-__device__ __forceinline__ void fill_start_cache(const BatchDev& b, unsigned long long idx0,
-                                                 unsigned long long nR, StartCache& sc) {
+// The next window of the warp's share (or of its next share) into half `half` of the window:
+// its number of walks, 0 when no walk is left.
+__device__ __forceinline__ uint32_t next_window(const GraphDev& g, const BatchDev& b,
+                                                WalkWindow& w, uint32_t half) {
   const uint32_t lane = threadIdx.x & 31;
-  const unsigned long long idx = idx0 + lane;
-  if (idx < nR) {
-    const unsigned long long entry = b.wr_entry[idx];
-    const uint32_t slot = (uint32_t)(entry >> 32);
-    sc.off[lane] = b.wr_offset[idx];
-    sc.wgt[lane] = b.wr_weight[idx];
-    sc.v[lane] = (uint32_t)entry;
-    sc.slot[lane] = slot;
-    sc.s[lane] = (uint32_t)b.sources[slot];
+  const unsigned long long W = b.totals[1], nR = b.totals[0];
+  unsigned long long pos = w.pos, stop = w.stop, entry = w.entry;
+  if (pos >= stop) {
+    const unsigned long long nwarps = (unsigned long long)gridDim.x * kWalkWarps;
+    const uint32_t share = share_walks(W, nwarps, kWalkShare);
+    const unsigned long long mine = w.next;
+    pos = mine * share;
+    if (pos >= W) return 0;
+    __syncwarp();
+    if (lane == 0) w.next = nwarps + atomicAdd(b.walk_next, 1ull);
+    stop = min(pos + share, W);
+    entry = warp_find_entry(b.wr_offset, nR, pos);
+  }
+  const unsigned long long i = entry + lane;
+  const bool live = i < nR;
+  // offsets relative to pos; the entry of walk pos has offset 0, the others follow
+  const unsigned long long o = live ? b.wr_offset[i] : ~0ull;
+  const unsigned long long past = entry + 32 < nR ? b.wr_offset[entry + 32] : W;
+  const uint32_t rel = o <= pos ? 0u : (uint32_t)min(o - pos, 0x7FFFFFFFull);
+  if (live) {
+    const unsigned long long ent = b.wr_entry[i], wgt = b.wr_weight[i];
+    const uint32_t slot = (uint32_t)(ent >> 32), v = (uint32_t)ent;
+    w.walk[half * 32 + lane] = make_uint4(v, (uint32_t)b.sources[slot], g.wid[v], (uint32_t)o);
+    w.end[half * 32 + lane] = make_uint4((uint32_t)wgt, (uint32_t)(wgt >> 32), slot, 0u);
+  }
+  const uint32_t cnt =
+      (uint32_t)min(min(stop, past) - pos, (unsigned long long)kWindowWalks);
+  for (uint32_t k = lane; k < cnt + lane; k += 32) {  // every lane takes part in every step
+    int lo = 0, hi = 31;  // largest entry whose offset is at most k
+#pragma unroll
+    for (int t = 0; t < 5; ++t) {
+      const int mid = (lo + hi + 1) >> 1;
+      if (__shfl_sync(kFull, rel, mid) <= k) lo = mid; else hi = mid - 1;
+    }
+    if (k < cnt) w.map[k] = (uint8_t)lo;
+  }
+  const uint32_t passed = (uint32_t)__popc(__ballot_sync(kFull, rel <= cnt));  // entries begun
+  __syncwarp();
+  if (lane == 0) {
+    w.pos = pos + cnt;
+    w.stop = stop;
+    w.entry = pos + cnt == past ? entry + 32 : entry + passed - 1;
   }
   __syncwarp();
+  return cnt;
 }
 
-// Per-walk state of the walk kernels.
-struct Walk {
-  uint32_t x, v, j, s, slot, steps, cb, i;
-  unsigned long long wgt;
-  bool have;
-};
-
-// Start walk w.i of the chunk (residual entry idx0 + smap[w.i]).
-__device__ __forceinline__ void start_walk(const BatchDev& b, const unsigned long long* off,
-                                           unsigned long long cbeg, unsigned long long idx0,
-                                           const uint16_t* smap, const StartCache& sc, Walk& w) {
-  const uint32_t e = smap[w.i];
-  if (e < (uint32_t)kStartCache) {
-    w.slot = sc.slot[e];
-    w.v = sc.v[e];
-    w.s = sc.s[e];
-    w.wgt = sc.wgt[e];
-    w.j = (uint32_t)(cbeg + w.i - sc.off[e]);
-  } else {
-    unsigned long long idx = idx0 + e;
-    if (!FORA_IN_RANGE(b.err, idx, b.totals[0])) idx = idx0;
-    const unsigned long long entry = b.wr_entry[idx];
-    w.slot = (uint32_t)(entry >> 32);
-    w.v = (uint32_t)entry;
-    w.j = (uint32_t)(cbeg + w.i - off[idx]);
-    w.s = (uint32_t)b.sources[w.slot];
-    w.wgt = b.wr_weight[idx];
+// Adds the moves of the lanes with `due` to the counters of their sources (every lane of the
+// warp calls it): one atomic when they are of one source.  (One per lane queued 2 * 10^5
+// atomics on the counter of a single-source query, 0.1 ms.)
+__device__ __forceinline__ void flush_moves(const BatchDev& b, bool due, uint32_t& moves,
+                                            uint32_t slot) {
+  const uint32_t some = __ballot_sync(kFull, due && moves > 0);
+  if (some == 0) return;
+  const uint32_t first = __shfl_sync(kFull, slot, __ffs(some) - 1);
+  if (__all_sync(kFull, !due || moves == 0 || slot == first)) {
+    const uint32_t sum = __reduce_add_sync(kFull, due ? moves : 0u);  // each below 2^26
+    if ((threadIdx.x & 31) == 0) atomicAdd(&b.stats[first].walk_steps, (unsigned long long)sum);
+  } else if (due && moves) {
+    atomicAdd(&b.stats[slot].walk_steps, (unsigned long long)moves);
   }
-  w.x = w.v;
-  w.steps = 0;
-  w.cb = 0;
+  if (due) moves = 0;
 }
 
-// One iteration of a walk on its Philox block o (block index w.cb - 1): plain walks take
-// the words as stop test, move, stop test, move; zero-hop walks as move, stop test, move,
-// stop test (the first move of a zero-hop walk has no stop test).  A rejected neighbour try
-// (probability below d / 2^32) moves the walk off this block alignment: walk_rest then
-// finishes it word by word.  Returns true when the walk stopped (at w.x); sets w.have =
-// false and capped when it ran into the step cap.
-template <bool kZeroHop>
-__device__ __forceinline__ bool walk_block(const GraphDev& g, uint4 o, uint2 key, uint32_t t_alpha,
-                                           Walk& w, bool& capped, uint32_t* err) {
-  bool stop = false;
-  uint32_t rb = 0, d = 0;
-  unsigned long long m = 0;
-  int rejected = -1;  // word index of a try that walk_rest has to decide
-  bool bad = false;   // a failed index check (FORA_DEBUG builds): the walk is dropped
-  const uint32_t u0 = kZeroHop ? 0u : o.x, mv0 = kZeroHop ? o.x : o.y;
-  const uint32_t t1 = kZeroHop ? o.y : o.z, mv1 = kZeroHop ? o.z : o.w;
-  if (!kZeroHop) stop = u0 < t_alpha;
-  if (!stop) {
-    if (w.steps >= kMaxSteps) { capped = true; w.have = false; return false; }
-    if (fast_move(g, mv0, w.x, rb, d, m, err, bad)) {
-      ++w.steps;
-      stop = t1 < t_alpha;
-      if (!stop) {
-        if (w.steps >= kMaxSteps) { capped = true; w.have = false; return false; }
-        if (fast_move(g, mv1, w.x, rb, d, m, err, bad)) {
-          ++w.steps;
-          if (kZeroHop) stop = o.w < t_alpha;
-        } else {
-          rejected = kZeroHop ? 2 : 3;
+// The walk kernel.  The flat walk range goes to the warps in shares, in order, so the walks in
+// flight at any time are a narrow window of the source-major walk space and their end sums
+// stay in L2.  A warp goes through its share in windows of up to 32 residual entries, staged in
+// shared memory with the entry of each walk; each lane runs one walk and takes the window's
+// next unstarted walk when it ends (walk lengths are geometric: with a fixed share of walks per
+// lane a warp would wait for its longest share).  A walk's registers are its record x, number j
+// and state st = (block << 6 | place of its entry in the window); the entry's data stay in the
+// window, whose other half takes the next entries once no running walk needs it, so no lane
+// waits for the last walk of a window.
+//
+// One loop iteration consumes exactly one Philox block of every walk, so the ten rounds run on
+// full warps: a plain walk takes the words as stop test, move, stop test, move, a zero-hop
+// walk as move, stop test, move, stop test (its first move has no stop test).  A walk that
+// stops inside a block leaves the block's remaining words unused, as its stream definition
+// does; every block before took two moves, so a walk at block c has made 2 c moves.  A
+// neighbour try that Lemire's method may reject moves the walk off this block alignment:
+// walk_rest finishes it.
+//
+// Bounds: one gathered sector per move at 3.0e11 a second (one per clock and SM) and one
+// reduction per walk at 2.0e11; the latency of an iteration's two dependent gathers (the
+// slowest of 32 lanes' sectors) and instruction issue keep it above them.  Hence one record
+// per move, the tests and moves without branches, and little state in registers: 40, for 4
+// blocks of 384 threads.  Measured against a kernel with two lookups per move, an 18-register
+// walk state, one counter atomic per lane and source, and chunks whose last walks the warp
+// waited for: 256 sources of a 2^20-node R-MAT graph (0.35 of the rule's r_max) 119.3 -> 63.2
+// ms, 1.75e11 moves/s; 64 of 2^18 14.5 -> 8.1 ms; 100 of a 200003-node graph without hubs 13.9
+// -> 7.1 ms; one of 2^20 0.99 -> 0.63 ms.  Two walks per lane (54 registers) took 70.4 ms of
+// the first, 320 or 448 threads 75 and 68, shares of 1024, 2048 or 8192 walks 71, 65.5, 65.6.
+//
+// kTally: the end of walk g is summed into b.acc; otherwise it is stored in b.walk_dest[g]
+// (a walk index) or summed and counted (b.wcount).
+constexpr uint32_t kIdle = 0xFFFFFFFFu;
+template <int kMinBlocks, bool kZeroHop, bool kTally>
+__global__ void __launch_bounds__(kWalkThreads, kMinBlocks) k_walks(GraphDev g, BatchDev b) {
+  __shared__ WalkWindow windows[kWalkWarps];
+  __shared__ uint2 cls[kMaxWalkClasses + 1];
+  if (*b.err) return;
+  load_classes(g, cls);
+  __syncthreads();
+  const uint32_t lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const uint32_t t_alpha = b.alpha_threshold;
+  WalkWindow& win = windows[wid];
+  if (lane == 0) {
+    win.pos = win.stop = 0;
+    win.next = (unsigned long long)blockIdx.x * kWalkWarps + wid;
+  }
+  __syncwarp();
+
+  uint32_t half = 0;                // the half of the window whose walks are being started
+  uint32_t cnt = 0, next_walk = 0;  // next_walk of the window's cnt walks are started
+  bool more = true;
+  uint32_t x = 0, j = 0, st = kIdle;
+  uint32_t moves = 0, mslot = 0xFFFFFFFFu;  // moves of this lane's walks of slot mslot
+  for (;;) {
+    if (next_walk >= cnt && more) {  // warp-uniform
+      // does a running walk need the other half?
+      if (!__any_sync(kFull, st != kIdle && ((st >> 5) & 1u) != half)) {
+        half ^= 1u;
+        cnt = next_window(g, b, win, half);
+        next_walk = 0;
+        more = cnt > 0;
+      }
+    }
+    const uint32_t idle = __ballot_sync(kFull, st == kIdle);
+    const uint32_t i = next_walk + (uint32_t)__popc(idle & ((1u << lane) - 1u));
+    if (st == kIdle && i < cnt) {
+      const uint32_t e = half * 32 + win.map[i];
+      const uint4 w = win.walk[e];
+      x = w.z;
+      j = (uint32_t)win.pos - cnt + i - w.w;
+      st = e;
+    }
+    next_walk = min(next_walk + (uint32_t)__popc(idle), cnt);
+    if (!__any_sync(kFull, st != kIdle)) {
+      if (!more) break;
+      continue;
+    }
+
+    const uint4 w = win.walk[st & 63u];
+    const uint4 o = philox_rk(make_uint4(st >> 6, j, w.x, w.y), b.round_key);
+    static_assert(kMaxSteps % 2 == 0, "the cap is met before a block's first move");
+    uint32_t steps = 2u * (st >> 6);
+    bool have = st != kIdle;
+    bool go = have && (kZeroHop || o.x >= t_alpha);  // makes the block's first move
+    if (go && steps >= kMaxSteps) {
+      atomicOr(b.err, kErrWalkCap);
+      have = go = false;
+    }
+    if (!FORA_IN_RANGE(b.err, walk_id(g, x), g.n)) have = go = false;
+    uint2 r = node_row(g, cls, x, go);
+    unsigned long long m = (unsigned long long)(kZeroHop ? o.x : o.y) * r.y;
+    bool again = go && (uint32_t)m < r.y;  // a try that may be rejected
+    const bool one = go && !again;
+    uint32_t e = r.x + (uint32_t)(m >> 32);
+    if (one && FORA_IN_RANGE(b.err, e, g.m)) x = g.wcol[e];
+    go = one && (kZeroHop ? o.y : o.z) >= t_alpha;  // makes the second
+    r = node_row(g, cls, x, go);
+    m = (unsigned long long)(kZeroHop ? o.z : o.w) * r.y;
+    const bool retry = go && (uint32_t)m < r.y;
+    const bool two = go && !retry;
+    again |= retry;
+    e = r.x + (uint32_t)(m >> 32);
+    if (two && FORA_IN_RANGE(b.err, e, g.m)) x = g.wcol[e];
+    steps += (one ? 1u : 0u) + (two ? 1u : 0u);
+    bool stop = have && !(kZeroHop ? two && o.w >= t_alpha : two);
+    if (__any_sync(kFull, again)) {  // rare
+      if (again) {
+        const unsigned long long end =
+            walk_rest(g.wcol, g.wesc, cls, (uint32_t)g.ncls, (uint32_t)g.wbits,
+                      (one ? 4 : 2) - (kZeroHop ? 1 : 0), (st >> 6) + 1, j, win.walk[st & 63u].x,
+                      win.walk[st & 63u].y, b.round_key[0], t_alpha, x, steps);
+        x = (uint32_t)end;
+        steps = (uint32_t)(end >> 32);
+        stop = (steps & kCapped) == 0;
+        if (!stop) {
+          atomicOr(b.err, kErrWalkCap);
+          have = false;
         }
       }
-    } else {
-      rejected = kZeroHop ? 0 : 1;
     }
+    uint32_t slot = 0;
+    if (stop) {
+      // the walk stops at x (Section 2.1): its weight is added there (Alg. 2), or its end is
+      // recorded in a walk index (Section 3.3); its moves count for its source
+      const uint32_t id = walk_id(g, x);
+      const uint4 end = win.end[st & 63u];
+      slot = end.z;
+      const unsigned long long at = (unsigned long long)slot * b.ends + end_place(g, id);
+      if (!kTally && b.walk_dest) {
+        b.walk_dest[j + win.walk[st & 63u].w] = id;  // an index has fewer than 2^32 walks
+      } else if (FORA_IN_RANGE(b.err, id, g.n) && FORA_IN_RANGE(b.err, slot, b.nsrc)) {
+        if (!kTally) atomicAdd(&b.wcount[at], 1u);
+        atomicAdd(&b.acc[at], ((unsigned long long)end.y << 32) | end.x);
+      }
+    }
+    const bool due = stop && (slot != mslot || moves >= 1u << 25);
+    if (__any_sync(kFull, due)) flush_moves(b, due, moves, mslot);
+    if (stop) {
+      mslot = slot;
+      moves += steps;
+    }
+    st = have && !stop ? st + 64u : kIdle;
   }
-  if (bad) { w.have = false; return false; }
-  if (rejected >= 0) {  // rare: decide the try and finish the walk word by word
-    const uint32_t end = walk_rest(g, o, rejected + 1, w.cb, w.j, w.v, w.s, key, t_alpha, w.x,
-                                   rb, d, m, &w.steps);
-    if (end == kCapped) { capped = true; w.have = false; return false; }
-    w.x = end;
-    stop = true;
-  }
-  return stop;
+  flush_moves(b, true, moves, mslot);
 }
 
-// The end of this lane's walk w: tally it (or store it in a walk index) and count its
-// moves for its source.
-__device__ __forceinline__ void finish_walk(const BatchDev& b, unsigned long long n,
-                                            unsigned long long cbeg, const Walk& w,
-                                            unsigned long long& steps_here, uint32_t& cur_slot) {
-  // the walk stops at x (Section 2.1): count it and add its weight (Alg. 2), or record
-  // its end in a walk index (Section 3.3)
-  if (b.walk_dest) {
-    b.walk_dest[cbeg + w.i] = w.x;
-  } else if (FORA_IN_RANGE(b.err, w.x, n) && FORA_IN_RANGE(b.err, w.slot, b.nsrc)) {
-    Tally* t = b.tally + (unsigned long long)w.slot * n + w.x;
-    if (b.want_count) atomicAdd(&t->cnt, 1u);
-    atomicAdd(&t->acc, w.wgt);
-  }
-  if (w.slot != cur_slot) {
-    if (steps_here) atomicAdd(&b.stats[cur_slot].walk_steps, steps_here);
-    steps_here = 0;
-    cur_slot = w.slot;
-  }
-  steps_here += w.steps;
-}
-
-// The walk kernel.  The flat walk range is cut into chunks of kChunk walks and chunk c goes
-// to warp c mod (number of warps), so the walks in flight at any time are a narrow window
-// of the source-major walk space and their end tallies stay in L2.  Per chunk the warp maps
-// every walk to its residual entry (map_chunk) and stages the chunk's first entries
-// (fill_start_cache); each lane runs one walk and takes the chunk's next unstarted walk
-// when its walk ends (walk lengths are geometric: with a fixed share of walks per lane a
-// warp would wait for its longest share).  One loop iteration consumes exactly one Philox
-// block of a lane's walk (walk_block), so every lane with a walk evaluates its Philox block
-// in the same iteration and the ten rounds, most of a walk's arithmetic, run on full warps;
-// a walk that stops inside a block leaves the block's remaining words unused, as its stream
-// definition does.
-template <int kMinBlocks, bool kZeroHop>
-__global__ void __launch_bounds__(kWalkThreads, kMinBlocks) k_walks(GraphDev g, BatchDev b) {
-  __shared__ uint16_t smap[kWalkWarps][kChunk];
-  __shared__ StartCache scache[kWalkWarps];
-  if (*b.err) return;
-  const unsigned long long W = b.totals[1];
-  const unsigned long long nR = b.totals[0];
-  const uint32_t lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  const uint32_t lt_mask = (1u << lane) - 1u;
+// Edge records of the walks (GraphDev::wcol), one warp per node.
+__global__ void k_walk_records(GraphDev g, uint32_t* wcol) {
   const unsigned long long warp = ((unsigned long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const unsigned long long nwarps = ((unsigned long long)gridDim.x * blockDim.x) >> 5;
-  const unsigned long long nchunks = (W + kChunk - 1) / kChunk;
-  const unsigned long long* off = b.wr_offset;
-  const unsigned long long n = (unsigned long long)g.n;
-  const uint2 key = make_uint2((uint32_t)b.seed, (uint32_t)(b.seed >> 32));
-  const uint32_t t_alpha = b.alpha_threshold;
-  StartCache& sc = scache[wid];
-  unsigned long long steps_here = 0;  // moves of this lane's walks of source `cur_slot`
-  uint32_t cur_slot = 0xFFFFFFFFu;
-  bool capped = false;
-
-  for (unsigned long long c = warp; c < nchunks; c += nwarps) {
-    const unsigned long long cbeg = c * kChunk;
-    const uint32_t cnt = (uint32_t)min((unsigned long long)kChunk, W - cbeg);
-    const unsigned long long idx0 = warp_find_entry(off, nR, cbeg);
-    map_chunk(off, nR, cbeg, cnt, idx0, smap[wid]);
-    fill_start_cache(b, idx0, nR, sc);
-
-    uint32_t next_walk = 32;  // warp-uniform: the chunk's next unstarted walk
-    Walk w;
-    w.i = lane;
-    w.have = w.i < cnt;
-    if (w.have) start_walk(b, off, cbeg, idx0, smap[wid], sc, w);
-    for (;;) {
-      bool stop = false;
-      if (w.have) {
-        const uint4 o = philox_rk(make_uint4(w.cb, w.j, w.v, w.s), b.round_key);
-        ++w.cb;
-        stop = walk_block<kZeroHop>(g, o, key, t_alpha, w, capped, b.err);
-      }
-      const bool ended = w.have && stop;
-      const uint32_t ends = __ballot_sync(kFull, ended);
-      if (ended) {
-        finish_walk(b, n, cbeg, w, steps_here, cur_slot);
-        w.i = next_walk + (uint32_t)__popc(ends & lt_mask);
-        w.have = w.i < cnt;
-        if (w.have) start_walk(b, off, cbeg, idx0, smap[wid], sc, w);
-      }
-      next_walk += (uint32_t)__popc(ends);
-      if (!__any_sync(kFull, w.have)) break;
-    }
-    __syncwarp();
+  const uint32_t lane = threadIdx.x & 31;
+  for (unsigned long long v = warp; v < (unsigned long long)g.n; v += nwarps) {
+    const uint32_t rec = g.wid[v], c = rec >> g.wbits, id = walk_id(g, rec);
+    const uint32_t rb = g.row[v], d = g.row[v + 1] - rb;
+    const uint32_t to = c < (uint32_t)g.ncls ? g.wcls[c].x + id * d : g.wesc[id].x;
+    for (uint32_t k = lane; k < d; k += 32) wcol[to + k] = g.wid[g.col[rb + k]];
   }
-  if (capped) atomicOr(b.err, kErrWalkCap);
-  if (steps_here) atomicAdd(&b.stats[cur_slot].walk_steps, steps_here);
 }
 
 // FORA+ (Section 3.3): the residue whose walk count is the index's omega_max(v).
@@ -578,25 +599,25 @@ __global__ void k_index_residue(GraphDev g, double* r, double rmax) {
 
 // The walk phase served from a walk index: walk j of residual entry (slot, v) ends at
 // idx_dest[idx_off[v] + j] (the j-th stored walk from v) instead of being simulated.
-// Walks map to entries as in k_walks (chunks of kChunk, a shared-memory map per warp).
+// A warp maps a chunk of walks to their entries in a shared-memory map.
 // A walk past v's stored walks (a residue above the index's r_max) sets kErrIndexRange
 // and is skipped.
-__global__ void __launch_bounds__(kWalkThreads) k_walks_indexed(GraphDev g, BatchDev b,
+constexpr int kChunk = 1024;  // walks a warp maps to their entries at a time
+__global__ void __launch_bounds__(kIndexedThreads) k_walks_indexed(GraphDev g, BatchDev b,
                                                                 const unsigned long long* idx_off,
                                                                 const uint32_t* idx_dest) {
-  __shared__ uint16_t smap[kWalkWarps][kChunk];
+  __shared__ uint16_t smap[kIndexedThreads / 32][kChunk];
   if (*b.err) return;
   const unsigned long long W = b.totals[1];
   const unsigned long long nR = b.totals[0];
   const uint32_t lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const unsigned long long warp = ((unsigned long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const unsigned long long nwarps = ((unsigned long long)gridDim.x * blockDim.x) >> 5;
-  const unsigned long long nchunks = (W + kChunk - 1) / kChunk;
+  const uint32_t chunk = share_walks(W, nwarps, kChunk);
   const unsigned long long* off = b.wr_offset;
   bool out_of_range = false;
-  for (unsigned long long c = warp; c < nchunks; c += nwarps) {
-    const unsigned long long cbeg = c * kChunk;
-    const uint32_t cnt = (uint32_t)min((unsigned long long)kChunk, W - cbeg);
+  for (unsigned long long cbeg = warp * chunk; cbeg < W; cbeg += nwarps * chunk) {
+    const uint32_t cnt = (uint32_t)min((unsigned long long)chunk, W - cbeg);
     const unsigned long long idx0 = warp_find_entry(off, nR, cbeg);
     unsigned long long idxw = idx0;
     for (uint32_t rb = 0; rb < cnt; rb += 32) {
@@ -623,23 +644,28 @@ __global__ void __launch_bounds__(kWalkThreads) k_walks_indexed(GraphDev g, Batc
         out_of_range = true;
         continue;
       }
-      Tally* t = b.tally + (unsigned long long)slot * (unsigned long long)g.n + idx_dest[pos];
-      if (b.want_count) atomicAdd(&t->cnt, 1u);
-      atomicAdd(&t->acc, b.wr_weight[idx]);
+      const unsigned long long at =
+          (unsigned long long)slot * b.ends + end_place(g, idx_dest[pos]);
+      if (b.want_count) atomicAdd(&b.wcount[at], 1u);
+      atomicAdd(&b.acc[at], b.wr_weight[idx]);
     }
     __syncwarp();
   }
   if (out_of_range) atomicOr(b.err, kErrIndexRange);
 }
 
-__global__ void k_unpack_tally(const Tally* __restrict__ t, uint32_t* cnt,
-                               unsigned long long* acc, unsigned long long count) {
+__global__ void k_unpack_ends(GraphDev g, BatchDev b, uint32_t* cnt, unsigned long long* acc) {
+  const unsigned long long n = (unsigned long long)g.n;
   const unsigned long long stride = (unsigned long long)gridDim.x * blockDim.x;
-  for (unsigned long long i = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x; i < count;
-       i += stride) {
-    const Tally v = t[i];
-    if (cnt) cnt[i] = v.cnt;
-    if (acc) acc[i] = v.acc;
+  for (int slot = blockIdx.y; slot < b.nsrc; slot += gridDim.y) {
+    const unsigned long long g0 = (unsigned long long)slot * n;
+    for (unsigned long long v = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x; v < n;
+         v += stride) {
+      const unsigned long long at =
+          (unsigned long long)slot * b.ends + end_place(g, walk_id(g, g.wid[v]));
+      if (cnt) cnt[g0 + v] = b.wcount[at];
+      if (acc) acc[g0 + v] = b.acc[at];
+    }
   }
 }
 
@@ -667,22 +693,30 @@ cudaError_t launch_residuals(const GraphDev& g, const BatchDev& b, cudaStream_t 
   return cudaGetLastError();
 }
 
-// Walk kernel instances for 3, 4 or 5 resident blocks of 256 threads per SM (the register
-// budget the compiler gets); b.walk_blocks picks one (launch shape only).
-template <int kMinBlocks, bool kZeroHop>
+// Walk kernel instances for 3, 4 or 5 resident blocks per SM (the register budget the
+// compiler gets); b.walk_blocks picks one (launch shape only).
+template <int kMinBlocks, bool kZeroHop, bool kTally>
 cudaError_t launch_walks_t(const GraphDev& g, const BatchDev& b, int num_sms, cudaStream_t st) {
-  const int per_sm = resident_blocks((const void*)k_walks<kMinBlocks, kZeroHop>, kWalkThreads);
+  const int per_sm =
+      resident_blocks((const void*)k_walks<kMinBlocks, kZeroHop, kTally>, kWalkThreads);
   if (per_sm == 0) return cudaErrorInvalidConfiguration;
-  k_walks<kMinBlocks, kZeroHop><<<num_sms * per_sm, kWalkThreads, 0, st>>>(g, b);
+  k_walks<kMinBlocks, kZeroHop, kTally><<<num_sms * per_sm, kWalkThreads, 0, st>>>(g, b);
   return cudaGetLastError();
 }
 
 template <bool kZeroHop>
 cudaError_t launch_walks_zh(const GraphDev& g, const BatchDev& b, int num_sms, cudaStream_t st) {
+  const bool tally = !b.walk_dest && !b.want_count;
   switch (b.walk_blocks) {
-    case 3: return launch_walks_t<3, kZeroHop>(g, b, num_sms, st);
-    case 5: return launch_walks_t<5, kZeroHop>(g, b, num_sms, st);
-    default: return launch_walks_t<4, kZeroHop>(g, b, num_sms, st);
+    case 3:
+      return tally ? launch_walks_t<3, kZeroHop, true>(g, b, num_sms, st)
+                   : launch_walks_t<3, kZeroHop, false>(g, b, num_sms, st);
+    case 5:
+      return tally ? launch_walks_t<5, kZeroHop, true>(g, b, num_sms, st)
+                   : launch_walks_t<5, kZeroHop, false>(g, b, num_sms, st);
+    default:
+      return tally ? launch_walks_t<4, kZeroHop, true>(g, b, num_sms, st)
+                   : launch_walks_t<4, kZeroHop, false>(g, b, num_sms, st);
   }
 }
 
@@ -699,18 +733,23 @@ cudaError_t launch_index_residue(const GraphDev& g, double* r, double rmax, cuda
 cudaError_t launch_walks_indexed(const GraphDev& g, const BatchDev& b, int num_sms,
                                  const unsigned long long* idx_off, const uint32_t* idx_dest,
                                  cudaStream_t st) {
-  const int per_sm = resident_blocks((const void*)k_walks_indexed, kWalkThreads);
+  const int per_sm = resident_blocks((const void*)k_walks_indexed, kIndexedThreads);
   if (per_sm == 0) return cudaErrorInvalidConfiguration;
-  k_walks_indexed<<<num_sms * per_sm, kWalkThreads, 0, st>>>(g, b, idx_off, idx_dest);
+  k_walks_indexed<<<num_sms * per_sm, kIndexedThreads, 0, st>>>(g, b, idx_off, idx_dest);
   return cudaGetLastError();
 }
 
-cudaError_t launch_unpack_tally(const Tally* t, uint32_t* cnt, unsigned long long* acc,
-                                uint64_t count, int num_sms, cudaStream_t st) {
-  uint64_t blocks = (count + 255) / 256;
-  if (blocks > (uint64_t)num_sms * 32) blocks = (uint64_t)num_sms * 32;
-  if (blocks == 0) return cudaSuccess;
-  k_unpack_tally<<<(unsigned)blocks, 256, 0, st>>>(t, cnt, acc, count);
+cudaError_t launch_unpack_ends(const GraphDev& g, const BatchDev& b, uint32_t* cnt,
+                               unsigned long long* acc, int num_sms, cudaStream_t st) {
+  uint64_t bx = ((uint64_t)g.n + 255) / 256;
+  const uint64_t most = ((uint64_t)num_sms * 32 + b.nsrc - 1) / b.nsrc;
+  if (bx > most) bx = most;
+  k_unpack_ends<<<dim3((unsigned)bx, (unsigned)b.nsrc), 256, 0, st>>>(g, b, cnt, acc);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_walk_records(const GraphDev& g, uint32_t* wcol, int num_sms, cudaStream_t st) {
+  k_walk_records<<<num_sms * 8, 256, 0, st>>>(g, wcol);
   return cudaGetLastError();
 }
 
