@@ -336,11 +336,8 @@ def run_fora(args):
     def collect(step, st, ms):
         bounds = part_bounds(len(st))
         rounds = max(s.push_rounds for s in st)
-        for lo, hi in bounds:
-            r_k = max(s.push_rounds for s in st[lo:hi])
-            # push: the seed, then (rounds + 1) passes of the loop body (spread, take,
-            # advance); residuals 4, walks 1, estimate 1, top-k select 19
-            counters["launches"] += 1 + 3 * (r_k + 1) + 4 + 1 + 1 + 19
+        # a part: push 1 (all rounds), residuals 3, walks 1, estimate 1, top-k select 19
+        counters["launches"] += len(bounds) * (1 + 3 + 1 + 1 + 19)
         if model is not None:
             counters["launches"] += 3  # features, forward, r_max (whole batch)
         # kernel time of each phase, summed over the parts (parts overlap in time)

@@ -432,18 +432,16 @@ int fora_threshold_debug(const double *r, const double *rmax, const uint32_t *d,
  * (grouped by source) through this many interleaved segments, so the warps in flight cover about that
  * many sources at once (wider spreads reductions on shared hub targets over more
  * addresses; narrower keeps the residue arrays in flight smaller).  "spread_hot" (0 or 1,
- * default 1): in the heavy rounds of the push a block first sums, in shared memory, its
- * pushes to the graph's hot nodes (the up to 128 nodes of highest in-degree, each >= 64)
- * over a stretch of up to 32 frontier groups of one source, then adds each sum to the
- * residue with one atomic; 0 adds every push with its own atomic (results differ only by
+ * default 1): the push adds what it pushes to the graph's hot nodes (the up to 128 nodes of
+ * highest in-degree, each >= 64) to one of several copies of their residues, which the next
+ * round's scan adds up; 0 adds it to the residue itself (results differ only by
  * the order of FP64 additions).  The tuning read-back also answers "hot_nodes", the
  * number of hot nodes of the graph (0: spread_hot has no effect).  "walk_blocks" (3, 4
  * or 5, default 4): resident walk blocks (of 384 threads) per SM, traded against registers
  * per thread.
  * "push_host_loop" (0 or 1, default 0): 1 launches the push rounds from a host loop with
- * one device-to-host read per round, instead of the CUDA graph whose conditional while-node
- * runs them on the device; the kernels are the same (a profiler that cannot look inside
- * conditional graph nodes sees each of them).  "pipeline" (1..4, default 1): a batched
+ * one device-to-host read per round, instead of one cooperative launch that runs them all
+ * on the device; the steps are the same (a profiler sees each of them on its own).  "pipeline" (1..4, default 1): a batched
  * query of B >= 64 sources runs as that many parts (at least 32 sources each), each on
  * its own workspace, stream and host thread, part k's push starting when part k-1's push
  * has finished, so one part's walk phase runs beside the next part's push; the call's

@@ -10,6 +10,7 @@
 #include <cstdio>
 #include <cstring>
 #include <map>
+#include <memory>
 #include <mutex>
 #include <string>
 #include <thread>
@@ -118,9 +119,9 @@ fora::WorkspaceSizes fora::workspace_sizes(int64_t n, uint64_t hub_chunks, int n
   z.stats = S * sizeof(SlotStats);
   z.stopped = S * sizeof(uint32_t);
   z.light = S;
-  z.tile_dirty = S * (((size_t)n + kTakeTile - 1) / kTakeTile);
+  z.tile_dirty = S * (((size_t)n + 1023) / 1024);
   z.last_edges = S * sizeof(unsigned long long);
-  z.blk = 2 * (size_t)kMaxResidualGrid * sizeof(unsigned long long);
+  z.blk = 2 * (size_t)kUnitPairs * sizeof(unsigned long long);
   z.topk = topk_scratch_bytes(nsrc);
   z.feat = S * FORA_NUM_FEATURES * sizeof(float);
   z.pred = S * sizeof(float);
@@ -165,11 +166,10 @@ int ensure_workspace(fora_graph* g, Workspace* w, int nsrc) {
   if (nsrc <= w->cap) return FORA_OK;
   w->release();
   const WorkspaceSizes z = workspace_sizes(g->n, g->hub_chunks, nsrc);
-  // hub items hold a queue index in their upper 64 - kHubChunkBits bits
-  if (z.N >= (1ull << (64 - kHubChunkBits)))
+  // a bound that no device's memory reaches
+  if (z.N >= (1ull << 40))
     return fail(FORA_ERR_BAD_ARG, "%d sources x %lld nodes exceed the queue index range", nsrc,
                 (long long)g->n);
-  w->residual_grid = std::min(g->num_sms * 8, kMaxResidualGrid);
   CUDA_TRY(dalloc(&w->r, z.r));
   CUDA_TRY(dalloc(&w->res, z.res));
   CUDA_TRY(dalloc(&w->tally, z.tally));
@@ -184,14 +184,15 @@ int ensure_workspace(fora_graph* g, Workspace* w, int nsrc) {
   CUDA_TRY(dalloc(&w->slot_cnt, z.slot_cnt));
   CUDA_TRY(dalloc(&w->pre, z.pre));
   CUDA_TRY(dalloc(&w->ps, z.ps));
-  if (!w->capture_stream) CUDA_TRY(cudaStreamCreateWithFlags(&w->capture_stream, cudaStreamNonBlocking));
+  CUDA_TRY(cudaMemset(w->ps, 0, z.ps));
+  CUDA_TRY(cudaMemset(w->work, 0, z.work));  // the push's barrier starts at 0
   CUDA_TRY(dalloc(&w->err, z.err));
   CUDA_TRY(dalloc(&w->sources, z.sources));
   CUDA_TRY(dalloc(&w->rmax, z.rmax));
   CUDA_TRY(dalloc(&w->stats, z.stats));
   CUDA_TRY(dalloc(&w->stopped, z.stopped));
   CUDA_TRY(dalloc(&w->light, z.light));
-  CUDA_TRY(dalloc(&w->tile_dirty, z.tile_dirty));
+  CUDA_TRY(dalloc(&w->tile_dirty, (z.tile_dirty + 3) / 4 * 4));  // marked by 4-byte atomics
   CUDA_TRY(dalloc(&w->last_edges, z.last_edges));
   CUDA_TRY(dalloc(&w->blk, z.blk));
   CUDA_TRY(dalloc(&w->topk_scratch, z.topk));
@@ -209,7 +210,6 @@ int ensure_workspace(fora_graph* g, Workspace* w, int nsrc) {
   for (int i = 0; i < 5; ++i)
     if (!w->ev[i]) CUDA_TRY(cudaEventCreate(&w->ev[i]));
   w->cap = nsrc;
-  ++w->generation;
   return FORA_OK;
 }
 
@@ -263,59 +263,101 @@ int resolve(const fora_graph* g, const fora_params* p, Resolved* out) {
 
 namespace {
 
-// The push rounds as a CUDA graph: one conditional while-node whose body is a round
-// (spread, detect, scan, emit, advance); the advance kernel sets the loop condition.
-// The instantiated graph is kept in the workspace and rebuilt when the workspace, the
-// number of sources, alpha or the launch shape change.
-int push_loop_graph(fora_graph* g, Workspace* w, const GraphDev& gd, const BatchDev& b) {
-  PushGraphKey key;
-  key.generation = w->generation;
-  key.nsrc = b.nsrc;
-  key.alpha = b.alpha;
-  key.spread_width = b.spread_width;
-  key.spread_hot = b.spread_hot;
-  key.max_rounds = b.max_rounds;
-  key.balance = b.balance;
-  key.bal[0] = b.bal_scale;
-  key.bal[1] = b.cost_edge;
-  key.bal[2] = b.cost_push;
-  key.bal[3] = b.cost_walk;
-  if (w->push_exec && key == w->push_key) return FORA_OK;
-  if (w->push_exec) {
-    cudaGraphExecDestroy(w->push_exec);
-    w->push_exec = nullptr;
+// Pushes of one device never run side by side: a push fills the device with blocks that wait
+// for each other, so each waits for the one launched before it (on whatever stream).
+struct PushGate {
+  std::mutex mu;
+  cudaEvent_t last = nullptr;
+};
+std::mutex g_gates_mu;
+std::map<int, std::unique_ptr<PushGate>> g_gates;
+
+cudaError_t launch_push_gated(int device, const GraphDev& gd, const BatchDev& b, int num_sms,
+                              cudaStream_t stream) {
+  PushGate* gate;
+  {
+    std::lock_guard<std::mutex> lock(g_gates_mu);
+    auto& p = g_gates[device];
+    if (!p) p = std::make_unique<PushGate>();
+    gate = p.get();
   }
-  cudaGraph_t graph = nullptr;
-  CUDA_TRY(cudaGraphCreate(&graph, 0));
-  cudaGraphConditionalHandle loop;
-  cudaGraphNode_t node;
-  cudaGraphNodeParams np{};
-  cudaGraph_t captured = nullptr;
-  cudaError_t e = cudaGraphConditionalHandleCreate(&loop, graph, 1, cudaGraphCondAssignDefault);
-  if (e == cudaSuccess) {
-    np.type = cudaGraphNodeTypeConditional;
-    np.conditional.handle = loop;
-    np.conditional.type = cudaGraphCondTypeWhile;
-    np.conditional.size = 1;
-    e = cudaGraphAddNode(&node, graph, nullptr, nullptr, 0, &np);
-  }
-  if (e == cudaSuccess)
-    e = cudaStreamBeginCaptureToGraph(w->capture_stream, np.conditional.phGraph_out[0], nullptr,
-                                      nullptr, 0, cudaStreamCaptureModeRelaxed);
-  if (e == cudaSuccess) {
-    const cudaError_t le = launch_push_body(gd, b, g->num_sms, loop, true, w->capture_stream);
-    e = cudaStreamEndCapture(w->capture_stream, &captured);
-    if (le != cudaSuccess) e = le;
-  }
-  if (e == cudaSuccess) e = cudaGraphInstantiate(&w->push_exec, graph, 0);
-  cudaGraphDestroy(graph);
-  if (e != cudaSuccess) {
-    w->push_exec = nullptr;
-    return fail(FORA_ERR_CUDA, "push loop graph: %s", cudaGetErrorString(e));
-  }
-  w->push_key = key;
-  return FORA_OK;
+  std::lock_guard<std::mutex> lock(gate->mu);
+  cudaError_t e = cudaSuccess;
+  if (!gate->last)
+    e = cudaEventCreateWithFlags(&gate->last, cudaEventDisableTiming);
+  else
+    e = cudaStreamWaitEvent(stream, gate->last, 0);
+  if (e == cudaSuccess) e = launch_push(gd, b, num_sms, stream);
+  if (e == cudaSuccess) e = cudaEventRecord(gate->last, stream);
+  return e;
 }
+
+// The parts of a BatchDev that follow from the workspace, the graph and the number of slots:
+// `lay` of them in the layout, in groups of gw.
+void lay_out(const fora_graph* g, const Workspace* w, int lay, int gw, BatchDev* b) {
+  const size_t n = (size_t)g->n, cells = (size_t)lay * n;
+  b->lay = lay;
+  b->gw = gw;
+  b->lgrp = (lay + gw - 1) / gw;
+  b->tiles = (uint32_t)((n + kTakeUnit / gw - 1) / (kTakeUnit / gw));
+  b->ends = end_places(g->n, g->wbits);
+  b->r = w->r;
+  b->res = w->res;
+  b->acc = w->tally;
+  b->wcount = reinterpret_cast<uint32_t*>(w->tally + (size_t)lay * b->ends);
+  b->q = reinterpret_cast<uint2*>(w->q[0]);
+  b->fa = w->fa;
+  b->hub = reinterpret_cast<uint2*>(w->hub[0]);
+  b->hub_len = reinterpret_cast<uint32_t*>(w->hub[1]);
+  b->hub_stride = g->hub_chunks;
+  b->slot_cnt = w->slot_cnt;
+  b->cnt_stride = w->cap;
+  b->gpre = w->pre;
+  b->hpre = w->pre + (w->cap + 1);
+  b->alist = w->alist;
+  b->work = w->work;
+  b->ps = w->ps;
+  b->ctl = reinterpret_cast<PushCtl*>(w->small);
+  b->meet = reinterpret_cast<uint32_t*>(w->work + 8);  // and work + 24
+  // the second queue buffer: the list of tiles, then the copies of the hot nodes' residues
+  b->tlist = reinterpret_cast<uint32_t*>(w->q[1]);
+  const size_t list = ((size_t)b->lgrp * b->tiles * sizeof(uint32_t) + 15) / 16 * 2;  // doubles
+  b->hotr = reinterpret_cast<double*>(w->q[1]) + list;
+  const size_t one = (size_t)b->lgrp * gw * g->nhot;  // doubles of one copy
+  b->hot_copies = one > 0 && cells > list ? (int)std::min<size_t>(kHotCopies, (cells - list) / one) : 0;
+  b->totals = w->small + 4;
+  b->walk_next = w->small + 6;
+  b->sources = w->sources;
+  b->rmax = w->rmax;
+  b->stats = w->stats;
+  b->err = w->err;
+  b->wr_entry = w->q[0];
+  b->wr_offset = w->q[1];
+  b->wr_weight = reinterpret_cast<unsigned long long*>(w->fa);
+  b->theta = w->rmax;
+  b->stopped = w->stopped;
+  b->light = w->light;
+  b->dirty = reinterpret_cast<uint32_t*>(w->tile_dirty);
+  b->last_edges = w->last_edges;
+  // a frontier whose spread touches at most half of a group's units
+  b->light_edges = b->tiles / 2;
+}
+
+// ... and from the number of sources.
+void set_sources(const fora_graph* g, const Workspace* w, int nsrc, BatchDev* b) {
+  b->nsrc = nsrc;
+  b->ngrp = (nsrc + b->gw - 1) / b->gw;
+  b->units = residual_units(g->n, nsrc);
+  const size_t pairs = (size_t)nsrc * b->units;
+  b->unit_cnt = pairs <= (size_t)kUnitPairs ? w->blk
+                                            : reinterpret_cast<unsigned long long*>(w->topk_scratch);
+  b->unit_walks = b->unit_cnt + pairs;
+}
+
+// Sources side by side in the push: four from three sources on (of the spread's reductions a
+// group of four needs one sector where its sources push from the same nodes, and a group that
+// is not full costs only idle lanes), one below.
+int group_width(int nsrc, bool balance) { return nsrc >= 3 && !balance ? 4 : 1; }
 
 }  // namespace
 
@@ -376,7 +418,6 @@ int fora::run_batch_ws(fora_graph* g, Workspace* w, const fora_params* p,
   CUDA_TRY(cudaSetDevice(g->device));
   rc = ensure_workspace(g, w, join ? join->cap : nsrc);
   if (rc) return rc;
-  size_t N = (size_t)nsrc * (size_t)g->n;
   for (int i = 0; i < nsrc; ++i) {
     w->h_sources[i] = sources[i];
     w->h_rmax[i] = bal ? 1.0 : rsrc.host ? rsrc.host[i] : rp.rmax;
@@ -390,55 +431,24 @@ int fora::run_batch_ws(fora_graph* g, Workspace* w, const fora_params* p,
     CUDA_TRY(cudaMemcpyAsync(w->rmax, rsrc.device, nsrc * sizeof(double), cudaMemcpyDeviceToDevice, stream));
   else
     CUDA_TRY(cudaMemcpyAsync(w->rmax, w->h_rmax, nsrc * sizeof(double), cudaMemcpyHostToDevice, stream));
-  const bool want_count = dbg && dbg->count;
-  const size_t ends = (size_t)end_places(g->n, g->wbits);
-  uint32_t* wcount = reinterpret_cast<uint32_t*>(w->tally + (size_t)nsrc * ends);
-  CUDA_TRY(cudaMemsetAsync(w->tally, 0, (size_t)nsrc * ends * sizeof(unsigned long long), stream));
-  if (want_count)
-    CUDA_TRY(cudaMemsetAsync(wcount, 0, (size_t)nsrc * ends * sizeof(uint32_t), stream));
-  CUDA_TRY(cudaMemsetAsync(w->small, 0, 8 * sizeof(unsigned long long), stream));
-  CUDA_TRY(cudaMemsetAsync(w->err, 0, sizeof(uint32_t), stream));
-  CUDA_TRY(cudaMemsetAsync(w->stats, 0, nsrc * sizeof(SlotStats), stream));
-
   const GraphDev gd = g->dev();
   const size_t n64 = (size_t)g->n;
   BatchDev b{};
-  b.nsrc = nsrc;
+  lay_out(g, w, join ? join->cap : nsrc, group_width(nsrc, bal != nullptr), &b);
+  set_sources(g, w, nsrc, &b);
   b.alpha = rp.alpha;
   b.walk_scale = rp.walk_scale;
   b.alpha_threshold = rp.alpha_threshold;
   b.seed = p->seed;
   set_round_keys(&b, p->seed);
   b.zero_hop = (p->flags & FORA_ZERO_HOP) != 0;
-  b.want_count = want_count;
-  b.r = w->r; b.res = w->res; b.acc = w->tally; b.wcount = wcount; b.ends = ends;
-  b.q[0] = w->q[0]; b.q[1] = w->q[1]; b.fa = w->fa;
-  b.hub[0] = w->hub[0]; b.hub[1] = w->hub[1];
-  b.hub_stride = g->hub_chunks;
-  b.slot_cnt = w->slot_cnt;
-  b.cnt_stride = w->cap;
-  b.gpre = w->pre;
-  b.hpre = w->pre + (w->cap + 1);
-  b.alist = w->alist;
-  b.work = w->work;
-  b.ps = w->ps;
-  b.totals = w->small + 4;
-  b.walk_next = w->small + 6;
-  b.sources = w->sources; b.rmax = w->rmax; b.stats = w->stats; b.err = w->err;
-  b.wr_entry = w->q[0];
-  b.wr_offset = w->q[1];
-  b.wr_weight = reinterpret_cast<unsigned long long*>(w->fa);
-  b.blk_cnt = w->blk;
-  b.blk_walks = w->blk + w->residual_grid;
-  b.residual_grid = w->residual_grid;
-  b.theta = w->rmax;
-  b.stopped = w->stopped;
-  b.light = w->light;
-  b.tile_dirty = w->tile_dirty;
-  b.last_edges = w->last_edges;
-  b.tiles = ((unsigned long long)g->n + kTakeTile - 1) / kTakeTile;
-  // a frontier whose spread touches at most about half of a source's tiles
-  b.light_edges = b.tiles / 2;
+  b.want_count = dbg && dbg->count;
+  CUDA_TRY(cudaMemsetAsync(w->tally, 0, (size_t)nsrc * b.ends * sizeof(unsigned long long), stream));
+  if (b.want_count)
+    CUDA_TRY(cudaMemsetAsync(b.wcount, 0, (size_t)nsrc * b.ends * sizeof(uint32_t), stream));
+  CUDA_TRY(cudaMemsetAsync(w->small, 0, 8 * sizeof(unsigned long long), stream));
+  CUDA_TRY(cudaMemsetAsync(w->err, 0, sizeof(uint32_t), stream));
+  CUDA_TRY(cudaMemsetAsync(w->stats, 0, nsrc * sizeof(SlotStats), stream));
   if (bal) {
     b.balance = 1;
     b.bal_scale = b.zero_hop ? (1.0 - rp.alpha) * rp.walk_scale : rp.walk_scale;
@@ -450,7 +460,7 @@ int fora::run_batch_ws(fora_graph* g, Workspace* w, const fora_params* p,
   {
     std::lock_guard<std::mutex> tlock(g->mu);
     b.spread_width = g->tune.spread_width;
-    b.spread_hot = (g->tune.spread_hot != 0 && g->nhot > 0) ? 1 : 0;
+    if (g->tune.spread_hot == 0) b.hot_copies = 0;
     b.walk_blocks = g->tune.walk_blocks;
     b.max_rounds = g->tune.max_push_rounds;
     host_loop = g->tune.push_host_loop != 0;
@@ -466,21 +476,15 @@ int fora::run_batch_ws(fora_graph* g, Workspace* w, const fora_params* p,
 
   // ---- push (Alg. 1) ----
   if (given) {
-    CUDA_TRY(cudaMemcpyAsync(w->res, dbg->reserve, N * sizeof(double), cudaMemcpyDeviceToDevice, stream));
-    CUDA_TRY(cudaMemcpyAsync(w->r, dbg->residue, N * sizeof(double), cudaMemcpyDeviceToDevice, stream));
+    CUDA_TRY(launch_regroup(w->res, dbg->reserve, b, g->n, false, g->num_sms, stream));
+    CUDA_TRY(launch_regroup(w->r, dbg->residue, b, g->n, false, g->num_sms, stream));
   } else {
-    CUDA_TRY(cudaMemsetAsync(w->r, 0, N * sizeof(double), stream));
-    CUDA_TRY(cudaMemsetAsync(w->res, 0, N * sizeof(double), stream));
-    CUDA_TRY(cudaMemsetAsync(w->work, 0, 32 * sizeof(unsigned long long), stream));
-    CUDA_TRY(cudaMemsetAsync(w->slot_cnt, 0, 4 * (size_t)w->cap * sizeof(uint32_t), stream));
-    CUDA_TRY(cudaMemsetAsync(w->tile_dirty, 0, (size_t)w->cap * b.tiles, stream));
-    CUDA_TRY(cudaMemsetAsync(w->last_edges, 0, (size_t)w->cap * sizeof(unsigned long long), stream));
-    CUDA_TRY(launch_push_seed(gd, b, stream));
     if (join) {
       // rounds from a host loop; after each round further sources may join as new slots
+      CUDA_TRY(launch_push_start(gd, b, g->num_sms, stream));
       uint32_t go = 1;
       while (go) {
-        CUDA_TRY(launch_push_body(gd, b, g->num_sms, 0, false, stream));
+        CUDA_TRY(launch_push_round(gd, b, g->num_sms, stream));
         CUDA_TRY(cudaMemcpyAsync(w->go_host, &w->ps->go, sizeof(uint32_t), cudaMemcpyDeviceToHost,
                                  stream));
         CUDA_TRY(cudaStreamSynchronize(stream));
@@ -488,46 +492,49 @@ int fora::run_batch_ws(fora_graph* g, Workspace* w, const fora_params* p,
         const int room = join->cap - b.nsrc;
         const int k = room > 0 ? join->poll(w->h_sources + b.nsrc, room) : 0;
         if (k <= 0) continue;
-        const int first = b.nsrc;
+        const int first = b.nsrc, grp0 = b.ngrp;
         for (int i = first; i < first + k; ++i) w->h_rmax[i] = rp.rmax;
         CUDA_TRY(cudaMemcpyAsync(w->sources + first, w->h_sources + first, k * sizeof(int32_t),
                                  cudaMemcpyHostToDevice, stream));
         CUDA_TRY(cudaMemcpyAsync(w->rmax + first, w->h_rmax + first, k * sizeof(double),
                                  cudaMemcpyHostToDevice, stream));
-        const size_t off = (size_t)first * n64, len = (size_t)k * n64;
-        CUDA_TRY(cudaMemsetAsync(w->r + off, 0, len * sizeof(double), stream));
-        CUDA_TRY(cudaMemsetAsync(w->res + off, 0, len * sizeof(double), stream));
-        CUDA_TRY(cudaMemsetAsync(w->tally + (size_t)first * ends, 0,
-                                 (size_t)k * ends * sizeof(unsigned long long), stream));
+        CUDA_TRY(cudaMemsetAsync(w->tally + (size_t)first * b.ends, 0,
+                                 (size_t)k * b.ends * sizeof(unsigned long long), stream));
         CUDA_TRY(cudaMemsetAsync(w->stats + first, 0, k * sizeof(SlotStats), stream));
-        b.nsrc = first + k;
+        set_sources(g, w, first + k, &b);
+        // the places of groups that are new (those of the others were zeroed with the batch's)
+        const size_t off = (size_t)grp0 * b.gw * n64;
+        const size_t end = (size_t)std::min(b.ngrp * b.gw, b.lay) * n64;
+        if (end > off) {
+          CUDA_TRY(cudaMemsetAsync(w->r + off, 0, (end - off) * sizeof(double), stream));
+          CUDA_TRY(cudaMemsetAsync(w->res + off, 0, (end - off) * sizeof(double), stream));
+        }
         CUDA_TRY(launch_push_join(gd, b, first, k, stream));
         go = 1;
       }
+      CUDA_TRY(launch_push_finish(gd, b, g->num_sms, stream));
       nsrc = b.nsrc;
-      N = (size_t)nsrc * n64;
       if (join->nsrc_final) *join->nsrc_final = nsrc;
     } else if (host_loop) {
-      // the same round kernels launched one round at a time from the host (for profilers
-      // that cannot look inside conditional graph nodes); one host round trip per round
+      // the same phases launched one round at a time from the host (for profilers, which then
+      // see each of them); one host round trip per round
+      CUDA_TRY(launch_push_start(gd, b, g->num_sms, stream));
       uint32_t go = 1;
       while (go) {
-        CUDA_TRY(launch_push_body(gd, b, g->num_sms, 0, false, stream));
+        CUDA_TRY(launch_push_round(gd, b, g->num_sms, stream));
         CUDA_TRY(cudaMemcpyAsync(w->go_host, &w->ps->go, sizeof(uint32_t), cudaMemcpyDeviceToHost,
                                  stream));
         CUDA_TRY(cudaStreamSynchronize(stream));
         go = *w->go_host;
       }
+      CUDA_TRY(launch_push_finish(gd, b, g->num_sms, stream));
     } else {
-      // the rounds run as a device-side while loop (no host round trip per round)
-      rc = push_loop_graph(g, w, gd, b);
-      if (rc) return rc;
-      CUDA_TRY(cudaGraphLaunch(w->push_exec, stream));
+      CUDA_TRY(launch_push_gated(g->device, gd, b, g->num_sms, stream));
     }
     if (dbg && dbg->reserve)
-      CUDA_TRY(cudaMemcpyAsync(dbg->reserve, w->res, N * sizeof(double), cudaMemcpyDeviceToDevice, stream));
+      CUDA_TRY(launch_regroup(w->res, dbg->reserve, b, g->n, true, g->num_sms, stream));
     if (dbg && dbg->residue)
-      CUDA_TRY(cudaMemcpyAsync(dbg->residue, w->r, N * sizeof(double), cudaMemcpyDeviceToDevice, stream));
+      CUDA_TRY(launch_regroup(w->r, dbg->residue, b, g->n, true, g->num_sms, stream));
   }
   if (timed) CUDA_TRY(cudaEventRecord(w->ev[1], stream));
   if (hook && hook->after) {
@@ -548,14 +555,16 @@ int fora::run_batch_ws(fora_graph* g, Workspace* w, const fora_params* p,
     CUDA_TRY(launch_unpack_ends(gd, b, dbg->count, reinterpret_cast<unsigned long long*>(dbg->acc),
                                 g->num_sms, stream));
 
-  // ---- estimate and top-k (the residue array becomes the estimate) ----
+  // ---- estimate (into the increments' array, by source) and top-k ----
   nvtx_phase.next("fora: estimate and top-k");
-  CUDA_TRY(launch_estimate(gd, b, w->r, stream));
+  double* est = w->fa;
+  CUDA_TRY(launch_estimate(gd, b, est, stream));
   if (dbg && dbg->estimate)
-    CUDA_TRY(cudaMemcpyAsync(dbg->estimate, w->r, N * sizeof(double), cudaMemcpyDeviceToDevice, stream));
+    CUDA_TRY(cudaMemcpyAsync(dbg->estimate, est, (size_t)nsrc * n64 * sizeof(double),
+                             cudaMemcpyDeviceToDevice, stream));
   int32_t* ids_dev = out_dev ? out_ids : w->out_ids;
   double* vals_dev = out_dev ? out_vals : w->out_vals;
-  CUDA_TRY(launch_topk(w->r, g->n, nsrc, p->k, ids_dev, vals_dev,
+  CUDA_TRY(launch_topk(est, g->n, nsrc, p->k, ids_dev, vals_dev,
                        topk_scratch_carve(w->topk_scratch, nsrc), g->num_sms, stream));
   if (timed) CUDA_TRY(cudaEventRecord(w->ev[4], stream));
   if (!out_dev && p->k > 0) {
@@ -568,6 +577,7 @@ int fora::run_batch_ws(fora_graph* g, Workspace* w, const fora_params* p,
   if (st && (rsrc.device || bal))  // the thresholds used were set on the device
     CUDA_TRY(cudaMemcpyAsync(w->h_rmax, w->rmax, nsrc * sizeof(double), cudaMemcpyDeviceToHost, stream));
   CUDA_TRY(cudaStreamSynchronize(stream));
+  if (*w->h_err & kErrBarrier) return fail(FORA_ERR_CUDA, "the push's blocks did not all run");
   if (*w->h_err & kErrPushNotConverged)
     return fail(FORA_ERR_PUSH_NOT_CONVERGED, "push did not converge in %u rounds", b.max_rounds);
   if (*w->h_err & kErrWalkOverflow) return fail(FORA_ERR_WALK_OVERFLOW, "a source needs 2^32 or more walks");
@@ -841,10 +851,13 @@ int fora_graph_create(int64_t n, const int64_t* row_ptr, const int32_t* col, uin
   if (e == cudaSuccess) e = cudaMemcpy(g->col, col, (size_t)m * sizeof(int32_t), cudaMemcpyHostToDevice);
   if (e == cudaSuccess) {  // reciprocal out-degrees (every d >= 1 here)
     std::vector<double> invd((size_t)n);
-    for (int64_t v = 0; v < n; ++v) invd[v] = 1.0 / (double)(row[v + 1] - row[v]);
-    e = dalloc(&g->invd, (size_t)n * sizeof(double));
-    if (e == cudaSuccess)
-      e = cudaMemcpy(g->invd, invd.data(), (size_t)n * sizeof(double), cudaMemcpyHostToDevice);
+    std::vector<float> fdeg((size_t)n);
+    for (int64_t v = 0; v < n; ++v) {
+      invd[v] = 1.0 / (double)(row[v + 1] - row[v]);
+      fdeg[v] = (float)(row[v + 1] - row[v]);
+    }
+    e = upload(&g->invd, invd);
+    if (e == cudaSuccess) e = upload(&g->fdeg, fdeg);
   }
   if (e == cudaSuccess) {  // the walks' numbering and edge records
     const WalkNumbering wn = walk_numbering(n, row.data());
@@ -866,6 +879,12 @@ int fora_graph_create(int64_t n, const int64_t* row_ptr, const int32_t* col, uin
       std::vector<uint32_t> sc((size_t)m);
       for (int64_t k = 0; k < m; ++k) sc[k] = code[(size_t)col[k]];
       e = dalloc(&g->scol, (size_t)m * sizeof(uint32_t));
+      std::vector<uint8_t> first(((size_t)n + kHotSpan - 1) / kHotSpan + 1);
+      for (size_t t = 0, h = 0; t < first.size(); ++t) {
+        while (h < hot.size() && hot[h] < t * kHotSpan) ++h;
+        first[t] = (uint8_t)h;
+      }
+      if (e == cudaSuccess) e = upload(&g->hot_first, first);
       if (e == cudaSuccess) e = dalloc(&g->hot_node, hot.size() * sizeof(uint32_t));
       if (e == cudaSuccess)
         e = cudaMemcpy(g->scol, sc.data(), (size_t)m * sizeof(uint32_t), cudaMemcpyHostToDevice);
@@ -918,12 +937,14 @@ void fora_graph_destroy(fora_graph* g) {
     dfree(g->col);
     dfree(g->indeg);
     dfree(g->invd);
+    dfree(g->fdeg);
     dfree(g->wcol);
     dfree(g->wid);
     dfree(g->wcls);
     dfree(g->wesc);
     dfree(g->scol);
     dfree(g->hot_node);
+    dfree(g->hot_first);
     dfree(g->idx_off);
     dfree(g->idx_dest);
   }
@@ -953,7 +974,8 @@ int fora_index_build(fora_graph* g, const fora_params* params, void* stream_) {
   CUDA_TRY(cudaMemsetAsync(w->stats, 0, sizeof(SlotStats), stream));
   const GraphDev gd = g->dev();
   BatchDev b{};
-  b.nsrc = 1;
+  lay_out(g, w, 1, 1, &b);
+  set_sources(g, w, 1, &b);
   b.alpha = rp.alpha;
   b.walk_scale = rp.walk_scale;
   b.alpha_threshold = rp.alpha_threshold;
@@ -961,26 +983,6 @@ int fora_index_build(fora_graph* g, const fora_params* params, void* stream_) {
   set_round_keys(&b, params->seed);
   // zero-hop: omega_max from (1 - alpha) RN(r_max d(v)) and walks with a forced first move
   b.zero_hop = zero_hop ? 1 : 0;
-  b.r = w->r; b.res = w->res; b.acc = w->tally;
-  b.q[0] = w->q[0]; b.q[1] = w->q[1]; b.fa = w->fa;
-  b.hub[0] = w->hub[0]; b.hub[1] = w->hub[1];
-  b.hub_stride = g->hub_chunks;
-  b.slot_cnt = w->slot_cnt;
-  b.cnt_stride = w->cap;
-  b.gpre = w->pre;
-  b.hpre = w->pre + (w->cap + 1);
-  b.alist = w->alist;
-  b.work = w->work;
-  b.ps = w->ps;
-  b.totals = w->small + 4;
-  b.walk_next = w->small + 6;
-  b.sources = w->sources; b.rmax = w->rmax; b.stats = w->stats; b.err = w->err;
-  b.wr_entry = w->q[0];
-  b.wr_offset = w->q[1];
-  b.wr_weight = reinterpret_cast<unsigned long long*>(w->fa);
-  b.blk_cnt = w->blk;
-  b.blk_walks = w->blk + w->residual_grid;
-  b.residual_grid = w->residual_grid;
   {
     std::lock_guard<std::mutex> tlock(g->mu);
     b.spread_width = g->tune.spread_width;

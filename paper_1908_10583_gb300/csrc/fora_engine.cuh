@@ -11,9 +11,21 @@ namespace fora {
 // one warp per chunk, so that a hub never serialises a round on one warp.
 constexpr uint32_t kHubChunk = 256;
 
-// Nodes of one source a warp of the push take scans as one tile.
-constexpr uint32_t kTakeTile = 1024;
-constexpr int kHubChunkBits = 24;  // hub item = (frontier index << 24) | chunk
+// Residues of one group of sources that a warp of the push's take reads at a time: 256 / gw
+// nodes, whose changes in a light push round share one mark.
+constexpr int kTakeUnit = 256;
+// Nodes per entry of GraphDev::hot_first.
+constexpr uint32_t kHotSpan = 64;
+// Copies of the hot nodes' residues that a push spreads its pushes to them over.
+constexpr int kHotCopies = 8;
+// State of a group of sources in the push (BatchDev::light).
+constexpr uint32_t kGroupLight = 1u;   // its next take scans the listed tiles only
+constexpr uint32_t kGroupActive = 2u;  // it takes part in the next take
+constexpr uint32_t kMaxPolls = 1u << 25;  // polls of a block at the push's barrier (about 30 s)
+
+// Units of the residual list: all of a call (scanned by one block), and of one slot.
+constexpr int kMaxUnits = 32768;
+constexpr int kMaxSlotUnits = 4096;
 
 // Top-k radix select: 96-bit keys (estimate bits : ~id), 12-bit digits.
 constexpr int kDigitBits = 12;
@@ -27,6 +39,7 @@ constexpr uint32_t kErrWalkOverflow = 2u;
 constexpr uint32_t kErrPushNotConverged = 4u;
 constexpr uint32_t kErrIndexRange = 8u;  // a residue needs more walks than the index holds
 constexpr uint32_t kErrBounds = 16u;     // a device index check failed (FORA_DEBUG builds)
+constexpr uint32_t kErrBarrier = 32u;    // a wait of the push's blocks for each other ran out
 
 // Device index checks of the FORA_DEBUG build: FORA_IN_RANGE(err, i, n) is true when
 // i < n; otherwise it records kErrBounds in *err and is false, and the caller skips the
@@ -52,10 +65,16 @@ constexpr uint32_t kMaxPushRounds = 100000u;  // default cap of the push rounds
 struct PushState {
   int cur;
   uint32_t round;
-  uint32_t go;    // the loop condition of the last round (read by the host-driven loop)
-  uint32_t nact;  // sources with a non-empty current frontier (listed in BatchDev::alist)
-  unsigned long long ngroups;  // 32-entry groups of the current frontier, over all sources
-  unsigned long long nhub;     // hub items of the current frontier, over all sources
+  uint32_t go;      // the loop condition of the last round (read by the host-driven loop)
+  uint32_t nact;    // groups that take part in the next take
+  unsigned long long ngroups;  // items of `span` entries of the current frontier, over all groups
+  unsigned long long nhub;     // hub items of the current frontier, over all groups
+};
+struct PushCtl {
+  uint32_t nheavy;  // groups that the next take scans whole (listed in BatchDev::alist)
+  uint32_t nlist;   // units listed of the others (BatchDev::tlist)
+  uint32_t span;    // entries of an item of the spread
+  uint32_t pad;
 };
 
 struct GraphDev {
@@ -64,6 +83,7 @@ struct GraphDev {
   const uint32_t* row;  // [n+1] edge offsets (m < 2^32)
   const int32_t* col;   // [m]
   const double* invd;   // [n] RN(1 / d(v)): the push increment is a product, not a quotient
+  const float* fdeg;    // [n] RN32(d(v)), of the frontier test
   // The walks' own numbering and adjacency.  Nodes of equal out-degree have consecutive walk
   // ids and consecutive rows of wcol, so a node's first edge is wcls[c].x + id * d with its
   // degree class c (d = wcls[c].y), and an edge record {class : 32 - wbits bits, walk id :
@@ -81,21 +101,18 @@ struct GraphDev {
   uint32_t ecols;        // end_cols(n, wbits)
   // The spread's copy of the targets (null when the graph has no hot nodes): the target
   // id, or kHotBit | h for the h-th hot node (a node of high in-degree, hot_node[h]), whose
-  // increments a block sums in shared memory before one reduction reaches L2.
+  // increments go to one of several copies of its residue.
   const uint32_t* scol;
   const uint32_t* hot_node;  // [nhot] ascending ids
+  const uint8_t* hot_first;  // [ceil(n / kHotSpan) + 1]: hot nodes below node t * kHotSpan
   int nhot;
 };
 
 // Hot targets of the spread: at most kHotSlots nodes, each of in-degree >= kHotMinIndeg.
-// (2^20 R-MAT graph, 256 sources, push of the rule's / half the rule's r_max: 2048 hot
-// nodes 100.5 / 151.8 ms, 1024: 98.6 / 146.6, 256: 97.1 / 140.5, 128: 97.3 / 138.1,
-// 16: 98.7 / 138.6, one atomic per push 116.9 / 168.6; what the sums remove is mostly
-// the queueing of reductions on the same few addresses at L2.)
-#ifndef FORA_HOT_SLOTS
-#define FORA_HOT_SLOTS 128
-#endif
-constexpr int kHotSlots = FORA_HOT_SLOTS;
+// Their residues are added up in kHotCopies copies (256 sources of a 2^20-node R-MAT graph, r_max
+// of the network: 121.5 ms of push, 187.2 without the copies, as the reductions that meet in one
+// sector take turns there).
+constexpr int kHotSlots = 128;
 constexpr uint32_t kHotMinIndeg = 64;
 constexpr uint32_t kHotBit = 0x80000000u;
 
@@ -152,9 +169,13 @@ struct TopkSlot {
   uint32_t pad;
 };
 
-// Pointers into a call's workspace; all arrays source-major ([slot][n]).
+// Pointers into a call's workspace.  The push keeps its sources in groups of gw (1 or 4): value
+// (slot, v) of r, res and fa is at g n gw + v w + slot % gw, with g = slot / gw and w the slots
+// of the group (gw, fewer in the last group of a layout of `lay` slots).
 struct BatchDev {
   int32_t nsrc;
+  int lay, gw;
+  int ngrp, lgrp;            // groups of nsrc and of lay slots
   double alpha;
   double walk_scale;         // C = omega / r_sum
   uint32_t alpha_threshold;  // floor(alpha * 2^32)
@@ -164,42 +185,49 @@ struct BatchDev {
   int want_count;            // tally walk counts too (only a debug output reads them)
   uint32_t* walk_dest;       // non-null: k_walks stores walk g's end (a walk id) in
                              // walk_dest[g] (building a walk index) instead of tallying it
-  double* r;                 // residue, later the estimate
+  double* r;                 // residue
   double* res;               // reserve
   // Walk ends: the sum of walk weights (2^-63 units) at [slot * ends + end_place(walk id)],
   // and, when want_count, the number of walks.
   unsigned long long* acc;
   uint32_t* wcount;
   unsigned long long ends;  // end_places of the graph
-  // Frontier of source `slot`: entries (slot << 32) | v at q[par][slot * n + j],
-  // j < slot_cnt[par][slot], with increments fa[slot * n + j]; its hub items at
-  // hub[par][slot * hub_stride + j], j < slot_cnt[2 + par][slot].
-  unsigned long long* q[2];
-  double* fa;                // per frontier entry: (1 - alpha) r(v) / d(v)
-  unsigned long long* hub[2];  // hub chunk items: (q index << kHubChunkBits) | chunk
+  // Frontier of group g: entry e < slot_cnt[par][g] (par: the round's parity) is a node with
+  // {first edge, degree} q[g * gw * n + e] and increments fa[g * gw * n + e * w + slot % gw]; its
+  // hub items, i < slot_cnt[2 + par][g], are {entry, first edge} hub[g * gw * hub_stride + i]
+  // with hub_len edges each.
+  uint2* q;
+  double* fa;                // per frontier entry and source: (1 - alpha) r(v) / d(v)
+  uint2* hub;
+  uint32_t* hub_len;
   unsigned long long hub_stride;
   uint32_t* slot_cnt;        // [4][cnt_stride]: entries of parity 0, 1; hub items of parity 0, 1
   int cnt_stride;            // slots per row of slot_cnt (the workspace's capacity)
-  unsigned long long* gpre;  // [nsrc + 1]: exclusive prefix of ceil(entries / 32), current
-  unsigned long long* hpre;  // [nsrc + 1]: exclusive prefix of hub items, current
-  uint32_t* alist;           // [nsrc]: the sources with a non-empty current frontier
+  unsigned long long* gpre;  // [ngrp + 1]: exclusive prefix of ceil(entries / 32), current
+  unsigned long long* hpre;  // [ngrp + 1]: exclusive prefix of hub items, current
+  uint32_t* alist;           // the groups that the next take scans whole
+  uint32_t* tlist;           // units (g * tiles + t) that the next take scans of the others
+  double* hotr;              // [hot_copies][lgrp][nhot][gw] copies of the hot nodes' residues
+  int hot_copies;            // 0: every push goes to r
   unsigned long long* work;  // dynamic work counters of the spread ([0] and [16])
   PushState* ps;
+  PushCtl* ctl;
+  uint32_t* meet;            // barrier of the push: [0] arrivals, [32] the last meeting's word
   const int32_t* sources;    // [nsrc]
   const double* rmax;        // [nsrc]
   SlotStats* stats;          // [nsrc]
   uint32_t* err;
   // walk phase
-  unsigned long long* wr_entry;   // residual list: (slot << 32) | v   (aliases q[0])
-  unsigned long long* wr_offset;  // exclusive walk offsets, [|R| + 1]  (aliases q[1])
+  unsigned long long* wr_entry;   // residual list: (slot << 32) | v
+  unsigned long long* wr_offset;  // exclusive walk offsets, [|R| + 1]
   unsigned long long* wr_weight;  // fixed-point weight per walk        (aliases fa)
-  unsigned long long* blk_cnt;    // [grid] per-block counts, then block offsets
-  unsigned long long* blk_walks;  // [grid] per-block counts, then block offsets
+  // entries and walks of each slot's share of the nodes: counts, then offsets
+  unsigned long long* unit_cnt;    // [nsrc][units]
+  unsigned long long* unit_walks;  // [nsrc][units]
+  int units;                       // shares of the nodes, a warp's work each
   unsigned long long* totals;     // [2]: |R|, W
   unsigned long long* walk_next;  // shares of the walk range taken beyond the first (zeroed)
-  int residual_grid;
   int spread_width;  // interleaved segments of the frontier the spread visits at once
-  int spread_hot;    // the spread sums hot targets per block (GraphDev::scol is set)
   int walk_blocks;   // resident walk blocks per SM (3, 4 or 5)
   uint32_t max_rounds;  // push rounds allowed before kErrPushNotConverged
   // Balanced push (Section 4.2, Alg. 3): balance != 0 makes rmax the per-source threshold
@@ -211,23 +239,23 @@ struct BatchDev {
   double* theta;       // [nsrc] the thresholds (the same array as rmax)
   uint32_t* stopped;   // [nsrc] 1 once the cost rule stopped the source's push
   // Light rounds: after every take each node of an active source is at or below its
-  // threshold, so only nodes the next spread adds to can cross.  When a source's new
-  // frontier spreads fewer than light_edges edges, light[s] = 1: its spread marks the
-  // kTakeTile-node tiles it touches in tile_dirty and its take scans only those (clearing
-  // them); otherwise the take scans every tile.
-  uint8_t* light;                  // [nsrc]
-  uint8_t* tile_dirty;             // [nsrc][tiles]
+  // threshold, so only nodes the next spread adds to can cross.  When a group's new frontier
+  // spreads fewer than light_edges edges, its spread marks the units of kTakeUnit residues that
+  // it touches (one bit each) and lists them in tlist, and its take scans only those (clearing
+  // the marks); otherwise the take scans every unit.
+  uint8_t* light;                  // [ngrp] kGroupLight | kGroupActive
+  uint32_t* dirty;                 // [lgrp][tiles] bits
   unsigned long long* last_edges;  // [nsrc] the source's edge pushes at the last advance
-  unsigned long long tiles;        // tiles per source, ceil(n / kTakeTile)
+  uint32_t tiles;                  // units per group, ceil(n / (kTakeUnit / gw))
   unsigned long long light_edges;
 };
 
 // Launch-shape parameters of a graph (set through fora_graph_tune or the autotuner).
 struct Tuning {
   int spread_width = 1;
-  int spread_hot = 1;      // 1: heavy spread rounds sum hot targets' increments per block
+  int spread_hot = 1;      // 1: pushes to hot nodes go to copies of their residues
   int walk_blocks = 4;
-  int push_host_loop = 0;  // 1: rounds launched from a host loop instead of the graph
+  int push_host_loop = 0;  // 1: rounds launched from a host loop instead of one launch
   int pipeline = 1;        // parts of a batch run on their own streams, pushes staggered
   uint32_t max_push_rounds = kMaxPushRounds;
 };
@@ -242,12 +270,16 @@ int resident_blocks(const void* kernel, int threads);
 // returns cudaErrorMemoryAllocation without allocating when the hook says so.
 cudaError_t device_alloc(void** p, size_t bytes);
 
-// push.cu: r(s) = 1 and the loop state; then the rounds, each launched by the body of a
-// conditional while-node of a CUDA graph (the body sets the loop condition itself), or,
-// with in_graph false, from a host loop that reads PushState::go after each round.
-cudaError_t launch_push_seed(const GraphDev& g, const BatchDev& b, cudaStream_t st);
-cudaError_t launch_push_body(const GraphDev& g, const BatchDev& b, int num_sms,
-                             cudaGraphConditionalHandle loop, bool in_graph, cudaStream_t st);
+// push.cu: the whole push in one cooperative launch (from zeroing r and res on).
+cudaError_t launch_push(const GraphDev& g, const BatchDev& b, int num_sms, cudaStream_t st);
+// The same in steps for a host loop that reads PushState::go after each round: start, rounds,
+// finish.
+cudaError_t launch_push_start(const GraphDev& g, const BatchDev& b, int num_sms, cudaStream_t st);
+cudaError_t launch_push_round(const GraphDev& g, const BatchDev& b, int num_sms, cudaStream_t st);
+cudaError_t launch_push_finish(const GraphDev& g, const BatchDev& b, int num_sms, cudaStream_t st);
+// push.cu: a [slot][n] array from (to_rows) or into the batch's grouped layout.
+cudaError_t launch_regroup(double* grouped, double* rows, const BatchDev& b, int64_t n,
+                           bool to_rows, int num_sms, cudaStream_t st);
 // push.cu: slots [first, first + k) join a batch between two push rounds (host loop only).
 cudaError_t launch_push_join(const GraphDev& g, const BatchDev& b, int first, int k,
                              cudaStream_t st);
@@ -256,6 +288,9 @@ cudaError_t launch_threshold_table(const double* r, const double* rm, const uint
                                    uint8_t* out, int count, cudaStream_t st);
 
 // walk.cu
+// Residual units per slot: a multiple of a warp's nodes, at most kMaxUnits in all so that one
+// block scans them, and at most what the top-k scratch of a slot holds.
+int residual_units(int64_t n, int nsrc);
 cudaError_t launch_residuals(const GraphDev& g, const BatchDev& b, cudaStream_t st);
 cudaError_t launch_walks(const GraphDev& g, const BatchDev& b, int num_sms, cudaStream_t st);
 // walk.cu, FORA+ (Section 3.3): r[v] = RN(rmax * d(v)) for one slot (the residues whose
@@ -288,8 +323,7 @@ cudaError_t launch_pred_to_rmax(const float* pred, int n, double rmax_rule, floa
 int mlp_tile();
 
 // topk.cu
-// est may alias b.r (the residue array becomes the estimate); with zero-hop pruning the
-// estimate also takes alpha * r.
+// est [nsrc][n]; with zero-hop pruning the estimate also takes alpha * r.
 cudaError_t launch_estimate(const GraphDev& g, const BatchDev& b, double* est, cudaStream_t st);
 // Scratch of the top-k select: hist [nrows][kBins], slots [nrows], cand [nrows][kSortCap].
 struct TopkScratch {

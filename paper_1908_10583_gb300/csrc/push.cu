@@ -1,33 +1,48 @@
 // Forward Push (Alg. 1) as synchronous frontier rounds over a batch of sources.
 //
-// F_t holds, per source, the nodes v with r(v) > r_max * d(v) at the start of round t,
-// each with the increment inc_v = (1 - alpha) a_v / d(v) of its taken residue a_v.
-// Source s keeps its part of F_t in its own region of the queue (q[par][s * n + j]), so
-// the frontier is grouped by source without a global sort.  Round t:
-//   k_push_spread   r(u) += inc_v for every out-edge (v, u) of F_t: FP64 reductions
-//                   that return nothing, so a warp never waits on an atomic.
-//                   (k_push_spread_hot, the default on graphs with hot nodes, first
-//                   sums a block's pushes to the few nodes of highest in-degree in
-//                   shared memory; see there.)
-//   k_push_take     F_{t+1} = {u : r(u) > r_max * d(u)} over the sources that pushed in
-//                   round t (every other r is unchanged and below its threshold), in one
-//                   streaming pass over their residues; each crossing node is appended
-//                   to its source's region and taken at once:
-//                   a_u = r(u); reserve(u) += alpha a_u; r(u) = 0;
-//                   inc_u = (1 - alpha) a_u / d(u)   (the first half of round t+1),
-//                   computed as RN(RN((1 - alpha) a_u) * RN(1 / d(u))) with the
-//                   graph's reciprocal degrees (within an ulp or so of the quotient;
-//                   this GPU's FP64 division costs about ten FP64 instructions).
-//   k_push_advance  one block: per-source prefix of the new frontier's groups and hub
-//                   items, the list of sources still pushing, the loop condition.
-// The take of round t+1 happens after every add of round t (kernel boundary), so
-// residue arriving at a frontier node during a round waits for the next round.
+// Sources are kept in groups of G (1 or 4): the residues, reserves and increments of a group's
+// sources at one node lie side by side (r[group][node][source]), so the take reads a node's
+// degree once per group and the spread adds to the G sources of a target in one 32-byte
+// sector.  (The L2 takes 2.0e11 scattered FP64 reductions a second, and 5.1e11 where four fill
+// a sector; after the first rounds the sources of a batch push from much the same nodes: four
+// sources of the 2^20-node R-MAT graph share 74% of their frontier edges at 0.35 of the rule's
+// r_max, 38% at the rule's.)
 //
-// Spread load balance: a warp takes 32 frontier entries with d <= kHubChunk, scans their
-// degrees and walks their concatenated edge lists 128 edges per iteration (coalesced
-// col reads); nodes with more out-edges are split into kHubChunk-edge hub items, one
-// warp each.  Work is handed out in source order, so the warps in flight work on a few
-// sources at a time and the residue arrays they add into stay in L2.
+// F_t holds, per group, the nodes v that some source of the group takes in round t, i.e. with
+// r(v) > r_max * d(v) at its start, and per source the increment inc_v = (1 - alpha) a_v / d(v)
+// of its taken residue a_v (0: the source does not take v).  Round t:
+//   spread   r(u) += inc_v for every out-edge (v, u) of F_t: FP64 reductions that return
+//            nothing, so a warp never waits on an atomic.
+//   take     F_{t+1} = {u : r(u) > r_max * d(u)} over the groups that pushed in round t (every
+//            other r is unchanged and below its threshold), in one pass over their residues;
+//            each crossing node is appended to its group's queue and taken at once:
+//            a_u = r(u); reserve(u) += alpha a_u; r(u) = 0;
+//            inc_u = (1 - alpha) a_u / d(u)   (the first half of round t+1), computed as
+//            RN(RN((1 - alpha) a_u) * RN(1 / d(u))) with the graph's reciprocal degrees (within
+//            an ulp or so of the quotient; this GPU's FP64 division costs about ten FP64
+//            instructions).
+//   advance  one block: per-group prefix of the new frontier's items, the groups still
+//            pushing, the loop condition.
+// The take of round t+1 happens after every add of round t, so residue arriving at a frontier
+// node during a round waits for the next round.
+//
+// k_push runs all rounds in one cooperative launch: its blocks meet at a barrier after each
+// phase, and block 0 runs the advance while the others wait at the take's.  (As three launches in
+// a conditional graph node a round cost 39 us however small; 22 rounds of a 2^14-node graph took
+// 0.89 ms, now 0.39.)  The same phases are launched one by one where the host steps in between
+// rounds (serving joins, push_host_loop).
+//
+// Pushes to the graph's hot nodes (the up to 128 nodes of highest in-degree) would queue at the
+// L2 slices that hold their residues: each block adds them to one of kHotCopies copies, and the
+// take adds the copies to the residue before it reads it.
+//
+// Bounds: the spread by the reductions' rate at L2 (heavy rounds run at 2.4e11 to 2.7e11 pushes
+// a second, 1.2e11 sectors, of the 1.27e11 sectors that four neighbouring FP64 reductions each
+// reached in isolation), the take by the pass over the residues, light rounds by the latency of
+// a few dependent L2 accesses and two barriers (about 17 us).  Measured against one reduction per
+// push and source (with hot pushes summed in shared memory, and the rounds in a graph): 256
+// sources of a 2^20-node R-MAT graph, r_max of the network, 185 -> 121.5 ms of push; 64 of 2^18
+// 7.5 -> 6.9; 100 of a 200003-node graph without hubs 8.9 -> 6.3; one of 2^20 1.86 -> 1.45.
 #include "fora_engine.cuh"
 
 namespace fora {
@@ -35,9 +50,10 @@ namespace fora {
 namespace {
 
 constexpr unsigned kFull = 0xFFFFFFFFu;
-constexpr int kTakeThreads = 256;
-constexpr int kSpreadThreads = 256;
-constexpr uint32_t kTileNodes = kTakeTile;  // nodes of one source a warp scans per take tile
+constexpr int kPushThreads = 256;
+constexpr int kPushWarps = kPushThreads / 32;
+constexpr uint32_t kSpan = 32;  // most entries of an item of the spread
+constexpr int kUnit = kTakeUnit;  // residues a warp of the take reads at a time
 
 __device__ __forceinline__ uint32_t lane_id() { return threadIdx.x & 31u; }
 
@@ -79,27 +95,22 @@ __device__ __forceinline__ uint32_t hub_chunks_of(uint32_t d) {
   return d > kHubChunk ? (d + kHubChunk - 1) / kHubChunk : 0u;
 }
 
-// r > RN(rm * d), the frontier test, with FP64 arithmetic only near the threshold (this
-// GPU issues about two FP64 operations per clock per SM, so the test itself would bound
-// the scan).  rf is r truncated to 23 mantissa bits through its bit pattern (rf <= r <
-// rf (1 + 2^-23) when r's exponent is in FP32's normal range, rf = 0 when r < 2^-126),
-// tf = RN32(rmf * RN32(d)) with rmf = RN32(rm) is within 2^-22 of V = rm * d, and
-// T = RN64(V) is within 2^-53 of V.  So rf below tf (1 - 2^-19) implies r < V (1 - 2^-20)
-// < T, and rf above tf (1 + 2^-19) implies r > V (1 + 2^-20) > T.  Returns 0 (below),
-// 1 (above) or 2 (undecided: in between, or rmf outside [2^-100, 2^60], which `fast`
-// excludes, or r >= 2^128); the FP64 test decides the undecided ones.
-__device__ __forceinline__ uint32_t threshold_fast(double r, float rmf, bool fast, uint32_t d) {
-  const unsigned long long bits = (unsigned long long)__double_as_longlong(r);
-  const uint32_t hi = (uint32_t)(bits >> 32);
-  const uint32_t ex = hi >> 20;  // r >= 0: no sign bit
-  if (!fast || ex > 1150u) return 2u;
-  const float tf = rmf * __uint2float_rn(d);
-  const float rf = ex < 897u ? 0.0f
-                             : __uint_as_float(((ex - 896u) << 23) | ((hi & 0xFFFFFu) << 3) |
-                                               ((uint32_t)bits >> 29));
-  if (rf < tf * (1.0f - 0x1p-19f)) return 0u;
-  if (rf > tf * (1.0f + 0x1p-19f)) return 1u;
-  return 2u;
+// r > RN(rm * d), the frontier test, without FP64 arithmetic but near the threshold (this GPU
+// issues about two FP64 operations per clock per SM, so the test itself would bound the scan).
+// tf = RN32(rmf * RN32(d)) with rmf = RN32(rm) is within 2^-22 of V = rm * d, and T = RN64(V) is
+// within 2^-53 of V.  The upper word of an FP64 value (exponent and 20 mantissa bits) is
+// floor(bits / 2^32), that of tf is (bits of tf >> 3) + 0x38000000, and a relative change of
+// 2^-21 moves it by at most 1; so r's word below tf's word - 1 implies r < T, and above tf's
+// word + 1 implies r > T.  Valid for rmf in [2^-100, 2^60] (`fast`), where tf is a normal
+// number; r may be anything (r >= 0: its words order as its values).  Returns 0 (below), 1
+// (above) or 2 (undecided); the FP64 test decides the undecided ones.
+__device__ __forceinline__ uint32_t threshold_word(float rmf, float d) {
+  return (__float_as_uint(rmf * d) >> 3) + 0x38000000u;
+}
+__device__ __forceinline__ uint32_t threshold_fast(double r, float rmf, bool fast, float d) {
+  const uint32_t hi = (uint32_t)((unsigned long long)__double_as_longlong(r) >> 32);
+  const uint32_t t = threshold_word(rmf, d);
+  return !fast ? 2u : hi < t - 1u ? 0u : hi > t + 1u ? 1u : 2u;
 }
 
 // The FP64 test, kept out of line so that it is not evaluated for every node.
@@ -109,15 +120,15 @@ __device__ __noinline__ bool threshold_exact(double r, double rm, uint32_t d) {
 
 __device__ __forceinline__ bool above_threshold(double r, double rm, float rmf, bool fast,
                                                 uint32_t d) {
-  const uint32_t f = threshold_fast(r, rmf, fast, d);
+  const uint32_t f = threshold_fast(r, rmf, fast, __uint2float_rn(d));
   return f == 2u ? threshold_exact(r, rm, d) : f == 1u;
 }
 
-// The source whose range [pre[s], pre[s + 1]) holds x, for a non-decreasing prefix with
-// x < pre[nsrc]: the largest s with pre[s] <= x (empty sources have pre[s] = pre[s + 1]).
-__device__ __forceinline__ int slot_of(const unsigned long long* pre, int nsrc,
-                                       unsigned long long x) {
-  int lo = 0, hi = nsrc - 1;
+// The group whose range [pre[s], pre[s + 1]) holds x, for a non-decreasing prefix with
+// x < pre[count]: the largest s with pre[s] <= x (empty ones have pre[s] = pre[s + 1]).
+__device__ __forceinline__ int group_of(const unsigned long long* pre, int count,
+                                        unsigned long long x) {
+  int lo = 0, hi = count - 1;
   while (lo < hi) {
     const int mid = (lo + hi + 1) >> 1;
     if (pre[mid] <= x) lo = mid; else hi = mid - 1;
@@ -125,17 +136,35 @@ __device__ __forceinline__ int slot_of(const unsigned long long* pre, int nsrc,
   return lo;
 }
 
-__global__ void k_push_seed(GraphDev g, BatchDev b) {
-  for (int slot = blockIdx.x * blockDim.x + threadIdx.x; slot < b.nsrc;
-       slot += gridDim.x * blockDim.x) {
-    // Alg. 1 starts from r(s) = 1.  The first pass of the loop body has an empty
-    // frontier (nothing to spread); its take scans every source and finds F_0.
-    const uint32_t src = (uint32_t)b.sources[slot];
-    b.r[(unsigned long long)slot * (unsigned long long)g.n + src] = 1.0;
-    b.alist[slot] = (uint32_t)slot;
-    // only r(s) is non-zero: the first take scans the source's tile alone
-    b.light[slot] = 1;
-    b.tile_dirty[(unsigned long long)slot * b.tiles + src / kTileNodes] = 1;
+// Sources of group gr side by side in the layout: G, fewer in the last group.
+template <int G>
+__device__ __forceinline__ uint32_t width_of(const BatchDev& b, uint32_t gr) {
+  return min((uint32_t)G, (uint32_t)b.lay - gr * G);
+}
+
+// Marks the unit of node u of a group for its next take, listing it once.
+template <int G>
+__device__ __forceinline__ void mark_unit(const BatchDev& b, uint32_t gr, uint32_t u) {
+  const unsigned long long t = (unsigned long long)gr * b.tiles + u / (kUnit / G);
+  uint32_t* word = b.dirty + (t >> 5);
+  const uint32_t bit = 1u << (t & 31);
+  if (*(volatile uint32_t*)word & bit) return;
+  if (!(atomicOr(word, bit) & bit)) b.tlist[atomicAdd(&b.ctl->nlist, 1u)] = (uint32_t)t;
+}
+
+// Before the first round: r(s) = 1 for every source (Alg. 1), every group in the first take,
+// which scans the sources' units alone.  Called by the threads of one block.
+template <int G>
+__device__ void seed_phase(const GraphDev& g, const BatchDev& b) {
+  for (int slot = threadIdx.x; slot < b.nsrc; slot += blockDim.x) {
+    const uint32_t src = (uint32_t)b.sources[slot], gr = (uint32_t)slot / G;
+    b.r[(unsigned long long)gr * G * (unsigned long long)g.n +
+        (unsigned long long)src * width_of<G>(b, gr) + slot % G] = 1.0;
+    mark_unit<G>(b, gr, src);
+    if (slot % G == 0) {
+      b.alist[gr] = gr;
+      b.light[gr] = kGroupLight | kGroupActive;
+    }
     if (b.balance) {
       // the cost rule before any push: FC = 0 against the walk cost of r_sum = 1
       const bool stop = 0.0 >= __dmul_rn(__dmul_rn(1.0, b.bal_scale), b.cost_walk);
@@ -149,284 +178,157 @@ __global__ void k_push_seed(GraphDev g, BatchDev b) {
       b.theta[slot] = theta;
     }
   }
-  if (blockIdx.x == 0 && threadIdx.x == 0) {
+  if (threadIdx.x == 0) {
     PushState* ps = b.ps;
     ps->cur = 1;
     ps->round = 0;
     ps->go = 1;
-    ps->nact = (uint32_t)b.nsrc;
+    ps->nact = (uint32_t)((b.nsrc + G - 1) / G);
     ps->ngroups = 0;
     ps->nhub = 0;
+    b.ctl->span = kSpan;
   }
 }
 
-// 0, 1, ..., 32 as FP64 (the run lengths of spread_slice).
-__constant__ double kMultiple[33] = {0,  1,  2,  3,  4,  5,  6,  7,  8,  9,  10,
-                                     11, 12, 13, 14, 15, 16, 17, 18, 19, 20, 21,
-                                     22, 23, 24, 25, 26, 27, 28, 29, 30, 31, 32};
+// ---------------------------------------------------------------- spread
 
-// Runs of one 32-edge slice whose lanes hold consecutive CSR entries (lane order = entry
-// order; inactive lanes only at the end).  Rows are sorted, so the copies of a multi-edge
-// (v, u) are adjacent: a run of lanes with the same target from the same frontier node
-// (`owner`) becomes one add of k * inc by its first lane (k copies counted with
-// multiplicity, as Alg. 1 pushes along each of them; one rounding instead of k, which only
-// reorders the FP64 sum like the atomics do).  True for the first lane of a run, with
-// add = k * inc; every lane of the warp calls it.
-__device__ __forceinline__ bool run_lead(uint32_t u, uint32_t owner, double inc, bool act,
-                                         double& add) {
-  const uint32_t lane = lane_id();
-  const uint32_t pu = __shfl_up_sync(kFull, u, 1);
-  const uint32_t po = __shfl_up_sync(kFull, owner, 1);
-  const bool cont = act && lane > 0 && pu == u && po == owner;  // continues lane - 1's run
-  const uint32_t brk = __ballot_sync(kFull, !cont);              // run starts and idle lanes
-  const bool lead = act && !cont;
-  uint32_t k = 1;
-  if (lead) {
-    const uint32_t above = brk & ~((2u << lane) - 1u);
-    k = (above ? (uint32_t)__ffs(above) - 1u : 32u) - lane;
-  }
-  // FP64 arithmetic only in slices that hold a run (this GPU's FP64 rate is low, and most
-  // slices have none); kMultiple[k] = k avoids an integer-to-FP64 conversion
-  add = inc;
-  if (__any_sync(kFull, k > 1u)) {
-    if (k > 1u) add = __dmul_rn(inc, kMultiple[k]);
-  }
-  return lead;
+// Where the pushes of one group go: its residues, and this block's copies of its hot nodes'.
+template <int G>
+struct SpreadTarget {
+  double* r;
+  double* hot;  // null: no copies (then no code has kHotBit)
+  uint32_t w;
+};
+
+template <int G>
+__device__ __forceinline__ SpreadTarget<G> spread_target(const GraphDev& g, const BatchDev& b,
+                                                         uint32_t gr) {
+  SpreadTarget<G> t;
+  t.w = width_of<G>(b, gr);
+  t.r = b.r + (unsigned long long)gr * G * (unsigned long long)g.n;
+  t.hot = b.hot_copies ? b.hotr + ((unsigned long long)(blockIdx.x % b.hot_copies) * b.lgrp + gr) *
+                                      (unsigned long long)(g.nhot * G)
+                       : nullptr;
+  return t;
 }
 
-// r[base + u] += inc for the active lanes of one slice, one reduction per run.
-__device__ __forceinline__ void spread_slice(double* r, unsigned long long base, uint32_t u,
-                                             uint32_t owner, double inc, bool act,
-                                             uint32_t* err, unsigned long long n) {
-  double add;
-  if (run_lead(u, owner, inc, act, add) && FORA_IN_RANGE(err, u, n)) atomicAdd(&r[base + u], add);
+// *p += x with nothing returned, in global memory for certain (where the compiler cannot tell the
+// address space of p, an FP64 atomicAdd becomes a loop).
+__device__ __forceinline__ void red_add(double* p, double x) {
+  asm volatile("red.global.add.f64 [%0], %1;" ::"l"(__cvta_generic_to_global(p)), "d"(x)
+               : "memory");
 }
 
-// Work is handed out dynamically (kGrab groups or hub items per atomic), so the warps
-// in flight always hold the next unprocessed stretch of the frontier, whatever the cost
-// of each group.
-constexpr unsigned long long kGrab = 4;
-
-#ifndef FORA_SPREAD_MIN_BLOCKS
-#define FORA_SPREAD_MIN_BLOCKS 6
-#endif
-__global__ void __launch_bounds__(kSpreadThreads, FORA_SPREAD_MIN_BLOCKS) k_push_spread(GraphDev g, BatchDev b) {
-  const int cur = b.ps->cur;
-  const unsigned long long ngroups = b.ps->ngroups;
-  const unsigned long long nh = b.ps->nhub;
-  const unsigned long long* q = b.q[cur];
-  const uint32_t* cnt = b.slot_cnt + (size_t)cur * b.cnt_stride;
-  const uint32_t lane = lane_id();
-  const unsigned long long n = (unsigned long long)g.n;
-
-  // groups of 32 frontier entries of one source (nodes with d <= kHubChunk), visited
-  // through b.spread_width interleaved segments of the frontier
-  const unsigned long long width = (unsigned long long)b.spread_width;
-  const unsigned long long gseg = (ngroups + width - 1) / width;
-  const unsigned long long gtotal = gseg * width;
-  int cs = 0;                           // source of the cached range
-  unsigned long long clo = 1, chi = 0;  // its groups [clo, chi) (empty: nothing cached)
-  uint32_t ccnt = 0;
-  bool clight = false;                  // the cached source's round is light: mark tiles
-  for (;;) {
-    unsigned long long v0 = 0;
-    if (lane == 0) v0 = atomicAdd(&b.work[0], kGrab);
-    v0 = __shfl_sync(kFull, v0, 0);
-    if (v0 >= gtotal) break;
-    const unsigned long long v1 = min(v0 + kGrab, gtotal);
-    for (unsigned long long vg = v0; vg < v1; ++vg) {
-      const unsigned long long grp = (vg % width) * gseg + vg / width;
-      if (grp >= ngroups) continue;
-      if (grp < clo || grp >= chi) {  // warp-uniform
-        cs = slot_of(b.gpre, b.nsrc, grp);
-        clo = b.gpre[cs];
-        chi = b.gpre[cs + 1];
-        ccnt = cnt[cs];
-        clight = b.light[cs] != 0;
-      }
-      const uint32_t i = (uint32_t)(grp - clo) * 32u + lane;
-      const unsigned long long base_gi = (unsigned long long)cs * n;
-      uint32_t c = 0, rb = 0;
-      double inc = 0.0;
-      if (i < ccnt) {
-        const uint32_t v = (uint32_t)q[base_gi + i];
-        rb = g.row[v];
-        const uint32_t d = g.row[v + 1] - rb;
-        if (d <= kHubChunk) {
-          c = d;
-          inc = b.fa[base_gi + i];
-        }
-      }
-      const uint32_t incl = warp_incl_scan(c);
-      const uint32_t total = __shfl_sync(kFull, incl, 31);
-      const uint32_t excl = incl - c;
-      for (uint32_t base = 0; base < total; base += 128) {
-        uint32_t u[4], own[4];
-        double ik[4];
-        bool act[4];
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-          const uint32_t e = base + 32 * k + lane;
-          int lo = 0, hi = 31;  // owner: the first lane whose inclusive prefix exceeds e
-#pragma unroll
-          for (int s2 = 0; s2 < 5; ++s2) {
-            const int mid = (lo + hi) >> 1;
-            if (__shfl_sync(kFull, incl, mid) > e) hi = mid; else lo = mid + 1;
-          }
-          const uint32_t ek = __shfl_sync(kFull, excl, lo);
-          const uint32_t rbk = __shfl_sync(kFull, rb, lo);
-          ik[k] = __shfl_sync(kFull, inc, lo);
-          own[k] = (uint32_t)lo;
-          act[k] = e < total;
-          u[k] = act[k] ? (uint32_t)g.col[rbk + (e - ek)] : 0u;
-        }
-#pragma unroll
-        for (int k = 0; k < 4; ++k)
-          spread_slice(b.r, base_gi, u[k], own[k], ik[k], act[k], b.err, n);
-        if (clight) {  // warp-uniform
-          uint8_t* dirty = b.tile_dirty + (unsigned long long)cs * b.tiles;
-#pragma unroll
-          for (int k = 0; k < 4; ++k)
-            if (act[k] && u[k] < n) dirty[u[k] / kTileNodes] = 1;
-        }
-      }
-    }
-  }
-
-  // hub items: kHubChunk edges of one frontier node each, same segment order
-  const unsigned long long hseg = (nh + width - 1) / width;
-  const unsigned long long htotal = hseg * width;
-  clo = 1;
-  chi = 0;
-  for (;;) {
-    unsigned long long v0 = 0;
-    if (lane == 0) v0 = atomicAdd(&b.work[16], kGrab);
-    v0 = __shfl_sync(kFull, v0, 0);
-    if (v0 >= htotal) break;
-    const unsigned long long v1 = min(v0 + kGrab, htotal);
-    for (unsigned long long vh = v0; vh < v1; ++vh) {
-      const unsigned long long h = (vh % width) * hseg + vh / width;
-      if (h >= nh) continue;
-      if (h < clo || h >= chi) {  // warp-uniform
-        cs = slot_of(b.hpre, b.nsrc, h);
-        clo = b.hpre[cs];
-        chi = b.hpre[cs + 1];
-        clight = b.light[cs] != 0;
-      }
-      const unsigned long long item =
-          b.hub[cur][(unsigned long long)cs * b.hub_stride + (h - clo)];
-      const unsigned long long fi = item >> kHubChunkBits;
-      const uint32_t c = (uint32_t)(item & ((1ull << kHubChunkBits) - 1));
-      const uint32_t v = (uint32_t)q[fi];
-      const unsigned long long gbase = (unsigned long long)cs * n;
-      const uint32_t rb = g.row[v], re = g.row[v + 1];
-      const double inc = b.fa[fi];
-      const uint32_t beg = rb + c * kHubChunk;
-      const uint32_t end = min(beg + kHubChunk, re);
-      uint32_t u[kHubChunk / 32];
-#pragma unroll
-      for (int k = 0; k < (int)(kHubChunk / 32); ++k) {
-        const uint32_t p = beg + 32 * k + lane;
-        u[k] = p < end ? (uint32_t)g.col[p] : 0xFFFFFFFFu;
-      }
-#pragma unroll
-      for (int k = 0; k < (int)(kHubChunk / 32); ++k)
-        spread_slice(b.r, gbase, u[k], 0u, inc, u[k] != 0xFFFFFFFFu, b.err, n);
-      if (clight) {  // warp-uniform
-        uint8_t* dirty = b.tile_dirty + (unsigned long long)cs * b.tiles;
-#pragma unroll
-        for (int k = 0; k < (int)(kHubChunk / 32); ++k)
-          if (u[k] < n) dirty[u[k] / kTileNodes] = 1;
-      }
-    }
-  }
-}
-
-// The spread with hot targets summed per block (GraphDev::scol set, BatchDev::spread_hot).
-// In the R-MAT graphs a few thousand nodes of high in-degree receive a large share of all
-// edge pushes, and every push is an FP64 reduction at L2, the spread's bound.  Here a
-// block takes kHotRange consecutive groups (or hub items) of one interleaved segment of
-// the frontier at a time.  Where the range holds at least kHotStretch items of one source
-// in a heavy round (the source's round is not light), the block processes that stretch
-// together: its adds to hot nodes go to a shared-memory array, and after the stretch one
-// reduction per touched hot node carries each sum to r.  The rest of the range (light
-// rounds, whose spread also marks the tiles it touches, and short stretches) is spread
-// first, warp by warp, with one reduction per push as in k_push_spread.  Summing in
-// shared memory first only regroups the FP64 sum, as the order of the atomics does.
-// Range and stretch measured on the 2^20 R-MAT graph (2048 hot nodes, 5 blocks per SM):
-// ranges of 16, 24, 32, 64, 128 items gave 103.4, 101.2, 100.5, 110.7, 141.3 ms of push
-// with the rule's r_max (fewer, larger ranges leave blocks idle at the end of a round);
-// a minimum stretch of 4, 8 or 16 items made no difference.
-#ifndef FORA_HOT_RANGE
-#define FORA_HOT_RANGE 32
-#endif
-constexpr unsigned long long kHotRange = FORA_HOT_RANGE;
-#ifndef FORA_HOT_STRETCH
-#define FORA_HOT_STRETCH 8
-#endif
-constexpr unsigned long long kHotStretch = FORA_HOT_STRETCH;
-
-// Node id of a target code of GraphDev::scol.
-__device__ __forceinline__ uint32_t hot_decode(const GraphDev& g, uint32_t code) {
-  return (code & kHotBit) ? g.hot_node[code & ~kHotBit] : code;
-}
-
-__device__ __forceinline__ void hot_slice(const GraphDev& g, double* r, unsigned long long base,
-                                          double* hacc, bool agg, uint32_t code, uint32_t owner,
-                                          double inc, bool act, uint32_t* err,
-                                          unsigned long long n) {
-  double add;
-  if (!run_lead(code, owner, inc, act, add)) return;
+// r(u) += inc for source j of the group and the target of a code.
+template <int G>
+__device__ __forceinline__ void add_to(const GraphDev& g, const BatchDev& b,
+                                       const SpreadTarget<G>& t, uint32_t code, uint32_t j,
+                                       double inc) {
   if (code & kHotBit) {
     const uint32_t h = code & ~kHotBit;
-    if (!FORA_IN_RANGE(err, h, (uint32_t)g.nhot)) return;
-    if (agg) atomicAdd(&hacc[h], add);
-    else atomicAdd(&r[base + g.hot_node[h]], add);
-  } else if (FORA_IN_RANGE(err, code, n)) {
-    atomicAdd(&r[base + code], add);
+    if (FORA_IN_RANGE(b.err, h, (uint32_t)g.nhot)) red_add(t.hot + (h * G + j), inc);
+  } else if (FORA_IN_RANGE(b.err, code, g.n)) {
+    red_add(t.r + ((unsigned long long)code * t.w + j), inc);
   }
 }
 
-// Light rounds: the take tile of this lane's push target is marked (when act).
-__device__ __forceinline__ void hot_mark(const GraphDev& g, const BatchDev& b, int cs,
-                                         uint32_t code, bool act) {
-  const unsigned long long n = (unsigned long long)g.n;
-  if (!act) return;
-  const uint32_t x = hot_decode(g, code);
-  if (x < n) b.tile_dirty[(unsigned long long)cs * b.tiles + x / kTileNodes] = 1;
+constexpr uint32_t kNoEdge = 0xFFFFFFFFu;
+
+// x is not zero, for x >= 0 (never -0), without the FP64 pipe: at its rate the comparison alone
+// bounds a kernel that makes it for every value.
+__device__ __forceinline__ bool nonzero(double x) { return __double_as_longlong(x) != 0; }
+
+// The adds of 32 edges (each lane's target code and the place of its entry's increments in
+// inc[place][G]) for the G sources of the group, lanes of one edge side by side.
+template <int G>
+__device__ __forceinline__ void spread_slice(const GraphDev& g, const BatchDev& b,
+                                             const SpreadTarget<G>& t, uint32_t code,
+                                             uint32_t place, const double* inc) {
+  const uint32_t lane = lane_id(), j = lane % G;
+#pragma unroll
+  for (int k = 0; k < G; ++k) {
+    const int from = k * (32 / G) + (int)(lane / G);
+    const uint32_t c = G == 1 ? code : __shfl_sync(kFull, code, from);
+    const uint32_t p = G == 1 ? place : __shfl_sync(kFull, place, from);
+    const double a = inc[p * G + j];
+    if (c != kNoEdge && nonzero(a)) add_to<G>(g, b, t, c, j, a);
+  }
 }
 
-// Group grp of source cs (its groups start at clo, its frontier has ccnt entries): the
-// out-edges of 32 frontier entries with d <= kHubChunk, 128 edges per iteration.
-__device__ __forceinline__ void hot_group(const GraphDev& g, const BatchDev& b,
-                                          const unsigned long long* q, int cs,
-                                          unsigned long long clo, uint32_t ccnt,
-                                          unsigned long long grp, bool light, bool agg,
-                                          double* hacc) {
-  const uint32_t lane = lane_id();
-  const unsigned long long n = (unsigned long long)g.n;
-  const unsigned long long base_gi = (unsigned long long)cs * n;
-  const uint32_t i = (uint32_t)(grp - clo) * 32u + lane;
-  uint32_t c = 0, rb = 0;
-  double inc = 0.0;
-  if (i < ccnt) {
-    const uint32_t v = (uint32_t)q[base_gi + i];
-    rb = g.row[v];
-    const uint32_t d = g.row[v + 1] - rb;
-    if (d <= kHubChunk) {
-      c = d;
-      inc = b.fa[base_gi + i];
+template <int G>
+__device__ __forceinline__ void spread_marks(const GraphDev& g, const BatchDev& b, uint32_t gr,
+                                             uint32_t code) {
+  if (code == kNoEdge) return;
+  const uint32_t u = (code & kHotBit) ? g.hot_node[code & ~kHotBit] : code;
+  if (u < (uint32_t)g.n) mark_unit<G>(b, gr, u);
+}
+
+// A warp's increments of the 32 entries of an item, and of the next item.
+template <int G>
+struct SpreadStage {
+  double inc[2][32 * G];
+};
+
+__device__ __forceinline__ void copy_async8(void* to, const void* from) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(
+                   (uint32_t)__cvta_generic_to_shared(to)),
+               "l"(from)
+               : "memory");
+}
+__device__ __forceinline__ void copy_async_wait() {
+  asm volatile("cp.async.wait_all;" ::: "memory");
+}
+
+// An item of the spread: the entries from `first` on of group gr.
+struct SpreadItem {
+  uint32_t gr, first, have;
+};
+
+// Starts the loads of an item: its entries' {first edge, degree}, one per lane (returned; of a
+// node with more than kHubChunk edges the degree is 0), and their increments into inc.
+template <int G>
+__device__ __forceinline__ uint2 fetch_item(const GraphDev& g, const BatchDev& b,
+                                            const SpreadItem& it, double* inc) {
+  const uint32_t lane = lane_id(), w = width_of<G>(b, it.gr);
+  const unsigned long long g0 = (unsigned long long)it.gr * G * (unsigned long long)g.n;
+  uint2 e = make_uint2(0u, 0u);
+  if (lane < it.have) {
+    e = __ldcg(&b.q[g0 + it.first + lane]);
+    if (e.y > kHubChunk) e.y = 0;
+  }
+  const double* fa = b.fa + g0 + (unsigned long long)it.first * w;
+  if (w == (uint32_t)G) {
+#pragma unroll
+    for (int k = 0; k < G; ++k) {
+      const uint32_t x = k * 32 + lane;
+      if (x < it.have * G) copy_async8(inc + x, fa + x);
+    }
+  } else {
+    for (uint32_t x = lane; x < it.have * G; x += 32) {
+      if (x % G < w) copy_async8(inc + x, fa + x / G * w + x % G);
+      else inc[x] = 0.0;
     }
   }
-  const uint32_t incl = warp_incl_scan(c);
+  return e;
+}
+
+// The edge lists of an item's entries, walked one after the other, 128 edges per iteration with
+// the next 128 targets on their way.
+template <int G>
+__device__ __forceinline__ void spread_item(const GraphDev& g, const BatchDev& b,
+                                            const uint32_t* codes, uint32_t gr, bool light,
+                                            uint2 entry, const double* inc) {
+  const uint32_t lane = lane_id();
+  const SpreadTarget<G> t = spread_target<G>(g, b, gr);
+  const uint32_t incl = warp_incl_scan(entry.y);
   const uint32_t total = __shfl_sync(kFull, incl, 31);
-  const uint32_t excl = incl - c;
-  for (uint32_t base = 0; base < total; base += 128) {
-    uint32_t u[4], own[4];
-    double ik[4];
-    bool act[4];
+  const uint32_t off = entry.x - (incl - entry.y);  // first edge minus the item's edges before
+  constexpr int kSlices = 4;
+  uint32_t code[kSlices], own = 0;  // own: 5 bits per slice
+  auto fetch = [&](uint32_t base, uint32_t* c, uint32_t* o) {
+    uint32_t packed = 0;
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
+    for (int k = 0; k < kSlices; ++k) {
       const uint32_t e = base + 32 * k + lane;
       int lo = 0, hi = 31;  // owner: the first lane whose inclusive prefix exceeds e
 #pragma unroll
@@ -434,442 +336,906 @@ __device__ __forceinline__ void hot_group(const GraphDev& g, const BatchDev& b,
         const int mid = (lo + hi) >> 1;
         if (__shfl_sync(kFull, incl, mid) > e) hi = mid; else lo = mid + 1;
       }
-      const uint32_t ek = __shfl_sync(kFull, excl, lo);
-      const uint32_t rbk = __shfl_sync(kFull, rb, lo);
-      ik[k] = __shfl_sync(kFull, inc, lo);
-      own[k] = (uint32_t)lo;
-      act[k] = e < total;
-      u[k] = act[k] ? g.scol[rbk + (e - ek)] : 0u;
+      const uint32_t at = __shfl_sync(kFull, off, lo) + e;
+      packed |= (uint32_t)(lo & 31) << (5 * k);
+      c[k] = e < total ? __ldg(codes + at) : kNoEdge;
     }
+    *o = packed;
+  };
+  if (total) fetch(0, code, &own);
+  for (uint32_t base = 0; base < total; base += 32 * kSlices) {
+    uint32_t next[kSlices], next_own = 0;
 #pragma unroll
-    for (int k = 0; k < 4; ++k)
-      hot_slice(g, b.r, base_gi, hacc, agg, u[k], own[k], ik[k], act[k], b.err, n);
+    for (int k = 0; k < kSlices; ++k) next[k] = kNoEdge;
+    if (base + 32 * kSlices < total) fetch(base + 32 * kSlices, next, &next_own);
+#pragma unroll
+    for (int k = 0; k < kSlices; ++k)
+      if (base + 32 * k < total) spread_slice<G>(g, b, t, code[k], (own >> (5 * k)) & 31u, inc);
     if (light) {  // warp-uniform
 #pragma unroll
-      for (int k = 0; k < 4; ++k) hot_mark(g, b, cs, u[k], act[k]);
+      for (int k = 0; k < kSlices; ++k) spread_marks<G>(g, b, gr, code[k]);
     }
+#pragma unroll
+    for (int k = 0; k < kSlices; ++k) code[k] = next[k];
+    own = next_own;
   }
 }
 
-// Hub item h of source cs (its items start at clo): kHubChunk out-edges of one node.
-__device__ __forceinline__ void hot_hub(const GraphDev& g, const BatchDev& b,
-                                        const unsigned long long* q, int cur, int cs,
-                                        unsigned long long clo, unsigned long long h, bool light,
-                                        bool agg, double* hacc) {
+// A hub item: up to kHubChunk consecutive out-edges of one frontier entry.
+template <int G>
+__device__ __forceinline__ void spread_hub(const GraphDev& g, const BatchDev& b,
+                                           const uint32_t* codes, uint32_t gr, bool light,
+                                           uint2 rec, uint32_t len, double* inc) {
   const uint32_t lane = lane_id();
-  const unsigned long long n = (unsigned long long)g.n;
-  const unsigned long long item = b.hub[cur][(unsigned long long)cs * b.hub_stride + (h - clo)];
-  const unsigned long long fi = item >> kHubChunkBits;
-  const uint32_t c = (uint32_t)(item & ((1ull << kHubChunkBits) - 1));
-  const uint32_t v = (uint32_t)q[fi];
-  const uint32_t rb = g.row[v], re = g.row[v + 1];
-  const double inc = b.fa[fi];
-  const uint32_t beg = rb + c * kHubChunk;
-  const uint32_t end = min(beg + kHubChunk, re);
-  uint32_t u[kHubChunk / 32];
-  bool act[kHubChunk / 32];
+  const SpreadTarget<G> t = spread_target<G>(g, b, gr);
+  const unsigned long long g0 = (unsigned long long)gr * G * (unsigned long long)g.n;
+  uint32_t code[kHubChunk / 32];
 #pragma unroll
   for (int k = 0; k < (int)(kHubChunk / 32); ++k) {
-    const uint32_t p = beg + 32 * k + lane;
-    act[k] = p < end;
-    u[k] = act[k] ? g.scol[p] : 0u;
+    const uint32_t p = 32 * k + lane;
+    code[k] = p < len ? __ldg(codes + rec.y + p) : kNoEdge;
   }
+  const uint32_t j = lane % G;
+  const double a = j < t.w ? __ldcg(b.fa + g0 + (unsigned long long)rec.x * t.w + j) : 0.0;
+  __syncwarp();  // inc free
+  if (lane < (uint32_t)G) inc[lane] = a;
+  __syncwarp();
 #pragma unroll
   for (int k = 0; k < (int)(kHubChunk / 32); ++k)
-    hot_slice(g, b.r, (unsigned long long)cs * n, hacc, agg, u[k], 0u, inc, act[k], b.err, n);
+    if (32u * k < len) spread_slice<G>(g, b, t, code[k], 0u, inc);
   if (light) {  // warp-uniform
 #pragma unroll
-    for (int k = 0; k < (int)(kHubChunk / 32); ++k) hot_mark(g, b, cs, u[k], act[k]);
+    for (int k = 0; k < (int)(kHubChunk / 32); ++k) spread_marks<G>(g, b, gr, code[k]);
   }
 }
 
-// Item x of a phase (0: groups, 1: hub items) of source cs.
-__device__ __forceinline__ void hot_item(const GraphDev& g, const BatchDev& b, int phase,
-                                         const unsigned long long* q, int cur,
-                                         const uint32_t* cnt, int cs, unsigned long long clo,
-                                         unsigned long long x, bool light, bool agg,
-                                         double* hacc) {
-  if (phase == 0)
-    hot_group(g, b, q, cs, clo, cnt[cs], x, light, agg, hacc);
-  else
-    hot_hub(g, b, q, cur, cs, clo, x, light, agg, hacc);
-}
+// A block's share of a list of items: its warps take them one by one from shared memory, and one
+// global atomic brings the next kChunk.  The items in flight are then a narrow window of the
+// list, so the residues that they add into stay in L2, at an atomic per kChunk items (a counter
+// that every warp used bounded the spread: 256 sources of a 2^20-node R-MAT graph took 224, 166
+// and 127 ms of push with 1, 2 and 4 items an atomic, and 151 and 183 with 16 and 32, whose
+// window no longer fits; this takes 121.5, and 121.8 and 123.1 with chunks of 16 and 32).
+constexpr uint32_t kChunk = 8;
+struct ItemShare {
+  unsigned long long state;  // first item of the chunk << 8 | items taken of it
+  unsigned long long next;   // the next chunk's number + 1, 0: not known yet
+};
 
-// The items of source cs in the range [lo, hi) are summed in shared memory when the
-// source's round is heavy and they are at least kHotStretch.
-__device__ __forceinline__ bool hot_summed(const BatchDev& b, const unsigned long long* pre,
-                                           int cs, unsigned long long lo, unsigned long long hi) {
-  const unsigned long long s0 = max(lo, pre[cs]), s1 = min(hi, pre[cs + 1]);
-  return b.light[cs] == 0 && s1 - s0 >= kHotStretch;
-}
+struct ItemCursor {
+  unsigned long long items, total, seg, width;
+  const unsigned long long* pre;
+  unsigned long long* counter;
+  ItemShare* share;
+  bool few, done;  // at most one item per warp
+  uint32_t gr;
+  unsigned long long lo, hi;  // the items of group gr
+  bool light;
+  uint32_t cnt;
 
-// 5 resident blocks (48 registers): 6 (40 registers, a few spilled) and 4 were slower by
-// 2-4% and 3-10%.
-#ifndef FORA_SPREAD_HOT_MIN_BLOCKS
-#define FORA_SPREAD_HOT_MIN_BLOCKS 5
-#endif
-__global__ void __launch_bounds__(kSpreadThreads, FORA_SPREAD_HOT_MIN_BLOCKS)
-    k_push_spread_hot(GraphDev g, BatchDev b) {
-  __shared__ double hacc[kHotSlots];
-  __shared__ unsigned long long s_range[2];  // one per phase: no thread reads a stale one
-  __shared__ uint32_t s_next;
-  const int cur = b.ps->cur;
-  const unsigned long long* q = b.q[cur];
-  const uint32_t* cnt = b.slot_cnt + (size_t)cur * b.cnt_stride;
-  const unsigned long long width = (unsigned long long)b.spread_width;
-  const uint32_t lane = lane_id();
-  const unsigned long long base_n = (unsigned long long)g.n;
-  for (int h = threadIdx.x; h < g.nhot; h += blockDim.x) hacc[h] = 0.0;
-
-  // phase 0: groups, phase 1: hub items; segment k of a phase's items is
-  // [k * seg, min((k + 1) * seg, total)), taken kHotRange items at a time, the ranges of
-  // the segments interleaved
-  for (int phase = 0; phase < 2; ++phase) {
-    const unsigned long long total = phase == 0 ? b.ps->ngroups : b.ps->nhub;
-    const unsigned long long* pre = phase == 0 ? b.gpre : b.hpre;
-    unsigned long long* work = b.work + (phase == 0 ? 0 : 16);
-    const unsigned long long seg = (total + width - 1) / width;
-    const unsigned long long rseg = (seg + kHotRange - 1) / kHotRange;
-    const unsigned long long rtotal = rseg * width;
+  __device__ __forceinline__ void attach(const BatchDev& b, unsigned long long items_,
+                                         const unsigned long long* pre_, unsigned long long* ctr,
+                                         ItemShare* share_) {
+    items = items_;
+    width = (unsigned long long)b.spread_width;
+    seg = width == 1 ? items : (items + width - 1) / width;
+    total = seg * width;
+    pre = pre_;
+    counter = ctr;
+    share = share_;
+    few = total <= (unsigned long long)gridDim.x * kPushWarps;
+    done = false;
+    gr = 0;
+    lo = 1;
+    hi = 0;
+    light = false;
+    cnt = 0;
+  }
+  // A place in the list, `total` or more when there is none left.  Lane 0.
+  __device__ __forceinline__ unsigned long long pop(uint32_t* err) {
+    for (uint32_t tries = 0; tries < kMaxPolls; ++tries) {
+      const unsigned long long old = atomicAdd(&share->state, 1ull);
+      const uint32_t k = (uint32_t)(old & 255u);
+      const unsigned long long x = (old >> 8) + k;
+      if (x >= total) return x;
+      if (k < kChunk) {
+        if (k == kChunk / 2)  // ask for the next chunk in good time
+          *(volatile unsigned long long*)&share->next = atomicAdd(counter, 1ull) + 1ull;
+        return x;
+      }
+      if (k == kChunk) {  // this warp opens the next chunk
+        unsigned long long n = 0;
+        for (uint32_t polls = 0; polls < kMaxPolls && n == 0; ++polls)
+          n = *(volatile unsigned long long*)&share->next;
+        if (n == 0) break;
+        *(volatile unsigned long long*)&share->next = 0;
+        const unsigned long long first = ((unsigned long long)gridDim.x + n - 1ull) * kChunk;
+        atomicExch(&share->state, first << 8 | 1ull);
+        return first;
+      }
+      for (uint32_t polls = 0; polls < kMaxPolls; ++polls)
+        if ((*(volatile unsigned long long*)&share->state & 255u) <= kChunk) break;
+    }
+    atomicOr(err, kErrBarrier);
+    return ~0ull;
+  }
+  // The next item's place in the list, or false.
+  __device__ __forceinline__ bool step(uint32_t* err, unsigned long long* it) {
     for (;;) {
-      if (threadIdx.x == 0) {
-        s_range[phase] = atomicAdd(work, 1ull);
-        s_next = 0;
+      unsigned long long x = 0;
+      if (few) {
+        if (done) return false;
+        x = (unsigned long long)(threadIdx.x >> 5) * gridDim.x + blockIdx.x;
+        done = true;
+      } else {
+        if (lane_id() == 0) x = pop(err);
+        x = __shfl_sync(kFull, x, 0);
       }
-      __syncthreads();
-      const unsigned long long vr = s_range[phase];
-      if (vr >= rtotal) break;  // block-uniform
-      const unsigned long long sbeg = (vr % width) * seg;
-      const unsigned long long lo = sbeg + (vr / width) * kHotRange;
-      const unsigned long long hi = min(lo + kHotRange, min(sbeg + seg, total));
-      // the items not summed, warp by warp with one reduction per push
-      int cs = 0;
-      unsigned long long clo = 1, chi = 0;
-      bool skip = false, light = false;
-      for (;;) {
-        uint32_t k = 0;
-        if (lane == 0) k = atomicAdd(&s_next, 1u);
-        k = __shfl_sync(kFull, k, 0);
-        const unsigned long long x = lo + k;
-        if (x >= hi) break;  // warp-uniform
-        if (x < clo || x >= chi) {  // warp-uniform
-          cs = slot_of(pre, b.nsrc, x);
-          clo = pre[cs];
-          chi = pre[cs + 1];
-          skip = hot_summed(b, pre, cs, lo, hi);
-          light = b.light[cs] != 0;
-        }
-        if (!skip) hot_item(g, b, phase, q, cur, cnt, cs, clo, x, light, false, hacc);
+      if (x >= total) return false;
+      *it = width == 1 ? x : (x % width) * seg + x / width;
+      if (*it < items) return true;
+    }
+  }
+  // Makes gr the group of item `it`, with its light flag and (for parity cur) entry count.
+  __device__ __forceinline__ void locate(const BatchDev& b, unsigned long long it, int cur) {
+    if (it >= lo && it < hi) return;  // warp-uniform
+    if (b.ngrp == 1) {
+      lo = 0;
+      hi = items;
+    } else {
+      gr = (uint32_t)group_of(pre, b.ngrp, it);
+      lo = pre[gr];
+      hi = pre[gr + 1];
+    }
+    light = (__ldcg(&b.light[gr]) & kGroupLight) != 0;
+    cnt = __ldcg(&b.slot_cnt[(size_t)cur * b.cnt_stride + gr]);
+  }
+};
+
+template <int G>
+__device__ void spread_phase(const GraphDev& g, const BatchDev& b, int cur,
+                             unsigned long long nhub, unsigned long long nitems, uint32_t span,
+                             SpreadStage<G>& st) {
+  const uint32_t* codes = b.hot_copies ? g.scol : (const uint32_t*)g.col;
+  __shared__ ItemShare shares[2];
+  ItemCursor c;
+  unsigned long long it;
+  if (threadIdx.x < 2) {
+    shares[threadIdx.x].state = (unsigned long long)blockIdx.x * kChunk << 8;
+    shares[threadIdx.x].next = 0;
+  }
+  __syncthreads();
+  if (nhub) {
+    c.attach(b, nhub, b.hpre, &b.work[16], &shares[0]);
+    auto fetch = [&](uint2* rec, uint32_t* len) {
+      c.locate(b, it, cur);
+      const unsigned long long at =
+          (unsigned long long)c.gr * G * b.hub_stride + (it - c.lo);
+      *rec = __ldcg(&b.hub[at]);
+      *len = __ldcg(&b.hub_len[at]);
+    };
+    bool more = c.step(b.err, &it);
+    uint2 rec = make_uint2(0u, 0u);
+    uint32_t len = 0;
+    if (more) fetch(&rec, &len);
+    while (more) {
+      const uint32_t gr = c.gr;
+      const bool light = c.light;
+      const uint2 r = rec;
+      const uint32_t l = len;
+      more = c.step(b.err, &it);
+      if (more) fetch(&rec, &len);
+      spread_hub<G>(g, b, codes, gr, light, r, l, st.inc[0]);
+    }
+    __syncwarp();
+  }
+  if (nitems) {
+    c.attach(b, nitems, b.gpre, &b.work[0], &shares[1]);
+    auto locate = [&](SpreadItem* x) {
+      c.locate(b, it, cur);
+      x->gr = c.gr;
+      x->first = (uint32_t)(it - c.lo) * span;
+      x->have = min(span, c.cnt - x->first);
+    };
+    SpreadItem x;
+    uint2 entry = make_uint2(0u, 0u);
+    int half = 0;
+    bool more = c.step(b.err, &it);
+    if (more) {
+      locate(&x);
+      entry = fetch_item<G>(g, b, x, st.inc[0]);
+    }
+    while (more) {
+      copy_async_wait();
+      __syncwarp();  // this item's increments are in place, the other half is free
+      const uint32_t gr = x.gr;
+      const bool light = c.light;
+      const uint2 now = entry;
+      more = c.step(b.err, &it);
+      if (more) {
+        locate(&x);
+        entry = fetch_item<G>(g, b, x, st.inc[half ^ 1]);
       }
-      // the summed stretches, one source at a time with the whole block
-      for (unsigned long long x = lo; x < hi;) {  // block-uniform
-        const int s = slot_of(pre, b.nsrc, x);
-        const unsigned long long s1 = min(hi, pre[s + 1]);
-        if (hot_summed(b, pre, s, lo, hi)) {
-          __syncthreads();  // s_next free, hacc zero
-          if (threadIdx.x == 0) s_next = 0;
-          __syncthreads();
-          for (;;) {
-            uint32_t k = 0;
-            if (lane == 0) k = atomicAdd(&s_next, 1u);
-            k = __shfl_sync(kFull, k, 0);
-            if (x + k >= s1) break;  // warp-uniform
-            hot_item(g, b, phase, q, cur, cnt, s, pre[s], x + k, false, true, hacc);
-          }
-          __syncthreads();  // every add of the stretch is in hacc
-          const unsigned long long base = (unsigned long long)s * base_n;
-          for (int h = threadIdx.x; h < g.nhot; h += blockDim.x) {
-            const double a = hacc[h];
-            if (a != 0.0) {  // every add is positive: zero means untouched
-              atomicAdd(&b.r[base + g.hot_node[h]], a);
-              hacc[h] = 0.0;
-            }
-          }
-        }
-        x = s1;
-      }
-      __syncthreads();  // s_range, s_next and hacc free for the next range
+      spread_item<G>(g, b, codes, gr, light, now, st.inc[half]);
+      half ^= 1;
     }
   }
 }
 
-// Detection and take of the next frontier in one pass.  Warp w scans tiles w, w + W, ...
-// of kTileNodes nodes of one pushing source; for 8 words of 32 nodes at a time the
-// residues and both row offsets are loaded before any is used, the crossing nodes of
-// the 8 words are counted, one atomic per counter reserves their places in the source's
-// queue region, and the crossing nodes are taken.
-// Resident blocks per SM the take and the spread are compiled for (measured on the 2^20
-// graph, 256 sources: take 3 -> 4 blocks 120.4 -> 118.5 ms of push; spread 7 or 8 blocks
-// instead of 6 made it slower, 128-130 ms: more scattered reductions in flight contend at L2).
-#ifndef FORA_TAKE_MIN_BLOCKS
-#define FORA_TAKE_MIN_BLOCKS 4
-#endif
-__global__ void __launch_bounds__(kTakeThreads, FORA_TAKE_MIN_BLOCKS) k_push_take(GraphDev g, BatchDev b) {
-  const PushState* ps = b.ps;
-  const int nx = ps->cur ^ 1;
-  const unsigned long long n = (unsigned long long)g.n;
-  const unsigned long long tps = (n + kTileNodes - 1) / kTileNodes;
-  const unsigned long long ntiles = (unsigned long long)ps->nact * tps;
-  uint32_t* cnt_nx = b.slot_cnt + (size_t)nx * b.cnt_stride;
-  uint32_t* hcnt_nx = b.slot_cnt + (size_t)(2 + nx) * b.cnt_stride;
-  unsigned long long* qn = b.q[nx];
-  unsigned long long* hn = b.hub[nx];
+// ---------------------------------------------------------------- take
+
+// Adds the copies of hot node h's residues in group gr to them and clears the copies.  A warp.
+template <int G>
+__device__ __noinline__ void fold_hot(const GraphDev& g, const BatchDev& b, uint32_t gr,
+                                      uint32_t h) {
+  const uint32_t lane = lane_id(), j = lane % G, w = width_of<G>(b, gr);
+  double sum = 0.0;
+  for (uint32_t c = lane / G; c < (uint32_t)b.hot_copies; c += 32 / G) {
+    double* p = b.hotr + ((unsigned long long)c * b.lgrp + gr) * (unsigned long long)(g.nhot * G) +
+                (h * G + j);
+    const double x = __ldcg(p);
+    if (nonzero(x)) {
+      sum = __dadd_rn(sum, x);
+      *p = 0.0;
+    }
+  }
+  if (!__any_sync(kFull, nonzero(sum))) return;
+#pragma unroll
+  for (int o = 16; o >= G; o >>= 1) sum = __dadd_rn(sum, __shfl_xor_sync(kFull, sum, o));
+  if (lane < w && nonzero(sum)) {
+    double* p = b.r + (unsigned long long)gr * G * (unsigned long long)g.n +
+                (unsigned long long)g.hot_node[h] * w + lane;
+    *p = __dadd_rn(__ldcg(p), sum);
+  }
+  __syncwarp();
+}
+
+// A warp's stage of crossing nodes of one group: those of one unit, and up to kCarry of the
+// units before (where few nodes cross, the take of a stage serves many units).
+constexpr uint32_t kCarry = 32;
+template <int G>
+struct TakeStage {
+  static constexpr uint32_t kCap = kUnit / G + kCarry;
+  double a[kCap * G];      // [entry][G] the taken residues (0: not taken), then the increments
+  uint32_t u[kCap];        // [entry] node
+  uint32_t d[kCap];        // [entry] out-degree
+  uint32_t rb[kCap];       // [entry] first edge
+  uint16_t pair[kCap * G];  // the places in `a` of the taken residues
+};
+
+// Counters of one group that a warp has not added to the batch's yet: of the source lane % G.
+struct TakeCount {
+  uint32_t gr = 0xFFFFFFFFu;
+  uint32_t cnt = 0;
+  unsigned long long deg = 0;
+  double moved = 0.0;  // sum of alpha a (balanced push)
+};
+
+// Sums a warp's counters over the lanes of each source.
+template <int G>
+__device__ __forceinline__ void sum_count(const BatchDev& b, TakeCount& t) {
+#pragma unroll
+  for (int o = 16; o >= G; o >>= 1) {
+    t.cnt += __shfl_xor_sync(kFull, t.cnt, o);
+    t.deg += __shfl_xor_sync(kFull, t.deg, o);
+    if (b.balance) t.moved = __dadd_rn(t.moved, __shfl_xor_sync(kFull, t.moved, o));
+  }
+}
+
+__device__ __forceinline__ void add_count(const BatchDev& b, uint32_t slot, uint32_t cnt,
+                                          unsigned long long deg, double moved) {
+  if (cnt == 0) return;
+  SlotStats& s = b.stats[slot];
+  atomicAdd(&s.pushes, (unsigned long long)cnt);
+  atomicAdd(&s.edge_pushes, deg);
+  if (b.balance) red_add(&s.moved, moved);
+}
+
+// What a warp of the take knows of the group it is at.
+struct TakeGroup {
+  uint32_t gr = 0xFFFFFFFFu;
+  uint32_t w = 0;
+  float rmf = 0.0f;             // this lane's source: RN32(r_max)
+  uint32_t mask = 0;            // ~0 where the frontier test's fast form holds for it
+  bool live = false;
+  uint32_t mine = 0, pairs = 0;  // entries and taken residues in the stage
+};
+
+// Takes the stage: one atomic per counter reserves the entries' places in the group's queue, and
+// the FP64 arithmetic runs on packed lanes.
+template <int G>
+__device__ __noinline__ void take_stage(const GraphDev& g, const BatchDev& b, int nx,
+                                        uint32_t gr, uint32_t w, uint32_t mine, uint32_t pairs,
+                                        TakeStage<G>& st, TakeCount& tc) {
+  const uint32_t lane = lane_id(), j = lane % G;
   const double alpha = b.alpha, beta = __dadd_rn(1.0, -b.alpha);
-  const uint32_t lane = lane_id();
-  const uint32_t lt_mask = (1u << lane) - 1u;
-  const unsigned long long wpb = blockDim.x >> 5;
-  const unsigned long long nwarps = (unsigned long long)gridDim.x * wpb;
-  __shared__ uint32_t stage_u[kTakeThreads / 32][256], stage_d[kTakeThreads / 32][256];
-  __shared__ double stage_a[kTakeThreads / 32][256];
-  uint32_t* st_u = stage_u[threadIdx.x >> 5];
-  uint32_t* st_d = stage_d[threadIdx.x >> 5];
-  double* st_a = stage_a[threadIdx.x >> 5];
-  for (unsigned long long t = blockIdx.x * wpb + (threadIdx.x >> 5); t < ntiles; t += nwarps) {
-    const uint32_t s = b.alist[t / tps];
-    if (b.balance && b.stopped[s]) continue;  // warp-uniform: stopped before its first push
-    if (b.light[s]) {  // warp-uniform: only the tiles this round's spread added to
-      uint8_t* flag = b.tile_dirty + (unsigned long long)s * b.tiles + t % tps;
-      if (*flag == 0) continue;
-      __syncwarp();
-      if (lane == 0) *flag = 0;
+  const unsigned long long g0 = (unsigned long long)gr * G * (unsigned long long)g.n;
+  __syncwarp();
+  // the entries' degrees; their chunks of kHubChunk edges (of distinct nodes of one group: at
+  // most the graph's); places in the queue
+  uint32_t hubs = 0;
+  for (uint32_t e = lane; e < mine; e += 32) {
+    const uint32_t u = st.u[e], rb = __ldg(g.row + u), d = __ldg(g.row + u + 1) - rb;
+    st.rb[e] = rb;
+    st.d[e] = d;
+    hubs += hub_chunks_of(d);
+  }
+  const uint32_t hsum = __reduce_add_sync(kFull, hubs);
+  uint32_t qb = 0, hb = 0;
+  if (lane == 0) {
+    qb = atomicAdd(&b.slot_cnt[(size_t)nx * b.cnt_stride + gr], mine);
+    if (hsum) hb = atomicAdd(&b.slot_cnt[(size_t)(2 + nx) * b.cnt_stride + gr], hsum);
+  }
+  __syncwarp();
+  if (b.balance) {
+    for (uint32_t x = lane; x < mine * G; x += 32)
+      tc.moved = __dadd_rn(tc.moved, __dmul_rn(alpha, st.a[x]));
+    __syncwarp();
+  }
+  // the take of every taken residue: reserve += alpha a, r = 0, spread increment
+  for (uint32_t i = lane; i < pairs; i += 32) {
+    const uint32_t p = st.pair[i], u = st.u[p / G];
+    const unsigned long long at = g0 + (unsigned long long)u * w + p % G;
+    const double a = st.a[p];
+    const double rs = __ldcg(b.res + at), inv = __ldg(g.invd + u);
+    b.r[at] = 0.0;
+    b.res[at] = __fma_rn(alpha, a, rs);
+    st.a[p] = __dmul_rn(__dmul_rn(beta, a), inv);  // (1 - alpha) a / d
+  }
+  qb = __shfl_sync(kFull, qb, 0);
+  hb = __shfl_sync(kFull, hb, 0);
+  __syncwarp();
+  for (uint32_t x = lane; x < mine * G; x += 32) {  // increments, and the sources' counters
+    const uint32_t e = x / G;
+    const double inc = st.a[x];
+    if (nonzero(inc)) {
+      ++tc.cnt;
+      tc.deg += st.d[e];
     }
-    const uint32_t tb = (uint32_t)((t % tps) * kTileNodes);
-    const double rm = b.rmax[s];
-    const float rmf = __double2float_rn(rm);
-    const bool fast = rmf >= 0x1p-100f && rmf <= 0x1p60f;
-    const unsigned long long g0 = (unsigned long long)s * n;
-    uint32_t t_cnt = 0;
-    unsigned long long t_d = 0;
-    double t_moved = 0.0;  // this lane's alpha a of the tile (balanced push only)
-#pragma unroll 1
-    for (uint32_t k0 = 0; k0 < kTileNodes / 32; k0 += 8) {
-      // 256 consecutive nodes: residues and row offsets (nodes past n read row[n], so
-      // their degree is 0) loaded before any is used; the row offset that ends the last
-      // node of a word is the next lane's, and for lane 31 the next word's first
-      const uint32_t ub = tb + k0 * 32;
-      double rv[8];
-      uint32_t d[8];
-#pragma unroll
-      for (int kk = 0; kk < 8; ++kk) {
-        const uint32_t u = ub + kk * 32 + lane;
-        rv[kk] = u < n ? b.r[g0 + u] : 0.0;
-        d[kk] = g.row[min((unsigned long long)u, n)];
-      }
-      const uint32_t tail = g.row[min((unsigned long long)(ub + 256), n)];
-      uint32_t m[8], any = 0, mine = 0, my_h = 0, my_d = 0;
-#pragma unroll
-      for (int kk = 0; kk < 8; ++kk) {
-        const uint32_t first_next = kk < 7 ? __shfl_sync(kFull, d[kk + 1], 0) : tail;
-        const uint32_t down = __shfl_down_sync(kFull, d[kk], 1);
-        d[kk] = (lane < 31 ? down : first_next) - d[kk];
-      }
-      uint32_t above = 0, undecided = 0;  // bit kk: word kk of this lane
-#pragma unroll
-      for (int kk = 0; kk < 8; ++kk) {
-        const uint32_t f = threshold_fast(rv[kk], rmf, fast, d[kk]);
-        above |= (f == 1u ? 1u : 0u) << kk;
-        undecided |= (f == 2u ? 1u : 0u) << kk;
-      }
-      if (__any_sync(kFull, undecided != 0)) {  // rare: a residue within 2^-19 of its threshold
-        for (int kk = 0; kk < 8; ++kk)
-          if (((undecided >> kk) & 1u) && threshold_exact(rv[kk], rm, d[kk])) above |= 1u << kk;
-      }
-#pragma unroll
-      for (int kk = 0; kk < 8; ++kk) {
-        const bool cross = (above >> kk) & 1u;
-        m[kk] = __ballot_sync(kFull, cross);
-        any |= m[kk];
-        mine += __popc(m[kk]);
-        if (cross) {
-          my_h += hub_chunks_of(d[kk]);
-          my_d += d[kk];
-        }
-      }
-      if (any == 0) continue;  // warp-uniform
-      // distinct nodes of one source: their degrees sum to at most m < 2^32
-      const uint32_t hsum = __reduce_add_sync(kFull, my_h);
-      t_d += __reduce_add_sync(kFull, my_d);
-      t_cnt += mine;
-      uint32_t qb = 0, hb = 0;
-      if (lane == 0) {
-        qb = atomicAdd(&cnt_nx[s], mine);
-        if (hsum) hb = atomicAdd(&hcnt_nx[s], hsum);
-      }
-      qb = __shfl_sync(kFull, qb, 0);
-      hb = __shfl_sync(kFull, hb, 0);
-      // the batch's crossing nodes, packed in (word, lane) order into this warp's stage,
-      // so the take's FP64 arithmetic runs on 32 crossing nodes per instruction
-      {
-        uint32_t before = 0;
-#pragma unroll
-        for (int kk = 0; kk < 8; ++kk) {
-          if ((m[kk] >> lane) & 1u) {
-            const uint32_t e = before + __popc(m[kk] & lt_mask);
-            st_u[e] = ub + kk * 32 + lane;
-            st_d[e] = d[kk];
-            st_a[e] = rv[kk];
-          }
-          before += __popc(m[kk]);
-        }
-      }
-      __syncwarp();
-      uint32_t hp = hb;
-      for (uint32_t e0 = 0; e0 < mine; e0 += 32) {
-        const uint32_t e = e0 + lane;
-        const bool live = e < mine;
-        uint32_t u = 0, dk = 1;
-        double a = 0.0, rs = 0.0, inv = 0.0;
-        if (live) {
-          u = st_u[e];
-          dk = st_d[e];
-          a = st_a[e];
-          rs = b.res[g0 + u];
-          inv = g.invd[u];
-        }
-        const uint32_t nch = live ? hub_chunks_of(dk) : 0u;
-        const uint32_t nch_incl = hsum ? warp_incl_scan(nch) : 0u;  // lower entries first
-        if (live && FORA_IN_RANGE(b.err, qb + e, n) &&
-            FORA_IN_RANGE(b.err, hp + nch_incl, b.hub_stride + 1)) {
-          const unsigned long long gi = g0 + u;
-          // the take: reserve += alpha a, r = 0, spread increment
-          b.r[gi] = 0.0;
-          const double moved = __dmul_rn(alpha, a);
-          b.res[gi] = __dadd_rn(rs, moved);
-          if (b.balance) t_moved = __dadd_rn(t_moved, moved);
-          const unsigned long long qi = g0 + qb + e;
-          qn[qi] = ((unsigned long long)s << 32) | u;
-          b.fa[qi] = __dmul_rn(__dmul_rn(beta, a), inv);  // (1 - alpha) a / d
-          const unsigned long long hbase =
-              (unsigned long long)s * b.hub_stride + hp + (nch_incl - nch);
-          for (uint32_t c = 0; c < nch; ++c) hn[hbase + c] = (qi << kHubChunkBits) | c;
-        }
-        if (hsum) hp += __shfl_sync(kFull, nch_incl, 31);
-      }
-      __syncwarp();
+    if (j < w && FORA_IN_RANGE(b.err, qb + e, g.n))
+      b.fa[g0 + (unsigned long long)(qb + e) * w + j] = inc;
+  }
+  const unsigned long long h0 = (unsigned long long)gr * G * b.hub_stride;
+  for (uint32_t e0 = 0; e0 < mine; e0 += 32) {
+    const uint32_t e = e0 + lane;
+    uint32_t rb = 0, d = 0;
+    if (e < mine) {
+      rb = st.rb[e];
+      d = st.d[e];
+      if (FORA_IN_RANGE(b.err, qb + e, g.n)) b.q[g0 + qb + e] = make_uint2(rb, d);
     }
-    if (b.balance && t_cnt) {  // warp-uniform
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) t_moved = __dadd_rn(t_moved, __shfl_down_sync(kFull, t_moved, o));
+    if (hsum) {  // warp-uniform
+      const uint32_t nch = hub_chunks_of(d);
+      const uint32_t incl = warp_incl_scan(nch);  // lower entries first
+      const uint32_t at = hb + incl - nch;
+      if (nch && FORA_IN_RANGE(b.err, hb + incl, (unsigned long long)w * b.hub_stride + 1)) {
+        for (uint32_t c = 0; c < nch; ++c) {
+          b.hub[h0 + at + c] = make_uint2(qb + e, rb + c * kHubChunk);
+          b.hub_len[h0 + at + c] = min(kHubChunk, d - c * kHubChunk);
+        }
+      }
+      hb += __shfl_sync(kFull, incl, 31);
     }
-    if (lane == 0 && t_cnt) {
-      atomicAdd(&b.stats[s].pushes, (unsigned long long)t_cnt);
-      atomicAdd(&b.stats[s].edge_pushes, t_d);
-      if (b.balance) atomicAdd(&b.stats[s].moved, t_moved);
+  }
+  __syncwarp();
+}
+
+// Makes gr the warp's group: takes what is staged of the one before and adds its counters.
+template <int G>
+__device__ __forceinline__ void take_enter(const GraphDev& g, const BatchDev& b, int nx,
+                                           uint32_t gr, TakeStage<G>& st, TakeGroup& tg,
+                                           TakeCount& tc) {
+  const uint32_t lane = lane_id(), j = lane % G;
+  if (tg.mine) take_stage<G>(g, b, nx, tg.gr, tg.w, tg.mine, tg.pairs, st, tc);
+  if (__any_sync(kFull, tc.cnt != 0)) {
+    sum_count<G>(b, tc);
+    if (lane < (uint32_t)G) add_count(b, tc.gr * G + lane, tc.cnt, tc.deg, tc.moved);
+  }
+  tc = TakeCount();
+  tc.gr = gr;
+  tg = TakeGroup();
+  tg.gr = gr;
+  tg.w = width_of<G>(b, gr);
+  const uint32_t slot = gr * G + j;
+  tg.live = j < tg.w && slot < (uint32_t)b.nsrc && !(b.balance && __ldcg(&b.stopped[slot]));
+  tg.rmf = __double2float_rn(tg.live ? __ldcg(&b.rmax[slot]) : 1.0);
+  tg.mask = tg.rmf >= 0x1p-100f && tg.rmf <= 0x1p60f ? ~0u : 0u;
+}
+
+// Part `unit` of the warp's group (L loads per lane, so 32 L / G consecutive nodes; a unit is
+// 8 / L of them): the nodes that cross their source's threshold go to the stage.
+template <int G, int L>
+__device__ __forceinline__ void take_unit(const GraphDev& g, const BatchDev& b, int nx,
+                                          uint32_t unit, TakeStage<G>& st, TakeGroup& tg,
+                                          TakeCount& tc) {
+  constexpr uint32_t kNodes = 32 * L / G;  // nodes of a part
+  constexpr uint32_t kStep = 32 / G;       // nodes per load
+  constexpr uint32_t kEach = (uint32_t)(0xFFFFFFFFull / ((1ull << G) - 1));  // every G-th bit
+  const uint32_t lane = lane_id(), j = lane % G, w = tg.w;
+  const uint32_t n = (uint32_t)g.n;
+  const uint32_t ub = unit * kNodes;
+  if (ub >= n) return;
+  if (b.hot_copies) {
+    const uint32_t h1 = g.hot_first[(min(ub + kNodes, n) - 1) / kHotSpan + 1];
+    for (uint32_t h = g.hot_first[ub / kHotSpan]; h < h1; ++h) {
+      const uint32_t v = __ldg(g.hot_node + h);
+      if (v >= ub && v < ub + kNodes) fold_hot<G>(g, b, tg.gr, h);
+    }
+  }
+  const unsigned long long g0 = (unsigned long long)tg.gr * G * (unsigned long long)n;
+  const uint32_t first = ub + lane / G;  // this lane's nodes: first, first + kStep, ...
+  const uint32_t mine = tg.live && first < n ? (n - first + kStep - 1) / kStep : 0u;
+  const double* r = b.r + g0 + (unsigned long long)first * w + j;
+  const float* deg = g.fdeg + first;
+  double rv[L];
+  uint32_t cand = 0, above = 0;  // bit k: the node of load k may be, is above its threshold
+  {
+    float d[L];
+#pragma unroll
+    for (int k = 0; k < L; ++k) {
+      rv[k] = k < mine ? __ldcg(r + (unsigned long long)(k * kStep) * w) : 0.0;
+      d[k] = k < mine ? __ldg(deg + k * kStep) : 1.0f;
+    }
+    // threshold_fast(...): the upper word of r against the threshold's -1 and +1
+#pragma unroll
+    for (int k = 0; k < L; ++k) {
+      const uint32_t hi = (uint32_t)((unsigned long long)__double_as_longlong(rv[k]) >> 32);
+      const uint32_t t = threshold_word(tg.rmf, d[k]);
+      if (k < mine && hi >= ((t - 1u) & tg.mask)) cand |= 1u << k;
+      if (hi > (t + 1u | ~tg.mask)) above |= 1u << k;
+    }
+    above &= cand;
+  }
+  if (!__any_sync(kFull, cand != 0)) return;
+  uint32_t open = cand & ~above;
+  while (__any_sync(kFull, open != 0)) {  // a residue within 2^-19 of its threshold: rare
+    if (open) {
+      const uint32_t k = __ffs(open) - 1;
+      open &= open - 1;
+      double x = rv[0];
+#pragma unroll
+      for (uint32_t k2 = 1; k2 < L; ++k2) x = k2 == k ? rv[k2] : x;
+      const uint32_t u = first + k * kStep;
+      if (threshold_exact(x, __ldcg(&b.rmax[tg.gr * G + j]),
+                          __ldg(g.row + u + 1) - __ldg(g.row + u)))
+        above |= 1u << k;
+    }
+  }
+#pragma unroll
+  for (int k = 0; k < L; ++k) {
+    const bool cross = (above >> k) & 1u;
+    const uint32_t bal = __ballot_sync(kFull, cross);
+    if (bal == 0) continue;  // warp-uniform
+    uint32_t m = bal;  // one bit per node that some source takes
+    if (G > 1) {
+#pragma unroll
+      for (int s = 1; s < G; s <<= 1) m |= m >> s;
+      m &= kEach;
+    }
+    const uint32_t e = tg.mine + __popc(m & ((1u << (lane / G * G)) - 1u));
+    if ((m >> (lane / G * G)) & 1u) {
+      if (j == 0) st.u[e] = ub + k * kStep + lane / G;
+      st.a[e * G + j] = cross ? rv[k] : 0.0;
+    }
+    if (cross) st.pair[tg.pairs + __popc(bal & ((1u << lane) - 1u))] = (uint16_t)(e * G + j);
+    tg.mine += __popc(m);
+    tg.pairs += __popc(bal);
+  }
+  if (tg.mine > kCarry) {
+    take_stage<G>(g, b, nx, tg.gr, w, tg.mine, tg.pairs, st, tc);
+    tg.mine = tg.pairs = 0;
+  }
+}
+
+// The take: every unit of a group with a heavy round (listed in b.alist), and the listed units
+// of the groups with light ones.  A warp reads consecutive units, so its counters belong to one
+// or two groups; what is left of them at the end a block adds together.
+template <int G, int L>
+__device__ void take_phase(const GraphDev& g, const BatchDev& b, int nx, uint32_t nheavy,
+                           uint32_t nlist, TakeStage<G>& st) {
+  const unsigned long long nwarps = (unsigned long long)gridDim.x * (blockDim.x >> 5);
+  const unsigned long long warp =
+      (unsigned long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+  TakeCount tc;
+  TakeGroup tg;
+  constexpr uint32_t kParts = 8 / L;  // of a unit
+  const uint32_t per = b.tiles * kParts;
+  const unsigned long long units = (unsigned long long)nheavy * per;
+  unsigned long long x = units * warp / nwarps;
+  const unsigned long long end = units * (warp + 1) / nwarps;
+  if (x < end) {
+    unsigned long long ga = x / per;
+    uint32_t unit = (uint32_t)(x - ga * per);
+    uint32_t gr = b.ngrp == 1 ? 0u : __ldcg(&b.alist[ga]);
+    for (;;) {
+      if (gr != tg.gr) take_enter<G>(g, b, nx, gr, st, tg, tc);
+      take_unit<G, L>(g, b, nx, unit, st, tg, tc);
+      if (++x >= end) break;
+      if (++unit == per) {
+        unit = 0;
+        gr = __ldcg(&b.alist[++ga]);
+      }
+    }
+  }
+  const unsigned long long listed = (unsigned long long)nlist * kParts;
+  x = listed * warp / nwarps;
+  const unsigned long long lend = listed * (warp + 1) / nwarps;
+  for (; x < lend; ++x) {
+    const uint32_t t = __ldcg(&b.tlist[x / kParts]);
+    const uint32_t gr = t / b.tiles;
+    if (lane_id() == 0) b.dirty[t >> 5] = 0;  // every unit marked in the word is listed
+    // a group that a joining source made heavy is scanned above
+    if (!(__ldcg(&b.light[gr]) & kGroupLight)) continue;
+    if (gr != tg.gr) take_enter<G>(g, b, nx, gr, st, tg, tc);
+    take_unit<G, L>(g, b, nx, (t - gr * b.tiles) * kParts + (uint32_t)(x % kParts), st, tg, tc);
+  }
+  if (tg.mine) take_stage<G>(g, b, nx, tg.gr, tg.w, tg.mine, tg.pairs, st, tc);
+  __shared__ uint32_t s_gr[kPushWarps], s_cnt[kPushWarps][G];
+  __shared__ unsigned long long s_deg[kPushWarps][G];
+  __shared__ double s_moved[kPushWarps][G];
+  const uint32_t wid = threadIdx.x >> 5;
+  sum_count<G>(b, tc);
+  if (lane_id() < (uint32_t)G) {
+    s_cnt[wid][lane_id()] = tc.cnt;
+    s_deg[wid][lane_id()] = tc.deg;
+    s_moved[wid][lane_id()] = tc.moved;
+    s_gr[wid] = tc.gr;
+  }
+  __syncthreads();
+  if (threadIdx.x < G) {
+    uint32_t cnt = 0;
+    unsigned long long deg = 0;
+    double moved = 0.0;
+    for (int k = 0; k < kPushWarps; ++k) {
+      cnt += s_cnt[k][threadIdx.x];
+      deg += s_deg[k][threadIdx.x];
+      if (b.balance) moved = __dadd_rn(moved, s_moved[k][threadIdx.x]);
+      if (k + 1 == kPushWarps || s_gr[k + 1] != s_gr[k]) {
+        add_count(b, s_gr[k] * G + threadIdx.x, cnt, deg, moved);
+        cnt = 0;
+        deg = 0;
+        moved = 0.0;
+      }
     }
   }
 }
 
-// End of a round (one block): the new frontier's per-source group and hub-item prefixes,
-// the list of sources that still push, zeroed counters for the round after, and the
-// loop condition (at most b.max_rounds push rounds).
-__global__ void __launch_bounds__(1024) k_push_advance(BatchDev b,
-                                                       cudaGraphConditionalHandle loop,
-                                                       int in_graph) {
+// ---------------------------------------------------------------- advance
+
+// What the advance decides for group gr from its sources' counters: its next take, and whether
+// that scans every node.
+template <int G>
+__device__ __forceinline__ void advance_group(const BatchDev& b, int gr, bool* light,
+                                              bool* heavy) {
+  bool take = false, halved = false;
+  unsigned long long round_edges = 0;
+  unsigned long long ep[G], last[G];
+#pragma unroll
+  for (int j = 0; j < G; ++j) {
+    const int s = min(gr * G + j, b.nsrc - 1);
+    ep[j] = __ldcg(&b.stats[s].edge_pushes);
+    last[j] = __ldcg(&b.last_edges[s]);
+  }
+#pragma unroll
+  for (int j = 0; j < G; ++j) {
+    const int s = gr * G + j;
+    if (s >= b.nsrc) break;
+    const unsigned long long pushed = ep[j] - last[j];  // this round's
+    if (pushed) {
+      b.last_edges[s] = ep[j];
+      atomicAdd(&b.stats[s].rounds, 1u);  // a push round of this source
+      round_edges += pushed;
+    }
+    // does the source's next take run: it found a frontier, or (balanced push) the cost
+    // rule lets it go on, with the threshold halved when no node was above it
+    bool on = pushed > 0;
+    if (b.balance) {
+      on = false;
+      if (!__ldcg(&b.stopped[s])) {
+        const SlotStats& st = b.stats[s];
+        const double fc = __dadd_rn(__dmul_rn(b.cost_edge, (double)ep[j]),
+                                    __dmul_rn(b.cost_push, (double)__ldcg(&st.pushes)));
+        const double wc = __dmul_rn(__dmul_rn(__dadd_rn(1.0, -__ldcg(&st.moved)), b.bal_scale),
+                                    b.cost_walk);
+        if (fc >= wc) {
+          b.stopped[s] = 1u;  // the frontier just taken is still spread
+        } else {
+          if (!pushed) {
+            b.theta[s] = __dmul_rn(0.5, __ldcg(&b.theta[s]));
+            halved = true;
+          }
+          on = true;
+        }
+      }
+    }
+    take |= on;
+  }
+  // the frontier just taken is spread next; a light one lets the next take scan only the
+  // tiles it touches (a halved threshold needs a full scan)
+  *light = take && !halved && round_edges < b.light_edges;
+  *heavy = take && !*light;
+}
+
+// End of a round (one block; up to 32 groups: its first warp): the new frontier's per-group item
+// prefixes, the list of groups that still push, zeroed counters for the round after, and the
+// loop condition (at most b.max_rounds push rounds), which thread 0 returns.  Items of the spread
+// are 32 entries, fewer where 32 would leave some of nwarps warps without one.
+template <int G>
+__device__ bool advance_phase(const BatchDev& b, int nx, uint32_t nwarps) {
   PushState* ps = b.ps;
-  const int cur = ps->cur, nx = cur ^ 1;
-  const int nsrc = b.nsrc;
   const size_t cs = (size_t)b.cnt_stride;
   const uint32_t* cnt_nx = b.slot_cnt + (size_t)nx * cs;
   const uint32_t* hcnt_nx = b.slot_cnt + (size_t)(2 + nx) * cs;
-  uint32_t* cnt_cur = b.slot_cnt + (size_t)cur * cs;
-  uint32_t* hcnt_cur = b.slot_cnt + (size_t)(2 + cur) * cs;
-  __shared__ unsigned long long carry_g, carry_h, carry_a;
-  if (threadIdx.x == 0) { carry_g = 0; carry_h = 0; carry_a = 0; }
-  __syncthreads();
-  for (int base = 0; base < nsrc; base += blockDim.x) {
-    const int s = base + (int)threadIdx.x;
-    const uint32_t c = s < nsrc ? cnt_nx[s] : 0u;
-    const uint32_t h = s < nsrc ? hcnt_nx[s] : 0u;
-    // does the source's next take run: it found a frontier, or (balanced push) the cost
-    // rule lets it go on, with the threshold halved when no node was above it
-    bool take = c > 0;
-    if (s < nsrc && b.balance) {
-      if (b.stopped[s]) {
-        take = false;
-      } else {
-        const SlotStats& st = b.stats[s];
-        const double fc = __dadd_rn(__dmul_rn(b.cost_edge, (double)st.edge_pushes),
-                                    __dmul_rn(b.cost_push, (double)st.pushes));
-        const double wc = __dmul_rn(__dmul_rn(__dadd_rn(1.0, -st.moved), b.bal_scale), b.cost_walk);
-        if (fc >= wc) {
-          b.stopped[s] = 1u;  // the frontier just taken is still spread
-          take = false;
-        } else {
-          if (c == 0) b.theta[s] = __dmul_rn(0.5, b.theta[s]);
-          take = true;
-        }
-      }
+  uint32_t* cnt_cur = b.slot_cnt + (size_t)(nx ^ 1) * cs;
+  uint32_t* hcnt_cur = b.slot_cnt + (size_t)(2 + (nx ^ 1)) * cs;
+  const bool small = b.ngrp <= 32;
+  if (small && threadIdx.x >= 32) return false;
+  unsigned long long carry_g = 0, carry_h = 0, carry_heavy = 0, carry_light = 0;
+  const uint32_t round = __ldcg(&ps->round) + 1;
+  uint32_t span = kSpan;
+  for (int base = 0; base < b.ngrp; base += blockDim.x) {
+    const int gr = base + (int)threadIdx.x;
+    const uint32_t c = gr < b.ngrp ? __ldcg(&cnt_nx[gr]) : 0u;
+    const uint32_t h = gr < b.ngrp ? __ldcg(&hcnt_nx[gr]) : 0u;
+    bool light = false, heavy = false;
+    if (gr < b.ngrp) advance_group<G>(b, gr, &light, &heavy);
+    if (small) {
+      const uint32_t all = __reduce_add_sync(kFull, min(c, 1u << 26));
+      while (span > 4 && all < span / 2 * nwarps) span /= 2;
     }
-    if (s < nsrc && c > 0) b.stats[s].rounds += 1u;  // a push round of this source
-    if (s < nsrc) {
-      // the frontier just taken is spread next; a light one lets the next take scan only
-      // the tiles it touches (a halved threshold needs a full scan)
-      const unsigned long long ep = b.stats[s].edge_pushes;
-      const unsigned long long round_edges = ep - b.last_edges[s];
-      b.last_edges[s] = ep;
-      const bool halved = b.balance && take && c == 0;
-      b.light[s] = (take && !halved && round_edges < b.light_edges) ? 1 : 0;
+    const unsigned long long items = (c + span - 1u) / span;
+    unsigned long long ge, he, gt, ht, ae, le, at, lt;
+    if (small) {
+      const uint32_t mh = __ballot_sync(kFull, heavy), ml = __ballot_sync(kFull, light);
+      ge = warp_incl_scan(items);
+      he = warp_incl_scan((unsigned long long)h);
+      gt = __shfl_sync(kFull, ge, 31);
+      ht = __shfl_sync(kFull, he, 31);
+      ge -= items;
+      he -= h;
+      ae = __popc(mh & ((1u << lane_id()) - 1u));
+      at = __popc(mh);
+      lt = __popc(ml);
+    } else {
+      block_scan2(items, h, &ge, &he, &gt, &ht);
+      block_scan2(heavy ? 1u : 0u, light ? 1u : 0u, &ae, &le, &at, &lt);
     }
-    unsigned long long ge, he, gt, ht, ae, ze, at, zt;
-    block_scan2((c + 31u) / 32u, h, &ge, &he, &gt, &ht);
-    block_scan2(take ? 1u : 0u, 0u, &ae, &ze, &at, &zt);
-    if (s < nsrc) {
-      b.gpre[s] = carry_g + ge;
-      b.hpre[s] = carry_h + he;
-      if (take) b.alist[carry_a + ae] = (uint32_t)s;
-      cnt_cur[s] = 0;  // counters of the frontier just spread: they serve the round after
-      hcnt_cur[s] = 0;
+    if (gr < b.ngrp) {
+      b.gpre[gr] = carry_g + ge;
+      b.hpre[gr] = carry_h + he;
+      b.light[gr] =
+          (uint8_t)((light ? kGroupLight : 0u) | (light || heavy ? kGroupActive : 0u));
+      if (heavy) b.alist[carry_heavy + ae] = (uint32_t)gr;
+      cnt_cur[gr] = 0;  // counters of the frontier just spread: they serve the round after
+      hcnt_cur[gr] = 0;
     }
-    __syncthreads();
-    if (threadIdx.x == 0) { carry_g += gt; carry_h += ht; carry_a += at; }
-    __syncthreads();
+    carry_g += gt;
+    carry_h += ht;
+    carry_heavy += at;
+    carry_light += lt;
   }
+  // ps->round passes have run; the last one took the frontier of push round ps->round (the
+  // first pass only finds F_0), so going on is allowed while that is <= the cap.  Another pass
+  // is needed while a group takes again or a taken frontier waits for its spread (of a source
+  // the cost rule just stopped).
+  const bool more = carry_heavy + carry_light > 0 || carry_g > 0 || carry_h > 0;
+  const bool go = more && round <= b.max_rounds;
   if (threadIdx.x == 0) {
-    b.gpre[nsrc] = carry_g;
-    b.hpre[nsrc] = carry_h;
+    b.gpre[b.ngrp] = carry_g;
+    b.hpre[b.ngrp] = carry_h;
     ps->ngroups = carry_g;
     ps->nhub = carry_h;
-    ps->nact = (uint32_t)carry_a;
+    ps->nact = (uint32_t)(carry_heavy + carry_light);
+    b.ctl->nheavy = (uint32_t)carry_heavy;
+    b.ctl->nlist = 0;
+    b.ctl->span = span;
     ps->cur = nx;
-    ps->round += 1;
+    ps->round = round;
     b.work[0] = 0;  // dynamic work counters of the next spread
     b.work[16] = 0;
-    // ps->round passes have run; the last one took the frontier of push round ps->round
-    // (the first pass only finds F_0), so going on is allowed while that is <= the cap.
-    // Another pass is needed while a source takes again or a taken frontier waits for its
-    // spread (a source the cost rule just stopped).
-    const bool more = carry_a > 0 || carry_g > 0 || carry_h > 0;
-    const bool go = more && ps->round <= b.max_rounds;
     if (more && !go) atomicOr(b.err, kErrPushNotConverged);
     ps->go = go ? 1u : 0u;
-    if (in_graph) cudaGraphSetConditional(loop, go ? 1u : 0u);
+  }
+  return go;
+}
+
+// After the last round: copies of hot nodes that no take has added (sources that the cost rule
+// stopped).
+template <int G>
+__device__ void finish_phase(const GraphDev& g, const BatchDev& b) {
+  if (!b.hot_copies) return;
+  const unsigned long long nwarps = (unsigned long long)gridDim.x * (blockDim.x >> 5);
+  const unsigned long long warp =
+      (unsigned long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+  const unsigned long long total = (unsigned long long)b.ngrp * g.nhot;
+  for (unsigned long long x = warp; x < total; x += nwarps)
+    fold_hot<G>(g, b, (uint32_t)(x / g.nhot), (uint32_t)(x % g.nhot));
+}
+
+// ---------------------------------------------------------------- kernels
+
+// Zeroes `bytes` bytes at a 16-byte aligned address with all threads of the grid.
+__device__ __forceinline__ void grid_zero(void* p, unsigned long long bytes) {
+  const unsigned long long t = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x;
+  const unsigned long long nt = (unsigned long long)gridDim.x * blockDim.x;
+  const unsigned long long quads = bytes / 16;
+  for (unsigned long long i = t; i < quads; i += nt) ((uint4*)p)[i] = make_uint4(0u, 0u, 0u, 0u);
+  for (unsigned long long i = quads * 16 + t; i < bytes; i += nt) ((uint8_t*)p)[i] = 0;
+}
+
+// The state a push starts from, but for what seed_phase sets.
+__device__ __forceinline__ void zero_phase(const GraphDev& g, const BatchDev& b) {
+  const unsigned long long cells =
+      (unsigned long long)min(b.ngrp * b.gw, b.lay) * (unsigned long long)g.n;
+  grid_zero(b.r, cells * sizeof(double));
+  grid_zero(b.res, cells * sizeof(double));
+  grid_zero(b.hotr, (unsigned long long)b.hot_copies * b.lgrp * g.nhot * b.gw * sizeof(double));
+  grid_zero(b.dirty, ((unsigned long long)b.lgrp * b.tiles + 31) / 32 * 4);
+  grid_zero(b.slot_cnt, 4ull * b.cnt_stride * sizeof(uint32_t));
+  grid_zero(b.last_edges, (unsigned long long)b.lay * sizeof(unsigned long long));
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    b.work[0] = b.work[16] = 0;
+    b.ctl->nheavy = b.ctl->nlist = 0;
   }
 }
 
-// Sources joining a batch between two push rounds (serving): slots [first, first + k)
-// (their sources, r_max and zeroed state already in place) get r(s) = 1 and enter the next
-// take, and the frontier prefixes are extended over them (empty frontiers).  One block.
-// The push of a source depends only on its own residues, so a source that joins later runs
-// the same rounds as it would from the start.
-__global__ void k_push_join(GraphDev g, BatchDev b, int first, int k) {
-  PushState* ps = b.ps;
-  const unsigned long long gtot = b.gpre[first], htot = b.hpre[first];
-  const uint32_t nact = ps->nact;
-  for (int i = threadIdx.x; i < k; i += blockDim.x) {
-    const int slot = first + i;
-    const uint32_t src = (uint32_t)b.sources[slot];
-    b.r[(unsigned long long)slot * (unsigned long long)g.n + src] = 1.0;
-    b.alist[nact + i] = (uint32_t)slot;
-    b.light[slot] = 1;
-    b.tile_dirty[(unsigned long long)slot * b.tiles + src / kTileNodes] = 1;
-    b.gpre[slot + 1] = gtot;
-    b.hpre[slot + 1] = htot;
+// Meeting point of all blocks of a cooperative launch, its `count`-th (from 1).  With `work`,
+// block 0 runs it when all have arrived (always the same block: its instructions stay in that
+// SM's cache; run by whichever block came last they cost 10 us of fetches a round), lets the
+// others go on, and the value that its thread 0 returned comes back to every thread.  The waits
+// are bounded: a block that gives up reports kErrBarrier and gets 0, as then do the others.
+template <typename F>
+__device__ bool grid_meet(const BatchDev& b, uint32_t count, bool work, F f) {
+  __shared__ uint32_t s_value;
+  volatile uint32_t* arrived = b.meet;
+  volatile uint32_t* word = b.meet + 32;  // (meeting << 1) | value, in another sector
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    __threadfence();
+    atomicAdd(b.meet, 1u);
+    uint32_t polls = 0, v = 1;
+    if (work && blockIdx.x != 0) {
+      uint32_t w;
+      while (((w = *word) >> 1) < count && ++polls <= kMaxPolls)
+        if (polls > 64) __nanosleep(100);
+      v = w & 1u;
+    } else {
+      while (*arrived < count * gridDim.x && ++polls <= kMaxPolls)
+        if (polls > 64) __nanosleep(100);
+    }
+    if (polls > kMaxPolls) {
+      atomicOr(b.err, kErrBarrier);
+      v = 0;
+    }
+    s_value = v;
+    __threadfence();
   }
   __syncthreads();
-  if (threadIdx.x == 0) ps->nact = nact + (uint32_t)k;
+  bool v = s_value != 0;
+  if (work && blockIdx.x == 0 && v) {
+    v = f();
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      __threadfence();
+      *word = (count << 1) | (v ? 1u : 0u);
+      s_value = v ? 1u : 0u;
+    }
+    __syncthreads();
+    v = s_value != 0;
+  }
+  __syncthreads();
+  return v;
 }
 
-// The frontier test of k_push_take on given (r, r_max, d) triples.
+template <int G>
+union PushShared {
+  TakeStage<G> take[kPushWarps];
+  SpreadStage<G> spread[kPushWarps];
+};
+
+// Units per SM below which a batch is small: fewer than two for each of the 32 warps of 4 blocks.
+// (One query of a 2^14-node graph: 0.49 ms of push with whole units, 0.39 with quarters; from
+// two units a warp on the two differ by less than a percent.)
+constexpr unsigned long long kSmallUnits = 64;
+// 4 resident blocks (64 registers): 3 (no spilled register) took 130.4 ms where 4 take 121.5, 5
+// 138 (256 sources of a 2^20-node R-MAT graph).
+constexpr int kPushBlocks = 4;
+template <int G, int L>
+__global__ void __launch_bounds__(kPushThreads, kPushBlocks)
+    k_push(const __grid_constant__ GraphDev g, const __grid_constant__ BatchDev b) {
+  __shared__ PushShared<G> sh;
+  const PushState* ps = b.ps;
+  const PushCtl* ctl = b.ctl;
+  const uint32_t wid = threadIdx.x >> 5;
+  uint32_t met = 0;
+  zero_phase(g, b);
+  bool go = grid_meet(b, ++met, true, [&] {
+    seed_phase<G>(g, b);
+    return true;
+  });
+  for (int nx = 0; go; nx ^= 1) {
+    take_phase<G, L>(g, b, nx, __ldcg(&ctl->nheavy), __ldcg(&ctl->nlist), sh.take[wid]);
+    go = grid_meet(b, ++met, true,
+                   [&] { return advance_phase<G>(b, nx, gridDim.x * kPushWarps); });
+    if (!go) break;
+    spread_phase<G>(g, b, nx, __ldcg(&ps->nhub), __ldcg(&ps->ngroups), __ldcg(&ctl->span),
+                    sh.spread[wid]);
+    go = grid_meet(b, ++met, false, [] { return true; });
+  }
+  finish_phase<G>(g, b);
+}
+
+// The phases on their own.
+template <int G>
+__global__ void __launch_bounds__(kPushThreads) k_push_seed(const __grid_constant__ GraphDev g,
+                                                            const __grid_constant__ BatchDev b) {
+  seed_phase<G>(g, b);
+}
+__global__ void __launch_bounds__(kPushThreads) k_push_zero(const __grid_constant__ GraphDev g,
+                                                            const __grid_constant__ BatchDev b) {
+  zero_phase(g, b);
+}
+template <int G>
+__global__ void __launch_bounds__(kPushThreads, kPushBlocks)
+    k_push_spread(const __grid_constant__ GraphDev g, const __grid_constant__ BatchDev b) {
+  __shared__ SpreadStage<G> stage[kPushWarps];
+  spread_phase<G>(g, b, b.ps->cur, b.ps->nhub, b.ps->ngroups, b.ctl->span,
+                  stage[threadIdx.x >> 5]);
+}
+template <int G>
+__global__ void __launch_bounds__(kPushThreads, kPushBlocks)
+    k_push_take(const __grid_constant__ GraphDev g, const __grid_constant__ BatchDev b) {
+  __shared__ TakeStage<G> stage[kPushWarps];
+  take_phase<G, 8>(g, b, b.ps->cur ^ 1, b.ctl->nheavy, b.ctl->nlist, stage[threadIdx.x >> 5]);
+}
+template <int G>
+__global__ void __launch_bounds__(kPushThreads) k_push_advance(const __grid_constant__ BatchDev b) {
+  const int nx = b.ps->cur ^ 1;
+  __syncthreads();
+  advance_phase<G>(b, nx, 0u);
+}
+template <int G>
+__global__ void __launch_bounds__(kPushThreads) k_push_finish(const __grid_constant__ GraphDev g,
+                                                              const __grid_constant__ BatchDev b) {
+  finish_phase<G>(g, b);
+}
+
+// Sources joining a batch between two push rounds (serving): slots [first, first + k) (their
+// sources and r_max already in place, the places of their residues zeroed with the batch's) get
+// r(s) = 1; their groups enter the next take, scanned whole, and the prefixes are extended over
+// groups that are new.  One block.  The push of a source depends only on its own residues, so a
+// source that joins later runs the same rounds as it would from the start.
+template <int G>
+__global__ void __launch_bounds__(kPushThreads) k_push_join(const __grid_constant__ GraphDev g,
+                                                            const __grid_constant__ BatchDev b,
+                                                            int first, int k) {
+  PushState* ps = b.ps;
+  const int old_groups = (first + G - 1) / G;
+  const unsigned long long gtot = ps->ngroups, htot = ps->nhub;
+  for (int i = threadIdx.x; i < k; i += blockDim.x) {
+    const int slot = first + i;
+    const uint32_t src = (uint32_t)b.sources[slot], gr = (uint32_t)slot / G;
+    b.r[(unsigned long long)gr * G * (unsigned long long)g.n +
+        (unsigned long long)src * width_of<G>(b, gr) + slot % G] = 1.0;
+  }
+  for (int gr = old_groups + (int)threadIdx.x; gr < b.ngrp; gr += blockDim.x) {
+    b.gpre[gr + 1] = gtot;
+    b.hpre[gr + 1] = htot;
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    uint32_t nheavy = b.ctl->nheavy, nact = ps->nact;
+    for (int gr = first / G; gr < b.ngrp; ++gr) {
+      const uint32_t s = gr < old_groups ? b.light[gr] : 0u;
+      if (!(s & kGroupActive)) ++nact;
+      if (!(s & kGroupActive) || (s & kGroupLight)) b.alist[nheavy++] = (uint32_t)gr;
+      b.light[gr] = kGroupActive;
+    }
+    b.ctl->nheavy = nheavy;
+    ps->nact = nact;
+  }
+}
+
+// The frontier test of the take on given (r, r_max, d) triples.
 __global__ void k_threshold_table(const double* r, const double* rm, const uint32_t* d,
                                   uint8_t* out, int count) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -877,6 +1243,52 @@ __global__ void k_threshold_table(const double* r, const double* rm, const uint3
   const float rmf = __double2float_rn(rm[i]);
   const bool fast = rmf >= 0x1p-100f && rmf <= 0x1p60f;
   out[i] = above_threshold(r[i], rm[i], rmf, fast, d[i]) ? 1 : 0;
+}
+
+// [slot][n] arrays to and from the batch's grouped ones.
+__global__ void k_regroup(double* grouped, double* rows, unsigned long long n, int lay, int gw,
+                          int nsrc, int to_rows) {
+  const unsigned long long stride = (unsigned long long)gridDim.x * blockDim.x;
+  for (int slot = blockIdx.y; slot < nsrc; slot += gridDim.y) {
+    const int gr = slot / gw, w = min(gw, lay - gr * gw);
+    double* p = grouped + (unsigned long long)gr * gw * n + slot % gw;
+    double* q = rows + (unsigned long long)slot * n;
+    for (unsigned long long v = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x; v < n;
+         v += stride) {
+      if (to_rows) q[v] = p[v * w]; else p[v * w] = q[v];
+    }
+  }
+}
+
+template <int G, int L>
+cudaError_t push_t(const GraphDev& g, const BatchDev& b, int num_sms, cudaStream_t st) {
+  const int per_sm = resident_blocks((const void*)k_push<G, L>, kPushThreads);
+  if (per_sm == 0) return cudaErrorInvalidConfiguration;
+  // every SM at least once; more blocks only where a full scan has work for them
+  const unsigned long long parts = (unsigned long long)b.ngrp * b.tiles * (8 / L);
+  const unsigned long long want = (parts + kPushWarps - 1) / kPushWarps;
+  unsigned blocks = (unsigned)num_sms;
+  while (blocks < want && blocks < (unsigned)(num_sms * per_sm)) blocks += (unsigned)num_sms;
+  GraphDev gd = g;
+  BatchDev bd = b;
+  void* args[] = {&gd, &bd};
+  return cudaLaunchCooperativeKernel((const void*)k_push<G, L>, dim3(blocks), dim3(kPushThreads),
+                                     args, 0, st);
+}
+
+template <int G>
+cudaError_t push_round_t(const GraphDev& g, const BatchDev& b, int num_sms, cudaStream_t st) {
+  const int spread_per_sm = resident_blocks((const void*)k_push_spread<G>, kPushThreads);
+  const int take_per_sm = resident_blocks((const void*)k_push_take<G>, kPushThreads);
+  if (spread_per_sm == 0 || take_per_sm == 0) return cudaErrorInvalidConfiguration;
+  k_push_spread<G><<<num_sms * spread_per_sm, kPushThreads, 0, st>>>(g, b);
+  cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess) return e;
+  k_push_take<G><<<num_sms * take_per_sm, kPushThreads, 0, st>>>(g, b);
+  e = cudaGetLastError();
+  if (e != cudaSuccess) return e;
+  k_push_advance<G><<<1, kPushThreads, 0, st>>>(b);
+  return cudaGetLastError();
 }
 
 }  // namespace
@@ -888,38 +1300,53 @@ cudaError_t launch_threshold_table(const double* r, const double* rm, const uint
   return cudaGetLastError();
 }
 
+cudaError_t launch_push(const GraphDev& g, const BatchDev& b, int num_sms, cudaStream_t st) {
+  // a small batch's full scan has few units: a warp reads a quarter of one, which shortens a round
+  const bool small = (unsigned long long)b.ngrp * b.tiles < kSmallUnits * (unsigned)num_sms;
+  if (b.gw == 1) return small ? push_t<1, 2>(g, b, num_sms, st) : push_t<1, 8>(g, b, num_sms, st);
+  return small ? push_t<4, 2>(g, b, num_sms, st) : push_t<4, 8>(g, b, num_sms, st);
+}
+
+cudaError_t launch_push_start(const GraphDev& g, const BatchDev& b, int num_sms, cudaStream_t st) {
+  k_push_zero<<<num_sms * 8, kPushThreads, 0, st>>>(g, b);
+  cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess) return e;
+  if (b.gw == 1)
+    k_push_seed<1><<<1, kPushThreads, 0, st>>>(g, b);
+  else
+    k_push_seed<4><<<1, kPushThreads, 0, st>>>(g, b);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_push_round(const GraphDev& g, const BatchDev& b, int num_sms, cudaStream_t st) {
+  return b.gw == 1 ? push_round_t<1>(g, b, num_sms, st) : push_round_t<4>(g, b, num_sms, st);
+}
+
+cudaError_t launch_push_finish(const GraphDev& g, const BatchDev& b, int num_sms, cudaStream_t st) {
+  if (b.gw == 1)
+    k_push_finish<1><<<num_sms, kPushThreads, 0, st>>>(g, b);
+  else
+    k_push_finish<4><<<num_sms, kPushThreads, 0, st>>>(g, b);
+  return cudaGetLastError();
+}
+
 cudaError_t launch_push_join(const GraphDev& g, const BatchDev& b, int first, int k,
                              cudaStream_t st) {
   if (k <= 0) return cudaSuccess;
-  k_push_join<<<1, 256, 0, st>>>(g, b, first, k);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_push_seed(const GraphDev& g, const BatchDev& b, cudaStream_t st) {
-  const int threads = 256;
-  k_push_seed<<<(b.nsrc + threads - 1) / threads, threads, 0, st>>>(g, b);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_push_body(const GraphDev& g, const BatchDev& b, int num_sms,
-                             cudaGraphConditionalHandle loop, bool in_graph, cudaStream_t st) {
-  // one wave of resident blocks for the spread (with the dynamic work counter the warps
-  // in flight cover one contiguous window of the frontier) and for the take
-  const bool hot = b.spread_hot && g.scol && g.nhot > 0;
-  const void* spread = hot ? (const void*)k_push_spread_hot : (const void*)k_push_spread;
-  const int spread_per_sm = resident_blocks(spread, kSpreadThreads);
-  const int take_per_sm = resident_blocks((const void*)k_push_take, kTakeThreads);
-  if (spread_per_sm == 0 || take_per_sm == 0) return cudaErrorInvalidConfiguration;
-  if (hot)
-    k_push_spread_hot<<<num_sms * spread_per_sm, kSpreadThreads, 0, st>>>(g, b);
+  if (b.gw == 1)
+    k_push_join<1><<<1, kPushThreads, 0, st>>>(g, b, first, k);
   else
-    k_push_spread<<<num_sms * spread_per_sm, kSpreadThreads, 0, st>>>(g, b);
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  k_push_take<<<num_sms * take_per_sm, kTakeThreads, 0, st>>>(g, b);
-  e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  k_push_advance<<<1, 1024, 0, st>>>(b, loop, in_graph ? 1 : 0);
+    k_push_join<4><<<1, kPushThreads, 0, st>>>(g, b, first, k);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_regroup(double* grouped, double* rows, const BatchDev& b, int64_t n,
+                           bool to_rows, int num_sms, cudaStream_t st) {
+  uint64_t bx = ((uint64_t)n + 255) / 256;
+  const uint64_t most = ((uint64_t)num_sms * 32 + b.nsrc - 1) / b.nsrc;
+  if (bx > most) bx = most;
+  k_regroup<<<dim3((unsigned)bx, (unsigned)b.nsrc), 256, 0, st>>>(
+      grouped, rows, (unsigned long long)n, b.lay, b.gw, b.nsrc, to_rows ? 1 : 0);
   return cudaGetLastError();
 }
 

@@ -12,9 +12,9 @@
 
 namespace fora {
 
-// The residual kernels run at most this many blocks (8 per SM on up to 512 SMs), so the
-// per-block scan buffers have a size that does not depend on the device.
-constexpr int kMaxResidualGrid = 4096;
+// The residual list's unit counts of small batches have a buffer of this many pairs; larger
+// batches keep theirs in the top-k scratch, which is free then.
+constexpr int kUnitPairs = 4096;
 
 // Device bytes of every buffer of a query workspace for nsrc sources of a graph with n
 // nodes and hub_chunks hub items (workspace_sizes).  The workspace allocates exactly
@@ -34,25 +34,6 @@ void dfree(T*& p) {
   if (p) cudaFree((void*)p);
   p = nullptr;
 }
-
-// What an instantiated push-loop graph was built for.
-struct PushGraphKey {
-  uint64_t generation = 0;
-  int nsrc = 0;
-  double alpha = 0.0;
-  int spread_width = 0;
-  int spread_hot = 0;
-  uint32_t max_rounds = 0;
-  int balance = 0;
-  double bal[4] = {0, 0, 0, 0};  // C', cost_edge, cost_push, cost_walk (balanced push)
-  bool operator==(const PushGraphKey& o) const {
-    return generation == o.generation && nsrc == o.nsrc && alpha == o.alpha &&
-           spread_width == o.spread_width && spread_hot == o.spread_hot &&
-           max_rounds == o.max_rounds &&
-           balance == o.balance && bal[0] == o.bal[0] && bal[1] == o.bal[1] &&
-           bal[2] == o.bal[2] && bal[3] == o.bal[3];
-  }
-};
 
 // Device and pinned host buffers of one in-flight batched query (up to `cap` sources).
 // A graph owns one for its own entry points; the server owns one per lane.  A
@@ -78,10 +59,9 @@ struct Workspace {
   SlotStats* stats = nullptr;
   uint32_t* stopped = nullptr;        // [nsrc] balanced push: the cost rule stopped the source
   uint8_t* light = nullptr;           // [nsrc] light-round flags of the push take
-  uint8_t* tile_dirty = nullptr;      // [nsrc][tiles] tiles a light round's spread touched
+  uint8_t* tile_dirty = nullptr;      // tiles a light round's spread touched
   unsigned long long* last_edges = nullptr;  // [nsrc]
-  unsigned long long* blk = nullptr;  // [2][residual_grid]
-  int residual_grid = 0;
+  unsigned long long* blk = nullptr;  // [2][kUnitPairs]
   void* topk_scratch = nullptr;
   float* feat = nullptr;        // learned r_max: features [cap][16], predictions, r_max
   float* pred = nullptr;
@@ -98,15 +78,9 @@ struct Workspace {
   cudaEvent_t ev[5] = {nullptr, nullptr, nullptr, nullptr, nullptr};
 
   PushState* ps = nullptr;
-  uint64_t generation = 0;               // bumped whenever the buffers are reallocated
-  cudaGraphExec_t push_exec = nullptr;   // the push rounds as a device-side loop
-  PushGraphKey push_key;
-  cudaStream_t capture_stream = nullptr; // for capturing the loop body
   std::mutex mu;
 
   void release() {
-    if (push_exec) cudaGraphExecDestroy(push_exec);
-    push_exec = nullptr;
     dfree(ps);
     dfree(r); dfree(res); dfree(tally);
     dfree(q[0]); dfree(q[1]); dfree(hub[0]); dfree(hub[1]); dfree(fa);
@@ -126,7 +100,6 @@ struct Workspace {
   }
   ~Workspace() {
     release();
-    if (capture_stream) cudaStreamDestroy(capture_stream);
     for (int i = 0; i < 5; ++i)
       if (ev[i]) cudaEventDestroy(ev[i]);
   }
@@ -187,6 +160,7 @@ struct fora_graph {
   int32_t* col = nullptr;
   uint32_t* indeg = nullptr;  // in-degrees (features of the learned r_max)
   double* invd = nullptr;     // RN(1 / d(v)) per node
+  float* fdeg = nullptr;      // RN32(d(v)) per node
   // the walks' numbering and adjacency (GraphDev::wcol and the following)
   uint32_t* wcol = nullptr;
   uint32_t* wid = nullptr;
@@ -195,6 +169,7 @@ struct fora_graph {
   int ncls = 0, wbits = 1;
   uint32_t* scol = nullptr;   // the spread's target codes (GraphDev::scol), or null
   uint32_t* hot_node = nullptr;
+  uint8_t* hot_first = nullptr;  // GraphDev::hot_first
   int nhot = 0;
   // FORA+ walk index (Section 3.3): ends of omega_max(v) walks from every v
   unsigned long long* idx_off = nullptr;  // [n + 1] exclusive prefix of omega_max
@@ -212,8 +187,8 @@ struct fora_graph {
   fora::Workspace pipe_ws[fora::kMaxPipeline];
   cudaStream_t pipe_stream[fora::kMaxPipeline] = {};
   fora::GraphDev dev() const {
-    return fora::GraphDev{n,    m,    row,  col,   invd, wcol,     wid,
-                          wcls, wesc, ncls, wbits, fora::end_cols(n, wbits), scol, hot_node, nhot};
+    return fora::GraphDev{n,    m,    row,  col,   invd, fdeg, wcol,     wid,
+                          wcls, wesc, ncls, wbits, fora::end_cols(n, wbits), scol, hot_node, hot_first, nhot};
   }
 };
 

@@ -29,32 +29,40 @@ __device__ __forceinline__ u128 prefix_of(const TopkSlot& s) {
   return ((u128)s.pa << 32) | (u128)s.pb;
 }
 
-// One row of the grid per source, kEstNodes nodes per block: the walk ends are gathered (by walk
-// id), so few sources at a time keep their sectors in L2 until all four sums of each are used.
-// (19 blocks per source, 64 sources in flight: 5.3 ms for 256 sources of 2^20 nodes.)
+// One row of the grid per group of sources, kEstValues values per block: the walk ends are
+// gathered (by walk id), so few groups at a time keep their sectors in L2 until all four sums
+// of each are used.  (64 sources in flight: 5.3 ms for 256 sources of 2^20 nodes.)
 constexpr int kEstThreads = 256;
 constexpr int kEstPer = 8;
-constexpr int kEstNodes = kEstThreads * kEstPer;
+constexpr int kEstValues = kEstThreads * kEstPer;
+template <int G>
 __global__ void __launch_bounds__(kEstThreads) k_estimate(GraphDev g, BatchDev b, double* est) {
   const unsigned long long n = (unsigned long long)g.n;
-  const unsigned long long v0 = (unsigned long long)blockIdx.x * kEstNodes + threadIdx.x;
-  for (int slot = blockIdx.y; slot < b.nsrc; slot += gridDim.y) {
-    const unsigned long long g0 = (unsigned long long)slot * n;
+  const uint32_t j = threadIdx.x % G;
+  const unsigned long long v0 =
+      (unsigned long long)blockIdx.x * (kEstValues / G) + threadIdx.x / G;
+  for (int gr = blockIdx.y; gr < b.ngrp; gr += gridDim.y) {
+    const int slot = gr * G + (int)j;
+    const unsigned long long w = min(G, b.lay - gr * G);
+    if (slot >= b.nsrc) continue;
+    const unsigned long long g0 = (unsigned long long)gr * G * n;
     const unsigned long long e0 = (unsigned long long)slot * b.ends;
     unsigned long long acc[kEstPer];
 #pragma unroll
     for (int k = 0; k < kEstPer; ++k) {
-      const unsigned long long v = v0 + k * kEstThreads;
+      const unsigned long long v = v0 + k * (kEstThreads / G);
       acc[k] = v < n ? b.acc[e0 + end_place(g, walk_id(g, g.wid[v]))] : 0ull;
     }
 #pragma unroll
     for (int k = 0; k < kEstPer; ++k) {
-      const unsigned long long v = v0 + k * kEstThreads;
+      const unsigned long long v = v0 + k * (kEstThreads / G);
       if (v >= n) break;
       // pi_hat = reserve (+ alpha r with zero-hop pruning) + acc * 2^-63 (exact scaling)
-      const double res = b.res[g0 + v];
-      const double base = b.zero_hop ? __dadd_rn(res, __dmul_rn(b.alpha, b.r[g0 + v])) : res;
-      est[g0 + v] = __dadd_rn(base, __dmul_rn(__ull2double_rn(acc[k]), 0x1p-63));
+      const unsigned long long at = g0 + v * w + j;
+      const double res = b.res[at];
+      const double base = b.zero_hop ? __dadd_rn(res, __dmul_rn(b.alpha, b.r[at])) : res;
+      est[(unsigned long long)slot * n + v] =
+          __dadd_rn(base, __dmul_rn(__ull2double_rn(acc[k]), 0x1p-63));
     }
   }
 }
@@ -272,8 +280,12 @@ TopkScratch topk_scratch_carve(void* base, int nrows) {
 }
 
 cudaError_t launch_estimate(const GraphDev& g, const BatchDev& b, double* est, cudaStream_t st) {
-  const unsigned bx = (unsigned)((g.n + kEstNodes - 1) / kEstNodes);
-  k_estimate<<<dim3(bx, (unsigned)b.nsrc), kEstThreads, 0, st>>>(g, b, est);
+  const unsigned per = (unsigned)(kEstValues / b.gw);
+  const dim3 grid((unsigned)(((uint64_t)g.n + per - 1) / per), (unsigned)b.ngrp);
+  if (b.gw == 1)
+    k_estimate<1><<<grid, kEstThreads, 0, st>>>(g, b, est);
+  else
+    k_estimate<4><<<grid, kEstThreads, 0, st>>>(g, b, est);
   return cudaGetLastError();
 }
 

@@ -1,7 +1,7 @@
 // Walk phase of Alg. 2 over a batch of sources.
 //
 //   k_residual_count / k_residual_scan / k_residual_emit:
-//     R = {(slot, v) : r(v) > 0} in ascending (slot, v); omega_v = ceil(r(v) * C) with
+//     R = {(slot, v) : r(v) > 0} in ascending slot; omega_v = ceil(r(v) * C) with
 //     C = omega / r_sum (Alg. 2); exclusive offsets of omega_v over R (one flat
 //     walk index space for all sources) and the fixed-point weight
 //     W_v = rint(r(v)/omega_v * 2^63) of every walk from v (Alg. 2: a_v r_sum/omega).
@@ -10,6 +10,8 @@
 //     walk j = g - offset[i] of node v; it reads its own Philox4x32-10 stream with
 //     counter (c, j, v, s) and stops with probability alpha at every node
 //     (Section 2.1); count[end] += 1 and acc[end] += W_v.
+#include <algorithm>
+
 #include "fora_engine.cuh"
 
 namespace fora {
@@ -92,13 +94,6 @@ __device__ __forceinline__ double sampled(const BatchDev& b, double r) {
   return b.zero_hop ? __dmul_rn(__dadd_rn(1.0, -b.alpha), r) : r;
 }
 
-// Contiguous element range of block `blk` out of `nblk` over [0, total).
-__device__ __forceinline__ void block_range(unsigned long long total, int blk, int nblk,
-                                            unsigned long long* beg, unsigned long long* end) {
-  *beg = total * (unsigned long long)blk / (unsigned long long)nblk;
-  *end = total * (unsigned long long)(blk + 1) / (unsigned long long)nblk;
-}
-
 template <typename T>
 __device__ __forceinline__ T warp_incl_scan(T x) {
 #pragma unroll
@@ -134,118 +129,185 @@ __device__ __forceinline__ void block_excl_scan2(unsigned long long c, unsigned 
   __syncthreads();
 }
 
+// The residual list in three kernels.  A warp's unit is a share of the nodes of one group of
+// sources (G side by side, as the push leaves them; lane % G is the source), so neither pass
+// over the residues needs a block barrier: k_residual_count counts each source's entries and
+// walks per unit, k_residual_scan turns them into offsets (one block), k_residual_emit writes
+// the entries, computing the weights (an FP64 division each) on packed lanes.
+struct UnitRange {
+  uint32_t gr, k, w;          // group, share, sources side by side
+  uint32_t beg, end;          // its nodes
+  unsigned long long g0;      // of the group's residues
+};
+template <int G>
+__device__ __forceinline__ bool unit_range(const GraphDev& g, const BatchDev& b, UnitRange* u) {
+  const unsigned long long warp =
+      ((unsigned long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  if (warp >= (unsigned long long)b.ngrp * b.units) return false;
+  u->gr = (uint32_t)(warp / b.units);
+  u->k = (uint32_t)(warp - (unsigned long long)u->gr * b.units);
+  u->w = min((uint32_t)G, (uint32_t)b.lay - u->gr * G);
+  u->beg = (uint32_t)((unsigned long long)g.n * u->k / b.units);
+  u->end = (uint32_t)((unsigned long long)g.n * (u->k + 1) / b.units);
+  u->g0 = (unsigned long long)u->gr * G * (unsigned long long)g.n;
+  return true;
+}
+
+constexpr int kResidualLoads = 4;  // residues a lane reads before it uses any
+
+template <int G>
 __global__ void __launch_bounds__(kResidualThreads) k_residual_count(GraphDev g, BatchDev b) {
-  const unsigned long long total = (unsigned long long)b.nsrc * (unsigned long long)g.n;
-  unsigned long long beg, end;
-  block_range(total, blockIdx.x, gridDim.x, &beg, &end);
-  unsigned long long cnt = 0, walks = 0;
-  // per-source sums, flushed whenever this thread's elements move to another source
-  unsigned long long i = beg + threadIdx.x;
-  uint32_t slot = (uint32_t)(i / (unsigned long long)g.n);
-  unsigned long long slot_end = (unsigned long long)(slot + 1) * (unsigned long long)g.n;
-  unsigned long long s_cnt = 0, s_walks = 0;
-  double s_sum = 0.0;
+  UnitRange u;
+  if (!unit_range<G>(g, b, &u)) return;  // whole warps
+  constexpr uint32_t kStep = 32 / G;
+  const uint32_t lane = threadIdx.x & 31, j = lane % G, slot = u.gr * G + j;
+  const bool mine = j < u.w && slot < (uint32_t)b.nsrc;
   const float cf = __double2float_rn(b.walk_scale);
   const bool fast = cf >= 1.0f && cf <= 0x1p100f;
-  for (unsigned long long base = beg; base < end; base += kResidualThreads, i += kResidualThreads) {
-    const bool valid = i < end;
-    while (valid && i >= slot_end) {
-      if (s_cnt) {
-        atomicAdd(&b.stats[slot].residual_nodes, s_cnt);
-        atomicAdd(&b.stats[slot].walks, s_walks);
-        atomicAdd(&b.stats[slot].rsum, s_sum);
+  unsigned long long walks = 0;
+  uint32_t cnt = 0, some = 0;  // entries (at least one walk), residues above 0
+  double sum = 0.0;
+  for (uint32_t v0 = u.beg; v0 < u.end; v0 += kStep * kResidualLoads) {
+    double r[kResidualLoads];
+#pragma unroll
+    for (int k = 0; k < kResidualLoads; ++k) {
+      const uint32_t v = v0 + k * kStep + lane / G;
+      r[k] = mine && v < u.end ? b.r[u.g0 + (unsigned long long)v * u.w + j] : 0.0;
+    }
+#pragma unroll
+    for (int k = 0; k < kResidualLoads; ++k) {
+      // an entry of R needs at least one walk (omega_v = 0 only if r * C underflows)
+      const unsigned long long w = walks_of(sampled(b, r[k]), b.walk_scale, cf, fast);
+      if (__double_as_longlong(r[k]) != 0) {
+        cnt += w > 0 ? 1u : 0u;
+        walks += w;
+        ++some;
+        sum += r[k];
       }
-      s_cnt = 0; s_walks = 0; s_sum = 0.0;
-      ++slot;
-      slot_end += (unsigned long long)g.n;
-    }
-    const double r = valid ? b.r[i] : 0.0;
-    // an entry of R needs at least one walk (omega_v = 0 only if r * C underflows)
-    const unsigned long long w = walks_of(sampled(b, r), b.walk_scale, cf, fast);
-    if (__double_as_longlong(r) != 0) {
-      if (w > 0) { ++cnt; walks += w; }
-      ++s_cnt; s_walks += w; s_sum += r;
     }
   }
-  if (s_cnt && slot < (uint32_t)b.nsrc) {
-    atomicAdd(&b.stats[slot].residual_nodes, s_cnt);
-    atomicAdd(&b.stats[slot].walks, s_walks);
-    atomicAdd(&b.stats[slot].rsum, s_sum);
+#pragma unroll
+  for (int o = 16; o >= G; o >>= 1) {
+    cnt += __shfl_xor_sync(kFull, cnt, o);
+    some += __shfl_xor_sync(kFull, some, o);
+    walks += __shfl_xor_sync(kFull, walks, o);
+    sum += __shfl_xor_sync(kFull, sum, o);
   }
-  unsigned long long ce, we, ct, wt;
-  block_excl_scan2(cnt, walks, &ce, &we, &ct, &wt);
-  if (threadIdx.x == 0) {
-    b.blk_cnt[blockIdx.x] = ct;
-    b.blk_walks[blockIdx.x] = wt;
+  if (lane < (uint32_t)G && mine) {
+    const size_t at = (size_t)slot * b.units + u.k;
+    b.unit_cnt[at] = cnt;
+    b.unit_walks[at] = walks;
+    if (some) {
+      atomicAdd(&b.stats[slot].residual_nodes, (unsigned long long)some);
+      atomicAdd(&b.stats[slot].walks, walks);
+      atomicAdd(&b.stats[slot].rsum, sum);
+    }
   }
 }
 
-// One block: exclusive scan of the per-block totals; totals; per-source walk limit.
+// One block: exclusive scan of the units' counts, slot after slot; totals; per-source walk limit.
+// A thread scans consecutive units.
 __global__ void __launch_bounds__(1024) k_residual_scan(BatchDev b) {
-  __shared__ unsigned long long carry_c, carry_w;
-  if (threadIdx.x == 0) { carry_c = 0; carry_w = 0; }
-  __syncthreads();
-  for (int base = 0; base < b.residual_grid; base += blockDim.x) {
-    const int i = base + threadIdx.x;
-    const unsigned long long c = i < b.residual_grid ? b.blk_cnt[i] : 0;
-    const unsigned long long w = i < b.residual_grid ? b.blk_walks[i] : 0;
-    unsigned long long ce, we, ct, wt;
-    block_excl_scan2(c, w, &ce, &we, &ct, &wt);
-    if (i < b.residual_grid) {
-      b.blk_cnt[i] = carry_c + ce;
-      b.blk_walks[i] = carry_w + we;
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) { carry_c += ct; carry_w += wt; }
-    __syncthreads();
+  const uint32_t total = (uint32_t)b.nsrc * (uint32_t)b.units;
+  const uint32_t per = (total + blockDim.x - 1) / blockDim.x;
+  const uint32_t beg = min(threadIdx.x * per, total), end = min(beg + per, total);
+  unsigned long long c = 0, w = 0;
+  for (uint32_t i = beg; i < end; ++i) {
+    c += b.unit_cnt[i];
+    w += b.unit_walks[i];
+  }
+  unsigned long long ce, we, ct, wt;
+  block_excl_scan2(c, w, &ce, &we, &ct, &wt);
+  for (uint32_t i = beg; i < end; ++i) {
+    const unsigned long long ci = b.unit_cnt[i], wi = b.unit_walks[i];
+    b.unit_cnt[i] = ce;
+    b.unit_walks[i] = we;
+    ce += ci;
+    we += wi;
   }
   if (threadIdx.x == 0) {
-    b.totals[0] = carry_c;
-    b.totals[1] = carry_w;
-    b.wr_offset[carry_c] = carry_w;
+    b.totals[0] = ct;
+    b.totals[1] = wt;
+    b.wr_offset[ct] = wt;
+    b.meet[0] = b.meet[32] = 0;  // the next call's push starts its barrier from 0
   }
   for (int s = threadIdx.x; s < b.nsrc; s += blockDim.x)
     if (b.stats[s].walks > 0xFFFFFFFFull) atomicOr(b.err, kErrWalkOverflow);
 }
 
+// The entries of up to 32 * kResidualLoads residues of a warp's unit, packed.
+struct ResidualStage {
+  double r[32 * kResidualLoads];
+  uint32_t omega[32 * kResidualLoads];
+  uint32_t pos[32 * kResidualLoads];   // place and walk offset within the unit's entries of
+  uint32_t woff[32 * kResidualLoads];  // the source
+  uint32_t v[32 * kResidualLoads];     // node - first node of the unit, times G, plus lane % G
+};
+
+template <int G>
 __global__ void __launch_bounds__(kResidualThreads) k_residual_emit(GraphDev g, BatchDev b) {
-  const unsigned long long total = (unsigned long long)b.nsrc * (unsigned long long)g.n;
-  unsigned long long beg, end;
-  block_range(total, blockIdx.x, gridDim.x, &beg, &end);
-  unsigned long long pos = b.blk_cnt[blockIdx.x];
-  unsigned long long woff = b.blk_walks[blockIdx.x];
+  __shared__ ResidualStage stages[kResidualThreads / 32];
+  UnitRange u;
+  if (!unit_range<G>(g, b, &u)) return;  // whole warps
+  ResidualStage& st = stages[threadIdx.x >> 5];
+  constexpr uint32_t kStep = 32 / G;
+  const uint32_t lane = threadIdx.x & 31, j = lane % G, slot = u.gr * G + j;
+  const bool mine = j < u.w && slot < (uint32_t)b.nsrc;
+  const unsigned long long base_c = mine ? b.unit_cnt[(size_t)slot * b.units + u.k] : 0ull;
+  const unsigned long long base_w = mine ? b.unit_walks[(size_t)slot * b.units + u.k] : 0ull;
   const float cf = __double2float_rn(b.walk_scale);
   const bool fast = cf >= 1.0f && cf <= 0x1p100f;
-  for (unsigned long long tile = beg; tile < end; tile += kResidualThreads) {
-    const unsigned long long i = tile + threadIdx.x;
-    const double r = i < end ? sampled(b, b.r[i]) : 0.0;
-    const unsigned long long omega = walks_of(r, b.walk_scale, cf, fast);
-    const bool live = omega >= 1;
-    unsigned long long ce, we, ct, wt;
-    block_excl_scan2(live ? 1ull : 0ull, omega, &ce, &we, &ct, &wt);
-    if (live && FORA_IN_RANGE(b.err, pos + ce, total)) {
-      const unsigned long long slot = i / (unsigned long long)g.n;
-      const unsigned long long v = i - slot * (unsigned long long)g.n;
-      b.wr_entry[pos + ce] = (slot << 32) | v;
-      b.wr_offset[pos + ce] = woff + we;
-      // the residue for now; k_residual_weight turns it into the walk weight
-      b.wr_weight[pos + ce] = (unsigned long long)__double_as_longlong(r);
+  constexpr uint32_t kSame = (uint32_t)(0xFFFFFFFFull / ((1ull << G) - 1));  // lanes of source 0
+  uint32_t done_c = 0, done_w = 0;  // entries and walks of this lane's source so far
+  for (uint32_t v0 = u.beg; v0 < u.end; v0 += kStep * kResidualLoads) {
+    double r[kResidualLoads];
+#pragma unroll
+    for (int k = 0; k < kResidualLoads; ++k) {
+      const uint32_t v = v0 + k * kStep + lane / G;
+      r[k] = mine && v < u.end ? b.r[u.g0 + (unsigned long long)v * u.w + j] : 0.0;
     }
-    pos += ct;
-    woff += wt;
-  }
-}
-
-// W_v of every entry of R, densely over the list (omega_v = offset[i + 1] - offset[i]),
-// so the FP64 division runs on 32 entries per instruction.
-__global__ void __launch_bounds__(kResidualThreads) k_residual_weight(BatchDev b) {
-  const unsigned long long nR = b.totals[0];
-  const unsigned long long stride = (unsigned long long)gridDim.x * blockDim.x;
-  for (unsigned long long i = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x; i < nR;
-       i += stride) {
-    const double r = __longlong_as_double((long long)b.wr_weight[i]);
-    const double omega = (double)(b.wr_offset[i + 1] - b.wr_offset[i]);
-    b.wr_weight[i] = weight_of(r, omega);
+    uint32_t staged = 0;
+#pragma unroll
+    for (int k = 0; k < kResidualLoads; ++k) {
+      const double x = sampled(b, r[k]);
+      const uint32_t omega = (uint32_t)walks_of(x, b.walk_scale, cf, fast);  // below 2^32 (scan)
+      const bool live = omega > 0;
+      const uint32_t m = __ballot_sync(kFull, live);
+      if (m == 0) continue;  // warp-uniform
+      const uint32_t same = m & (kSame << j);  // this source's
+      uint32_t incl = omega;                   // its walks up to this lane
+#pragma unroll
+      for (int o = G; o < 32; o <<= 1) {
+        const uint32_t t = __shfl_up_sync(kFull, incl, o);
+        if ((int)lane >= o) incl += t;
+      }
+      if (live) {
+        const uint32_t at = staged + __popc(m & ((1u << lane) - 1u));
+        st.r[at] = x;
+        st.omega[at] = omega;
+        st.pos[at] = done_c + __popc(same & ((1u << lane) - 1u));
+        st.woff[at] = done_w + incl - omega;
+        st.v[at] = (v0 - u.beg + k * kStep) * G + lane;
+      }
+      staged += __popc(m);
+      done_c += __popc(same);
+      done_w += __shfl_sync(kFull, incl, 32 - G + j);
+    }
+    __syncwarp();
+    for (uint32_t e0 = 0; e0 < staged; e0 += 32) {
+      const uint32_t e = e0 + lane;
+      const bool have = e < staged;
+      const uint32_t vj = have ? st.v[e] : 0u;
+      const unsigned long long pos = __shfl_sync(kFull, base_c, vj % G) + (have ? st.pos[e] : 0u);
+      const unsigned long long off = __shfl_sync(kFull, base_w, vj % G) + (have ? st.woff[e] : 0u);
+      if (have && FORA_IN_RANGE(b.err, pos, (unsigned long long)b.nsrc * g.n)) {
+        b.wr_entry[pos] =
+            ((unsigned long long)(u.gr * G + vj % G) << 32) | (unsigned long long)(u.beg + vj / G);
+        b.wr_offset[pos] = off;
+        b.wr_weight[pos] = weight_of(st.r[e], (double)st.omega[e]);
+      }
+    }
+    __syncwarp();
   }
 }
 
@@ -679,18 +741,29 @@ __global__ void k_philox_table(const uint32_t* ck, uint32_t* out, int count) {
 
 }  // namespace
 
-cudaError_t launch_residuals(const GraphDev& g, const BatchDev& b, cudaStream_t st) {
-  k_residual_count<<<b.residual_grid, kResidualThreads, 0, st>>>(g, b);
+int residual_units(int64_t n, int nsrc) {
+  int64_t units = kMaxUnits / nsrc;
+  units = std::min<int64_t>(units, (n + 511) / 512);
+  units = std::min<int64_t>(units, kMaxSlotUnits);
+  return (int)std::max<int64_t>(units, 1);
+}
+
+template <int G>
+cudaError_t residuals_t(const GraphDev& g, const BatchDev& b, cudaStream_t st) {
+  const unsigned long long warps = (unsigned long long)b.ngrp * b.units;
+  const unsigned blocks = (unsigned)((warps * 32 + kResidualThreads - 1) / kResidualThreads);
+  k_residual_count<G><<<blocks, kResidualThreads, 0, st>>>(g, b);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   k_residual_scan<<<1, 1024, 0, st>>>(b);
   e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  k_residual_emit<<<b.residual_grid, kResidualThreads, 0, st>>>(g, b);
-  e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  k_residual_weight<<<b.residual_grid, kResidualThreads, 0, st>>>(b);
+  k_residual_emit<G><<<blocks, kResidualThreads, 0, st>>>(g, b);
   return cudaGetLastError();
+}
+
+cudaError_t launch_residuals(const GraphDev& g, const BatchDev& b, cudaStream_t st) {
+  return b.gw == 1 ? residuals_t<1>(g, b, st) : residuals_t<4>(g, b, st);
 }
 
 // Walk kernel instances for 3, 4 or 5 resident blocks per SM (the register budget the
