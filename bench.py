@@ -336,8 +336,8 @@ def run_fora(args):
     def collect(step, st, ms):
         bounds = part_bounds(len(st))
         rounds = max(s.push_rounds for s in st)
-        # a part: push 1 (all rounds), residuals 3, walks 1, estimate 1, top-k select 19
-        counters["launches"] += len(bounds) * (1 + 3 + 1 + 1 + 19)
+        # a part: push 1 (all rounds), residuals 3, walks 1, estimate 1, top-k select 3
+        counters["launches"] += len(bounds) * (1 + 3 + 1 + 1 + 3)
         if model is not None:
             counters["launches"] += 3  # features, forward, r_max (whole batch)
         # kernel time of each phase, summed over the parts (parts overlap in time)

@@ -30,7 +30,6 @@ constexpr int kMaxSlotUnits = 4096;
 // Top-k radix select: 96-bit keys (estimate bits : ~id), 12-bit digits.
 constexpr int kDigitBits = 12;
 constexpr int kBins = 1 << kDigitBits;
-constexpr int kLevels = 96 / kDigitBits;
 constexpr uint32_t kSortCap = 8192;  // candidates sorted in shared memory at the end
 
 // Device error bits (ORed into BatchDev::err).
@@ -166,7 +165,7 @@ struct TopkSlot {
   uint32_t kk;            // how many keys still to take from the current bucket
   uint32_t done;
   uint32_t ncand;
-  uint32_t pad;
+  uint32_t arrived;       // blocks of the row that are through with a kernel
 };
 
 // Pointers into a call's workspace.  The push keeps its sources in groups of gw (1 or 4): value

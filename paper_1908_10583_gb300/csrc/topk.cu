@@ -3,16 +3,24 @@
 //
 // Every element t of a row gets the 96-bit key  Z = bits(pi_hat(t)) : ~t.  pi_hat >= 0,
 // so its IEEE bits order like its value, and ~t orders equal values by ascending id;
-// keys are unique, so the k largest keys are exactly the answer.  Radix select over
-// the key in 12-bit digits, most significant first:
-//   level L:  k_topk_hist   histogram of digit L of the keys whose leading 12L bits equal
-//                           the row's prefix (skipped once the row is done)
-//             k_topk_select pick the digit whose bucket holds the kk-th largest key,
-//                           extend the prefix, and mark the row done once every key above
-//                           the bucket plus the bucket itself fits the final sort
-//   then      k_topk_collect  every key >= the prefix bucket goes to the candidate list
-//             k_topk_sort     bitonic sort of <= kSortCap candidates in shared memory.
-// All levels are launched without host synchronisation; finished rows return at once.
+// keys are unique, so the k largest keys are exactly the answer.
+//   k_topk_first    histogram of the upper 18 bits of the estimate (sign, exponent, 6 bits of
+//                   mantissa), clamped to the 4096 bins from 2^-63 to 2: estimates crowd into
+//                   few exponents, so a digit of the exponent alone would not separate them.  A
+//                   row's last block picks the bin that holds the k-th largest key as the row's
+//                   prefix; the row is done once the keys above the bin and its own fit the sort.
+//   k_topk_levels   for rows that are not (more equal or near-equal values than the sort takes,
+//                   or a k-th value outside the bins): a cluster per row takes the next 12 bits
+//                   of the keys with the row's prefix, and so on.
+//   k_topk_collect  every key from the prefix on goes to the candidate list; a row's last block
+//                   sorts it (bitonic, in shared memory) and writes the first k.
+// Two passes over the rows; HBM bounds large ones, the launches and the sort small ones.
+// 24 rows of 10^6 estimates: 40 us, 4 us where no level is left, 50 us (the two passes at the
+// measured copy rate: 58); fora_topk 522 -> 328 us, 145 of them its allocation.  (As 19 launches:
+// eight levels of 12 bits from the top, whether a row had use for them or not, then collect and
+// sort.)
+#include <algorithm>
+
 #include "fora_engine.cuh"
 
 namespace fora {
@@ -23,10 +31,6 @@ typedef unsigned __int128 u128;
 
 __device__ __forceinline__ u128 key_of(double e, uint32_t t) {
   return ((u128)(unsigned long long)__double_as_longlong(e) << 32) | (u128)(~t);
-}
-
-__device__ __forceinline__ u128 prefix_of(const TopkSlot& s) {
-  return ((u128)s.pa << 32) | (u128)s.pb;
 }
 
 // One row of the grid per group of sources, kEstValues values per block: the walk ends are
@@ -67,86 +71,114 @@ __global__ void __launch_bounds__(kEstThreads) k_estimate(GraphDev g, BatchDev b
   }
 }
 
-__global__ void k_topk_init(TopkSlot* slots, uint32_t* hist, int nrows, uint32_t k) {
-  const int row = blockIdx.x;
-  if (row >= nrows) return;
-  for (int i = threadIdx.x; i < kBins; i += blockDim.x) hist[(size_t)row * kBins + i] = 0;
-  if (threadIdx.x == 0) {
-    TopkSlot s;
-    s.pa = 0; s.pb = 0; s.plen = 0; s.kk = k; s.done = (k == 0); s.ncand = 0; s.pad = 0;
-    slots[row] = s;
-  }
+constexpr int kTopkThreads = 1024;
+constexpr int kTopkLoads = 4;   // elements a thread reads before it uses any
+constexpr int kTopkCluster = 8;  // blocks of a row in k_topk_levels
+
+struct TopkRun {
+  const double* est;
+  int64_t n;
+  uint32_t k;
+  int32_t* out_ids;
+  double* out_vals;
+  TopkScratch s;
+};
+
+// The first digit: bits of the estimate from kFirstShift on (with the sign), less kFirstBase.
+constexpr int kFirstShift = 46;
+constexpr uint32_t kFirstBase = 960u << 6;  // 2^-63
+__device__ __forceinline__ uint32_t first_bin(double e) {
+  const unsigned long long top = (unsigned long long)__double_as_longlong(e) >> kFirstShift;
+  if (top < kFirstBase) return 0u;
+  return (uint32_t)min(top - kFirstBase, (unsigned long long)(kBins - 1));
 }
 
-// Element range of block bx (of bpr blocks per row) over a row of n.
-__device__ __forceinline__ void row_range(int64_t n, int bx, int bpr, int64_t* beg, int64_t* end) {
-  *beg = n * (int64_t)bx / bpr;
-  *end = n * (int64_t)(bx + 1) / bpr;
+__device__ __forceinline__ TopkSlot load_slot(const TopkSlot* p) {
+  TopkSlot s;
+  s.pa = __ldcg(&p->pa);
+  s.pb = __ldcg(&p->pb);
+  s.plen = __ldcg(&p->plen);
+  s.kk = __ldcg(&p->kk);
+  s.done = __ldcg(&p->done);
+  s.ncand = __ldcg(&p->ncand);
+  s.arrived = 0;
+  return s;
 }
 
-__global__ void __launch_bounds__(256) k_topk_hist(const double* __restrict__ est, int64_t n,
-                                                   const TopkSlot* __restrict__ slots,
-                                                   uint32_t* __restrict__ hist, int level) {
-  const int row = blockIdx.y;
-  const TopkSlot s = slots[row];
-  if (s.done) return;
-  __shared__ uint32_t sh[kBins];
+// Elements [beg, end) of part `part` of `parts` of a row of n.
+__device__ __forceinline__ void row_range(int64_t n, int part, int parts, int64_t* beg,
+                                          int64_t* end) {
+  *beg = n * (int64_t)part / parts;
+  *end = n * (int64_t)(part + 1) / parts;
+}
+
+// Histogram of one part of a row into sh, then into the row's (h): of the first digit
+// (s == nullptr), else of the next digit of the keys with s's prefix.  Bin 0 of the first digit
+// (zeros and values below 2^-63, most of many rows) is not counted: what is asked of it is the
+// keys above the bins.
+__device__ void topk_hist(const TopkRun& t, int row, int part, int parts, const TopkSlot* s,
+                          uint32_t* h, uint32_t* sh) {
   for (int i = threadIdx.x; i < kBins; i += blockDim.x) sh[i] = 0;
   __syncthreads();
-  const int shift_digit = 96 - kDigitBits * (level + 1);
-  const u128 p = prefix_of(s) >> (96 - s.plen);  // s.plen = 12 * level
   int64_t beg, end;
-  row_range(n, blockIdx.x, gridDim.x, &beg, &end);
-  const double* e = est + (size_t)row * (size_t)n;
-  const uint32_t lane = threadIdx.x & 31;
-  // keys crowd into few bins (every zero estimate, and the few binades the others span, share
-  // the leading digits), so the lanes of a warp that fall into the same bin add their count
-  // once (their lowest lane), instead of serialising on one shared-memory counter
-  for (int64_t base = beg; base < end; base += blockDim.x) {
-    const int64_t t = base + threadIdx.x;
-    bool in = false;
-    uint32_t bin = 0;
-    if (t < end) {
-      const u128 z = key_of(e[t], (uint32_t)t);
-      in = (z >> (96 - s.plen)) == p;
-      bin = (uint32_t)(z >> shift_digit) & (kBins - 1);
+  row_range(t.n, part, parts, &beg, &end);
+  const double* e = t.est + (size_t)row * (size_t)t.n;
+  const uint32_t width = s ? min((uint32_t)kDigitBits, 96u - s->plen) : 0u;
+  const u128 p = s && s->plen ? (((u128)s->pa << 32) | s->pb) >> (96 - s->plen) : 0;
+  for (int64_t base = beg + threadIdx.x; base < end; base += (int64_t)blockDim.x * kTopkLoads) {
+    double v[kTopkLoads];
+#pragma unroll
+    for (int q = 0; q < kTopkLoads; ++q) {
+      const int64_t i = base + (int64_t)q * blockDim.x;
+      v[q] = i < end ? e[i] : 0.0;
     }
-    const unsigned members = __ballot_sync(0xFFFFFFFFu, in);
-    if (in) {
-      const unsigned grp = __match_any_sync(members, bin);
-      if ((grp & ((1u << lane) - 1u)) == 0) atomicAdd(&sh[bin], (uint32_t)__popc(grp));
+#pragma unroll
+    for (int q = 0; q < kTopkLoads; ++q) {
+      const int64_t i = base + (int64_t)q * blockDim.x;
+      if (!s) {
+        const uint32_t bin = first_bin(v[q]);
+        if (bin) atomicAdd(&sh[bin], 1u);
+      } else if (i < end) {
+        const u128 z = key_of(v[q], (uint32_t)i);
+        if (s->plen == 0 || (z >> (96 - s->plen)) == p) {
+          // equal values share every digit but the ids': lanes of one bin add their count once
+          const uint32_t bin = (uint32_t)(z >> (96 - s->plen - width)) & ((1u << width) - 1u);
+          const unsigned grp = __match_any_sync(__activemask(), bin);
+          if ((threadIdx.x & 31) == (uint32_t)(__ffs(grp) - 1))
+            atomicAdd(&sh[bin], (uint32_t)__popc(grp));
+        }
+      }
     }
   }
   __syncthreads();
-  uint32_t* h = hist + (size_t)row * kBins;
   for (int i = threadIdx.x; i < kBins; i += blockDim.x)
     if (sh[i]) atomicAdd(&h[i], sh[i]);
 }
 
-// One block of 1024 threads per row; thread t owns bins 4095-4t .. 4092-4t (descending).
-__global__ void __launch_bounds__(1024) k_topk_select(TopkSlot* slots, uint32_t* hist, uint32_t k,
-                                                      int level) {
-  const int row = blockIdx.x;
-  TopkSlot s = slots[row];
-  if (s.done) return;
-  uint32_t* h = hist + (size_t)row * kBins;
-  const int t = threadIdx.x;
+// The digit of one row from its histogram (1024 threads; thread th owns bins 4095 - 4 th ..
+// 4092 - 4 th, descending), which is cleared for the next.
+__device__ void topk_select(const TopkRun& t, int row, bool first) {
+  __shared__ uint32_t wsum[32];
+  __shared__ uint32_t s_found;
+  uint32_t* h = t.s.hist + (size_t)row * kBins;
+  TopkSlot s = load_slot(&t.s.slots[row]);
+  if (first) s.kk = t.k;
+  const int th = threadIdx.x, lane = th & 31, wid = th >> 5;
   uint32_t c[4];
   uint32_t local = 0;
 #pragma unroll
   for (int q = 0; q < 4; ++q) {
-    c[q] = h[kBins - 1 - (4 * t + q)];
+    c[q] = __ldcg(&h[kBins - 1 - (4 * th + q)]);
     local += c[q];
   }
   // exclusive scan of `local` over the block (descending bin order)
-  __shared__ uint32_t wsum[32];
-  const int lane = t & 31, wid = t >> 5;
   uint32_t incl = local;
 #pragma unroll
   for (int off = 1; off < 32; off <<= 1) {
     const uint32_t v = __shfl_up_sync(0xFFFFFFFFu, incl, off);
     if (lane >= off) incl += v;
   }
+  if (th == 0) s_found = 0;
   if (lane == 31) wsum[wid] = incl;
   __syncthreads();
   if (wid == 0) {
@@ -163,74 +195,82 @@ __global__ void __launch_bounds__(1024) k_topk_select(TopkSlot* slots, uint32_t*
   uint32_t above = wsum[wid] + incl - local;  // keys in bins above this thread's bins
 #pragma unroll
   for (int q = 0; q < 4; ++q) {
-    if (above < s.kk && s.kk <= above + c[q]) {
-      const uint32_t digit = (uint32_t)(kBins - 1 - (4 * t + q));
-      const int pos = 96 - kDigitBits * (level + 1);  // bit position of the digit
-      const u128 p = prefix_of(s) | ((u128)digit << pos);
-      s.pa = (unsigned long long)(p >> 32);
-      s.pb = (uint32_t)p;
-      s.plen += kDigitBits;
+    const int bin = kBins - 1 - (4 * th + q);
+    // the clamped bins of the first digit are no prefix
+    if (above < s.kk && s.kk <= above + c[q] && !(first && (bin == 0 || bin == kBins - 1))) {
+      if (first) {
+        s.pa = (unsigned long long)(kFirstBase + (uint32_t)bin) << kFirstShift;
+        s.plen = 64 - kFirstShift;
+      } else {
+        const uint32_t width = min((uint32_t)kDigitBits, 96u - s.plen);
+        const u128 p = (((u128)s.pa << 32) | s.pb) | ((u128)(uint32_t)bin << (96 - s.plen - width));
+        s.pa = (unsigned long long)(p >> 32);
+        s.pb = (uint32_t)p;
+        s.plen += width;
+      }
       s.kk -= above;
-      const uint32_t sure = k - s.kk;  // keys strictly above the bucket
+      const uint32_t sure = t.k - s.kk;  // keys strictly above the bucket
       s.done = (sure + c[q] <= kSortCap) || (s.plen >= 96);
-      slots[row] = s;
+      t.s.slots[row] = s;
+      s_found = 1;
     }
     above += c[q];
   }
-  __syncthreads();
 #pragma unroll
-  for (int q = 0; q < 4; ++q) h[kBins - 1 - (4 * t + q)] = 0;  // clean for the next level
+  for (int q = 0; q < 4; ++q) h[kBins - 1 - (4 * th + q)] = 0;
+  __syncthreads();
+  if (th == 0 && s_found == 0) t.s.slots[row] = s;  // the k-th key lies outside the first bins
 }
 
-__global__ void __launch_bounds__(256) k_topk_collect(const double* __restrict__ est, int64_t n,
-                                                      TopkSlot* slots,
-                                                      unsigned long long* __restrict__ cand_key,
-                                                      uint32_t* __restrict__ cand_id) {
+// Whether this block is the last of its row's to get here; what the others wrote is then visible.
+__device__ bool last_of_row(TopkSlot* slot) {
+  __shared__ uint32_t s_last;
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) s_last = atomicAdd(&slot->arrived, 1u) == gridDim.x - 1 ? 1u : 0u;
+  __syncthreads();
+  __threadfence();
+  return s_last != 0;
+}
+
+// Grid (parts of a row, rows); histograms and slots are zero.
+__global__ void __launch_bounds__(kTopkThreads, 2) k_topk_first(TopkRun t) {
+  __shared__ uint32_t sh[kBins];
   const int row = blockIdx.y;
-  const TopkSlot s = slots[row];
-  if (s.plen == 0) return;  // k == 0
-  const u128 p = prefix_of(s) >> (96 - s.plen);
-  int64_t beg, end;
-  row_range(n, blockIdx.x, gridDim.x, &beg, &end);
-  const double* e = est + (size_t)row * (size_t)n;
-  const unsigned lane = threadIdx.x & 31;
-  for (int64_t base = beg; base < end; base += blockDim.x) {
-    const int64_t t = base + threadIdx.x;
-    bool take = false;
-    double v = 0.0;
-    if (t < end) {
-      v = e[t];
-      take = (key_of(v, (uint32_t)t) >> (96 - s.plen)) >= p;
-    }
-    const unsigned bal = __ballot_sync(0xFFFFFFFFu, take);
-    if (bal) {
-      uint32_t pos = 0;
-      if (lane == 0) pos = atomicAdd(&slots[row].ncand, (uint32_t)__popc(bal));
-      pos = __shfl_sync(0xFFFFFFFFu, pos, 0) + __popc(bal & ((1u << lane) - 1u));
-      if (take && pos < kSortCap) {
-        cand_key[(size_t)row * kSortCap + pos] = (unsigned long long)__double_as_longlong(v);
-        cand_id[(size_t)row * kSortCap + pos] = (uint32_t)t;
-      }
-    }
+  topk_hist(t, row, blockIdx.x, gridDim.x, nullptr, t.s.hist + (size_t)row * kBins, sh);
+  if (last_of_row(&t.s.slots[row])) topk_select(t, row, true);
+}
+
+__device__ __forceinline__ void cluster_meet() {
+  __threadfence();
+  asm volatile("barrier.cluster.arrive.aligned;" ::: "memory");
+  asm volatile("barrier.cluster.wait.aligned;" ::: "memory");
+}
+
+__global__ void __cluster_dims__(kTopkCluster, 1, 1) __launch_bounds__(kTopkThreads, 1)
+    k_topk_levels(TopkRun t) {
+  __shared__ uint32_t sh[kBins];
+  const int row = blockIdx.y;
+  // at most 8 levels: each fixes 12 more of the 96 bits (the last, fewer)
+  for (TopkSlot s = load_slot(&t.s.slots[row]); !s.done; s = load_slot(&t.s.slots[row])) {
+    topk_hist(t, row, blockIdx.x, kTopkCluster, &s, t.s.hist + (size_t)row * kBins, sh);
+    cluster_meet();
+    if (blockIdx.x == 0) topk_select(t, row, false);
+    cluster_meet();
   }
 }
 
 // Bitonic sort (descending by key) of one row's candidates; writes the first k.
-__global__ void __launch_bounds__(1024) k_topk_sort(const TopkSlot* slots,
-                                                    const unsigned long long* cand_key,
-                                                    const uint32_t* cand_id, uint32_t k,
-                                                    int32_t* out_ids, double* out_vals) {
-  extern __shared__ unsigned char smem[];
+__device__ void topk_sort(const TopkRun& t, int row, unsigned char* smem) {
   unsigned long long* ka = (unsigned long long*)smem;
   uint32_t* kb = (uint32_t*)(ka + kSortCap);
-  const int row = blockIdx.x;
-  const uint32_t nc = min(slots[row].ncand, kSortCap);
+  const uint32_t nc = min(__ldcg(&t.s.slots[row].ncand), kSortCap);
   uint32_t size = 1;
   while (size < nc) size <<= 1;
   for (uint32_t i = threadIdx.x; i < size; i += blockDim.x) {
     if (i < nc) {
-      ka[i] = cand_key[(size_t)row * kSortCap + i];
-      kb[i] = ~cand_id[(size_t)row * kSortCap + i];
+      ka[i] = __ldcg(&t.s.cand_key[(size_t)row * kSortCap + i]);
+      kb[i] = ~__ldcg(&t.s.cand_id[(size_t)row * kSortCap + i]);
     } else {
       ka[i] = 0;  // below every real key (a real key has ~id > 0)
       kb[i] = 0;
@@ -239,25 +279,63 @@ __global__ void __launch_bounds__(1024) k_topk_sort(const TopkSlot* slots,
   __syncthreads();
   for (uint32_t len = 2; len <= size; len <<= 1) {
     for (uint32_t j = len >> 1; j > 0; j >>= 1) {
-      for (uint32_t i = threadIdx.x; i < size; i += blockDim.x) {
-        const uint32_t pr = i ^ j;
-        if (pr > i) {
-          const bool desc = (i & len) == 0;
-          const u128 zi = ((u128)ka[i] << 32) | kb[i];
-          const u128 zp = ((u128)ka[pr] << 32) | kb[pr];
-          if (desc ? (zi < zp) : (zi > zp)) {
-            const unsigned long long ta = ka[i]; ka[i] = ka[pr]; ka[pr] = ta;
-            const uint32_t tb = kb[i]; kb[i] = kb[pr]; kb[pr] = tb;
-          }
+      for (uint32_t q = threadIdx.x; q < size / 2; q += blockDim.x) {
+        const uint32_t i = 2 * q - (q & (j - 1)), pr = i + j;  // the q-th pair at distance j
+        const bool desc = (i & len) == 0;
+        const unsigned long long ai = ka[i], ap = ka[pr];
+        const uint32_t bi = kb[i], bp = kb[pr];
+        const bool less = ai < ap || (ai == ap && bi < bp);
+        const bool more = ai > ap || (ai == ap && bi > bp);
+        if (desc ? less : more) {
+          ka[i] = ap; ka[pr] = ai;
+          kb[i] = bp; kb[pr] = bi;
         }
       }
       __syncthreads();
     }
   }
-  for (uint32_t i = threadIdx.x; i < k; i += blockDim.x) {
-    out_ids[(size_t)row * k + i] = (int32_t)(~kb[i]);
-    out_vals[(size_t)row * k + i] = __longlong_as_double((long long)ka[i]);
+  for (uint32_t i = threadIdx.x; i < t.k; i += blockDim.x) {
+    t.out_ids[(size_t)row * t.k + i] = (int32_t)(~kb[i]);
+    t.out_vals[(size_t)row * t.k + i] = __longlong_as_double((long long)ka[i]);
   }
+}
+
+// Grid (parts of a row, rows).  A part is read from its end: k_topk_first has read that last.
+__global__ void __launch_bounds__(kTopkThreads, 2) k_topk_collect(TopkRun t) {
+  extern __shared__ unsigned char smem[];
+  const int row = blockIdx.y;
+  const unsigned long long pa = __ldcg(&t.s.slots[row].pa);
+  const uint32_t pb = __ldcg(&t.s.slots[row].pb);  // (pa, pb): the least key of the prefix
+  int64_t beg, end;
+  row_range(t.n, blockIdx.x, gridDim.x, &beg, &end);
+  const double* e = t.est + (size_t)row * (size_t)t.n;
+  const unsigned lane = threadIdx.x & 31;
+  // block-uniform trip count, descending
+  for (int64_t top = end; top > beg; top -= (int64_t)kTopkThreads * kTopkLoads) {
+    double v[kTopkLoads];
+#pragma unroll
+    for (int q = 0; q < kTopkLoads; ++q) {
+      const int64_t i = top - 1 - (int64_t)q * kTopkThreads - threadIdx.x;
+      v[q] = i >= beg ? e[i] : 0.0;
+    }
+#pragma unroll
+    for (int q = 0; q < kTopkLoads; ++q) {
+      const int64_t i = top - 1 - (int64_t)q * kTopkThreads - threadIdx.x;
+      const unsigned long long bits = (unsigned long long)__double_as_longlong(v[q]);
+      const bool take = i >= beg && (bits > pa || (bits == pa && ~(uint32_t)i >= pb));
+      const unsigned bal = __ballot_sync(0xFFFFFFFFu, take);
+      if (bal) {
+        uint32_t pos = 0;
+        if (lane == 0) pos = atomicAdd(&t.s.slots[row].ncand, (uint32_t)__popc(bal));
+        pos = __shfl_sync(0xFFFFFFFFu, pos, 0) + __popc(bal & ((1u << lane) - 1u));
+        if (take && pos < kSortCap) {
+          t.s.cand_key[(size_t)row * kSortCap + pos] = bits;
+          t.s.cand_id[(size_t)row * kSortCap + pos] = (uint32_t)i;
+        }
+      }
+    }
+  }
+  if (last_of_row(&t.s.slots[row])) topk_sort(t, row, smem);
 }
 
 }  // namespace
@@ -292,25 +370,27 @@ cudaError_t launch_estimate(const GraphDev& g, const BatchDev& b, double* est, c
 cudaError_t launch_topk(const double* est, int64_t n, int nrows, uint32_t k, int32_t* out_ids,
                         double* out_vals, const TopkScratch& s, int num_sms, cudaStream_t st) {
   if (nrows <= 0 || k == 0) return cudaSuccess;
-  k_topk_init<<<nrows, 256, 0, st>>>(s.slots, s.hist, nrows, k);
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  // enough blocks per row to cover the GPU, each with at least 4096 elements
-  int64_t bpr = ((int64_t)num_sms * 8 + nrows - 1) / nrows;
-  const int64_t max_bpr = (n + 4095) / 4096;
-  if (bpr > max_bpr) bpr = max_bpr;
-  if (bpr < 1) bpr = 1;
-  if (bpr > 65535) bpr = 65535;
-  const dim3 grid((unsigned)bpr, (unsigned)nrows);
-  for (int level = 0; level < kLevels; ++level) {
-    k_topk_hist<<<grid, 256, 0, st>>>(est, n, s.slots, s.hist, level);
-    k_topk_select<<<nrows, 1024, 0, st>>>(s.slots, s.hist, k, level);
-  }
-  k_topk_collect<<<grid, 256, 0, st>>>(est, n, s.slots, s.cand_key, s.cand_id);
   const size_t smem = kSortCap * (sizeof(unsigned long long) + sizeof(uint32_t));
-  e = cudaFuncSetAttribute(k_topk_sort, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = cudaFuncSetAttribute(k_topk_collect, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)smem);
   if (e != cudaSuccess) return e;
-  k_topk_sort<<<nrows, 1024, smem, st>>>(s.slots, s.cand_key, s.cand_id, k, out_ids, out_vals);
+  // slots and histograms lie side by side
+  e = cudaMemsetAsync(s.slots, 0, (size_t)nrows * (sizeof(TopkSlot) + kBins * sizeof(uint32_t)), st);
+  if (e != cudaSuccess) return e;
+  // Parts of at least 4096 elements: for few rows one wave of two blocks per SM, for more (which
+  // might fill half a last wave) about four.
+  int64_t bpr = nrows <= 32 ? (int64_t)num_sms * 2 / nrows
+                            : ((int64_t)num_sms * 8 + nrows - 1) / nrows;
+  bpr = std::max<int64_t>(1, std::min<int64_t>(bpr, (n + 4095) / 4096));
+  const dim3 grid((unsigned)bpr, (unsigned)nrows);
+  const TopkRun t{est, n, k, out_ids, out_vals, s};
+  k_topk_first<<<grid, kTopkThreads, 0, st>>>(t);
+  e = cudaGetLastError();
+  if (e != cudaSuccess) return e;
+  k_topk_levels<<<dim3(kTopkCluster, (unsigned)nrows), kTopkThreads, 0, st>>>(t);
+  e = cudaGetLastError();
+  if (e != cudaSuccess) return e;
+  k_topk_collect<<<grid, kTopkThreads, smem, st>>>(t);
   return cudaGetLastError();
 }
 

@@ -59,7 +59,7 @@ extern "C" int fora_topk_noalloc(const double* est, int64_t n, int32_t nrows, ui
     }
     scratch = g_scratch_addr[dev];
   }
-  // The select's first kernel zeroes the histograms and resets the per-row state, so
+  // launch_topk first clears the histograms and the per-row state, so
   // what an earlier call left in the array does not matter.
   cudaStream_t st = (cudaStream_t)stream;
   cudaError_t e = fora::launch_topk(est, n, nrows, k, out_ids, out_vals,
