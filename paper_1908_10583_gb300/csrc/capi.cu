@@ -1293,8 +1293,9 @@ struct ModelScratch {
   float* partial = nullptr;
   float* loss = nullptr;
   int32_t* idx = nullptr;
+  float2* corr = nullptr;
   ~ModelScratch() {
-    dfree(x); dfree(t); dfree(y); dfree(partial); dfree(loss); dfree(idx);
+    dfree(x); dfree(t); dfree(y); dfree(partial); dfree(loss); dfree(idx); dfree(corr);
   }
 };
 
@@ -1382,10 +1383,9 @@ int fora_model_gradient(fora_model* m, const float* x, const float* t, int32_t n
   std::lock_guard<std::mutex> lock(m->mu);
   CUDA_TRY(cudaSetDevice(m->device));
   ModelScratch s;
-  const int tiles = (n + mlp_tile() - 1) / mlp_tile();
   CUDA_TRY(cudaMalloc(&s.x, (size_t)n * FORA_NUM_FEATURES * sizeof(float)));
   CUDA_TRY(cudaMalloc(&s.t, (size_t)n * sizeof(float)));
-  CUDA_TRY(cudaMalloc(&s.partial, (size_t)tiles * FORA_MODEL_PARAMS * sizeof(float)));
+  CUDA_TRY(cudaMalloc(&s.partial, mlp_partial_floats(n) * sizeof(float)));
   CUDA_TRY(cudaMalloc(&s.loss, (size_t)n * sizeof(float)));
   CUDA_TRY(cudaMemcpy(s.x, x, (size_t)n * FORA_NUM_FEATURES * sizeof(float), cudaMemcpyHostToDevice));
   CUDA_TRY(cudaMemcpy(s.t, t, (size_t)n * sizeof(float), cudaMemcpyHostToDevice));
@@ -1420,16 +1420,22 @@ int fora_model_train(fora_model* m, const float* x, const float* t, int32_t n, i
   CUDA_TRY(cudaMemcpy(m->norm, norm.data(), 2 * F * sizeof(float), cudaMemcpyHostToDevice));
   ModelScratch s;
   const int b = batch < n ? batch : n;
-  const int tiles = (b + mlp_tile() - 1) / mlp_tile();
+  // a launch an epoch where one cluster takes a batch, else three a step
+  const bool fits = mlp_train_fits(b);
+  const int steps = (n + b - 1) / b;
   CUDA_TRY(cudaMalloc(&s.x, (size_t)n * F * sizeof(float)));
   CUDA_TRY(cudaMalloc(&s.t, (size_t)n * sizeof(float)));
   CUDA_TRY(cudaMalloc(&s.idx, (size_t)n * sizeof(int32_t)));
-  CUDA_TRY(cudaMalloc(&s.partial, (size_t)tiles * FORA_MODEL_PARAMS * sizeof(float)));
+  if (fits)
+    CUDA_TRY(cudaMalloc(&s.corr, (size_t)steps * sizeof(float2)));
+  else
+    CUDA_TRY(cudaMalloc(&s.partial, mlp_partial_floats(b) * sizeof(float)));
   CUDA_TRY(cudaMalloc(&s.loss, (size_t)n * sizeof(float)));
   CUDA_TRY(cudaMemcpy(s.x, x, (size_t)n * F * sizeof(float), cudaMemcpyHostToDevice));
   CUDA_TRY(cudaMemcpy(s.t, t, (size_t)n * sizeof(float), cudaMemcpyHostToDevice));
   std::vector<int32_t> perm(n);
   std::vector<float> l(n);
+  std::vector<float2> corr(fits ? steps : 0);
   uint64_t st = seed;
   for (int ep = 0; ep < epochs; ++ep) {
     for (int i = 0; i < n; ++i) perm[i] = i;
@@ -1438,11 +1444,18 @@ int fora_model_train(fora_model* m, const float* x, const float* t, int32_t n, i
       const int32_t tmp = perm[i]; perm[i] = perm[j]; perm[j] = tmp;
     }
     CUDA_TRY(cudaMemcpy(s.idx, perm.data(), (size_t)n * sizeof(int32_t), cudaMemcpyHostToDevice));
-    for (int off = 0; off < n; off += b) {
-      const int cnt = (n - off) < b ? (n - off) : b;
-      CUDA_TRY(launch_mlp_grad(m->master, m->norm, s.x, s.t, s.idx + off, cnt, s.partial,
-                               s.loss + off, m->grad, 0));
-      CUDA_TRY(launch_adam(m->master, m->adam_m, m->adam_v, m->grad, ++m->step, lr, 0));
+    if (fits) {
+      for (int k = 0; k < steps; ++k) corr[k] = adam_correction(++m->step);
+      CUDA_TRY(cudaMemcpy(s.corr, corr.data(), (size_t)steps * sizeof(float2), cudaMemcpyHostToDevice));
+      CUDA_TRY(launch_mlp_epoch(m->master, m->adam_m, m->adam_v, m->norm, s.x, s.t, s.idx, s.corr, n,
+                                b, lr, s.loss, 0));
+    } else {
+      for (int off = 0; off < n; off += b) {
+        const int cnt = (n - off) < b ? (n - off) : b;
+        CUDA_TRY(launch_mlp_grad(m->master, m->norm, s.x, s.t, s.idx + off, cnt, s.partial,
+                                 s.loss + off, m->grad, 0));
+        CUDA_TRY(launch_adam(m->master, m->adam_m, m->adam_v, m->grad, ++m->step, lr, 0));
+      }
     }
     if (loss_per_epoch) {
       CUDA_TRY(cudaMemcpy(l.data(), s.loss, (size_t)n * sizeof(float), cudaMemcpyDeviceToHost));

@@ -315,11 +315,17 @@ cudaError_t launch_mlp_forward(const float* master, const float* norm, const flo
 cudaError_t launch_mlp_grad(const float* master, const float* norm, const float* X,
                             const float* T, const int32_t* idx, int n, float* partial,
                             float* loss_partial, float* grad, cudaStream_t st);
+float2 adam_correction(int step);
+bool mlp_train_fits(int batch);
+cudaError_t launch_mlp_epoch(float* master, float* m, float* v, const float* norm, const float* X,
+                             const float* T, const int32_t* idx, const float2* corrections, int n,
+                             int batch, float lr, float* loss, cudaStream_t st);
+size_t mlp_partial_floats(int n);
 cudaError_t launch_adam(float* master, float* m, float* v, const float* grad, int step, float lr,
                         cudaStream_t st);
 cudaError_t launch_pred_to_rmax(const float* pred, int n, double rmax_rule, float lo, float hi,
                                 double* rmax, cudaStream_t st);
-int mlp_tile();
+
 
 // topk.cu
 // est [nsrc][n]; with zero-hop pruning the estimate also takes alpha * r.
