@@ -270,7 +270,8 @@ int resident_blocks(const void* kernel, int threads);
 cudaError_t device_alloc(void** p, size_t bytes);
 
 // push.cu: the whole push in one cooperative launch (from zeroing r and res on).
-cudaError_t launch_push(const GraphDev& g, const BatchDev& b, int num_sms, cudaStream_t st);
+cudaError_t launch_push(const GraphDev& g, const BatchDev& b, int num_sms, bool resume,
+                        const uint32_t* pause, cudaStream_t st);
 // The same in steps for a host loop that reads PushState::go after each round: start, rounds,
 // finish.
 cudaError_t launch_push_start(const GraphDev& g, const BatchDev& b, int num_sms, cudaStream_t st);

@@ -29,8 +29,9 @@
 // k_push runs all rounds in one cooperative launch: its blocks meet at a barrier after each
 // phase, and block 0 runs the advance while the others wait at the take's.  (As three launches in
 // a conditional graph node a round cost 39 us however small; 22 rounds of a 2^14-node graph took
-// 0.89 ms, now 0.39.)  The same phases are launched one by one where the host steps in between
-// rounds (serving joins, push_host_loop).
+// 0.89 ms, now 0.39.)  A serving batch that requests
+// join pauses the launch after a round and resumes it.  The same phases are launched one by one
+// by push_host_loop.
 //
 // Pushes to the graph's hot nodes (the up to 128 nodes of highest in-degree) would queue at the
 // L2 slices that hold their residues: each block adds them to one of kHotCopies copies, and the
@@ -1139,29 +1140,46 @@ constexpr unsigned long long kSmallUnits = 64;
 // 4 resident blocks (64 registers): 3 (no spilled register) took 130.4 ms where 4 take 121.5, 5
 // 138 (256 sources of a 2^20-node R-MAT graph).
 constexpr int kPushBlocks = 4;
-template <int G, int L>
+// With kJoin sources can join between rounds: a non-zero word at `pause` (host memory that the
+// device reads) ends the launch after its round, and with `resume` the push goes on where such a
+// launch left it.  (A template parameter: with the second entry into the loop a launch for one
+// source of a small graph spills 148 bytes, without it 116.)
+template <int G, int L, bool kJoin>
 __global__ void __launch_bounds__(kPushThreads, kPushBlocks)
-    k_push(const __grid_constant__ GraphDev g, const __grid_constant__ BatchDev b) {
+    k_push(const __grid_constant__ GraphDev g, const __grid_constant__ BatchDev b, int resume,
+           const volatile uint32_t* pause) {
   __shared__ PushShared<G> sh;
   const PushState* ps = b.ps;
   const PushCtl* ctl = b.ctl;
   const uint32_t wid = threadIdx.x >> 5;
   uint32_t met = 0;
-  zero_phase(g, b);
-  bool go = grid_meet(b, ++met, true, [&] {
-    seed_phase<G>(g, b);
-    return true;
-  });
-  for (int nx = 0; go; nx ^= 1) {
-    take_phase<G, L>(g, b, nx, __ldcg(&ctl->nheavy), __ldcg(&ctl->nlist), sh.take[wid]);
-    go = grid_meet(b, ++met, true,
-                   [&] { return advance_phase<G>(b, nx, gridDim.x * kPushWarps); });
-    if (!go) break;
+  int nx = 0;
+  bool go = true, take = true;
+  if (kJoin && resume) {
+    nx = __ldcg(&ps->cur);
+    take = false;
+  } else {
+    zero_phase(g, b);
+    go = grid_meet(b, ++met, true, [&] {
+      seed_phase<G>(g, b);
+      return true;
+    });
+  }
+  for (; go; nx ^= 1) {
+    if (!kJoin || take) {
+      take_phase<G, L>(g, b, nx, __ldcg(&ctl->nheavy), __ldcg(&ctl->nlist), sh.take[wid]);
+      go = grid_meet(b, ++met, true, [&] {
+        const uint32_t stop = kJoin && threadIdx.x == 0 ? *pause : 0u;
+        return advance_phase<G>(b, nx, gridDim.x * kPushWarps) && !stop;
+      });
+      if (!go) break;
+    }
+    take = true;
     spread_phase<G>(g, b, nx, __ldcg(&ps->nhub), __ldcg(&ps->ngroups), __ldcg(&ctl->span),
                     sh.spread[wid]);
     go = grid_meet(b, ++met, false, [] { return true; });
   }
-  finish_phase<G>(g, b);
+  if (!kJoin || !__ldcg(&ps->go)) finish_phase<G>(g, b);
 }
 
 // The phases on their own.
@@ -1232,6 +1250,7 @@ __global__ void __launch_bounds__(kPushThreads) k_push_join(const __grid_constan
     }
     b.ctl->nheavy = nheavy;
     ps->nact = nact;
+    b.meet[0] = b.meet[32] = 0;  // the launch that resumes starts its barrier from 0
   }
 }
 
@@ -1260,9 +1279,11 @@ __global__ void k_regroup(double* grouped, double* rows, unsigned long long n, i
   }
 }
 
-template <int G, int L>
-cudaError_t push_t(const GraphDev& g, const BatchDev& b, int num_sms, cudaStream_t st) {
-  const int per_sm = resident_blocks((const void*)k_push<G, L>, kPushThreads);
+template <int G, int L, bool kJoin>
+cudaError_t push_t(const GraphDev& g, const BatchDev& b, int num_sms, bool resume,
+                   const uint32_t* pause, cudaStream_t st) {
+  const void* kernel = (const void*)k_push<G, L, kJoin>;
+  const int per_sm = resident_blocks(kernel, kPushThreads);
   if (per_sm == 0) return cudaErrorInvalidConfiguration;
   // every SM at least once; more blocks only where a full scan has work for them
   const unsigned long long parts = (unsigned long long)b.ngrp * b.tiles * (8 / L);
@@ -1271,9 +1292,21 @@ cudaError_t push_t(const GraphDev& g, const BatchDev& b, int num_sms, cudaStream
   while (blocks < want && blocks < (unsigned)(num_sms * per_sm)) blocks += (unsigned)num_sms;
   GraphDev gd = g;
   BatchDev bd = b;
-  void* args[] = {&gd, &bd};
-  return cudaLaunchCooperativeKernel((const void*)k_push<G, L>, dim3(blocks), dim3(kPushThreads),
-                                     args, 0, st);
+  int rs = resume ? 1 : 0;
+  void* args[] = {&gd, &bd, &rs, &pause};
+  return cudaLaunchCooperativeKernel(kernel, dim3(blocks), dim3(kPushThreads), args, 0, st);
+}
+
+template <int G>
+cudaError_t push_any(const GraphDev& g, const BatchDev& b, int num_sms, bool resume,
+                     const uint32_t* pause, cudaStream_t st) {
+  // a small batch's full scan has few units: a warp reads a quarter of one, which shortens a round
+  const bool small = (unsigned long long)b.ngrp * b.tiles < kSmallUnits * (unsigned)num_sms;
+  if (pause)
+    return small ? push_t<G, 2, true>(g, b, num_sms, resume, pause, st)
+                 : push_t<G, 8, true>(g, b, num_sms, resume, pause, st);
+  return small ? push_t<G, 2, false>(g, b, num_sms, false, nullptr, st)
+               : push_t<G, 8, false>(g, b, num_sms, false, nullptr, st);
 }
 
 template <int G>
@@ -1300,11 +1333,10 @@ cudaError_t launch_threshold_table(const double* r, const double* rm, const uint
   return cudaGetLastError();
 }
 
-cudaError_t launch_push(const GraphDev& g, const BatchDev& b, int num_sms, cudaStream_t st) {
-  // a small batch's full scan has few units: a warp reads a quarter of one, which shortens a round
-  const bool small = (unsigned long long)b.ngrp * b.tiles < kSmallUnits * (unsigned)num_sms;
-  if (b.gw == 1) return small ? push_t<1, 2>(g, b, num_sms, st) : push_t<1, 8>(g, b, num_sms, st);
-  return small ? push_t<4, 2>(g, b, num_sms, st) : push_t<4, 8>(g, b, num_sms, st);
+cudaError_t launch_push(const GraphDev& g, const BatchDev& b, int num_sms, bool resume,
+                        const uint32_t* pause, cudaStream_t st) {
+  return b.gw == 1 ? push_any<1>(g, b, num_sms, resume, pause, st)
+                   : push_any<4>(g, b, num_sms, resume, pause, st);
 }
 
 cudaError_t launch_push_start(const GraphDev& g, const BatchDev& b, int num_sms, cudaStream_t st) {

@@ -74,7 +74,9 @@ struct Workspace {
   uint32_t* h_err = nullptr;
   int32_t* h_sources = nullptr;
   double* h_rmax = nullptr;
-  uint32_t* go_host = nullptr;  // PushState::go of the host-driven push loop
+  // pinned: [0] PushState::go of the host-driven push loop; [1] pauses a push that sources can
+  // join, [2] is its err
+  uint32_t* go_host = nullptr;
   cudaEvent_t ev[5] = {nullptr, nullptr, nullptr, nullptr, nullptr};
 
   PushState* ps = nullptr;
