@@ -59,6 +59,9 @@ int fora::report_error(int code, const char* fmt, ...) {
 
 namespace {
 
+std::mutex g_pools_mu;
+std::map<int, cudaMemPool_t> g_pools;  // by device (scratch_alloc)
+
 std::mutex g_occ_mu;
 std::map<std::pair<int, const void*>, int> g_occ;  // (device, kernel) -> blocks per SM
 
@@ -80,6 +83,45 @@ int fora::resident_blocks(const void* kernel, int threads) {
   if (per_sm < 1) per_sm = 1;
   g_occ[key] = per_sm;
   return per_sm;
+}
+
+cudaError_t fora::scratch_alloc(void** p, size_t bytes, cudaStream_t st) {
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  cudaMemPool_t pool = nullptr;
+  {
+    std::lock_guard<std::mutex> lock(g_pools_mu);
+    const auto it = g_pools.find(dev);
+    if (it != g_pools.end()) {
+      pool = it->second;
+    } else {
+      cudaMemPoolProps props = {};
+      props.allocType = cudaMemAllocationTypePinned;
+      props.location.type = cudaMemLocationTypeDevice;
+      props.location.id = dev;
+      e = cudaMemPoolCreate(&pool, &props);
+      if (e != cudaSuccess) return e;
+      uint64_t kept = kScratchKept;
+      e = cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &kept);
+      if (e != cudaSuccess) {
+        cudaMemPoolDestroy(pool);
+        return e;
+      }
+      g_pools[dev] = pool;
+    }
+  }
+  return cudaMallocFromPoolAsync(p, bytes, pool, st);
+}
+
+void fora::scratch_free(void* p, cudaStream_t st) {
+  if (p) cudaFreeAsync(p, st);
+}
+
+void fora::scratch_trim(int device) {
+  std::lock_guard<std::mutex> lock(g_pools_mu);
+  const auto it = g_pools.find(device);
+  if (it != g_pools.end()) cudaMemPoolTrimTo(it->second, 0);
 }
 
 cudaError_t fora::device_alloc(void** p, size_t bytes) {
@@ -953,6 +995,7 @@ void fora_graph_destroy(fora_graph* g) {
     dfree(g->idx_off);
     dfree(g->idx_dest);
   }
+  scratch_trim(g->device);
   delete g;
 }
 
@@ -1186,10 +1229,10 @@ int fora_topk(const double* est, int64_t n, int32_t nrows, uint32_t k, int32_t* 
   CUDA_TRY(cudaGetDevice(&dev));
   CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
   void* scratch = nullptr;
-  CUDA_TRY(cudaMallocAsync(&scratch, topk_scratch_bytes(nrows), st));
+  CUDA_TRY(scratch_alloc(&scratch, topk_scratch_bytes(nrows), st));
   const cudaError_t e = launch_topk(est, n, nrows, k, out_ids, out_vals, topk_scratch_carve(scratch, nrows),
                                     sms, st);
-  cudaFreeAsync(scratch, st);
+  scratch_free(scratch, st);
   CUDA_TRY(e);
   CUDA_TRY(cudaStreamSynchronize(st));
   return FORA_OK;
@@ -1291,6 +1334,7 @@ uint64_t splitmix(uint64_t* s) {
 }
 
 // Device buffers of one model call (inputs, targets, partials) on the default stream.
+// Buffers of a call on the default stream.
 struct ModelScratch {
   float* x = nullptr;
   float* t = nullptr;
@@ -1299,8 +1343,13 @@ struct ModelScratch {
   float* loss = nullptr;
   int32_t* idx = nullptr;
   float2* corr = nullptr;
+  template <typename T>
+  cudaError_t get(T** p, size_t count) {
+    return scratch_alloc(reinterpret_cast<void**>(p), count * sizeof(T), 0);
+  }
   ~ModelScratch() {
-    dfree(x); dfree(t); dfree(y); dfree(partial); dfree(loss); dfree(idx); dfree(corr);
+    for (void* p : {(void*)x, (void*)t, (void*)y, (void*)partial, (void*)loss, (void*)idx, (void*)corr})
+      scratch_free(p, 0);
   }
 };
 
@@ -1374,8 +1423,8 @@ int fora_model_predict(fora_model* m, const float* x, int32_t n, float* y) {
   std::lock_guard<std::mutex> lock(m->mu);
   CUDA_TRY(cudaSetDevice(m->device));
   ModelScratch s;
-  CUDA_TRY(cudaMalloc(&s.x, (size_t)n * FORA_NUM_FEATURES * sizeof(float)));
-  CUDA_TRY(cudaMalloc(&s.y, (size_t)n * sizeof(float)));
+  CUDA_TRY(s.get(&s.x, (size_t)n * FORA_NUM_FEATURES));
+  CUDA_TRY(s.get(&s.y, (size_t)n));
   CUDA_TRY(cudaMemcpy(s.x, x, (size_t)n * FORA_NUM_FEATURES * sizeof(float), cudaMemcpyHostToDevice));
   CUDA_TRY(launch_mlp_forward(m->master, m->norm, s.x, n, s.y, 0));
   CUDA_TRY(cudaMemcpy(y, s.y, (size_t)n * sizeof(float), cudaMemcpyDeviceToHost));
@@ -1388,10 +1437,10 @@ int fora_model_gradient(fora_model* m, const float* x, const float* t, int32_t n
   std::lock_guard<std::mutex> lock(m->mu);
   CUDA_TRY(cudaSetDevice(m->device));
   ModelScratch s;
-  CUDA_TRY(cudaMalloc(&s.x, (size_t)n * FORA_NUM_FEATURES * sizeof(float)));
-  CUDA_TRY(cudaMalloc(&s.t, (size_t)n * sizeof(float)));
-  CUDA_TRY(cudaMalloc(&s.partial, mlp_partial_floats(n) * sizeof(float)));
-  CUDA_TRY(cudaMalloc(&s.loss, (size_t)n * sizeof(float)));
+  CUDA_TRY(s.get(&s.x, (size_t)n * FORA_NUM_FEATURES));
+  CUDA_TRY(s.get(&s.t, (size_t)n));
+  CUDA_TRY(s.get(&s.partial, mlp_partial_floats(n)));
+  CUDA_TRY(s.get(&s.loss, (size_t)n));
   CUDA_TRY(cudaMemcpy(s.x, x, (size_t)n * FORA_NUM_FEATURES * sizeof(float), cudaMemcpyHostToDevice));
   CUDA_TRY(cudaMemcpy(s.t, t, (size_t)n * sizeof(float), cudaMemcpyHostToDevice));
   CUDA_TRY(launch_mlp_grad(m->master, m->norm, s.x, s.t, nullptr, n, s.partial, s.loss, m->grad, 0));
@@ -1415,10 +1464,16 @@ int fora_model_train(fora_model* m, const float* x, const float* t, int32_t n, i
   // feature normalisation from the training inputs
   const int F = FORA_NUM_FEATURES;
   std::vector<float> norm(2 * F);
+  double s1[FORA_NUM_FEATURES] = {}, s2[FORA_NUM_FEATURES] = {};
+  for (int r = 0; r < n; ++r) {  // the features' sums side by side
+    const float* row = x + (size_t)r * F;
+    for (int i = 0; i < F; ++i) {
+      s1[i] += row[i];
+      s2[i] += (double)row[i] * row[i];
+    }
+  }
   for (int i = 0; i < F; ++i) {
-    double s1 = 0, s2 = 0;
-    for (int r = 0; r < n; ++r) { s1 += x[(size_t)r * F + i]; s2 += (double)x[(size_t)r * F + i] * x[(size_t)r * F + i]; }
-    const double mean = s1 / n, var = s2 / n - mean * mean;
+    const double mean = s1[i] / n, var = s2[i] / n - mean * mean;
     norm[i] = (float)mean;
     norm[F + i] = var > 1e-12 ? (float)sqrt(var) : 1.0f;
   }
@@ -1428,26 +1483,29 @@ int fora_model_train(fora_model* m, const float* x, const float* t, int32_t n, i
   // a launch an epoch where one cluster takes a batch, else three a step
   const bool fits = mlp_train_fits(b);
   const int steps = (n + b - 1) / b;
-  CUDA_TRY(cudaMalloc(&s.x, (size_t)n * F * sizeof(float)));
-  CUDA_TRY(cudaMalloc(&s.t, (size_t)n * sizeof(float)));
-  CUDA_TRY(cudaMalloc(&s.idx, (size_t)n * sizeof(int32_t)));
+  CUDA_TRY(s.get(&s.x, (size_t)n * F));
+  CUDA_TRY(s.get(&s.t, (size_t)n));
+  CUDA_TRY(s.get(&s.idx, (size_t)n));
   if (fits)
-    CUDA_TRY(cudaMalloc(&s.corr, (size_t)steps * sizeof(float2)));
+    CUDA_TRY(s.get(&s.corr, (size_t)steps));
   else
-    CUDA_TRY(cudaMalloc(&s.partial, mlp_partial_floats(b) * sizeof(float)));
-  CUDA_TRY(cudaMalloc(&s.loss, (size_t)n * sizeof(float)));
+    CUDA_TRY(s.get(&s.partial, mlp_partial_floats(b)));
+  CUDA_TRY(s.get(&s.loss, (size_t)n));
   CUDA_TRY(cudaMemcpy(s.x, x, (size_t)n * F * sizeof(float), cudaMemcpyHostToDevice));
   CUDA_TRY(cudaMemcpy(s.t, t, (size_t)n * sizeof(float), cudaMemcpyHostToDevice));
   std::vector<int32_t> perm(n);
   std::vector<float> l(n);
   std::vector<float2> corr(fits ? steps : 0);
   uint64_t st = seed;
-  for (int ep = 0; ep < epochs; ++ep) {
+  auto shuffle = [&] {
     for (int i = 0; i < n; ++i) perm[i] = i;
     for (int i = n - 1; i > 0; --i) {  // seeded Fisher-Yates
       const int j = (int)(splitmix(&st) % (uint64_t)(i + 1));
       const int32_t tmp = perm[i]; perm[i] = perm[j]; perm[j] = tmp;
     }
+  };
+  shuffle();
+  for (int ep = 0; ep < epochs; ++ep) {
     CUDA_TRY(cudaMemcpy(s.idx, perm.data(), (size_t)n * sizeof(int32_t), cudaMemcpyHostToDevice));
     if (fits) {
       for (int k = 0; k < steps; ++k) corr[k] = adam_correction(++m->step);
@@ -1462,6 +1520,7 @@ int fora_model_train(fora_model* m, const float* x, const float* t, int32_t n, i
         CUDA_TRY(launch_adam(m->master, m->adam_m, m->adam_v, m->grad, ++m->step, lr, 0));
       }
     }
+    if (ep + 1 < epochs) shuffle();  // while the device runs the epoch
     if (loss_per_epoch) {
       CUDA_TRY(cudaMemcpy(l.data(), s.loss, (size_t)n * sizeof(float), cudaMemcpyDeviceToHost));
       double sum = 0.0;

@@ -142,9 +142,19 @@ struct PipeHook {
 };
 constexpr int kMaxPipeline = 4;
 
+// Device memory of short calls (the select alone, the network's), in the order of a stream.  It
+// comes from a pool of the library's, one per device, that keeps up to kScratchKept bytes between
+// calls, for any thread and stream, and gives them back when a graph is destroyed.  (Out of the
+// device's default pool, which keeps nothing over a synchronise, the scratch of 24 rows took 145
+// of the 328 us of fora_topk.)
+constexpr uint64_t kScratchKept = 64ull << 20;
+cudaError_t scratch_alloc(void** p, size_t bytes, cudaStream_t st);
+void scratch_free(void* p, cudaStream_t st);
+void scratch_trim(int device);
+
 // Admission of further sources while a batch is in its push rounds (the serving lanes):
-// the rounds run from a host loop, and after each round `poll` may write up to `room`
-// sources to `dst` (HOST) and returns how many; they join the batch as its next slots and
+// `poll`, called again and again meanwhile, may write up to `room` sources to `dst` (HOST) and
+// returns how many; after the running round they join the batch as its next slots and
 // their queries run exactly as they would alone.  The batch then has *nsrc_final sources
 // (outputs and stats are sized for `cap`).
 struct JoinHook {

@@ -16,7 +16,7 @@
 //                   sorts it (bitonic, in shared memory) and writes the first k.
 // Two passes over the rows; HBM bounds large ones, the launches and the sort small ones.
 // 24 rows of 10^6 estimates: 40 us, 4 us where no level is left, 50 us (the two passes at the
-// measured copy rate: 58); fora_topk 522 -> 328 us, 145 of them its allocation.  (As 19 launches:
+// measured copy rate: 58); fora_topk 522 -> 128 us.  (As 19 launches:
 // eight levels of 12 bits from the top, whether a row had use for them or not, then collect and
 // sort.)
 #include <algorithm>
