@@ -485,7 +485,11 @@ int fora::run_batch_ws(fora_graph* g, Workspace* w, const fora_params* p,
   set_round_keys(&b, p->seed);
   b.zero_hop = (p->flags & FORA_ZERO_HOP) != 0;
   b.want_count = dbg && dbg->count;
-  CUDA_TRY(cudaMemsetAsync(w->tally, 0, (size_t)nsrc * b.ends * sizeof(unsigned long long), stream));
+  b.side_by_side = indexed;
+  // of whole groups: a source that joins one finds its sums at 0
+  CUDA_TRY(cudaMemsetAsync(w->tally, 0,
+                           (size_t)std::min(b.ngrp * b.gw, b.lay) * b.ends * sizeof(unsigned long long),
+                           stream));
   if (b.want_count)
     CUDA_TRY(cudaMemsetAsync(b.wcount, 0, (size_t)nsrc * b.ends * sizeof(uint32_t), stream));
   CUDA_TRY(cudaMemsetAsync(w->small, 0, 8 * sizeof(unsigned long long), stream));
@@ -547,8 +551,6 @@ int fora::run_batch_ws(fora_graph* g, Workspace* w, const fora_params* p,
                                  cudaMemcpyHostToDevice, stream));
         CUDA_TRY(cudaMemcpyAsync(w->rmax + first, w->h_rmax + first, k * sizeof(double),
                                  cudaMemcpyHostToDevice, stream));
-        CUDA_TRY(cudaMemsetAsync(w->tally + (size_t)first * b.ends, 0,
-                                 (size_t)k * b.ends * sizeof(unsigned long long), stream));
         CUDA_TRY(cudaMemsetAsync(w->stats + first, 0, k * sizeof(SlotStats), stream));
         set_sources(g, w, first + k, &b);
         // the places of groups that are new (those of the others were zeroed with the batch's)
@@ -557,6 +559,9 @@ int fora::run_batch_ws(fora_graph* g, Workspace* w, const fora_params* p,
         if (end > off) {
           CUDA_TRY(cudaMemsetAsync(w->r + off, 0, (end - off) * sizeof(double), stream));
           CUDA_TRY(cudaMemsetAsync(w->res + off, 0, (end - off) * sizeof(double), stream));
+          const size_t from = (size_t)grp0 * b.gw * b.ends;
+          const size_t to = (size_t)std::min(b.ngrp * b.gw, b.lay) * b.ends;
+          CUDA_TRY(cudaMemsetAsync(w->tally + from, 0, (to - from) * sizeof(unsigned long long), stream));
         }
         CUDA_TRY(launch_push_join(gd, b, first, k, stream));
       }

@@ -191,6 +191,7 @@ struct BatchDev {
   unsigned long long* acc;
   uint32_t* wcount;
   unsigned long long ends;  // end_places of the graph
+  int side_by_side;         // the sums of a group's sources lie side by side (indexed walks)
   // Frontier of group g: entry e < slot_cnt[par][g] (par: the round's parity) is a node with
   // {first edge, degree} q[g * gw * n + e] and increments fa[g * gw * n + e * w + slot % gw]; its
   // hub items, i < slot_cnt[2 + par][g], are {entry, first edge} hub[g * gw * hub_stride + i]
@@ -248,6 +249,20 @@ struct BatchDev {
   uint32_t tiles;                  // units per group, ceil(n / (kTakeUnit / gw))
   unsigned long long light_edges;
 };
+
+// The sums of a slot's walk ends: that of place p at first + p * step.
+struct EndSums {
+  unsigned long long first, step;
+  __device__ __forceinline__ unsigned long long at(uint32_t place) const {
+    return first + (unsigned long long)place * step;
+  }
+};
+__device__ __forceinline__ EndSums end_sums(const BatchDev& b, int slot) {
+  if (!b.side_by_side) return EndSums{(unsigned long long)slot * b.ends, 1ull};
+  const int gr = slot / b.gw;
+  return EndSums{(unsigned long long)gr * b.gw * b.ends + (unsigned long long)(slot % b.gw),
+                 (unsigned long long)min(b.gw, b.lay - gr * b.gw)};
+}
 
 // Launch-shape parameters of a graph (set through fora_graph_tune or the autotuner).
 struct Tuning {

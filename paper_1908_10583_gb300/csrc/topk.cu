@@ -50,12 +50,12 @@ __global__ void __launch_bounds__(kEstThreads) k_estimate(GraphDev g, BatchDev b
     const unsigned long long w = min(G, b.lay - gr * G);
     if (slot >= b.nsrc) continue;
     const unsigned long long g0 = (unsigned long long)gr * G * n;
-    const unsigned long long e0 = (unsigned long long)slot * b.ends;
+    const EndSums sums = end_sums(b, slot);
     unsigned long long acc[kEstPer];
 #pragma unroll
     for (int k = 0; k < kEstPer; ++k) {
       const unsigned long long v = v0 + k * (kEstThreads / G);
-      acc[k] = v < n ? b.acc[e0 + end_place(g, walk_id(g, g.wid[v]))] : 0ull;
+      acc[k] = v < n ? b.acc[sums.at(end_place(g, walk_id(g, g.wid[v])))] : 0ull;
     }
 #pragma unroll
     for (int k = 0; k < kEstPer; ++k) {

@@ -659,85 +659,163 @@ __global__ void k_index_residue(GraphDev g, double* r, double rmax) {
     r[v] = __dmul_rn(rmax, (double)(g.row[v + 1] - g.row[v]));
 }
 
-// The walk phase served from a walk index: walk j of residual entry (slot, v) ends at
-// idx_dest[idx_off[v] + j] (the j-th stored walk from v) instead of being simulated.
-// A warp maps a chunk of walks to their entries in a shared-memory map.
-// A walk past v's stored walks (a residue above the index's r_max) sets kErrIndexRange
-// and is skipped.
-constexpr int kChunk = 1024;  // walks a warp maps to their entries at a time
-// Walks whose dependent loads (entry, index offset, destination) a lane has in flight.  64 sources
-// of a 2^20-node graph, 1.57e9 stored walks: 12.4 ms with 1, 11.5 with 2, 11.2 with 4, 13.3 with 8
-// (128 registers).  The additions to the tallies bound it: 1.4e11 a second is what scattered 8-byte
-// atomics with this graph's skew reach on their own.
-constexpr int kIndexedPer = 4;
-__global__ void __launch_bounds__(kIndexedThreads) k_walks_indexed(GraphDev g, BatchDev b,
-                                                                const unsigned long long* idx_off,
-                                                                const uint32_t* idx_dest) {
-  __shared__ uint16_t smap[kIndexedThreads / 32][kChunk];
-  if (*b.err) return;
-  const unsigned long long W = b.totals[1];
-  const unsigned long long nR = b.totals[0];
-  const uint32_t lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  const unsigned long long warp = ((unsigned long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const unsigned long long nwarps = ((unsigned long long)gridDim.x * blockDim.x) >> 5;
-  const uint32_t chunk = share_walks(W, nwarps, kChunk);
-  const unsigned long long* off = b.wr_offset;
-  bool out_of_range = false;
-  for (unsigned long long cbeg = warp * chunk; cbeg < W; cbeg += nwarps * chunk) {
-    const uint32_t cnt = (uint32_t)min((unsigned long long)chunk, W - cbeg);
-    const unsigned long long idx0 = warp_find_entry(off, nR, cbeg);
-    unsigned long long idxw = idx0;
-    for (uint32_t rb = 0; rb < cnt; rb += 32) {
-      const unsigned long long gw = cbeg + rb + lane;
-      const unsigned long long o = idxw + lane < nR ? off[idxw + lane] : ~0ull;
-      int lo = 0, hi = 31;  // largest j with off[idxw + j] <= gw
+// The walk phase served from a walk index: walk j of the residue (slot, v) ends at
+// idx_dest[idx_off[v] + j] (the j-th stored walk from v) instead of being simulated.  The sources
+// of a group that hold a residue at v share its first walks, so the kernels go through the
+// residues by node and a warp adds, for each of 32 / G walks, the weights of the G sources to
+// their sums, which lie side by side (BatchDev::side_by_side): one sector takes all four.  The
+// additions bound it: 7.2 ms for 64 sources of a 2^20-node graph, 1.57e9 walks, 2.2e11 a second.
+// (Source by source, from a list of entries, they took 11.2 ms: 1.4e11 a second, what scattered
+// 8-byte atomics with this graph's skew reach; the list took 0.9 ms more.)
+// k_indexed_nodes takes the nodes of up to kIndexedMost walks and lists the others, whose walks
+// k_indexed_hubs takes in chunks of kIndexedMost.
+// A residue of more walks than are stored (above the index's r_max) sets kErrIndexRange; only the
+// stored ones are taken.
+constexpr uint32_t kIndexedMost = 1024;
+constexpr int kIndexedPer = 4;    // steps of a warp (of 32 / G walks) whose loads are in flight
+constexpr int kIndexedLoads = 8;  // residues a lane reads before it uses any
+constexpr int kListBits = 36;     // of *walk_next: chunks listed, below them; nodes listed, above
+
+// This lane's source of group gr: its residue's walks and weight at node v, at most the stored
+// ones.  Every lane of the warp must call it.
+template <int G>
+__device__ __forceinline__ void indexed_entry(const BatchDev& b, double r, uint32_t stored,
+                                              uint32_t* omega, unsigned long long* weight) {
+  const float cf = __double2float_rn(b.walk_scale);
+  const bool fast = cf >= 1.0f && cf <= 0x1p100f;
+  const double x = sampled(b, r);
+  const uint32_t w = (uint32_t)walks_of(x, b.walk_scale, cf, fast);  // below 2^32 (scan)
+  *weight = w ? weight_of(x, (double)w) : 0ull;
+  if (w > stored) atomicOr(b.err, kErrIndexRange);
+  *omega = min(w, stored);
+}
+
+// Adds the walk that ends at dest to this lane's source's sum (source j of w in the group).
+__device__ __forceinline__ void add_end(const GraphDev& g, const BatchDev& b,
+                                        unsigned long long base, uint32_t w, uint32_t j,
+                                        uint32_t dest, unsigned long long weight) {
+  const unsigned long long at = base + (unsigned long long)end_place(g, dest) * w + j;
+  if (b.want_count) atomicAdd(&b.wcount[at], 1u);
+  atomicAdd(&b.acc[at], weight);
+}
+
+template <int G>
+__global__ void __launch_bounds__(kIndexedThreads) k_indexed_nodes(
+    GraphDev g, BatchDev b, const unsigned long long* idx_off, const uint32_t* idx_dest) {
+  if (__any_sync(kFull, *b.err != 0)) return;  // whole warps
+  constexpr uint32_t kPer = 32 / G;                // nodes of a batch, walks of a step
+  constexpr uint32_t kNodes = kPer * kIndexedLoads;  // of a warp
+  const uint32_t lane = threadIdx.x & 31, j = lane % G, q = lane / G;
+  const unsigned long long n = (unsigned long long)g.n, units = (n + kNodes - 1) / kNodes;
+  const unsigned long long warp =
+      ((unsigned long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  if (warp >= units * (unsigned long long)b.ngrp) return;  // whole warps
+  const uint32_t gr = (uint32_t)(warp / units);
+  const uint32_t v0 = (uint32_t)((warp - gr * units) * kNodes);
+  const uint32_t w = min((uint32_t)G, (uint32_t)b.lay - gr * G);
+  const bool mine = j < w && gr * G + j < (uint32_t)b.nsrc;
+  const unsigned long long g0 = (unsigned long long)gr * G * n;
+  const unsigned long long base = (unsigned long long)gr * G * b.ends;
+  double r[kIndexedLoads];
 #pragma unroll
-      for (int s = 0; s < 5; ++s) {
-        const int mid = (lo + hi + 1) >> 1;
-        if (__shfl_sync(kFull, o, mid) <= gw) lo = mid; else hi = mid - 1;
-      }
-      const unsigned long long mine = idxw + (unsigned long long)lo;
-      smap[wid][rb + lane] = (uint16_t)(mine - idx0);
-      idxw = __shfl_sync(kFull, mine, 31);
-    }
-    __syncwarp();
-    for (uint32_t i0 = lane; i0 < cnt; i0 += 32 * kIndexedPer) {
-      unsigned long long idx[kIndexedPer], entry[kIndexedPer], j[kIndexedPer];
-      unsigned long long beg[kIndexedPer], end[kIndexedPer];
-      uint32_t dest[kIndexedPer];
+  for (int k = 0; k < kIndexedLoads; ++k) {
+    const unsigned long long v = v0 + k * kPer + q;
+    r[k] = mine && v < n ? b.r[g0 + v * w + j] : 0.0;
+  }
 #pragma unroll
-      for (int q = 0; q < kIndexedPer; ++q) {
-        const uint32_t i = min(i0 + 32u * q, cnt - 1u);
-        idx[q] = idx0 + smap[wid][i];
-        entry[q] = b.wr_entry[idx[q]];
-        j[q] = cbeg + i - off[idx[q]];
-      }
+  for (int k = 0; k < kIndexedLoads; ++k) {
+    if (!__any_sync(kFull, __double_as_longlong(r[k]) != 0)) continue;
+    const uint32_t v = (uint32_t)min((unsigned long long)(v0 + k * kPer + q), n - 1);
+    const unsigned long long off = idx_off[v];
+    uint32_t omega;
+    unsigned long long weight;
+    indexed_entry<G>(b, r[k], (uint32_t)(idx_off[v + 1] - off), &omega, &weight);
+    uint32_t most = omega;  // of the node's sources
 #pragma unroll
-      for (int q = 0; q < kIndexedPer; ++q) {
-        beg[q] = idx_off[(uint32_t)entry[q]];
-        end[q] = idx_off[(uint32_t)entry[q] + 1u];
-      }
-#pragma unroll
-      for (int q = 0; q < kIndexedPer; ++q) {
-        beg[q] += j[q];
-        if (beg[q] < end[q]) {
-          dest[q] = idx_dest[beg[q]];
-        } else if (i0 + 32u * q < cnt) {
-          out_of_range = true;
+    for (int o = 1; o < G; o <<= 1) most = max(most, __shfl_xor_sync(kFull, most, o));
+    if (most > kIndexedMost) {
+      if (j == 0) {
+        const unsigned long long chunks = (most + kIndexedMost - 1) / kIndexedMost;
+        const unsigned long long at = atomicAdd(b.walk_next, (1ull << kListBits) | chunks);
+        const unsigned long long i = at >> kListBits;
+        if (FORA_IN_RANGE(b.err, i, (unsigned long long)b.nsrc * n)) {
+          b.wr_entry[i] = (unsigned long long)gr << 32 | v;
+          b.wr_offset[i] = at & ((1ull << kListBits) - 1ull);
         }
       }
-#pragma unroll
-      for (int q = 0; q < kIndexedPer; ++q) {
-        if (i0 + 32u * q >= cnt || beg[q] >= end[q]) continue;
-        const unsigned long long at =
-            (entry[q] >> 32) * (unsigned long long)b.ends + end_place(g, dest[q]);
-        if (b.want_count) atomicAdd(&b.wcount[at], 1u);
-        atomicAdd(&b.acc[at], b.wr_weight[idx[q]]);
-      }
+      most = 0;
     }
-    __syncwarp();
+    // the batch's nodes have ceil(most / kPer) steps each, one after the other
+    const uint32_t steps = (most + kPer - 1) / kPer;
+    uint32_t incl = steps;
+#pragma unroll
+    for (int o = G; o < 32; o <<= 1) {
+      const uint32_t t = __shfl_up_sync(kFull, incl, o);
+      if ((int)lane >= o) incl += t;
+    }
+    const uint32_t total = __shfl_sync(kFull, incl, 31);
+    for (uint32_t t0 = 0; t0 < total; t0 += kIndexedPer) {
+      uint32_t dest[kIndexedPer];
+      unsigned long long add[kIndexedPer];
+      bool have[kIndexedPer];
+#pragma unroll
+      for (int u = 0; u < kIndexedPer; ++u) {
+        const uint32_t t = min(t0 + u, total - 1u);
+        const uint32_t node = __popc(__ballot_sync(kFull, j == 0 && incl <= t));
+        const uint32_t first = __shfl_sync(kFull, incl - steps, node * G);
+        const uint32_t walk = (t - first) * kPer + q;
+        const unsigned long long at = __shfl_sync(kFull, off, node * G) + walk;
+        add[u] = __shfl_sync(kFull, weight, node * G + j);
+        have[u] = walk < __shfl_sync(kFull, omega, node * G + j) && t0 + u < total;
+        dest[u] = have[u] ? idx_dest[at] : 0u;
+      }
+#pragma unroll
+      for (int u = 0; u < kIndexedPer; ++u)
+        if (have[u]) add_end(g, b, base, w, j, dest[u], add[u]);
+    }
   }
-  if (out_of_range) atomicOr(b.err, kErrIndexRange);
+}
+
+template <int G>
+__global__ void __launch_bounds__(kIndexedThreads) k_indexed_hubs(
+    GraphDev g, BatchDev b, const unsigned long long* idx_off, const uint32_t* idx_dest) {
+  if (__any_sync(kFull, *b.err != 0)) return;  // whole warps
+  constexpr uint32_t kPer = 32 / G;
+  const uint32_t lane = threadIdx.x & 31, j = lane % G, q = lane / G;
+  const unsigned long long listed = *b.walk_next;
+  const unsigned long long nodes = listed >> kListBits;
+  const unsigned long long chunks = listed & ((1ull << kListBits) - 1ull);
+  const unsigned long long nwarps = (unsigned long long)gridDim.x * (blockDim.x >> 5);
+  for (unsigned long long x = ((unsigned long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+       x < chunks; x += nwarps) {
+    const unsigned long long i = warp_find_entry(b.wr_offset, nodes, x);
+    const unsigned long long entry = b.wr_entry[i];
+    const uint32_t gr = (uint32_t)(entry >> 32), v = (uint32_t)entry;
+    const uint32_t w = min((uint32_t)G, (uint32_t)b.lay - gr * G);
+    const bool mine = j < w && gr * G + j < (uint32_t)b.nsrc;
+    const unsigned long long base = (unsigned long long)gr * G * b.ends;
+    const double r =
+        mine ? b.r[(unsigned long long)gr * G * g.n + (unsigned long long)v * w + j] : 0.0;
+    const unsigned long long off = idx_off[v];
+    uint32_t omega;
+    unsigned long long weight;
+    indexed_entry<G>(b, r, (uint32_t)(idx_off[v + 1] - off), &omega, &weight);
+    const unsigned long long beg = (x - b.wr_offset[i]) * kIndexedMost;
+    const uint32_t end = (uint32_t)min((unsigned long long)omega, beg + kIndexedMost);
+#pragma unroll 1
+    for (uint32_t k = (uint32_t)beg; k < (uint32_t)beg + kIndexedMost; k += kPer * kIndexedPer) {
+      if (!__any_sync(kFull, k < end)) break;
+      uint32_t dest[kIndexedPer];
+#pragma unroll
+      for (int u = 0; u < kIndexedPer; ++u) {
+        const uint32_t walk = k + u * kPer + q;
+        dest[u] = walk < end ? idx_dest[off + walk] : 0u;
+      }
+#pragma unroll
+      for (int u = 0; u < kIndexedPer; ++u)
+        if (k + u * kPer + q < end) add_end(g, b, base, w, j, dest[u], weight);
+    }
+  }
 }
 
 __global__ void k_unpack_ends(GraphDev g, BatchDev b, uint32_t* cnt, unsigned long long* acc) {
@@ -745,10 +823,10 @@ __global__ void k_unpack_ends(GraphDev g, BatchDev b, uint32_t* cnt, unsigned lo
   const unsigned long long stride = (unsigned long long)gridDim.x * blockDim.x;
   for (int slot = blockIdx.y; slot < b.nsrc; slot += gridDim.y) {
     const unsigned long long g0 = (unsigned long long)slot * n;
+    const EndSums sums = end_sums(b, slot);
     for (unsigned long long v = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x; v < n;
          v += stride) {
-      const unsigned long long at =
-          (unsigned long long)slot * b.ends + end_place(g, walk_id(g, g.wid[v]));
+      const unsigned long long at = sums.at(end_place(g, walk_id(g, g.wid[v])));
       if (cnt) cnt[g0 + v] = b.wcount[at];
       if (acc) acc[g0 + v] = b.acc[at];
     }
@@ -781,7 +859,7 @@ cudaError_t residuals_t(const GraphDev& g, const BatchDev& b, cudaStream_t st) {
   if (e != cudaSuccess) return e;
   k_residual_scan<<<1, 1024, 0, st>>>(b);
   e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
+  if (e != cudaSuccess || b.side_by_side) return e;  // indexed walks need no list
   k_residual_emit<G><<<blocks, kResidualThreads, 0, st>>>(g, b);
   return cudaGetLastError();
 }
@@ -827,13 +905,28 @@ cudaError_t launch_index_residue(const GraphDev& g, double* r, double rmax, cuda
   return cudaGetLastError();
 }
 
+template <int G>
+cudaError_t walks_indexed_t(const GraphDev& g, const BatchDev& b, int num_sms,
+                            const unsigned long long* idx_off, const uint32_t* idx_dest,
+                            cudaStream_t st) {
+  constexpr unsigned long long kNodes = 32 / G * kIndexedLoads, kWarps = kIndexedThreads / 32;
+  const unsigned long long warps =
+      ((unsigned long long)g.n + kNodes - 1) / kNodes * (unsigned long long)b.ngrp;
+  k_indexed_nodes<G><<<(unsigned)((warps + kWarps - 1) / kWarps), kIndexedThreads, 0, st>>>(
+      g, b, idx_off, idx_dest);
+  cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess) return e;
+  const int per_sm = resident_blocks((const void*)k_indexed_hubs<G>, kIndexedThreads);
+  if (per_sm == 0) return cudaErrorInvalidConfiguration;
+  k_indexed_hubs<G><<<num_sms * per_sm, kIndexedThreads, 0, st>>>(g, b, idx_off, idx_dest);
+  return cudaGetLastError();
+}
+
 cudaError_t launch_walks_indexed(const GraphDev& g, const BatchDev& b, int num_sms,
                                  const unsigned long long* idx_off, const uint32_t* idx_dest,
                                  cudaStream_t st) {
-  const int per_sm = resident_blocks((const void*)k_walks_indexed, kIndexedThreads);
-  if (per_sm == 0) return cudaErrorInvalidConfiguration;
-  k_walks_indexed<<<num_sms * per_sm, kIndexedThreads, 0, st>>>(g, b, idx_off, idx_dest);
-  return cudaGetLastError();
+  return b.gw == 1 ? walks_indexed_t<1>(g, b, num_sms, idx_off, idx_dest, st)
+                   : walks_indexed_t<4>(g, b, num_sms, idx_off, idx_dest, st);
 }
 
 cudaError_t launch_unpack_ends(const GraphDev& g, const BatchDev& b, uint32_t* cnt,

@@ -1,0 +1,46 @@
+"""Indexed walks of groups of sources (1 or 4 side by side, the last group not full): nodes of
+few walks, of walks around a warp's step and a chunk of 1024, and hubs of many chunks, against the
+oracle on given residues."""
+import numpy as np
+import pytest
+
+import inputs
+import oracle
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+import paper_1908_10583_gb300 as fora  # noqa: E402
+from tests.test_gpu_index import _debug  # noqa: E402
+from tests.test_gpu_parity import _built  # noqa: E402,F401
+
+SEED, RMAX = 11, 1e-3
+
+
+# node counts around the nodes of a warp (64 in groups of four, 256 alone)
+@pytest.mark.parametrize("n,nsrc", [(1, 1), (63, 3), (65, 4), (255, 2), (257, 1), (300, 6), (300, 9)])
+def test_indexed_walks_of_groups_are_bit_exact(n, nsrc):
+    rng = np.random.default_rng(1000 * n + nsrc)
+    edges = [(v, int(u)) for v in range(n) for u in rng.integers(0, n, 1 + rng.poisson(3))]
+    edges += [(v, int(u)) for v in range(min(3, n)) for u in rng.integers(0, n, 700 * (v + 1))]
+    rp, col = inputs.csr_from_edges(n, edges)
+    deg = np.diff(rp)
+    g = fora.Graph(rp, col)
+    # C is about 6e4: 60 walks for an edge, up to 1e5 for a hub
+    g.build_index(fora.Params.make(k=1, delta=1e-3, pf=1e-3, rmax=RMAX, seed=SEED))
+    rmax, C, _ = g.index_info()
+    off, dest = oracle.walk_index(rp, col, 0.2, C, rmax, SEED)
+    walks = rng.choice([0.0, 0.5, 1, 7, 8, 9, 31, 32, 33, 1023, 1024, 1025, 2049, 1e9], (nsrc, n))
+    r = np.minimum(walks / C, rmax * deg)
+    r[0] = rmax * deg  # every stored walk
+    res = rng.random((nsrc, n))
+    p = fora.Params.make(k=1, delta=1e-3, pf=1e-3, rmax=RMAX, seed=1, flags=fora.FORA_USE_INDEX)
+    sources = rng.integers(0, n, nsrc).astype(np.int32)
+    _, _, st, out = _debug(g, sources, p, given=(res, r))
+    for i in range(nsrc):
+        cnt, acc, wst = oracle.walk_phase_indexed(n, C, r[i], off, dest)
+        np.testing.assert_array_equal(out["count"][i], cnt)
+        np.testing.assert_array_equal(out["acc"][i], acc)
+        np.testing.assert_array_equal(out["estimate"][i], oracle.estimate(res[i], acc))
+        assert st[i].walks == wst.walks
+    g.close()
