@@ -830,7 +830,12 @@ __device__ __forceinline__ void take_unit(const GraphDev& g, const BatchDev& b, 
 // The take: every unit of a group with a heavy round (listed in b.alist), and the listed units
 // of the groups with light ones.  A warp reads consecutive units, so its counters belong to one
 // or two groups; what is left of them at the end a block adds together.
-template <int G, int L>
+// Without groups (the balanced push) sources may differ much in what they take, and in large
+// scans a warp's units come from four places of the list: the balanced push of 256 sources of a
+// 2^20-node graph 317 -> 299 ms.  100 of 2^18, whose warps scan 21 units a round, 33.3 -> 33.9: so
+// from 48 units a warp on, and a kernel of its own, as the loop costs the others 3%.
+constexpr unsigned long long kFarUnits = 48;
+template <int G, int L, bool kFar>
 __device__ void take_phase(const GraphDev& g, const BatchDev& b, int nx, uint32_t nheavy,
                            uint32_t nlist, TakeStage<G>& st) {
   const unsigned long long nwarps = (unsigned long long)gridDim.x * (blockDim.x >> 5);
@@ -841,9 +846,14 @@ __device__ void take_phase(const GraphDev& g, const BatchDev& b, int nx, uint32_
   constexpr uint32_t kParts = 8 / L;  // of a unit
   const uint32_t per = b.tiles * kParts;
   const unsigned long long units = (unsigned long long)nheavy * per;
-  unsigned long long x = units * warp / nwarps;
-  const unsigned long long end = units * (warp + 1) / nwarps;
-  if (x < end) {
+  // A warp scans a stretch of consecutive units, with kFar four stretches a quarter of the list
+  // apart where they are long.
+  const unsigned pieces = kFar && units >= kFarUnits * nwarps ? 4u : 1u;
+  for (unsigned k = 0; k < pieces; ++k) {
+    const unsigned long long at = k * nwarps + warp, of = pieces * nwarps;
+    unsigned long long x = units * at / of;
+    const unsigned long long end = units * (at + 1) / of;
+    if (x >= end) continue;
     unsigned long long ga = x / per;
     uint32_t unit = (uint32_t)(x - ga * per);
     uint32_t gr = b.ngrp == 1 ? 0u : __ldcg(&b.alist[ga]);
@@ -858,7 +868,7 @@ __device__ void take_phase(const GraphDev& g, const BatchDev& b, int nx, uint32_
     }
   }
   const unsigned long long listed = (unsigned long long)nlist * kParts;
-  x = listed * warp / nwarps;
+  unsigned long long x = listed * warp / nwarps;
   const unsigned long long lend = listed * (warp + 1) / nwarps;
   for (; x < lend; ++x) {
     const uint32_t t = __ldcg(&b.tlist[x / kParts]);
@@ -1144,7 +1154,7 @@ constexpr int kPushBlocks = 4;
 // device reads) ends the launch after its round, and with `resume` the push goes on where such a
 // launch left it.  (A template parameter: with the second entry into the loop a launch for one
 // source of a small graph spills 148 bytes, without it 116.)
-template <int G, int L, bool kJoin>
+template <int G, int L, bool kJoin, bool kFar = false>
 __global__ void __launch_bounds__(kPushThreads, kPushBlocks)
     k_push(const __grid_constant__ GraphDev g, const __grid_constant__ BatchDev b, int resume,
            const volatile uint32_t* pause) {
@@ -1167,7 +1177,7 @@ __global__ void __launch_bounds__(kPushThreads, kPushBlocks)
   }
   for (; go; nx ^= 1) {
     if (!kJoin || take) {
-      take_phase<G, L>(g, b, nx, __ldcg(&ctl->nheavy), __ldcg(&ctl->nlist), sh.take[wid]);
+      take_phase<G, L, kFar>(g, b, nx, __ldcg(&ctl->nheavy), __ldcg(&ctl->nlist), sh.take[wid]);
       go = grid_meet(b, ++met, true, [&] {
         const uint32_t stop = kJoin && threadIdx.x == 0 ? *pause : 0u;
         return advance_phase<G>(b, nx, gridDim.x * kPushWarps) && !stop;
@@ -1203,7 +1213,7 @@ template <int G>
 __global__ void __launch_bounds__(kPushThreads, kPushBlocks)
     k_push_take(const __grid_constant__ GraphDev g, const __grid_constant__ BatchDev b) {
   __shared__ TakeStage<G> stage[kPushWarps];
-  take_phase<G, 8>(g, b, b.ps->cur ^ 1, b.ctl->nheavy, b.ctl->nlist, stage[threadIdx.x >> 5]);
+  take_phase<G, 8, false>(g, b, b.ps->cur ^ 1, b.ctl->nheavy, b.ctl->nlist, stage[threadIdx.x >> 5]);
 }
 template <int G>
 __global__ void __launch_bounds__(kPushThreads) k_push_advance(const __grid_constant__ BatchDev b) {
@@ -1279,10 +1289,10 @@ __global__ void k_regroup(double* grouped, double* rows, unsigned long long n, i
   }
 }
 
-template <int G, int L, bool kJoin>
+template <int G, int L, bool kJoin, bool kFar = false>
 cudaError_t push_t(const GraphDev& g, const BatchDev& b, int num_sms, bool resume,
                    const uint32_t* pause, cudaStream_t st) {
-  const void* kernel = (const void*)k_push<G, L, kJoin>;
+  const void* kernel = (const void*)k_push<G, L, kJoin, kFar>;
   const int per_sm = resident_blocks(kernel, kPushThreads);
   if (per_sm == 0) return cudaErrorInvalidConfiguration;
   // every SM at least once; more blocks only where a full scan has work for them
@@ -1305,8 +1315,11 @@ cudaError_t push_any(const GraphDev& g, const BatchDev& b, int num_sms, bool res
   if (pause)
     return small ? push_t<G, 2, true>(g, b, num_sms, resume, pause, st)
                  : push_t<G, 8, true>(g, b, num_sms, resume, pause, st);
-  return small ? push_t<G, 2, false>(g, b, num_sms, false, nullptr, st)
-               : push_t<G, 8, false>(g, b, num_sms, false, nullptr, st);
+  if (small) return push_t<G, 2, false>(g, b, num_sms, false, nullptr, st);
+  const unsigned long long warps = (unsigned long long)num_sms * kPushBlocks * kPushWarps;
+  if (G == 1 && (unsigned long long)b.ngrp * b.tiles >= kFarUnits * warps)
+    return push_t<G, 8, false, G == 1>(g, b, num_sms, false, nullptr, st);
+  return push_t<G, 8, false>(g, b, num_sms, false, nullptr, st);
 }
 
 template <int G>
