@@ -28,8 +28,8 @@ if ROOT not in sys.path:
 
 METRIC = "SSPPR queries/s and p99 latency at ε=0.5, batched+learned r_max vs plain FORA"
 UNIT = "queries/s"
-WALK_BYTES_PER_MOVE = 12      # row_ptr pair (8 B) + col entry (4 B)
-WALK_BYTES_PER_WALK = 24      # count RMW (4+4 B) + acc RMW (8+8 B)
+WALK_BYTES_PER_MOVE = 4       # edge record
+WALK_BYTES_PER_WALK = 16      # sum RMW (8+8 B)
 WALK_BYTES_PER_ENTRY = 24     # residual entry, offset, weight (8 B each)
 PUSH_BYTES_PER_EDGE = 20      # col entry (4 B) + FP64 read-modify-write of r(u) (16 B)
 PUSH_BYTES_PER_VERTEX = 44    # row pair, r(v) read and zero, reserve RMW, queue append
@@ -500,7 +500,7 @@ def run_fora(args):
                 "traffic": profiled_traffic("k_walks", args.workload, launches_per_step),
                 "algorithmic_bytes_per_launch": bytes_per_launch,
                 "launches_per_step": launches_per_step}
-    # the walk kernel is bound by issue and latency rather than by DRAM: its issue-slot and
+    # the walk kernel is bound by L2 gathers rather than by DRAM: its issue-slot and
     # L2 fractions from the committed ncu section capture of the same kernel (64 sources)
     wp = profile_values("k_walks", args.workload)
     if "issue_active_frac" in wp:
@@ -509,9 +509,7 @@ def run_fora(args):
         roofline["issue_l2_source"] = "ncu section capture, profiles/k_walks_" + args.workload + ".txt"
     # the push phase (all its rounds: spread, take, advance) against the same peak
     achieved_push = (sum(push_bytes) / len(push_bytes)) / (statistics.mean(push_ms) / 1e3) / 1e9
-    spread_kernel = ("k_push_spread_hot" if tuning.get("spread_hot") and tuning.get("hot_nodes")
-                     else "k_push_spread")
-    roofline_push = {"bound": "hbm", "kernels": spread_kernel + "+k_push_take+k_push_advance",
+    roofline_push = {"bound": "hbm", "kernels": "k_push",
                      "achieved": achieved_push, "peak": peak, "peak_kind": peak_kind,
                      "unit": "GB/s", "frac": achieved_push / peak,
                      "traffic": profiled_traffic("push", args.workload, 1, "dram_bytes_per_step"),
