@@ -848,27 +848,32 @@ __device__ void take_phase(const GraphDev& g, const BatchDev& b, int nx, uint32_
   const unsigned long long units = (unsigned long long)nheavy * per;
   // A warp scans a stretch of consecutive units, with kFar four stretches a quarter of the list
   // apart where they are long.
+  unsigned long long x = units * warp / nwarps;
+  unsigned long long end = units * (warp + 1) / nwarps;
   const unsigned pieces = kFar && units >= kFarUnits * nwarps ? 4u : 1u;
-  for (unsigned k = 0; k < pieces; ++k) {
-    const unsigned long long at = k * nwarps + warp, of = pieces * nwarps;
-    unsigned long long x = units * at / of;
-    const unsigned long long end = units * (at + 1) / of;
-    if (x >= end) continue;
-    unsigned long long ga = x / per;
-    uint32_t unit = (uint32_t)(x - ga * per);
-    uint32_t gr = b.ngrp == 1 ? 0u : __ldcg(&b.alist[ga]);
-    for (;;) {
-      if (gr != tg.gr) take_enter<G>(g, b, nx, gr, st, tg, tc);
-      take_unit<G, L>(g, b, nx, unit, st, tg, tc);
-      if (++x >= end) break;
-      if (++unit == per) {
-        unit = 0;
-        gr = __ldcg(&b.alist[++ga]);
+  for (unsigned k = 0;;) {
+    if (kFar && pieces > 1) {
+      x = units * (k * nwarps + warp) / (pieces * nwarps);
+      end = units * (k * nwarps + warp + 1) / (pieces * nwarps);
+    }
+    if (x < end) {
+      unsigned long long ga = x / per;
+      uint32_t unit = (uint32_t)(x - ga * per);
+      uint32_t gr = b.ngrp == 1 ? 0u : __ldcg(&b.alist[ga]);
+      for (;;) {
+        if (gr != tg.gr) take_enter<G>(g, b, nx, gr, st, tg, tc);
+        take_unit<G, L>(g, b, nx, unit, st, tg, tc);
+        if (++x >= end) break;
+        if (++unit == per) {
+          unit = 0;
+          gr = __ldcg(&b.alist[++ga]);
+        }
       }
     }
+    if (!kFar || ++k >= pieces) break;
   }
   const unsigned long long listed = (unsigned long long)nlist * kParts;
-  unsigned long long x = listed * warp / nwarps;
+  x = listed * warp / nwarps;
   const unsigned long long lend = listed * (warp + 1) / nwarps;
   for (; x < lend; ++x) {
     const uint32_t t = __ldcg(&b.tlist[x / kParts]);
