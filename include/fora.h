@@ -446,7 +446,10 @@ int fora_threshold_debug(const double *r, const double *rmax, const uint32_t *d,
  * its own workspace, stream and host thread, part k's push starting when part k-1's push
  * has finished, so one part's walk phase runs beside the next part's push; the call's
  * stream waits for all parts, and each part's stats carry that part's phase times.
- * Results do not depend on it.  "max_push_rounds" (1..100000, default 100000): the cap
+ * Results do not depend on it.  "index_groups" (0..65535, default 0): the groups of sources
+ * that one pass of the walk phase from an index takes, 0 (and any larger value) as many as its
+ * list of long residues can count (fora_index_list_groups).  Results do not depend on it.
+ * "max_push_rounds" (1..100000, default 100000): the cap
  * on the push rounds of Alg. 1 (the loop is bounded so that it cannot run away); a query
  * whose push needs more rounds stops there and returns FORA_ERR_PUSH_NOT_CONVERGED.
  * Unknown keys and out-of-range values return FORA_ERR_BAD_ARG.
@@ -509,6 +512,15 @@ int fora_index_destroy(fora_graph *g);
  * [1, 65535] or a decreasing row_ptr.
  */
 int fora_workspace_bytes(int64_t n, const int64_t *row_ptr, int32_t nsrc, uint64_t *bytes);
+
+/*
+ * How many groups of `width` sources one pass of the walk phase from an index can take on a
+ * graph of n nodes: its list of the residues of more than 1024 walks counts the listed nodes
+ * in 28 bits and their chunks of 1024 walks in 36, and a source has fewer than 2^32 walks.
+ * Larger batches take several passes.  Host arithmetic only (no device needed).
+ * FORA_ERR_BAD_ARG for n outside [1, 2^31), width outside [1, 32] or a null pointer.
+ */
+int fora_index_list_groups(int64_t n, int32_t width, int64_t *groups);
 
 /*
  * Fault injection for tests: the nth device allocation the library makes from now on

@@ -188,6 +188,8 @@ def load():
         L.fora_index_destroy.argtypes = [P]
         L.fora_workspace_bytes.restype = I
         L.fora_workspace_bytes.argtypes = [i64, P, i32, P]
+        L.fora_index_list_groups.restype = I
+        L.fora_index_list_groups.argtypes = [i64, i32, P]
         L.fora_hot_nodes.restype = I
         L.fora_hot_nodes.argtypes = [i64, P, P, P, i32, P]
         L.fora_debug_checks.restype = I
@@ -496,6 +498,13 @@ def hot_nodes(row_ptr, col) -> np.ndarray:
     _check(load().fora_hot_nodes(len(rp) - 1, rp.ctypes.data, c.ctypes.data, out.ctypes.data,
                                  len(out), ctypes.byref(count)))
     return out[:count.value]
+
+
+def index_list_groups(n: int, width: int) -> int:
+    """Groups of sources that one pass of the indexed walks takes (fora_index_list_groups)."""
+    out = ctypes.c_int64()
+    _check(load().fora_index_list_groups(int(n), int(width), ctypes.byref(out)))
+    return out.value
 
 
 def debug_fail_alloc(nth: int):

@@ -503,8 +503,10 @@ int fora::run_batch_ws(fora_graph* g, Workspace* w, const fora_params* p,
     b.cost_walk = bal->walk;
   }
   bool host_loop;
+  int index_groups;
   {
     std::lock_guard<std::mutex> tlock(g->mu);
+    index_groups = g->tune.index_groups;
     b.spread_width = g->tune.spread_width;
     if (g->tune.spread_hot == 0) b.hot_copies = 0;
     b.walk_blocks = g->tune.walk_blocks;
@@ -599,7 +601,7 @@ int fora::run_batch_ws(fora_graph* g, Workspace* w, const fora_params* p,
   CUDA_TRY(launch_residuals(gd, b, stream));
   if (timed) CUDA_TRY(cudaEventRecord(w->ev[2], stream));
   if (indexed)
-    CUDA_TRY(launch_walks_indexed(gd, b, g->num_sms, g->idx_off, g->idx_dest, stream));
+    CUDA_TRY(launch_walks_indexed(gd, b, g->num_sms, index_groups, g->idx_off, g->idx_dest, stream));
   else
     CUDA_TRY(launch_walks(gd, b, g->num_sms, stream));
   if (timed) CUDA_TRY(cudaEventRecord(w->ev[3], stream));
@@ -1307,6 +1309,11 @@ int fora_graph_tune(fora_graph* g, const char* key, int64_t value) {
     g->tune.push_host_loop = (int)value;
     return FORA_OK;
   }
+  if (strcmp(key, "index_groups") == 0) {
+    if (value < 0 || value > 65535) return fail(FORA_ERR_BAD_ARG, "index_groups must be in [0, 65535]");
+    g->tune.index_groups = (int)value;
+    return FORA_OK;
+  }
   if (strcmp(key, "max_push_rounds") == 0) {
     if (value < 1 || value > (int64_t)kMaxPushRounds)
       return fail(FORA_ERR_BAD_ARG, "max_push_rounds must be in [1, %u]", kMaxPushRounds);
@@ -1715,8 +1722,16 @@ int fora_graph_tuning(fora_graph* g, const char* key, int64_t* value) {
   if (strcmp(key, "walk_blocks") == 0) { *value = g->tune.walk_blocks; return FORA_OK; }
   if (strcmp(key, "pipeline") == 0) { *value = g->tune.pipeline; return FORA_OK; }
   if (strcmp(key, "push_host_loop") == 0) { *value = g->tune.push_host_loop; return FORA_OK; }
+  if (strcmp(key, "index_groups") == 0) { *value = g->tune.index_groups; return FORA_OK; }
   if (strcmp(key, "max_push_rounds") == 0) { *value = g->tune.max_push_rounds; return FORA_OK; }
   return fail(FORA_ERR_BAD_ARG, "unknown tuning key '%s'", key);
+}
+
+int fora_index_list_groups(int64_t n, int32_t width, int64_t* groups) {
+  if (n < 1 || n > 0x7FFFFFFF || width < 1 || width > 32 || !groups)
+    return fail(FORA_ERR_BAD_ARG, "bad arguments");
+  *groups = index_list_groups(n, width);
+  return FORA_OK;
 }
 
 int fora_workspace_bytes(int64_t n, const int64_t* row_ptr, int32_t nsrc, uint64_t* bytes) {

@@ -32,6 +32,20 @@ constexpr int kDigitBits = 12;
 constexpr int kBins = 1 << kDigitBits;
 constexpr uint32_t kSortCap = 8192;  // candidates sorted in shared memory at the end
 
+// Indexed walks: residues of more than kIndexedMost walks are listed, in a list whose length is
+// counted in one word: the listed nodes from bit kListBits on, their chunks of kIndexedMost walks
+// below.  A list serves at most index_list_groups groups of sources, so that neither count can
+// leave its bits: a source has fewer than 2^32 walks (kErrWalkOverflow), so a group of gw sources
+// lists at most gw * 2^32 / kIndexedMost nodes, and their chunks are at most as many again.
+constexpr uint32_t kIndexedMost = 1024;
+constexpr int kListBits = 36;
+inline int64_t index_list_groups(int64_t n, int gw) {
+  const int64_t most = (int64_t)gw * ((1ll << 32) / kIndexedMost);
+  const int64_t nodes = n < most ? n : most, chunks = nodes + most;
+  const int64_t a = ((1ll << (64 - kListBits)) - 1) / nodes, b = ((1ll << kListBits) - 1) / chunks;
+  return a < b ? a : b;
+}
+
 // Device error bits (ORed into BatchDev::err).
 constexpr uint32_t kErrWalkCap = 1u;
 constexpr uint32_t kErrWalkOverflow = 2u;
@@ -192,6 +206,7 @@ struct BatchDev {
   uint32_t* wcount;
   unsigned long long ends;  // end_places of the graph
   int side_by_side;         // the sums of a group's sources lie side by side (indexed walks)
+  int first_grp, end_grp;   // groups of this launch of the indexed walks
   // Frontier of group g: entry e < slot_cnt[par][g] (par: the round's parity) is a node with
   // {first edge, degree} q[g * gw * n + e] and increments fa[g * gw * n + e * w + slot % gw]; its
   // hub items, i < slot_cnt[2 + par][g], are {entry, first edge} hub[g * gw * hub_stride + i]
@@ -269,6 +284,7 @@ struct Tuning {
   int spread_width = 1;
   int spread_hot = 1;      // 1: pushes to hot nodes go to copies of their residues
   int walk_blocks = 4;
+  int index_groups = 0;    // groups per list of the indexed walks, 0: index_list_groups
   int push_host_loop = 0;  // 1: rounds launched from a host loop instead of one launch
   int pipeline = 1;        // parts of a batch run on their own streams, pushes staggered
   uint32_t max_push_rounds = kMaxPushRounds;
@@ -311,7 +327,8 @@ cudaError_t launch_walks(const GraphDev& g, const BatchDev& b, int num_sms, cuda
 // walk.cu, FORA+ (Section 3.3): r[v] = RN(rmax * d(v)) for one slot (the residues whose
 // omega_v are the index's omega_max(v)), and the walk phase served from an index.
 cudaError_t launch_index_residue(const GraphDev& g, double* r, double rmax, cudaStream_t st);
-cudaError_t launch_walks_indexed(const GraphDev& g, const BatchDev& b, int num_sms,
+// Several lists of at most `groups` groups of sources each where one cannot hold them all.
+cudaError_t launch_walks_indexed(const GraphDev& g, const BatchDev& b, int num_sms, int groups,
                                  const unsigned long long* idx_off, const uint32_t* idx_dest,
                                  cudaStream_t st);
 // The walk ends of a batch as [nsrc][n] arrays over node ids (either output may be null).

@@ -668,13 +668,12 @@ __global__ void k_index_residue(GraphDev g, double* r, double rmax) {
 // (Source by source, from a list of entries, they took 11.2 ms: 1.4e11 a second, what scattered
 // 8-byte atomics with this graph's skew reach; the list took 0.9 ms more.)
 // k_indexed_nodes takes the nodes of up to kIndexedMost walks and lists the others, whose walks
-// k_indexed_hubs takes in chunks of kIndexedMost.
+// k_indexed_hubs takes in chunks of kIndexedMost; a list serves as many groups as it can count
+// (index_list_groups), so large batches take the two kernels more than once.
 // A residue of more walks than are stored (above the index's r_max) sets kErrIndexRange; only the
 // stored ones are taken.
-constexpr uint32_t kIndexedMost = 1024;
 constexpr int kIndexedPer = 4;    // steps of a warp (of 32 / G walks) whose loads are in flight
 constexpr int kIndexedLoads = 8;  // residues a lane reads before it uses any
-constexpr int kListBits = 36;     // of *walk_next: chunks listed, below them; nodes listed, above
 
 // This lane's source of group gr: its residue's walks and weight at node v, at most the stored
 // ones.  Every lane of the warp must call it.
@@ -709,9 +708,9 @@ __global__ void __launch_bounds__(kIndexedThreads) k_indexed_nodes(
   const unsigned long long n = (unsigned long long)g.n, units = (n + kNodes - 1) / kNodes;
   const unsigned long long warp =
       ((unsigned long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  if (warp >= units * (unsigned long long)b.ngrp) return;  // whole warps
-  const uint32_t gr = (uint32_t)(warp / units);
-  const uint32_t v0 = (uint32_t)((warp - gr * units) * kNodes);
+  if (warp >= units * (unsigned long long)(b.end_grp - b.first_grp)) return;  // whole warps
+  const uint32_t gr = (uint32_t)b.first_grp + (uint32_t)(warp / units);
+  const uint32_t v0 = (uint32_t)(warp % units * kNodes);
   const uint32_t w = min((uint32_t)G, (uint32_t)b.lay - gr * G);
   const bool mine = j < w && gr * G + j < (uint32_t)b.nsrc;
   const unsigned long long g0 = (unsigned long long)gr * G * n;
@@ -906,27 +905,38 @@ cudaError_t launch_index_residue(const GraphDev& g, double* r, double rmax, cuda
 }
 
 template <int G>
-cudaError_t walks_indexed_t(const GraphDev& g, const BatchDev& b, int num_sms,
+cudaError_t walks_indexed_t(const GraphDev& g, BatchDev b, int num_sms, int groups,
                             const unsigned long long* idx_off, const uint32_t* idx_dest,
                             cudaStream_t st) {
   constexpr unsigned long long kNodes = 32 / G * kIndexedLoads, kWarps = kIndexedThreads / 32;
-  const unsigned long long warps =
-      ((unsigned long long)g.n + kNodes - 1) / kNodes * (unsigned long long)b.ngrp;
-  k_indexed_nodes<G><<<(unsigned)((warps + kWarps - 1) / kWarps), kIndexedThreads, 0, st>>>(
-      g, b, idx_off, idx_dest);
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
   const int per_sm = resident_blocks((const void*)k_indexed_hubs<G>, kIndexedThreads);
   if (per_sm == 0) return cudaErrorInvalidConfiguration;
-  k_indexed_hubs<G><<<num_sms * per_sm, kIndexedThreads, 0, st>>>(g, b, idx_off, idx_dest);
-  return cudaGetLastError();
+  for (int first = 0; first < b.ngrp; first = b.end_grp) {
+    cudaError_t e = cudaSuccess;
+    if (first > 0) e = cudaMemsetAsync(b.walk_next, 0, sizeof(*b.walk_next), st);
+    if (e != cudaSuccess) return e;
+    b.first_grp = first;
+    b.end_grp = groups < b.ngrp - first ? first + groups : b.ngrp;
+    const unsigned long long warps = ((unsigned long long)g.n + kNodes - 1) / kNodes *
+                                     (unsigned long long)(b.end_grp - first);
+    k_indexed_nodes<G><<<(unsigned)((warps + kWarps - 1) / kWarps), kIndexedThreads, 0, st>>>(
+        g, b, idx_off, idx_dest);
+    e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    k_indexed_hubs<G><<<num_sms * per_sm, kIndexedThreads, 0, st>>>(g, b, idx_off, idx_dest);
+    e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
 }
 
-cudaError_t launch_walks_indexed(const GraphDev& g, const BatchDev& b, int num_sms,
+cudaError_t launch_walks_indexed(const GraphDev& g, const BatchDev& b, int num_sms, int groups,
                                  const unsigned long long* idx_off, const uint32_t* idx_dest,
                                  cudaStream_t st) {
-  return b.gw == 1 ? walks_indexed_t<1>(g, b, num_sms, idx_off, idx_dest, st)
-                   : walks_indexed_t<4>(g, b, num_sms, idx_off, idx_dest, st);
+  const int64_t most = index_list_groups(g.n, b.gw);
+  if (groups < 1 || groups > most) groups = (int)std::min<int64_t>(most, b.ngrp);
+  return b.gw == 1 ? walks_indexed_t<1>(g, b, num_sms, groups, idx_off, idx_dest, st)
+                   : walks_indexed_t<4>(g, b, num_sms, groups, idx_off, idx_dest, st);
 }
 
 cudaError_t launch_unpack_ends(const GraphDev& g, const BatchDev& b, uint32_t* cnt,

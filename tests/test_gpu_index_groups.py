@@ -44,3 +44,32 @@ def test_indexed_walks_of_groups_are_bit_exact(n, nsrc):
         np.testing.assert_array_equal(out["estimate"][i], oracle.estimate(res[i], acc))
         assert st[i].walks == wst.walks
     g.close()
+
+
+@pytest.mark.parametrize("groups", [1, 2])
+@pytest.mark.parametrize("nsrc", [2, 9, 16])
+def test_indexed_walks_in_several_lists_are_the_same(groups, nsrc):
+    """Lists of one or two groups (of four groups, the last not full, or of single sources)."""
+    n = 300
+    rng = np.random.default_rng(nsrc)
+    edges = [(v, int(u)) for v in range(n) for u in rng.integers(0, n, 1 + rng.poisson(3))]
+    edges += [(v, int(u)) for v in range(3) for u in rng.integers(0, n, 700 * (v + 1))]
+    rp, col = inputs.csr_from_edges(n, edges)
+    deg = np.diff(rp)
+    g = fora.Graph(rp, col)
+    g.build_index(fora.Params.make(k=1, delta=1e-3, pf=1e-3, rmax=RMAX, seed=SEED))
+    rmax, C, _ = g.index_info()
+    off, dest = oracle.walk_index(rp, col, 0.2, C, rmax, SEED)
+    walks = rng.choice([0.0, 1, 9, 1024, 1025, 2049, 1e9], (nsrc, n))
+    r = np.minimum(walks / C, rmax * deg)
+    r[0] = rmax * deg
+    res = rng.random((nsrc, n))
+    p = fora.Params.make(k=1, delta=1e-3, pf=1e-3, rmax=RMAX, seed=1, flags=fora.FORA_USE_INDEX)
+    sources = rng.integers(0, n, nsrc).astype(np.int32)
+    g.tune("index_groups", groups)
+    _, _, _, out = _debug(g, sources, p, given=(res, r))
+    for i in range(nsrc):
+        cnt, acc, _ = oracle.walk_phase_indexed(n, C, r[i], off, dest)
+        np.testing.assert_array_equal(out["count"][i], cnt)
+        np.testing.assert_array_equal(out["acc"][i], acc)
+    g.close()
