@@ -734,7 +734,7 @@ __global__ void __launch_bounds__(kIndexedThreads) k_indexed_nodes(
     for (int o = 1; o < G; o <<= 1) most = max(most, __shfl_xor_sync(kFull, most, o));
     if (most > kIndexedMost) {
       if (j == 0) {
-        const unsigned long long chunks = (most + kIndexedMost - 1) / kIndexedMost;
+        const unsigned long long chunks = (most - 1) / kIndexedMost + 1;
         const unsigned long long at = atomicAdd(b.walk_next, (1ull << kListBits) | chunks);
         const unsigned long long i = at >> kListBits;
         if (FORA_IN_RANGE(b.err, i, (unsigned long long)b.nsrc * n)) {
@@ -799,10 +799,11 @@ __global__ void __launch_bounds__(kIndexedThreads) k_indexed_hubs(
     uint32_t omega;
     unsigned long long weight;
     indexed_entry<G>(b, r, (uint32_t)(idx_off[v + 1] - off), &omega, &weight);
-    const unsigned long long beg = (x - b.wr_offset[i]) * kIndexedMost;
-    const uint32_t end = (uint32_t)min((unsigned long long)omega, beg + kIndexedMost);
+    const uint32_t beg = (uint32_t)(x - b.wr_offset[i]) * kIndexedMost;  // below 2^32
+    const uint32_t end = omega - min(omega, beg) < kIndexedMost ? omega : beg + kIndexedMost;
 #pragma unroll 1
-    for (uint32_t k = (uint32_t)beg; k < (uint32_t)beg + kIndexedMost; k += kPer * kIndexedPer) {
+    for (uint32_t s = 0; s < kIndexedMost; s += kPer * kIndexedPer) {
+      const uint32_t k = beg + s;  // the chunk's last walk is below 2^32, the next chunk need not be
       if (!__any_sync(kFull, k < end)) break;
       uint32_t dest[kIndexedPer];
 #pragma unroll

@@ -73,3 +73,26 @@ def test_indexed_walks_in_several_lists_are_the_same(groups, nsrc):
         np.testing.assert_array_equal(out["count"][i], cnt)
         np.testing.assert_array_equal(out["acc"][i], acc)
     g.close()
+
+
+def test_indexed_walks_of_a_node_with_almost_2_32_walks():
+    """One node with a self-loop holds all walks: the last chunk of them ends at 2^32."""
+    lo, hi = 1e-6, 1e-2
+    for _ in range(200):  # walks fall with eps
+        eps = 0.5 * (lo + hi)
+        lo, hi = (eps, hi) if oracle.walk_scale(eps, 1.0, 1e-3) > 2**32 - 512 else (lo, eps)
+    p = fora.Params.make(k=1, eps=hi, delta=1.0, pf=1e-3, rmax=1.0, seed=SEED)
+    g = fora.Graph(np.array([0, 1]), np.array([0]))
+    walks = int(np.ceil(g.resolve(p)[1]))
+    assert 2**32 - 1024 < walks < 2**32 and walks % 1024
+    if torch.cuda.mem_get_info()[0] < 6 * walks:
+        pytest.skip("the index takes 17 GB")
+    g.build_index(p)
+    p.flags = fora.FORA_USE_INDEX
+    _, _, st, out = _debug(g, [0], p)
+    assert st[0].walks == walks
+    # the residue 1 as `walks` walks of weight rint(2^63 / walks), all of them ending at the node
+    weight = int(np.rint(np.float64(1.0) / np.float64(walks) * np.float64(2.0**63)))
+    assert int(out["acc"][0, 0]) == walks * weight
+    assert int(out["count"][0, 0]) == walks
+    g.close()
