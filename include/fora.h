@@ -440,11 +440,16 @@ int fora_threshold_debug(const double *r, const double *rmax, const uint32_t *d,
  * or 5, default 4): resident walk blocks (of 384 threads) per SM, traded against registers
  * per thread.
  * "push_host_loop" (0 or 1, default 0): 1 launches the push rounds from a host loop with
- * one device-to-host read per round, instead of one cooperative launch that runs them all
- * on the device; the steps are the same (a profiler sees each of them on its own).  "pipeline" (1..4, default 1): a batched
+ * one device-to-host read per round, instead of a launch that runs many of them
+ * on the device; the steps are the same (a profiler sees each of them on its own).
+ * "push_slice" (0..1000000, default 1000): a push that is expected to take longer than twice
+ * this many microseconds is a sequence of launches that end after the round in which they have
+ * run so long (0: one round each), and after the spread of a longer round, so that work of other
+ * streams and calls starts in between; the host thread of a synchronous call enqueues them as the
+ * push goes on.  Results do not depend on it.  "pipeline" (1..4, default 1): a batched
  * query of B >= 64 sources runs as that many parts (at least 32 sources each), each on
- * its own workspace, stream and host thread, part k's push starting when part k-1's push
- * has finished, so one part's walk phase runs beside the next part's push; the call's
+ * its own workspace, stream and host thread, part k's push (in one launch) starting when part
+ * k-1's push has finished, and part k-1's walk phase as the device has room beside it; the call's
  * stream waits for all parts, and each part's stats carry that part's phase times.
  * Results do not depend on it.  "index_groups" (0..65535, default 0): the groups of sources
  * that one pass of the walk phase from an index takes, 0 (and any larger value) as many as its

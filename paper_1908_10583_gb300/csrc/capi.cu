@@ -220,14 +220,13 @@ int ensure_workspace(fora_graph* g, Workspace* w, int nsrc) {
   CUDA_TRY(dalloc(&w->fa, z.fa));
   CUDA_TRY(dalloc(&w->hub[0], z.hub));
   CUDA_TRY(dalloc(&w->hub[1], z.hub));
-  CUDA_TRY(dalloc(&w->small, z.small));
-  CUDA_TRY(dalloc(&w->work, z.work));
+  CUDA_TRY(dalloc(&w->small, z.small + z.work));  // cleared together
+  w->work = w->small + z.small / sizeof(*w->small);
   CUDA_TRY(dalloc(&w->alist, z.alist));
   CUDA_TRY(dalloc(&w->slot_cnt, z.slot_cnt));
   CUDA_TRY(dalloc(&w->pre, z.pre));
   CUDA_TRY(dalloc(&w->ps, z.ps));
   CUDA_TRY(cudaMemset(w->ps, 0, z.ps));
-  CUDA_TRY(cudaMemset(w->work, 0, z.work));  // the push's barrier starts at 0
   CUDA_TRY(dalloc(&w->err, z.err));
   CUDA_TRY(dalloc(&w->sources, z.sources));
   CUDA_TRY(dalloc(&w->rmax, z.rmax));
@@ -248,9 +247,13 @@ int ensure_workspace(fora_graph* g, Workspace* w, int nsrc) {
   CUDA_TRY(cudaMallocHost(&w->h_err, sizeof(uint32_t)));
   CUDA_TRY(cudaMallocHost(&w->h_sources, nsrc * sizeof(int32_t)));
   CUDA_TRY(cudaMallocHost(&w->h_rmax, nsrc * sizeof(double)));
-  CUDA_TRY(cudaMallocHost(&w->go_host, 3 * sizeof(uint32_t)));
+  CUDA_TRY(cudaMallocHost(&w->go_host, sizeof(uint32_t)));
+  CUDA_TRY(cudaMallocHost(&w->push_err, sizeof(uint32_t)));
+  CUDA_TRY(cudaMallocHost(&w->push_host, sizeof(PushHost)));
   for (int i = 0; i < 5; ++i)
     if (!w->ev[i]) CUDA_TRY(cudaEventCreate(&w->ev[i]));
+  for (int i = 0; i < 2; ++i)
+    if (!w->part_ev[i]) CUDA_TRY(cudaEventCreateWithFlags(&w->part_ev[i], cudaEventDisableTiming));
   w->cap = nsrc;
   return FORA_OK;
 }
@@ -305,32 +308,47 @@ int resolve(const fora_graph* g, const fora_params* p, Resolved* out) {
 
 namespace {
 
-// Pushes of one device never run side by side: a push fills the device with blocks that wait
-// for each other, so each waits for the one launched before it (on whatever stream).
-struct PushGate {
-  std::mutex mu;
-  cudaEvent_t last = nullptr;
-};
-std::mutex g_gates_mu;
-std::map<int, std::unique_ptr<PushGate>> g_gates;
+// About how long a push takes, in microseconds, from what it costs at the device's rates: an edge
+// push costs 1 / (2e11 s), and the scans of its heavy rounds read each residue some 40 times.
+// Section 3.2 counts 1 / r_max edge pushes per source.
+double push_estimate(const double* rmax, int nsrc, int64_t n) {
+  double edges = 0.0;
+  for (int i = 0; i < nsrc; ++i) edges += 1.0 / rmax[i];
+  return edges / 2e5 + (double)nsrc * (double)n * 40.0 * 8.0 / 6e6;
+}
+// Launches that an asynchronous call enqueues for a long push, at most.
+constexpr int kAsyncParts = 64;
 
-cudaError_t launch_push_gated(int device, const GraphDev& gd, const BatchDev& b, int num_sms,
-                              bool resume, const uint32_t* pause, cudaStream_t stream) {
-  PushGate* gate;
-  {
-    std::lock_guard<std::mutex> lock(g_gates_mu);
-    auto& p = g_gates[device];
-    if (!p) p = std::make_unique<PushGate>();
-    gate = p.get();
-  }
-  std::lock_guard<std::mutex> lock(gate->mu);
+// A push that is expected to take longer than two slices, as a sequence of launches of about a
+// slice each, so that work of other streams starts between them.  The host keeps one launch
+// ahead of the one that is running (the last does nothing), so the device does not wait for it.
+// An asynchronous call enqueues as many as the estimate tells, and one without a limit.
+cudaError_t push_in_parts(const GraphDev& gd, const BatchDev& b, const fora_graph* g, Workspace* w,
+                          uint32_t slice, double estimate, bool async, cudaStream_t stream) {
+  PushPart part{0, 0, slice, 0, async ? nullptr : w->push_host};
   cudaError_t e = cudaSuccess;
-  if (!gate->last)
-    e = cudaEventCreateWithFlags(&gate->last, cudaEventDisableTiming);
-  else
-    e = cudaStreamWaitEvent(stream, gate->last, 0);
-  if (e == cudaSuccess) e = launch_push(gd, b, num_sms, resume, pause, stream);
-  if (e == cudaSuccess) e = cudaEventRecord(gate->last, stream);
+  auto next = [&] {
+    if (part.host) part.host->go[part.turn] = 1;
+    e = launch_push(gd, b, g->num_sms, &part, stream);
+    if (e == cudaSuccess && part.host) e = cudaEventRecord(w->part_ev[part.turn], stream);
+    part.resume = 1;
+    part.turn ^= 1;
+  };
+  if (async) {
+    const double parts = slice ? estimate / slice : kAsyncParts;
+    for (int i = 0; i < kAsyncParts && i < parts && e == cudaSuccess; ++i) next();
+    part.slice = kNoSlice;
+    if (e == cudaSuccess) next();
+    return e;
+  }
+  w->push_host->stop = 0;
+  next();
+  while (e == cudaSuccess) {
+    next();
+    // part.turn is now the turn of the launch before that one
+    if (e == cudaSuccess) e = cudaEventSynchronize(w->part_ev[part.turn]);
+    if (e == cudaSuccess && !*(volatile uint32_t*)&w->push_host->go[part.turn]) break;
+  }
   return e;
 }
 
@@ -360,7 +378,7 @@ void lay_out(const fora_graph* g, const Workspace* w, int lay, int gw, BatchDev*
   b->work = w->work;
   b->ps = w->ps;
   b->ctl = reinterpret_cast<PushCtl*>(w->small);
-  b->meet = reinterpret_cast<uint32_t*>(w->work + 8);  // and work + 24
+  b->meet = reinterpret_cast<uint32_t*>(w->work + 4);  // up to work + 28, around work[16]
   // the second queue buffer: the list of tiles, then the copies of the hot nodes' residues
   b->tlist = reinterpret_cast<uint32_t*>(w->q[1]);
   const size_t list = ((size_t)b->lgrp * b->tiles * sizeof(uint32_t) + 15) / 16 * 2;  // doubles
@@ -492,7 +510,8 @@ int fora::run_batch_ws(fora_graph* g, Workspace* w, const fora_params* p,
                            stream));
   if (b.want_count)
     CUDA_TRY(cudaMemsetAsync(b.wcount, 0, (size_t)nsrc * b.ends * sizeof(uint32_t), stream));
-  CUDA_TRY(cudaMemsetAsync(w->small, 0, 8 * sizeof(unsigned long long), stream));
+  // with `work`, behind it
+  CUDA_TRY(cudaMemsetAsync(w->small, 0, (8 + 32) * sizeof(unsigned long long), stream));
   CUDA_TRY(cudaMemsetAsync(w->err, 0, sizeof(uint32_t), stream));
   CUDA_TRY(cudaMemsetAsync(w->stats, 0, nsrc * sizeof(SlotStats), stream));
   if (bal) {
@@ -504,6 +523,7 @@ int fora::run_batch_ws(fora_graph* g, Workspace* w, const fora_params* p,
   }
   bool host_loop;
   int index_groups;
+  uint32_t slice;
   {
     std::lock_guard<std::mutex> tlock(g->mu);
     index_groups = g->tune.index_groups;
@@ -512,6 +532,7 @@ int fora::run_batch_ws(fora_graph* g, Workspace* w, const fora_params* p,
     b.walk_blocks = g->tune.walk_blocks;
     b.max_rounds = g->tune.max_push_rounds;
     host_loop = g->tune.push_host_loop != 0;
+    slice = (uint32_t)g->tune.push_slice;
   }
 
   if (hook && hook->before && hook->before->wait())  // the earlier part's push is done
@@ -528,25 +549,27 @@ int fora::run_batch_ws(fora_graph* g, Workspace* w, const fora_params* p,
     CUDA_TRY(launch_regroup(w->r, dbg->residue, b, g->n, false, g->num_sms, stream));
   } else {
     if (join) {
-      // While the push runs the host looks for requests; when some arrive it pauses the push
+      // While the push runs the host looks for requests; when some arrive it ends the launch
       // after the round that is running, and they join as new slots.  (With a host round trip
       // after every round, whether anyone had come or not, 24 requests to a 2^16-node graph took
       // 4.13 ms, with this 3.39, 0.5 of them the batching window.)
-      for (bool resume = false;; resume = true) {
-        __atomic_store_n(w->go_host + 1, 0u, __ATOMIC_RELEASE);
-        CUDA_TRY(launch_push_gated(g->device, gd, b, g->num_sms, resume, w->go_host + 1, stream));
-        CUDA_TRY(cudaMemcpyAsync(w->go_host + 2, w->err, sizeof(uint32_t), cudaMemcpyDeviceToHost,
-                                 stream));
+      for (PushPart part{0, 0, slice, 1, w->push_host};; part.resume = 1, part.turn ^= 1) {
+        __atomic_store_n(&w->push_host->stop, 0u, __ATOMIC_RELEASE);
+        w->push_host->go[part.turn] = 1;
+        CUDA_TRY(launch_push(gd, b, g->num_sms, &part, stream));
+        CUDA_TRY(cudaMemcpyAsync(w->push_err, w->err, sizeof(uint32_t), cudaMemcpyDeviceToHost, stream));
         const int room = join->cap - b.nsrc;
         int k = 0;
         cudaError_t state;
         do {
           state = cudaStreamQuery(stream);
           if (k < room) k += join->poll(w->h_sources + b.nsrc + k, room - k);
-          if (k > 0) __atomic_store_n(w->go_host + 1, 1u, __ATOMIC_RELEASE);
+          if (k > 0) __atomic_store_n(&w->push_host->stop, 1u, __ATOMIC_RELEASE);
         } while (state == cudaErrorNotReady);
         CUDA_TRY(state);
-        if (k == 0 || (w->go_host[2] & kErrBarrier)) break;  // not paused: it is through
+        if (*w->push_err & kErrBarrier) break;
+        if (k == 0 && w->push_host->go[part.turn]) continue;  // the slice is over
+        if (k == 0) break;
         const int first = b.nsrc, grp0 = b.ngrp;
         for (int i = first; i < first + k; ++i) w->h_rmax[i] = rp.rmax;
         CUDA_TRY(cudaMemcpyAsync(w->sources + first, w->h_sources + first, k * sizeof(int32_t),
@@ -583,7 +606,16 @@ int fora::run_batch_ws(fora_graph* g, Workspace* w, const fora_params* p,
       }
       CUDA_TRY(launch_push_finish(gd, b, g->num_sms, stream));
     } else {
-      CUDA_TRY(launch_push_gated(g->device, gd, b, g->num_sms, false, nullptr, stream));
+      // where the thresholds are found on the device, some third of the rule's r_max
+      std::vector<double> guess;
+      if (bal || rsrc.device) guess.assign(nsrc, rp.rmax / 3);
+      const double us = push_estimate(guess.empty() ? w->h_rmax : guess.data(), nsrc, g->n);
+      // (a part of a pipelined batch is not cut: its own walks of the part before would start in
+      // between, and beside each other both are slower, 248 ms for 256 sources of 2^20, not 234)
+      if (us > 2.0 * slice && !hook)
+        CUDA_TRY(push_in_parts(gd, b, g, w, slice, us, async, stream));
+      else
+        CUDA_TRY(launch_push(gd, b, g->num_sms, nullptr, stream));
     }
     if (dbg && dbg->reserve)
       CUDA_TRY(launch_regroup(w->res, dbg->reserve, b, g->n, true, g->num_sms, stream));
@@ -667,9 +699,11 @@ int fora::run_batch_ws(fora_graph* g, Workspace* w, const fora_params* p,
 namespace {
 
 // A batch in `parts` parts, each on its own workspace and stream, driven by its own host
-// thread; part k's push waits for part k-1's push to finish, so part k-1's walks (bound
-// by instruction issue) run beside part k's push (bound by L2 reductions).  The caller's
-// stream waits for every part, so work queued on it afterwards sees the results.
+// thread; part k's push waits for part k-1's push to finish, and part k-1's walks start as the
+// blocks of part k's push leave their SMs.  (Both are bound by L2 now, so little is gained: 256
+// sources of 2^20, rule's r_max, 231.6 ms in one part, 233.6 in two, 261 in four; 64 of 2^25 8.71 s
+// in one or two.)  The caller's stream waits for every part, so work queued on it afterwards sees
+// the results.
 constexpr int kMinPartSources = 32;
 
 int run_batch_pipelined(fora_graph* g, const fora_params* p, const int32_t* sources, int nsrc,
@@ -1309,6 +1343,11 @@ int fora_graph_tune(fora_graph* g, const char* key, int64_t value) {
     g->tune.push_host_loop = (int)value;
     return FORA_OK;
   }
+  if (strcmp(key, "push_slice") == 0) {
+    if (value < 0 || value > 1000000) return fail(FORA_ERR_BAD_ARG, "push_slice must be in [0, 1000000]");
+    g->tune.push_slice = (int)value;
+    return FORA_OK;
+  }
   if (strcmp(key, "index_groups") == 0) {
     if (value < 0 || value > 65535) return fail(FORA_ERR_BAD_ARG, "index_groups must be in [0, 65535]");
     g->tune.index_groups = (int)value;
@@ -1722,6 +1761,7 @@ int fora_graph_tuning(fora_graph* g, const char* key, int64_t* value) {
   if (strcmp(key, "walk_blocks") == 0) { *value = g->tune.walk_blocks; return FORA_OK; }
   if (strcmp(key, "pipeline") == 0) { *value = g->tune.pipeline; return FORA_OK; }
   if (strcmp(key, "push_host_loop") == 0) { *value = g->tune.push_host_loop; return FORA_OK; }
+  if (strcmp(key, "push_slice") == 0) { *value = g->tune.push_slice; return FORA_OK; }
   if (strcmp(key, "index_groups") == 0) { *value = g->tune.index_groups; return FORA_OK; }
   if (strcmp(key, "max_push_rounds") == 0) { *value = g->tune.max_push_rounds; return FORA_OK; }
   return fail(FORA_ERR_BAD_ARG, "unknown tuning key '%s'", key);

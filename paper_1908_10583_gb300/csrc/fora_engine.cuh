@@ -22,6 +22,12 @@ constexpr int kHotCopies = 8;
 constexpr uint32_t kGroupLight = 1u;   // its next take scans the listed tiles only
 constexpr uint32_t kGroupActive = 2u;  // it takes part in the next take
 constexpr uint32_t kMaxPolls = 1u << 25;  // polls of a block at the push's barrier (about 30 s)
+// Words (of 4 bytes) of a launch's part of BatchDev::meet.
+constexpr int kMeetArrived = 0;  // arrivals of its blocks
+constexpr int kMeetEntered = 1;  // blocks that have entered
+constexpr int kMeetReady = 2;    // blocks that have cleared their part of the state
+constexpr int kMeetWord = 8;     // 8 bytes, in another sector: the last meeting (k_push)
+constexpr int kMeetWords = 32;   // from one launch's part to the other's
 
 // Units of the residual list: all of a call (scanned by one block), and of one slot.
 constexpr int kMaxUnits = 32768;
@@ -78,16 +84,31 @@ constexpr uint32_t kMaxPushRounds = 100000u;  // default cap of the push rounds
 struct PushState {
   int cur;
   uint32_t round;
-  uint32_t go;      // the loop condition of the last round (read by the host-driven loop)
-  uint32_t nact;    // groups that take part in the next take
+  uint32_t go;      // the loop condition of the last round
+  float us;         // about how long the rest of the round takes with every block, microseconds
   unsigned long long ngroups;  // items of `span` entries of the current frontier, over all groups
   unsigned long long nhub;     // hub items of the current frontier, over all groups
 };
+// A launch that runs part of a push: it ends after the round in which `slice` microseconds have
+// passed or, when it may be stopped, a non-zero `stop` was seen, and after the spread of a round
+// that takes longer.
+struct PushHost {  // pinned host memory
+  uint32_t stop;   // written by the host
+  uint32_t go[2];  // 1: rounds are left after the launch with this turn
+};
+struct PushPart {
+  int resume;      // 0: from the start of the push, 1: where the launch before it ended
+  int turn;        // alternates between 0 and 1, from 0
+  uint32_t slice;  // kNoSlice: no limit
+  int stops;       // read host->stop every round
+  PushHost* host;  // may be null
+};
+constexpr uint32_t kNoSlice = 0xFFFFFFFFu;
 struct PushCtl {
   uint32_t nheavy;  // groups that the next take scans whole (listed in BatchDev::alist)
   uint32_t nlist;   // units listed of the others (BatchDev::tlist)
   uint32_t span;    // entries of an item of the spread
-  uint32_t pad;
+  uint32_t cut;     // the launch ends after the spread, and the next begins with the take
 };
 
 struct GraphDev {
@@ -227,7 +248,7 @@ struct BatchDev {
   unsigned long long* work;  // dynamic work counters of the spread ([0] and [16])
   PushState* ps;
   PushCtl* ctl;
-  uint32_t* meet;            // barrier of the push: [0] arrivals, [32] the last meeting's word
+  uint32_t* meet;            // [2][kMeetWords] meeting points of the push, by turn; zero before it
   const int32_t* sources;    // [nsrc]
   const double* rmax;        // [nsrc]
   SlotStats* stats;          // [nsrc]
@@ -286,6 +307,7 @@ struct Tuning {
   int walk_blocks = 4;
   int index_groups = 0;    // groups per list of the indexed walks, 0: index_list_groups
   int push_host_loop = 0;  // 1: rounds launched from a host loop instead of one launch
+  int push_slice = 1000;   // microseconds after which a long push starts another launch
   int pipeline = 1;        // parts of a batch run on their own streams, pushes staggered
   uint32_t max_push_rounds = kMaxPushRounds;
 };
@@ -300,9 +322,9 @@ int resident_blocks(const void* kernel, int threads);
 // returns cudaErrorMemoryAllocation without allocating when the hook says so.
 cudaError_t device_alloc(void** p, size_t bytes);
 
-// push.cu: the whole push in one cooperative launch (from zeroing r and res on).
-cudaError_t launch_push(const GraphDev& g, const BatchDev& b, int num_sms, bool resume,
-                        const uint32_t* pause, cudaStream_t st);
+// push.cu: the whole push in one launch (from zeroing r and res on), or a part of it.
+cudaError_t launch_push(const GraphDev& g, const BatchDev& b, int num_sms, const PushPart* part,
+                        cudaStream_t st);
 // The same in steps for a host loop that reads PushState::go after each round: start, rounds,
 // finish.
 cudaError_t launch_push_start(const GraphDev& g, const BatchDev& b, int num_sms, cudaStream_t st);

@@ -74,9 +74,10 @@ struct Workspace {
   uint32_t* h_err = nullptr;
   int32_t* h_sources = nullptr;
   double* h_rmax = nullptr;
-  // pinned: [0] PushState::go of the host-driven push loop; [1] pauses a push that sources can
-  // join, [2] is its err
-  uint32_t* go_host = nullptr;
+  uint32_t* go_host = nullptr;      // pinned: PushState::go of the host-driven push loop
+  uint32_t* push_err = nullptr;     // pinned: err after a launch of a push that sources can join
+  PushHost* push_host = nullptr;    // pinned
+  cudaEvent_t part_ev[2] = {};      // ends of a long push's launches, by turn
   cudaEvent_t ev[5] = {nullptr, nullptr, nullptr, nullptr, nullptr};
 
   PushState* ps = nullptr;
@@ -86,7 +87,7 @@ struct Workspace {
     dfree(ps);
     dfree(r); dfree(res); dfree(tally);
     dfree(q[0]); dfree(q[1]); dfree(hub[0]); dfree(hub[1]); dfree(fa);
-    dfree(small); dfree(work); dfree(alist); dfree(slot_cnt); dfree(pre); dfree(err); dfree(sources); dfree(rmax); dfree(stats); dfree(stopped); dfree(light); dfree(tile_dirty); dfree(last_edges); dfree(blk);
+    dfree(small); work = nullptr; dfree(alist); dfree(slot_cnt); dfree(pre); dfree(err); dfree(sources); dfree(rmax); dfree(stats); dfree(stopped); dfree(light); dfree(tile_dirty); dfree(last_edges); dfree(blk);
     if (topk_scratch) cudaFree(topk_scratch);
     topk_scratch = nullptr;
     dfree(out_ids); dfree(out_vals); dfree(feat); dfree(pred); dfree(rmax_learned);
@@ -96,14 +97,18 @@ struct Workspace {
     if (h_sources) cudaFreeHost(h_sources);
     if (h_rmax) cudaFreeHost(h_rmax);
     if (go_host) cudaFreeHost(go_host);
+    if (push_err) cudaFreeHost(push_err);
+    if (push_host) cudaFreeHost(push_host);
     h_counters = nullptr; h_stats = nullptr; h_err = nullptr; h_sources = nullptr; h_rmax = nullptr;
-    go_host = nullptr;
+    go_host = nullptr; push_err = nullptr; push_host = nullptr;
     cap = 0;
   }
   ~Workspace() {
     release();
     for (int i = 0; i < 5; ++i)
       if (ev[i]) cudaEventDestroy(ev[i]);
+    for (int i = 0; i < 2; ++i)
+      if (part_ev[i]) cudaEventDestroy(part_ev[i]);
   }
 };
 
@@ -112,8 +117,7 @@ struct Workspace {
 namespace fora {
 
 // Ordering between consecutive parts of a pipelined batch: the later part's push waits
-// on the device until the earlier part's push is done (so the earlier part's walks run
-// beside the later part's push).  The earlier part's host thread records `ev` after
+// on the device until the earlier part's push is done.  The earlier part's host thread records `ev` after
 // enqueueing its push and signals; it signals without recording if it stops early.
 struct PipeLink {
   std::mutex m;

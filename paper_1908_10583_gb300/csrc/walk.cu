@@ -229,7 +229,6 @@ __global__ void __launch_bounds__(1024) k_residual_scan(BatchDev b) {
     b.totals[0] = ct;
     b.totals[1] = wt;
     b.wr_offset[ct] = wt;
-    b.meet[0] = b.meet[32] = 0;  // the next call's push starts its barrier from 0
   }
   for (int s = threadIdx.x; s < b.nsrc; s += blockDim.x)
     if (b.stats[s].walks > 0xFFFFFFFFull) atomicOr(b.err, kErrWalkOverflow);
