@@ -125,7 +125,9 @@ __device__ void topk_hist(const TopkRun& t, int row, int part, int parts, const 
   const double* e = t.est + (size_t)row * (size_t)t.n;
   const uint32_t width = s ? min((uint32_t)kDigitBits, 96u - s->plen) : 0u;
   const u128 p = s && s->plen ? (((u128)s->pa << 32) | s->pb) >> (96 - s->plen) : 0;
-  for (int64_t base = beg + threadIdx.x; base < end; base += (int64_t)blockDim.x * kTopkLoads) {
+  // block-uniform trip count
+  for (int64_t top = beg; top < end; top += (int64_t)blockDim.x * kTopkLoads) {
+    const int64_t base = top + threadIdx.x;
     double v[kTopkLoads];
 #pragma unroll
     for (int q = 0; q < kTopkLoads; ++q) {
@@ -138,12 +140,14 @@ __device__ void topk_hist(const TopkRun& t, int row, int part, int parts, const 
       if (!s) {
         const uint32_t bin = first_bin(v[q]);
         if (bin) atomicAdd(&sh[bin], 1u);
-      } else if (i < end) {
+      } else {
         const u128 z = key_of(v[q], (uint32_t)i);
-        if (s->plen == 0 || (z >> (96 - s->plen)) == p) {
+        const bool in = i < end && (s->plen == 0 || (z >> (96 - s->plen)) == p);
+        const unsigned members = __ballot_sync(0xFFFFFFFFu, in);
+        if (in) {
           // equal values share every digit but the ids': lanes of one bin add their count once
           const uint32_t bin = (uint32_t)(z >> (96 - s->plen - width)) & ((1u << width) - 1u);
-          const unsigned grp = __match_any_sync(__activemask(), bin);
+          const unsigned grp = __match_any_sync(members, bin);
           if ((threadIdx.x & 31) == (uint32_t)(__ffs(grp) - 1))
             atomicAdd(&sh[bin], (uint32_t)__popc(grp));
         }
