@@ -10,15 +10,18 @@
 //                   row's last block picks the bin that holds the k-th largest key as the row's
 //                   prefix; the row is done once the keys above the bin and its own fit the sort.
 //   k_topk_levels   for rows that are not (more equal or near-equal values than the sort takes,
-//                   or a k-th value outside the bins): a cluster per row takes the next 12 bits
-//                   of the keys with the row's prefix, and so on.
+//                   or a k-th value outside the bins): the next 12 bits of the keys with the
+//                   row's prefix, and so on.  The blocks of a row take its parts as they come,
+//                   and whichever finishes a level's last part picks its digit.
 //   k_topk_collect  every key from the prefix on goes to the candidate list; a row's last block
 //                   sorts it (bitonic, in shared memory) and writes the first k.
 // Two passes over the rows; HBM bounds large ones, the launches and the sort small ones.
 // 24 rows of 10^6 estimates: 40 us, 4 us where no level is left, 50 us (the two passes at the
 // measured copy rate: 58); fora_topk 522 -> 128 us.  (As 19 launches:
 // eight levels of 12 bits from the top, whether a row had use for them or not, then collect and
-// sort.)
+// sort.)  fora_topk of rows whose k-th value is 0 (eight levels): one row of 2^25 values 0.92 ms,
+// 24 of 2^20 0.88, 256 of 2^14 0.48.  With eight blocks of a cluster for each row's levels, however
+// long the row, they took 10.9, 1.06 and 1.03, as 19 launches 1.26, 1.28 and 0.74.
 #include <algorithm>
 
 #include "fora_engine.cuh"
@@ -73,7 +76,6 @@ __global__ void __launch_bounds__(kEstThreads) k_estimate(GraphDev g, BatchDev b
 
 constexpr int kTopkThreads = 1024;
 constexpr int kTopkLoads = 4;   // elements a thread reads before it uses any
-constexpr int kTopkCluster = 8;  // blocks of a row in k_topk_levels
 
 struct TopkRun {
   const double* est;
@@ -112,14 +114,12 @@ __device__ __forceinline__ void row_range(int64_t n, int part, int parts, int64_
   *end = n * (int64_t)(part + 1) / parts;
 }
 
-// Histogram of one part of a row into sh, then into the row's (h): of the first digit
-// (s == nullptr), else of the next digit of the keys with s's prefix.  Bin 0 of the first digit
+// Counts one part of a row in sh: the first digit (s == nullptr), else the next digit of the keys
+// with s's prefix.  Bin 0 of the first digit
 // (zeros and values below 2^-63, most of many rows) is not counted: what is asked of it is the
 // keys above the bins.
 __device__ void topk_hist(const TopkRun& t, int row, int part, int parts, const TopkSlot* s,
-                          uint32_t* h, uint32_t* sh) {
-  for (int i = threadIdx.x; i < kBins; i += blockDim.x) sh[i] = 0;
-  __syncthreads();
+                          uint32_t* sh) {
   int64_t beg, end;
   row_range(t.n, part, parts, &beg, &end);
   const double* e = t.est + (size_t)row * (size_t)t.n;
@@ -154,6 +154,14 @@ __device__ void topk_hist(const TopkRun& t, int row, int part, int parts, const 
       }
     }
   }
+}
+
+// Clears sh; adds it to the row's histogram h.  By the whole block.
+__device__ __forceinline__ void topk_clear(uint32_t* sh) {
+  for (int i = threadIdx.x; i < kBins; i += blockDim.x) sh[i] = 0;
+  __syncthreads();
+}
+__device__ __forceinline__ void topk_flush(const uint32_t* sh, uint32_t* h) {
   __syncthreads();
   for (int i = threadIdx.x; i < kBins; i += blockDim.x)
     if (sh[i]) atomicAdd(&h[i], sh[i]);
@@ -226,6 +234,17 @@ __device__ void topk_select(const TopkRun& t, int row, bool first) {
   if (th == 0 && s_found == 0) t.s.slots[row] = s;  // the k-th key lies outside the first bins
 }
 
+// A row's levels: how many have been picked, and of each the parts that blocks have taken and
+// finished.  It lies at the start of the row's candidates, which k_topk_collect writes later.
+constexpr int kMaxLevels = 8;  // of 12 bits (the last, fewer)
+struct LevelWork {
+  uint32_t level;
+  uint32_t taken[kMaxLevels], done[kMaxLevels];
+};
+__device__ __forceinline__ LevelWork* level_work(const TopkRun& t, int row) {
+  return (LevelWork*)(t.s.cand_key + (size_t)row * kSortCap);
+}
+
 // Whether this block is the last of its row's to get here; what the others wrote is then visible.
 __device__ bool last_of_row(TopkSlot* slot) {
   __shared__ uint32_t s_last;
@@ -241,26 +260,75 @@ __device__ bool last_of_row(TopkSlot* slot) {
 __global__ void __launch_bounds__(kTopkThreads, 2) k_topk_first(TopkRun t) {
   __shared__ uint32_t sh[kBins];
   const int row = blockIdx.y;
-  topk_hist(t, row, blockIdx.x, gridDim.x, nullptr, t.s.hist + (size_t)row * kBins, sh);
-  if (last_of_row(&t.s.slots[row])) topk_select(t, row, true);
+  topk_clear(sh);
+  topk_hist(t, row, blockIdx.x, gridDim.x, nullptr, sh);
+  topk_flush(sh, t.s.hist + (size_t)row * kBins);
+  if (!last_of_row(&t.s.slots[row])) return;
+  topk_select(t, row, true);
+  LevelWork* lw = level_work(t, row);
+  for (int i = threadIdx.x; i < (int)(sizeof(LevelWork) / sizeof(uint32_t)); i += blockDim.x)
+    ((uint32_t*)lw)[i] = 0;
 }
 
-__device__ __forceinline__ void cluster_meet() {
-  __threadfence();
-  asm volatile("barrier.cluster.arrive.aligned;" ::: "memory");
-  asm volatile("barrier.cluster.wait.aligned;" ::: "memory");
-}
-
-__global__ void __cluster_dims__(kTopkCluster, 1, 1) __launch_bounds__(kTopkThreads, 1)
-    k_topk_levels(TopkRun t) {
+// Grid (parts of a row, rows).  A block takes parts of the row's level until none is left, adds its
+// counts, and waits for the blocks that hold the others; the one that finishes the last picks the
+// digit, clears the histogram and lets the row go on.  Only parts that a running block has taken
+// are waited for, so blocks that have not started hold nobody up, and a block that has waited too
+// long can leave: the block that finishes a level takes the next one's parts itself.
+constexpr uint32_t kLevelPolls = 1u << 20;
+__global__ void __launch_bounds__(kTopkThreads, 2) k_topk_levels(TopkRun t) {
   __shared__ uint32_t sh[kBins];
+  __shared__ uint32_t s_x;
   const int row = blockIdx.y;
-  // at most 8 levels: each fixes 12 more of the 96 bits (the last, fewer)
-  for (TopkSlot s = load_slot(&t.s.slots[row]); !s.done; s = load_slot(&t.s.slots[row])) {
-    topk_hist(t, row, blockIdx.x, kTopkCluster, &s, t.s.hist + (size_t)row * kBins, sh);
-    cluster_meet();
-    if (blockIdx.x == 0) topk_select(t, row, false);
-    cluster_meet();
+  if (__ldcg(&t.s.slots[row].done)) return;
+  LevelWork* lw = level_work(t, row);
+  if (threadIdx.x == 0) s_x = *(volatile uint32_t*)&lw->level;
+  __syncthreads();
+  for (uint32_t level = s_x; level < (uint32_t)kMaxLevels;) {
+    __threadfence();
+    // of this level for certain only once a part of it is taken (a level ends with its last part)
+    const TopkSlot s = load_slot(&t.s.slots[row]);
+    if (__syncthreads_or(s.done != 0)) return;
+    topk_clear(sh);
+    uint32_t mine = 0;
+    for (;;) {
+      if (threadIdx.x == 0) s_x = atomicAdd(&lw->taken[level], 1u);
+      __syncthreads();
+      const uint32_t part = s_x;
+      __syncthreads();
+      if (part >= gridDim.x) break;
+      topk_hist(t, row, (int)part, (int)gridDim.x, &s, sh);
+      ++mine;
+    }
+    bool last = false;
+    if (mine) {  // block-uniform
+      topk_flush(sh, t.s.hist + (size_t)row * kBins);
+      __threadfence();
+      __syncthreads();
+      if (threadIdx.x == 0) s_x = atomicAdd(&lw->done[level], mine) + mine;
+      __syncthreads();
+      last = s_x == gridDim.x;
+      __syncthreads();
+    }
+    if (last) {
+      __threadfence();
+      topk_select(t, row, false);
+      __threadfence();
+      __syncthreads();
+      if (threadIdx.x == 0) *(volatile uint32_t*)&lw->level = level + 1;
+      ++level;
+    } else {
+      if (threadIdx.x == 0) {
+        uint32_t now, polls = 0;
+        while ((now = *(volatile uint32_t*)&lw->level) <= level && ++polls <= kLevelPolls)
+          if (polls > 64) __nanosleep(50);
+        s_x = now;
+      }
+      __syncthreads();
+      if (s_x <= level) return;
+      level = s_x;
+      __syncthreads();
+    }
   }
 }
 
@@ -391,7 +459,9 @@ cudaError_t launch_topk(const double* est, int64_t n, int nrows, uint32_t k, int
   k_topk_first<<<grid, kTopkThreads, 0, st>>>(t);
   e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  k_topk_levels<<<dim3(kTopkCluster, (unsigned)nrows), kTopkThreads, 0, st>>>(t);
+  // a level's hand-over costs more than a short part's pass, so its parts are of 8192 or more
+  const dim3 level_grid((unsigned)std::min<int64_t>(bpr, (n + 8191) / 8192), (unsigned)nrows);
+  k_topk_levels<<<level_grid, kTopkThreads, 0, st>>>(t);
   e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   k_topk_collect<<<grid, kTopkThreads, smem, st>>>(t);

@@ -57,3 +57,40 @@ def test_more_rows_than_one_wave():
     got_ids, got_vals = fora.topk(torch.tensor(est).cuda(), 100)
     np.testing.assert_array_equal(np.asarray(got_ids.cpu()), ids)
     np.testing.assert_array_equal(np.asarray(got_vals.cpu()), vals)
+
+
+# few long rows (a part of each for every block of the device), and rows of one part
+@pytest.mark.parametrize("nrows,n,k", [(1, 3000001, 500), (2, 1 << 21, 4096), (3, 4096, 4096),
+                                       (33, 8191, 100)])
+def test_levels_over_the_whole_grid(nrows, n, k):
+    rng = np.random.default_rng(nrows)
+    for make in range(7):
+        est = np.stack([rows(n, rng)[(make + i) % 7] for i in range(nrows)])
+        ids, vals = expect(est, k)
+        for _ in range(2):
+            got_ids, got_vals = fora.topk(torch.tensor(est).cuda(), k)
+            np.testing.assert_array_equal(np.asarray(got_ids.cpu()), ids)
+            np.testing.assert_array_equal(np.asarray(got_vals.cpu()), vals)
+
+
+def test_a_long_row_of_few_values_above_zero_takes_no_longer_per_level_than_a_pass():
+    """The eight levels of a row whose k-th value is 0, against the two passes of a plain one: at
+    most 8 + 2 passes and their hand-overs."""
+    n = 1 << 25
+    zeros = torch.zeros((1, n), dtype=torch.float64, device="cuda")
+    zeros[0, ::n // 100] = 0.25
+    plain = torch.rand((1, n), dtype=torch.float64, device="cuda") ** 8
+
+    def ms(est):
+        best = 1e9
+        for _ in range(5):
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            a.record()
+            fora.topk(est, 500)
+            b.record()
+            b.synchronize()
+            best = min(best, a.elapsed_time(b))
+        return best
+
+    ms(plain)
+    assert ms(zeros) < 8 * ms(plain)
