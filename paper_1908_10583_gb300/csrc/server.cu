@@ -14,6 +14,7 @@
 #include <algorithm>
 #include <chrono>
 #include <condition_variable>
+#include <cstdlib>
 #include <cstring>
 #include <deque>
 #include <memory>
@@ -21,6 +22,7 @@
 #include <string>
 #include <thread>
 #include <unordered_map>
+#include <unordered_set>
 #include <vector>
 
 #include "fora.h"
@@ -197,6 +199,39 @@ struct fora_server {
   }
 };
 
+namespace {
+
+// The servers that are open.  At exit their lanes end before the process tears the device down:
+// they are threads with kernels in flight, whose memory must outlive them.  (A process that exited
+// with requests still running left the GPU a memory fault.)  The handler is registered with the
+// first server, after the CUDA runtime's own.
+struct OpenServers {
+  std::mutex mu;
+  std::unordered_set<fora_server*> all;
+};
+OpenServers& open_servers() {
+  static OpenServers* o = new OpenServers();  // outlives every handler
+  return *o;
+}
+
+// Ends the lanes after the batches that they are running.
+void stop_lanes(fora_server* s) {
+  {
+    std::lock_guard<std::mutex> lk(s->mu);
+    s->stop = true;
+  }
+  s->cv_work.notify_all();
+  for (auto& L : s->lanes)
+    if (L->th.joinable()) L->th.join();
+}
+
+void stop_open_servers() {
+  std::lock_guard<std::mutex> lk(open_servers().mu);
+  for (fora_server* s : open_servers().all) stop_lanes(s);
+}
+
+}  // namespace
+
 extern "C" {
 
 int fora_server_create(fora_graph* const* graphs, int32_t ngraphs, const fora_server_config* cfg,
@@ -243,6 +278,12 @@ int fora_server_create(fora_graph* const* graphs, int32_t ngraphs, const fora_se
     }
   }
   fora_server* srv = s.release();
+  {
+    std::lock_guard<std::mutex> lk(open_servers().mu);
+    static const int registered = std::atexit(stop_open_servers);
+    (void)registered;
+    open_servers().all.insert(srv);
+  }
   for (auto& L : srv->lanes) {
     Lane* lp = L.get();
     lp->th = std::thread([srv, lp] { srv->lane_loop(lp); });
@@ -254,12 +295,11 @@ int fora_server_create(fora_graph* const* graphs, int32_t ngraphs, const fora_se
 void fora_server_destroy(fora_server* s) {
   if (!s) return;
   {
-    std::lock_guard<std::mutex> lk(s->mu);
-    s->stop = true;
+    std::lock_guard<std::mutex> lk(open_servers().mu);
+    open_servers().all.erase(s);
   }
-  s->cv_work.notify_all();
+  stop_lanes(s);
   for (auto& L : s->lanes) {
-    if (L->th.joinable()) L->th.join();
     cudaSetDevice(s->graphs[L->graph]->device);
     {
       std::lock_guard<std::mutex> wl(L->ws.mu);

@@ -79,3 +79,28 @@ def test_arrivals_join_running_batches_and_match_the_query_alone():
         assert info.stats.walks == st1.walks and info.stats.pushes == st1.pushes
     server.close()
     g.close()
+
+
+def test_a_program_may_exit_with_requests_running():
+    """A program that leaves a server open, with requests running and queued, ends cleanly (its
+    lanes end with the batches that they run, before the device is torn down)."""
+    import os
+    import subprocess
+    import sys
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    fbuild.build()
+    program = """
+import inputs
+import paper_1908_10583_gb300 as fora
+g = fora.Graph(*inputs.rmat_csr(16, 16, 5))
+server = fora.Server([g], lanes_per_graph=2, max_batch=16, memory_budget_bytes=2 << 30)
+p = fora.Params.make(k=10)
+tickets = [server.submit(0, i, p) for i in range(5000)]
+server.wait(tickets[0], 10)
+import builtins
+builtins.keep = (g, server)  # alive up to the exit handlers
+"""
+    r = subprocess.run([sys.executable, "-c", program], capture_output=True, text=True, timeout=300,
+                       cwd=os.path.dirname(os.path.dirname(os.path.abspath(__file__))))
+    assert r.returncode == 0, r.stderr
