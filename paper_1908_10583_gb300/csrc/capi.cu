@@ -565,6 +565,7 @@ int fora::run_batch_ws(fora_graph* g, Workspace* w, const fora_params* p,
           state = cudaStreamQuery(stream);
           if (k < room) k += join->poll(w->h_sources + b.nsrc + k, room - k);
           if (k > 0) __atomic_store_n(&w->push_host->stop, 1u, __ATOMIC_RELEASE);
+          std::this_thread::yield();
         } while (state == cudaErrorNotReady);
         CUDA_TRY(state);
         if (*w->push_err & kErrBarrier) break;

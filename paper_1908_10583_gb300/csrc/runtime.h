@@ -157,7 +157,7 @@ void scratch_free(void* p, cudaStream_t st);
 void scratch_trim(int device);
 
 // Admission of further sources while a batch is in its push rounds (the serving lanes):
-// `poll`, called again and again meanwhile, may write up to `room` sources to `dst` (HOST) and
+// `poll`, called again and again meanwhile (so it is cheap while nothing is new), may write up to `room` sources to `dst` (HOST) and
 // returns how many; after the running round they join the batch as its next slots and
 // their queries run exactly as they would alone.  The batch then has *nsrc_final sources
 // (outputs and stats are sized for `cap`).

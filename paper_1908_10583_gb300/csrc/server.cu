@@ -12,6 +12,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <atomic>
 #include <chrono>
 #include <condition_variable>
 #include <cstdlib>
@@ -79,7 +80,8 @@ struct fora_server {
   fora_server_config cfg{};
   std::mutex mu;
   std::condition_variable cv_work, cv_done;
-  std::vector<std::deque<uint64_t>> queue;  // per graph
+  std::vector<std::deque<uint64_t>> queue;  // per graph, ascending tickets
+  std::unique_ptr<std::atomic<uint64_t>[]> newest;  // per graph: the last ticket queued
   std::unordered_map<uint64_t, Request> reqs;
   uint64_t next_ticket = 1;
   std::vector<std::unique_ptr<Lane>> lanes;
@@ -131,6 +133,7 @@ struct fora_server {
         r.info.start_ms = t_start;
         src[i] = r.source;
       }
+      uint64_t seen = newest[L->graph].load();  // every compatible one up to here is in
       ++lanes_busy;
       if (lanes_busy > max_lanes_busy) max_lanes_busy = lanes_busy;
       lk.unlock();
@@ -143,15 +146,20 @@ struct fora_server {
       vals.resize((size_t)L->cap * kmax);
       st.resize(L->cap);
       // continuous admission: between two push rounds, compatible requests that arrived
-      // meanwhile (k <= the batch's k) take free slots of this batch
+      // meanwhile (k <= the batch's k) take free slots of this batch.  The batch asks all the time
+      // while it waits for the device, so without a new request neither the lock is taken nor the
+      // queue looked through, and with one only the requests since the last look.
       JoinHook hook;
       hook.cap = L->cap;
       hook.nsrc_final = &nb;
       hook.poll = [&](int32_t* dst, int room) {
+        if (newest[L->graph].load(std::memory_order_acquire) <= seen) return 0;
         std::lock_guard<std::mutex> g2(mu);
         int added = 0;
         const double t_join = now_ms();
-        for (auto it = q.begin(); it != q.end() && added < room;) {
+        auto it = std::upper_bound(q.begin(), q.end(), seen);
+        seen = newest[L->graph].load();
+        while (it != q.end() && added < room) {
           Request& r = reqs[*it];
           if (compatible(r.params, first) && r.params.k <= kmax) {
             r.status = 1;
@@ -246,6 +254,7 @@ int fora_server_create(fora_graph* const* graphs, int32_t ngraphs, const fora_se
   s->graphs.assign(graphs, graphs + ngraphs);
   s->cfg = *cfg;
   s->queue.resize(ngraphs);
+  s->newest.reset(new std::atomic<uint64_t>[ngraphs]());
   size_t budget = cfg->memory_budget_bytes;
   if (budget == 0) {  // 80% of the free device memory
     size_t free_b = 0, total_b = 0;
@@ -334,6 +343,7 @@ int fora_server_submit(fora_server* s, int32_t graph, int32_t source, const fora
     r.params = *params;
     r.info.submit_ms = s->now_ms();
     s->queue[graph].push_back(t);
+    s->newest[graph].store(t, std::memory_order_release);
     *ticket = t;
   }
   s->cv_work.notify_all();

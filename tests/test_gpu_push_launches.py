@@ -62,20 +62,22 @@ def test_requests_join_a_push_of_a_launch_a_round():
     g.tune("push_slice", 0)
     server = fora.Server([g], lanes_per_graph=1, max_batch=16, memory_budget_bytes=2 << 30,
                          batch_window_ms=0.0, admit_during_push=True)
-    p = fora.Params.make(k=50, seed=21)
-    src = inputs.uniform_sources(g.n, 60, 2024)
-    tickets = []
-    for s in src:
-        tickets.append(server.submit(0, int(s), p))
-        time.sleep(0.0002)
-    results = [server.wait(t, 50) for t in tickets]
-    assert server.stats()["joined"] >= 1
-    for s, (ids, vals, info) in zip(src, results):
-        _, vals1, st1 = g.ssppr(int(s), p)
-        np.testing.assert_allclose(vals, vals1, rtol=0, atol=ATOL_PUSH)
-        assert info.stats.walks == st1.walks and info.stats.pushes == st1.pushes
-    server.close()
-    g.close()
+    try:
+        p = fora.Params.make(k=50, seed=21)
+        src = inputs.uniform_sources(g.n, 60, 2024)
+        tickets = []
+        for s in src:
+            tickets.append(server.submit(0, int(s), p))
+            time.sleep(0.0002)
+        results = [server.wait(t, 50) for t in tickets]
+        assert server.stats()["joined"] >= 1
+        for s, (ids, vals, info) in zip(src, results):
+            _, vals1, st1 = g.ssppr(int(s), p)
+            np.testing.assert_allclose(vals, vals1, rtol=0, atol=ATOL_PUSH)
+            assert info.stats.walks == st1.walks and info.stats.pushes == st1.pushes
+    finally:
+        server.close()
+        g.close()
 
 
 def test_a_kernel_that_holds_an_SM_does_not_hold_a_query():
@@ -131,15 +133,17 @@ def test_a_long_push_does_not_hold_queries_of_another_thread():
     th.start()
     time.sleep(0.2)
     waits = []
-    for i in range(40):
-        t0 = time.perf_counter()
-        _, vals, st = small.ssppr(i, ps, stream=b)
-        waits.append((time.perf_counter() - t0) * 1e3)
-        np.testing.assert_allclose(vals, alone[i][1], rtol=0, atol=ATOL_PUSH)
-        assert (st.pushes, st.walks) == (alone[i][2].pushes, alone[i][2].walks)
-        time.sleep(0.003)
-    stop.set()
-    th.join()
+    try:
+        for i in range(40):
+            t0 = time.perf_counter()
+            _, vals, st = small.ssppr(i, ps, stream=b)
+            waits.append((time.perf_counter() - t0) * 1e3)
+            np.testing.assert_allclose(vals, alone[i][1], rtol=0, atol=ATOL_PUSH)
+            assert (st.pushes, st.walks) == (alone[i][2].pushes, alone[i][2].walks)
+            time.sleep(0.003)
+    finally:
+        stop.set()
+        th.join()
     assert max(differ) <= ATOL_PUSH
     assert np.median(waits) < push_ms / 3, (np.median(waits), push_ms)
     big.close()

@@ -104,3 +104,34 @@ builtins.keep = (g, server)  # alive up to the exit handlers
     r = subprocess.run([sys.executable, "-c", program], capture_output=True, text=True, timeout=300,
                        cwd=os.path.dirname(os.path.dirname(os.path.abspath(__file__))))
     assert r.returncode == 0, r.stderr
+
+
+def test_a_backlog_does_not_hold_the_server_during_a_push():
+    """While a batch pushes, with 20000 requests of other parameters queued behind it, calls that
+    take the server's lock (here its counters, 200 times) return at once."""
+    import time
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    fbuild.build()
+    g = fora.Graph(*inputs.rmat_csr(20, 16, 2))
+    server = fora.Server([g], lanes_per_graph=1, max_batch=128, memory_budget_bytes=16 << 30,
+                         batch_window_ms=0.0, admit_during_push=True)
+    try:
+        # a push of more than half a second: 64 sources at a threshold that nearly every node
+        # crosses in every round
+        small = fora.Params.make(k=10, rmax=g.resolve(fora.Params.make())[0] / 1000)
+        long = [server.submit(0, i, small) for i in range(64)]
+        other = fora.Params.make(k=10, eps=0.4)
+        for i in range(20000):
+            server.submit(0, i, other)
+        took = []
+        for _ in range(200):
+            t0 = time.perf_counter()
+            done = server.stats()["completed"]
+            took.append((time.perf_counter() - t0) * 1e3)
+        assert done == 0, "the push ended before the calls"
+        server.wait(long[0], 10)
+        assert np.median(took) < 0.2, np.median(took)
+    finally:
+        server.close()
+        g.close()
