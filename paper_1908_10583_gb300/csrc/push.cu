@@ -229,6 +229,8 @@ __device__ __forceinline__ void red_add(double* p, double x) {
                : "memory");
 }
 
+constexpr uint32_t kNoEdge = 0xFFFFFFFFu;
+
 // r(u) += inc for source j of the group and the target of a code.
 template <int G>
 __device__ __forceinline__ void add_to(const GraphDev& g, const BatchDev& b,
@@ -242,19 +244,48 @@ __device__ __forceinline__ void add_to(const GraphDev& g, const BatchDev& b,
   }
 }
 
-constexpr uint32_t kNoEdge = 0xFFFFFFFFu;
-
 // x is not zero, for x >= 0 (never -0), without the FP64 pipe: at its rate the comparison alone
 // bounds a kernel that makes it for every value.
 __device__ __forceinline__ bool nonzero(double x) { return __double_as_longlong(x) != 0; }
 
+// 0, 1, ..., 32 as FP64: lengths of runs.
+__constant__ double kRunLength[33] = {0,  1,  2,  3,  4,  5,  6,  7,  8,  9,  10,
+                                      11, 12, 13, 14, 15, 16, 17, 18, 19, 20, 21,
+                                      22, 23, 24, 25, 26, 27, 28, 29, 30, 31, 32};
+
+// 32 consecutive edges of one source: rows are sorted, so the copies of a multi-edge lie in
+// neighbouring lanes, and their increments are added at once, k copies as k * inc by the first
+// (one rounding instead of k, which reorders the FP64 sum as the reductions do).
+// Only for large batches without groups: the balanced push of 256 sources of a 2^20-node R-MAT
+// graph, 4% of whose edges are copies (more of what hubs push), 295.6 -> 276.9 ms; a graph whose
+// edges all have 16 copies, 32 sources of 2^18 nodes, 14.2 -> 11.7.  In the small launches the
+// shuffles cost more than they save (one of 2^14 nodes 0.44 -> 0.46), and groups of four, whose
+// lanes of one edge lie side by side, are no slower without (64 sources, 16 copies: 6.1 ms, 6.1
+// where each copy of a source was merged).
+__device__ __forceinline__ void spread_runs(const GraphDev& g, const BatchDev& b,
+                                            const SpreadTarget<1>& t, uint32_t code,
+                                            uint32_t place, double inc) {
+  const uint32_t lane = lane_id();
+  const uint32_t code0 = __shfl_up_sync(kFull, code, 1), place0 = __shfl_up_sync(kFull, place, 1);
+  const bool goes_on = lane > 0 && code0 == code && place0 == place;
+  const uint32_t starts = __ballot_sync(kFull, !goes_on);
+  if (goes_on || code == kNoEdge || !nonzero(inc)) return;
+  const uint32_t later = starts & ~((2u << lane) - 1u);
+  const uint32_t k = (later ? (uint32_t)__ffs(later) - 1u : 32u) - lane;
+  add_to<1>(g, b, t, code, 0u, k > 1u ? __dmul_rn(inc, kRunLength[k]) : inc);
+}
+
 // The adds of 32 edges (each lane's target code and the place of its entry's increments in
 // inc[place][G]) for the G sources of the group, lanes of one edge side by side.
-template <int G>
+template <int G, bool kRuns>
 __device__ __forceinline__ void spread_slice(const GraphDev& g, const BatchDev& b,
                                              const SpreadTarget<G>& t, uint32_t code,
                                              uint32_t place, const double* inc) {
   const uint32_t lane = lane_id(), j = lane % G;
+  if constexpr (kRuns) {
+    spread_runs(g, b, t, code, place, inc[place]);
+    return;
+  }
 #pragma unroll
   for (int k = 0; k < G; ++k) {
     const int from = k * (32 / G) + (int)(lane / G);
@@ -324,7 +355,7 @@ __device__ __forceinline__ uint2 fetch_item(const GraphDev& g, const BatchDev& b
 
 // The edge lists of an item's entries, walked one after the other, 128 edges per iteration with
 // the next 128 targets on their way.
-template <int G>
+template <int G, bool kRuns>
 __device__ __forceinline__ void spread_item(const GraphDev& g, const BatchDev& b,
                                             const uint32_t* codes, uint32_t gr, bool light,
                                             uint2 entry, const double* inc) {
@@ -360,7 +391,7 @@ __device__ __forceinline__ void spread_item(const GraphDev& g, const BatchDev& b
     if (base + 32 * kSlices < total) fetch(base + 32 * kSlices, next, &next_own);
 #pragma unroll
     for (int k = 0; k < kSlices; ++k)
-      if (base + 32 * k < total) spread_slice<G>(g, b, t, code[k], (own >> (5 * k)) & 31u, inc);
+      if (base + 32 * k < total) spread_slice<G, kRuns>(g, b, t, code[k], (own >> (5 * k)) & 31u, inc);
     if (light) {  // warp-uniform
 #pragma unroll
       for (int k = 0; k < kSlices; ++k) spread_marks<G>(g, b, gr, code[k]);
@@ -372,7 +403,7 @@ __device__ __forceinline__ void spread_item(const GraphDev& g, const BatchDev& b
 }
 
 // A hub item: up to kHubChunk consecutive out-edges of one frontier entry.
-template <int G>
+template <int G, bool kRuns>
 __device__ __forceinline__ void spread_hub(const GraphDev& g, const BatchDev& b,
                                            const uint32_t* codes, uint32_t gr, bool light,
                                            uint2 rec, uint32_t len, double* inc) {
@@ -392,7 +423,7 @@ __device__ __forceinline__ void spread_hub(const GraphDev& g, const BatchDev& b,
   __syncwarp();
 #pragma unroll
   for (int k = 0; k < (int)(kHubChunk / 32); ++k)
-    if (32u * k < len) spread_slice<G>(g, b, t, code[k], 0u, inc);
+    if (32u * k < len) spread_slice<G, kRuns>(g, b, t, code[k], 0u, inc);
   if (light) {  // warp-uniform
 #pragma unroll
     for (int k = 0; k < (int)(kHubChunk / 32); ++k) spread_marks<G>(g, b, gr, code[k]);
@@ -502,7 +533,7 @@ struct ItemCursor {
   }
 };
 
-template <int G>
+template <int G, bool kRuns>
 __device__ void spread_phase(const GraphDev& g, const BatchDev& b, const Team& team, int cur,
                              unsigned long long nhub, unsigned long long nitems, uint32_t span,
                              SpreadStage<G>& st) {
@@ -536,7 +567,7 @@ __device__ void spread_phase(const GraphDev& g, const BatchDev& b, const Team& t
       const uint32_t l = len;
       more = c.step(b.err, &it);
       if (more) fetch(&rec, &len);
-      spread_hub<G>(g, b, codes, gr, light, r, l, st.inc[0]);
+      spread_hub<G, kRuns>(g, b, codes, gr, light, r, l, st.inc[0]);
     }
     __syncwarp();
   }
@@ -567,7 +598,7 @@ __device__ void spread_phase(const GraphDev& g, const BatchDev& b, const Team& t
         locate(&x);
         entry = fetch_item<G>(g, b, x, st.inc[half ^ 1]);
       }
-      spread_item<G>(g, b, codes, gr, light, now, st.inc[half]);
+      spread_item<G, kRuns>(g, b, codes, gr, light, now, st.inc[half]);
       half ^= 1;
     }
   }
@@ -1355,7 +1386,7 @@ __global__ void __launch_bounds__(kPushThreads, kPushBlocks)
       });
       if (!go) break;
     }
-    spread_phase<G>(g, b, ts.team, nx, __ldcg(&ps->nhub), __ldcg(&ps->ngroups), __ldcg(&ctl->span),
+    spread_phase<G, G == 1 && L == 8>(g, b, ts.team, nx, __ldcg(&ps->nhub), __ldcg(&ps->ngroups), __ldcg(&ctl->span),
                     sh.spread[wid]);
     if (threadIdx.x == 0) ts.begin = kBeginTake;
     if (kParts && __ldcg(&ctl->cut)) break;
@@ -1385,7 +1416,7 @@ template <int G>
 __global__ void __launch_bounds__(kPushThreads, kPushBlocks)
     k_push_spread(const __grid_constant__ GraphDev g, const __grid_constant__ BatchDev b) {
   __shared__ SpreadStage<G> stage[kPushWarps];
-  spread_phase<G>(g, b, Team{blockIdx.x, gridDim.x}, b.ps->cur, b.ps->nhub, b.ps->ngroups,
+  spread_phase<G, G == 1>(g, b, Team{blockIdx.x, gridDim.x}, b.ps->cur, b.ps->nhub, b.ps->ngroups,
                   b.ctl->span, stage[threadIdx.x >> 5]);
 }
 template <int G>
