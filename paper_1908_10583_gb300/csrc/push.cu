@@ -873,9 +873,12 @@ __device__ __forceinline__ void take_unit(const GraphDev& g, const BatchDev& b, 
 // of the groups with light ones.  A warp reads consecutive units, so its counters belong to one
 // or two groups; what is left of them at the end a block adds together.
 // Without groups (the balanced push) sources may differ much in what they take, and in large
-// scans a warp's units come from four places of the list: the balanced push of 256 sources of a
-// 2^20-node graph 317 -> 299 ms.  100 of 2^18, whose warps scan 21 units a round, 33.3 -> 33.9: so
-// from 48 units a warp on, and a kernel of its own, as the loop costs the others 3%.
+// scans a warp's units come from places far apart, kStretch at a time: the balanced push of 256
+// sources of a 2^20-node graph 317 ms with one stretch and 299 with four, 277 and 271 with four and
+// with stretches of kStretch since runs are added at once (64 sources 78.4 and 76.2).  100 of 2^18,
+// whose warps scan 21 units a round, 33.3 -> 33.9 with four: so from 48 units a warp on, and a
+// kernel of its own, as the loop costs the others 3%.
+constexpr unsigned kStretch = 13;
 constexpr unsigned long long kFarUnits = 48;
 template <int G, int L, bool kFar>
 __device__ void take_phase(const GraphDev& g, const BatchDev& b, const Team& team, int nx,
@@ -888,11 +891,11 @@ __device__ void take_phase(const GraphDev& g, const BatchDev& b, const Team& tea
   constexpr uint32_t kParts = 8 / L;  // of a unit
   const uint32_t per = b.tiles * kParts;
   const unsigned long long units = (unsigned long long)nheavy * per;
-  // A warp scans a stretch of consecutive units, with kFar four stretches a quarter of the list
-  // apart where they are long.
+  // A warp scans a stretch of consecutive units, with kFar several stretches far apart.
   unsigned long long x = units * warp / nwarps;
   unsigned long long end = units * (warp + 1) / nwarps;
-  const unsigned pieces = kFar && units >= kFarUnits * nwarps ? 4u : 1u;
+  const unsigned pieces =
+      kFar ? (unsigned)min(max(units / (nwarps * kStretch), 1ull), 64ull) : 1u;
   for (unsigned k = 0;;) {
     if (kFar && pieces > 1) {
       x = units * (k * nwarps + warp) / (pieces * nwarps);
