@@ -476,6 +476,11 @@ int fora::run_batch_ws(fora_graph* g, Workspace* w, const fora_params* p,
 
   std::lock_guard<std::mutex> lock(w->mu);
   CUDA_TRY(cudaSetDevice(g->device));
+  // a captured call would read its sources from the workspace's host buffers at every replay
+  cudaStreamCaptureStatus capture;
+  CUDA_TRY(cudaStreamIsCapturing(stream, &capture));
+  if (capture != cudaStreamCaptureStatusNone)
+    return fail(FORA_ERR_CUDA, "a query cannot be captured in a graph");
   rc = ensure_workspace(g, w, join ? join->cap : nsrc);
   if (rc) return rc;
   for (int i = 0; i < nsrc; ++i) {

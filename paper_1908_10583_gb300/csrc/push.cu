@@ -284,15 +284,15 @@ __device__ __forceinline__ void spread_slice(const GraphDev& g, const BatchDev& 
   const uint32_t lane = lane_id(), j = lane % G;
   if constexpr (kRuns) {
     spread_runs(g, b, t, code, place, inc[place]);
-    return;
-  }
+  } else {
 #pragma unroll
-  for (int k = 0; k < G; ++k) {
-    const int from = k * (32 / G) + (int)(lane / G);
-    const uint32_t c = G == 1 ? code : __shfl_sync(kFull, code, from);
-    const uint32_t p = G == 1 ? place : __shfl_sync(kFull, place, from);
-    const double a = inc[p * G + j];
-    if (c != kNoEdge && nonzero(a)) add_to<G>(g, b, t, c, j, a);
+    for (int k = 0; k < G; ++k) {
+      const int from = k * (32 / G) + (int)(lane / G);
+      const uint32_t c = G == 1 ? code : __shfl_sync(kFull, code, from);
+      const uint32_t p = G == 1 ? place : __shfl_sync(kFull, place, from);
+      const double a = inc[p * G + j];
+      if (c != kNoEdge && nonzero(a)) add_to<G>(g, b, t, c, j, a);
+    }
   }
 }
 

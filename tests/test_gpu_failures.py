@@ -151,3 +151,24 @@ def test_server_wait_times_out_and_the_request_still_completes(small):
     ids1, vals1, _ = g.ssppr(17, p)
     np.testing.assert_allclose(vals, vals1, rtol=0, atol=1e-12)
     s.close()
+
+
+def test_a_query_under_stream_capture_is_refused(small):
+    """Nothing is captured, and the graph answers afterwards."""
+    rp, col, g = small
+    p = fora.Params.make(k=20, seed=inputs.WALK_SEED)
+    src = inputs.uniform_sources(g.n, 5, 99)
+    ids0, vals0, _ = g.ssppr_batch(src, p)
+    out = [torch.empty((5, 20), dtype=t, device="cuda") for t in (torch.int32, torch.float64)]
+    pa = fora.Params.make(k=20, seed=inputs.WALK_SEED, flags=0x2)  # FORA_ASYNC
+    stream = torch.cuda.Stream()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=stream):
+        for q, stats in ((p, True), (pa, False)):
+            with pytest.raises(fora.FORAError) as e:
+                g.ssppr_batch(src, q, out_ids=out[0], out_vals=out[1], stats=stats, stream=stream)
+            assert e.value.code == fora.FORA_ERR_CUDA
+    ids1, vals1, _ = g.ssppr_batch(src, p)
+    np.testing.assert_array_equal(ids1, ids0)
+    np.testing.assert_allclose(vals1, vals0, rtol=0, atol=1e-12)
+    assert_still_answers(rp, col, g)
