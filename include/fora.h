@@ -133,9 +133,11 @@ typedef struct {
  * m = row_ptr[n] < 2^32 and d_out(v) >= 1 for every v (FORA_ERR_DANGLING: a walk of
  * Section 2.1 needs an out-neighbour at every node).  Edges are taken with
  * multiplicity; self-loops are allowed.  flags: 0.  Device memory: about
- * 4 (n + 1) + 8 m + 16 n bytes (4 m of them the walks' edge records), plus 4 m bytes of
- * target codes for the push when some node has in-degree >= 64 (the up to 128 nodes of
- * highest in-degree are marked in them, see "spread_hot").  Errors: FORA_ERR_BAD_ARG, FORA_ERR_DANGLING, FORA_ERR_OOM,
+ * 4 (n + 1) + 8 m + 20 n bytes (4 m of them the walks' edge records), 8 for each node whose
+ * degree has no class in those records (all but the lowest 1023 distinct degrees, or
+ * 2^(32 - ceil(log2 n)) - 1 if that is less), plus 4 m bytes of target codes for the push when
+ * some node has in-degree >= 64 (the up to 128 nodes of highest in-degree are marked in them,
+ * see "spread_hot").  Errors: FORA_ERR_BAD_ARG, FORA_ERR_DANGLING, FORA_ERR_OOM,
  * FORA_ERR_CUDA (no device); *out is NULL on any error.
  */
 int fora_graph_create(int64_t n, const int64_t *row_ptr, const int32_t *col, uint32_t flags,
@@ -461,8 +463,9 @@ int fora_threshold_debug(const double *r, const double *rmax, const uint32_t *d,
  */
 int fora_graph_tune(fora_graph *g, const char *key, int64_t value);
 
-/* The current value of a fora_graph_tune key (as set, or as the autotuner chose it).
- * Returns FORA_ERR_BAD_ARG for an unknown key or a null pointer. */
+/* The current value of a fora_graph_tune key (as set, or as the autotuner chose it), or of
+ * "hot_nodes" (see "spread_hot") or "push_launches", the launches of the push kernel by all
+ * calls on the graph so far.  Returns FORA_ERR_BAD_ARG for an unknown key or a null pointer. */
 int fora_graph_tuning(fora_graph *g, const char *key, int64_t *value);
 
 /*

@@ -319,17 +319,33 @@ double push_estimate(const double* rmax, int nsrc, int64_t n) {
 // Launches that an asynchronous call enqueues for a long push, at most.
 constexpr int kAsyncParts = 64;
 
+cudaError_t push_launch(fora_graph* g, const GraphDev& gd, const BatchDev& b, const PushPart* part,
+                        cudaStream_t stream) {
+  ++g->push_launches;
+  return launch_push(gd, b, g->num_sms, part, stream);
+}
+
+// A round of the push as kernels of its own, which the device runs as it has room, after a launch
+// that had none; `begun`: the push has been started.
+cudaError_t push_round_apart(const GraphDev& gd, const BatchDev& b, const fora_graph* g, bool* begun,
+                             cudaStream_t stream) {
+  cudaError_t e = cudaSuccess;
+  if (!*begun) e = launch_push_start(gd, b, g->num_sms, stream);
+  *begun = true;
+  return e == cudaSuccess ? launch_push_round(gd, b, g->num_sms, stream) : e;
+}
+
 // A push that is expected to take longer than two slices, as a sequence of launches of about a
 // slice each, so that work of other streams starts between them.  The host keeps one launch
 // ahead of the one that is running (the last does nothing), so the device does not wait for it.
 // An asynchronous call enqueues as many as the estimate tells, and one without a limit.
-cudaError_t push_in_parts(const GraphDev& gd, const BatchDev& b, const fora_graph* g, Workspace* w,
+cudaError_t push_in_parts(const GraphDev& gd, const BatchDev& b, fora_graph* g, Workspace* w,
                           uint32_t slice, double estimate, bool async, cudaStream_t stream) {
-  PushPart part{0, 0, slice, 0, async ? nullptr : w->push_host};
+  PushPart part{0, 0, slice, 0, async ? 1 : 0, async ? nullptr : w->push_host};
   cudaError_t e = cudaSuccess;
   auto next = [&] {
-    if (part.host) part.host->go[part.turn] = 1;
-    e = launch_push(gd, b, g->num_sms, &part, stream);
+    if (part.host) part.host->go[part.turn] = kPushLeft;
+    e = push_launch(g, gd, b, &part, stream);
     if (e == cudaSuccess && part.host) e = cudaEventRecord(w->part_ev[part.turn], stream);
     part.resume = 1;
     part.turn ^= 1;
@@ -341,14 +357,22 @@ cudaError_t push_in_parts(const GraphDev& gd, const BatchDev& b, const fora_grap
     if (e == cudaSuccess) next();
     return e;
   }
-  w->push_host->stop = 0;
+  bool begun = true, apart = false;
   next();
-  while (e == cudaSuccess) {
+  for (bool first = true; e == cudaSuccess; first = false) {
     next();
     // part.turn is now the turn of the launch before that one
     if (e == cudaSuccess) e = cudaEventSynchronize(w->part_ev[part.turn]);
-    if (e == cudaSuccess && !*(volatile uint32_t*)&w->push_host->go[part.turn]) break;
+    if (e != cudaSuccess) break;
+    const uint32_t state = *(volatile uint32_t*)&w->push_host->go[part.turn];
+    if (state == kPushDone) break;
+    if (state == kPushMissing) {
+      if (first) begun = false;
+      apart = true;
+      e = push_round_apart(gd, b, g, &begun, stream);
+    }
   }
+  if (e == cudaSuccess && apart) e = launch_push_finish(gd, b, g->num_sms, stream);
   return e;
 }
 
@@ -427,12 +451,15 @@ int fora::reserve_workspace(fora_graph* g, Workspace* w, int nsrc) {
   return ensure_workspace(g, w, nsrc);
 }
 
-// One batched query on workspace w (the whole phase sequence of include/fora.h).
-int fora::run_batch_ws(fora_graph* g, Workspace* w, const fora_params* p,
-                       const int32_t* sources, int nsrc, int32_t* out_ids, double* out_vals,
-                       fora_stats* st, const fora_debug_io* dbg, uint32_t dbg_flags,
-                       cudaStream_t stream, RmaxSource rsrc, const PipeHook* hook,
-                       const fora_balance* bal, const JoinHook* join) {
+namespace {
+
+// One batched query on workspace w (the whole phase sequence of include/fora.h).  *missing: the
+// device had no room for all blocks of the push at once, and nothing came of the call; with `apart`
+// the push runs as kernels that need none.
+int try_batch(fora_graph* g, Workspace* w, const fora_params* p, const int32_t* sources, int nsrc,
+              int32_t* out_ids, double* out_vals, fora_stats* st, const fora_debug_io* dbg,
+              uint32_t dbg_flags, cudaStream_t stream, RmaxSource rsrc, const PipeHook* hook,
+              const fora_balance* bal, const JoinHook* join, bool apart_only, bool* missing) {
   // a pipelined part always signals the next part, also when it stops early
   struct SignalOnExit {
     PipeLink* link;
@@ -536,7 +563,7 @@ int fora::run_batch_ws(fora_graph* g, Workspace* w, const fora_params* p,
     if (g->tune.spread_hot == 0) b.hot_copies = 0;
     b.walk_blocks = g->tune.walk_blocks;
     b.max_rounds = g->tune.max_push_rounds;
-    host_loop = g->tune.push_host_loop != 0;
+    host_loop = g->tune.push_host_loop != 0 || apart_only;
     slice = (uint32_t)g->tune.push_slice;
   }
 
@@ -558,10 +585,11 @@ int fora::run_batch_ws(fora_graph* g, Workspace* w, const fora_params* p,
       // after the round that is running, and they join as new slots.  (With a host round trip
       // after every round, whether anyone had come or not, 24 requests to a 2^16-node graph took
       // 4.13 ms, with this 3.39, 0.5 of them the batching window.)
-      for (PushPart part{0, 0, slice, 1, w->push_host};; part.resume = 1, part.turn ^= 1) {
+      bool begun = false, apart = false;
+      for (PushPart part{0, 0, slice, 1, 0, w->push_host};; part.resume = 1, part.turn ^= 1) {
         __atomic_store_n(&w->push_host->stop, 0u, __ATOMIC_RELEASE);
-        w->push_host->go[part.turn] = 1;
-        CUDA_TRY(launch_push(gd, b, g->num_sms, &part, stream));
+        w->push_host->go[part.turn] = kPushLeft;
+        CUDA_TRY(push_launch(g, gd, b, &part, stream));
         CUDA_TRY(cudaMemcpyAsync(w->push_err, w->err, sizeof(uint32_t), cudaMemcpyDeviceToHost, stream));
         const int room = join->cap - b.nsrc;
         int k = 0;
@@ -574,7 +602,13 @@ int fora::run_batch_ws(fora_graph* g, Workspace* w, const fora_params* p,
         } while (state == cudaErrorNotReady);
         CUDA_TRY(state);
         if (*w->push_err & kErrBarrier) break;
-        if (k == 0 && w->push_host->go[part.turn]) continue;  // the slice is over
+        const uint32_t left = w->push_host->go[part.turn];
+        if (left == kPushMissing) {
+          apart = true;
+          CUDA_TRY(push_round_apart(gd, b, g, &begun, stream));
+        }
+        begun = true;
+        if (k == 0 && left != kPushDone) continue;  // the slice is over
         if (k == 0) break;
         const int first = b.nsrc, grp0 = b.ngrp;
         for (int i = first; i < first + k; ++i) w->h_rmax[i] = rp.rmax;
@@ -596,6 +630,7 @@ int fora::run_batch_ws(fora_graph* g, Workspace* w, const fora_params* p,
         }
         CUDA_TRY(launch_push_join(gd, b, first, k, stream));
       }
+      if (apart) CUDA_TRY(launch_push_finish(gd, b, g->num_sms, stream));
       nsrc = b.nsrc;
       if (join->nsrc_final) *join->nsrc_final = nsrc;
     } else if (host_loop) {
@@ -618,10 +653,13 @@ int fora::run_batch_ws(fora_graph* g, Workspace* w, const fora_params* p,
       const double us = push_estimate(guess.empty() ? w->h_rmax : guess.data(), nsrc, g->n);
       // (a part of a pipelined batch is not cut: its own walks of the part before would start in
       // between, and beside each other both are slower, 248 ms for 256 sources of 2^20, not 234)
-      if (us > 2.0 * slice && !hook)
+      if (us > 2.0 * slice && !hook) {
         CUDA_TRY(push_in_parts(gd, b, g, w, slice, us, async, stream));
-      else
-        CUDA_TRY(launch_push(gd, b, g->num_sms, nullptr, stream));
+      } else {
+        // nobody could take up an asynchronous call's push, and a part's waits for its walks
+        const PushPart whole{0, 0, kNoSlice, 0, async || hook ? 1 : 0, nullptr};
+        CUDA_TRY(push_launch(g, gd, b, &whole, stream));
+      }
     }
     if (dbg && dbg->reserve)
       CUDA_TRY(launch_regroup(w->res, dbg->reserve, b, g->n, true, g->num_sms, stream));
@@ -669,6 +707,10 @@ int fora::run_batch_ws(fora_graph* g, Workspace* w, const fora_params* p,
   if (st && (rsrc.device || bal))  // the thresholds used were set on the device
     CUDA_TRY(cudaMemcpyAsync(w->h_rmax, w->rmax, nsrc * sizeof(double), cudaMemcpyDeviceToHost, stream));
   CUDA_TRY(cudaStreamSynchronize(stream));
+  if (*w->h_err & kErrMissing) {
+    *missing = true;
+    return FORA_OK;
+  }
   if (*w->h_err & kErrBarrier) return fail(FORA_ERR_CUDA, "the push's blocks did not all run");
   if (*w->h_err & kErrPushNotConverged)
     return fail(FORA_ERR_PUSH_NOT_CONVERGED, "push did not converge in %u rounds", b.max_rounds);
@@ -700,6 +742,21 @@ int fora::run_batch_ws(fora_graph* g, Workspace* w, const fora_params* p,
     }
   }
   return FORA_OK;
+}
+
+}  // namespace
+
+int fora::run_batch_ws(fora_graph* g, Workspace* w, const fora_params* p,
+                       const int32_t* sources, int nsrc, int32_t* out_ids, double* out_vals,
+                       fora_stats* st, const fora_debug_io* dbg, uint32_t dbg_flags,
+                       cudaStream_t stream, RmaxSource rsrc, const PipeHook* hook,
+                       const fora_balance* bal, const JoinHook* join) {
+  bool missing = false;
+  const int rc = try_batch(g, w, p, sources, nsrc, out_ids, out_vals, st, dbg, dbg_flags, stream,
+                           rsrc, hook, bal, join, false, &missing);
+  if (!missing) return rc;
+  return try_batch(g, w, p, sources, nsrc, out_ids, out_vals, st, dbg, dbg_flags, stream, rsrc, hook,
+                   bal, join, true, &missing);
 }
 
 namespace {
@@ -987,6 +1044,7 @@ int fora_graph_create(int64_t n, const int64_t* row_ptr, const int32_t* col, uin
       if (e == cudaSuccess) g->nhot = (int)hot.size();
     }
   }
+  if (e == cudaSuccess) e = load_push_phases();
   if (e == cudaSuccess) e = dalloc(&g->indeg, (size_t)n * sizeof(uint32_t));
   if (e == cudaSuccess) {
     const GraphDev gd = g->dev();
@@ -1391,7 +1449,6 @@ uint64_t splitmix(uint64_t* s) {
 }
 
 // Device buffers of one model call (inputs, targets, partials) on the default stream.
-// Buffers of a call on the default stream.
 struct ModelScratch {
   float* x = nullptr;
   float* t = nullptr;
@@ -1674,7 +1731,7 @@ int fora_graph_autotune(fora_graph* g, const fora_params* params, const int32_t*
     g->tune.pipeline = 1;  // phase times below are those of the whole batch
   }
   float pm = 0, wm = 0;
-  int rc = run(&pm, &wm);  // warm-up: workspace and push-loop graph
+  int rc = run(&pm, &wm);  // warm-up: workspace
   if (rc) return rc;
   // the push depends on spread_width only, the walk kernel on walk_blocks only
   int best_sw = 1, best_wb = 3;
@@ -1767,6 +1824,7 @@ int fora_graph_tuning(fora_graph* g, const char* key, int64_t* value) {
   if (strcmp(key, "walk_blocks") == 0) { *value = g->tune.walk_blocks; return FORA_OK; }
   if (strcmp(key, "pipeline") == 0) { *value = g->tune.pipeline; return FORA_OK; }
   if (strcmp(key, "push_host_loop") == 0) { *value = g->tune.push_host_loop; return FORA_OK; }
+  if (strcmp(key, "push_launches") == 0) { *value = g->push_launches.load(); return FORA_OK; }
   if (strcmp(key, "push_slice") == 0) { *value = g->tune.push_slice; return FORA_OK; }
   if (strcmp(key, "index_groups") == 0) { *value = g->tune.index_groups; return FORA_OK; }
   if (strcmp(key, "max_push_rounds") == 0) { *value = g->tune.max_push_rounds; return FORA_OK; }

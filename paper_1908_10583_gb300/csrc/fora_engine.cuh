@@ -59,6 +59,7 @@ constexpr uint32_t kErrPushNotConverged = 4u;
 constexpr uint32_t kErrIndexRange = 8u;  // a residue needs more walks than the index holds
 constexpr uint32_t kErrBounds = 16u;     // a device index check failed (FORA_DEBUG builds)
 constexpr uint32_t kErrBarrier = 32u;    // a wait of the push's blocks for each other ran out
+constexpr uint32_t kErrMissing = 64u;    // no push: the device had no room for all its blocks
 
 // Device index checks of the FORA_DEBUG build: FORA_IN_RANGE(err, i, n) is true when
 // i < n; otherwise it records kErrBounds in *err and is false, and the caller skips the
@@ -94,13 +95,17 @@ struct PushState {
 // that takes longer.
 struct PushHost {  // pinned host memory
   uint32_t stop;   // written by the host
-  uint32_t go[2];  // 1: rounds are left after the launch with this turn
+  uint32_t go[2];  // what the launch with this turn left: kPushDone, kPushLeft, kPushMissing
 };
+constexpr uint32_t kPushDone = 0u;     // the push is through
+constexpr uint32_t kPushLeft = 1u;     // rounds are left
+constexpr uint32_t kPushMissing = 2u;  // nothing done: the device had no room for all blocks
 struct PushPart {
   int resume;      // 0: from the start of the push, 1: where the launch before it ended
   int turn;        // alternates between 0 and 1, from 0
   uint32_t slice;  // kNoSlice: no limit
   int stops;       // read host->stop every round
+  int sure;        // a cooperative launch: all blocks run together, whenever they can
   PushHost* host;  // may be null
 };
 constexpr uint32_t kNoSlice = 0xFFFFFFFFu;
@@ -322,11 +327,15 @@ int resident_blocks(const void* kernel, int threads);
 // returns cudaErrorMemoryAllocation without allocating when the hook says so.
 cudaError_t device_alloc(void** p, size_t bytes);
 
-// push.cu: the whole push in one launch (from zeroing r and res on), or a part of it.
+// push.cu: the whole push in one launch (from zeroing r and res on), or a part of it.  Where the
+// device has no room for all its blocks at once nothing is done, and host->go or (without host)
+// kErrMissing tells.
 cudaError_t launch_push(const GraphDev& g, const BatchDev& b, int num_sms, const PushPart* part,
                         cudaStream_t st);
 // The same in steps for a host loop that reads PushState::go after each round: start, rounds,
-// finish.
+// finish.  They are loaded with the first graph: loaded when first launched they would wait for
+// whatever kernel is running, and it is beside such a kernel that they are needed.
+cudaError_t load_push_phases();
 cudaError_t launch_push_start(const GraphDev& g, const BatchDev& b, int num_sms, cudaStream_t st);
 cudaError_t launch_push_round(const GraphDev& g, const BatchDev& b, int num_sms, cudaStream_t st);
 cudaError_t launch_push_finish(const GraphDev& g, const BatchDev& b, int num_sms, cudaStream_t st);

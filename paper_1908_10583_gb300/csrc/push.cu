@@ -29,13 +29,17 @@
 // k_push runs the rounds in one launch: its blocks meet after each phase, and the first of them
 // runs the advance while the others wait at the take's.  (As three launches in a conditional graph
 // node a round cost 39 us however small; 22 rounds of a 2^14-node graph took 0.89 ms, now 0.39.)
-// The blocks at work are those that the device has room for, so nothing else on the device, of this
-// process or another, can hold a push back: a block enters when it starts, and takes part from the
-// next advance on; no block waits for one that has not started.  So that a push does not hold back
-// others either, a long one is a sequence of launches of about a millisecond, between which kernels
-// of other streams start (a single query beside batches of 256 sources of 2^20 nodes waited for the
-// whole push of one).  A serving batch that requests join ends its launch after a round and
-// resumes.  The same phases are launched one by one by push_host_loop.
+// A launch does its work only if all its blocks run at once: each enters as it starts, and when
+// some have not come after a tenth of a millisecond (other kernels hold their places) those that
+// have leave, and the host runs a round as kernels of its own, the phases one by one, which need no
+// places held, before it tries again.  So no block waits for one that has not started, and nothing
+// else on the device can hold a push back.  (Working on with the blocks that were there, and
+// admitting the others round by round, let lanes of a server block each other: a round begun by a
+// few blocks took 600 times as long, its late blocks holding the SMs meanwhile.)  So that a push
+// does not hold back others either, a long one is a sequence of launches of about a millisecond,
+// between which kernels of other streams start (a single query beside batches of 256 sources of
+// 2^20 nodes waited for the whole push of one).  A serving batch that requests join ends its launch
+// after a round and resumes.  The phases are launched one by one by push_host_loop too.
 //
 // Pushes to the graph's hot nodes (the up to 128 nodes of highest in-degree) would queue at the
 // L2 slices that hold their residues: each block adds them to one of kHotCopies copies, and the
@@ -194,11 +198,6 @@ __device__ void seed_phase(const GraphDev& g, const BatchDev& b) {
     b.ctl->span = kSpan;
   }
 }
-
-// The blocks at work: this block's place among them, and their number.
-struct Team {
-  uint32_t rank, size;
-};
 
 // ---------------------------------------------------------------- spread
 
@@ -440,7 +439,6 @@ constexpr uint32_t kChunk = 8;
 struct ItemShare {
   unsigned long long state;  // first item of the chunk << 8 | items taken of it
   unsigned long long next;   // the next chunk's number + 1, 0: not known yet
-  Team team;
 };
 
 struct ItemCursor {
@@ -464,7 +462,7 @@ struct ItemCursor {
     pre = pre_;
     counter = ctr;
     share = share_;
-    few = total <= (unsigned long long)share->team.size * kPushWarps;
+    few = total <= (unsigned long long)gridDim.x * kPushWarps;
     done = false;
     gr = 0;
     lo = 1;
@@ -490,7 +488,7 @@ struct ItemCursor {
           n = *(volatile unsigned long long*)&share->next;
         if (n == 0) break;
         *(volatile unsigned long long*)&share->next = 0;
-        const unsigned long long first = (share->team.size + n - 1ull) * kChunk;
+        const unsigned long long first = ((unsigned long long)gridDim.x + n - 1ull) * kChunk;
         atomicExch(&share->state, first << 8 | 1ull);
         return first;
       }
@@ -506,7 +504,7 @@ struct ItemCursor {
       unsigned long long x = 0;
       if (few) {
         if (done) return false;
-        x = (unsigned long long)(threadIdx.x >> 5) * share->team.size + share->team.rank;
+        x = (unsigned long long)(threadIdx.x >> 5) * gridDim.x + blockIdx.x;
         done = true;
       } else {
         if (lane_id() == 0) x = pop(err);
@@ -534,7 +532,7 @@ struct ItemCursor {
 };
 
 template <int G, bool kRuns>
-__device__ void spread_phase(const GraphDev& g, const BatchDev& b, const Team& team, int cur,
+__device__ void spread_phase(const GraphDev& g, const BatchDev& b, int cur,
                              unsigned long long nhub, unsigned long long nitems, uint32_t span,
                              SpreadStage<G>& st) {
   const uint32_t* codes = b.hot_copies ? g.scol : (const uint32_t*)g.col;
@@ -542,9 +540,8 @@ __device__ void spread_phase(const GraphDev& g, const BatchDev& b, const Team& t
   ItemCursor c;
   unsigned long long it;
   if (threadIdx.x < 2) {
-    shares[threadIdx.x].state = (unsigned long long)team.rank * kChunk << 8;
+    shares[threadIdx.x].state = (unsigned long long)blockIdx.x * kChunk << 8;
     shares[threadIdx.x].next = 0;
-    shares[threadIdx.x].team = team;
   }
   __syncthreads();
   if (nhub) {
@@ -881,11 +878,11 @@ __device__ __forceinline__ void take_unit(const GraphDev& g, const BatchDev& b, 
 constexpr unsigned kStretch = 13;
 constexpr unsigned long long kFarUnits = 48;
 template <int G, int L, bool kFar>
-__device__ void take_phase(const GraphDev& g, const BatchDev& b, const Team& team, int nx,
-                           uint32_t nheavy, uint32_t nlist, TakeStage<G>& st) {
-  const unsigned long long nwarps = (unsigned long long)team.size * (blockDim.x >> 5);
+__device__ void take_phase(const GraphDev& g, const BatchDev& b, int nx, uint32_t nheavy,
+                           uint32_t nlist, TakeStage<G>& st) {
+  const unsigned long long nwarps = (unsigned long long)gridDim.x * (blockDim.x >> 5);
   const unsigned long long warp =
-      (unsigned long long)team.rank * (blockDim.x >> 5) + (threadIdx.x >> 5);
+      (unsigned long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   TakeCount tc;
   TakeGroup tg;
   constexpr uint32_t kParts = 8 / L;  // of a unit
@@ -1104,11 +1101,11 @@ __device__ bool advance_phase(const GraphDev& g, const BatchDev& b, int nx, uint
 // After the last round: copies of hot nodes that no take has added (sources that the cost rule
 // stopped).
 template <int G>
-__device__ void finish_phase(const GraphDev& g, const BatchDev& b, const Team& team) {
+__device__ void finish_phase(const GraphDev& g, const BatchDev& b) {
   if (!b.hot_copies) return;
-  const unsigned long long nwarps = (unsigned long long)team.size * (blockDim.x >> 5);
+  const unsigned long long nwarps = (unsigned long long)gridDim.x * (blockDim.x >> 5);
   const unsigned long long warp =
-      (unsigned long long)team.rank * (blockDim.x >> 5) + (threadIdx.x >> 5);
+      (unsigned long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   const unsigned long long total = (unsigned long long)b.ngrp * g.nhot;
   for (unsigned long long x = warp; x < total; x += nwarps)
     fold_hot<G>(g, b, (uint32_t)(x / g.nhot), (uint32_t)(x % g.nhot));
@@ -1116,199 +1113,167 @@ __device__ void finish_phase(const GraphDev& g, const BatchDev& b, const Team& t
 
 // ---------------------------------------------------------------- kernels
 
-// Zeroes `bytes` bytes at a 16-byte aligned address with all threads of the team.
-__device__ __forceinline__ void team_zero(const Team& team, void* p, unsigned long long bytes) {
-  const unsigned long long t = (unsigned long long)team.rank * blockDim.x + threadIdx.x;
-  const unsigned long long nt = (unsigned long long)team.size * blockDim.x;
+// Zeroes `bytes` bytes at a 16-byte aligned address with all threads of the grid.
+__device__ __forceinline__ void grid_zero(void* p, unsigned long long bytes) {
+  const unsigned long long t = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x;
+  const unsigned long long nt = (unsigned long long)gridDim.x * blockDim.x;
   const unsigned long long quads = bytes / 16;
   for (unsigned long long i = t; i < quads; i += nt) ((uint4*)p)[i] = make_uint4(0u, 0u, 0u, 0u);
   for (unsigned long long i = quads * 16 + t; i < bytes; i += nt) ((uint8_t*)p)[i] = 0;
 }
 
 // The state a push starts from, but for what seed_phase sets.
-__device__ __forceinline__ void zero_phase(const GraphDev& g, const BatchDev& b,
-                                           const Team& team) {
+__device__ __forceinline__ void zero_phase(const GraphDev& g, const BatchDev& b) {
   const unsigned long long cells =
       (unsigned long long)min(b.ngrp * b.gw, b.lay) * (unsigned long long)g.n;
-  team_zero(team, b.r, cells * sizeof(double));
-  team_zero(team, b.res, cells * sizeof(double));
-  team_zero(team, b.hotr, (unsigned long long)b.hot_copies * b.lgrp * g.nhot * b.gw * sizeof(double));
-  team_zero(team, b.dirty, ((unsigned long long)b.lgrp * b.tiles + 31) / 32 * 4);
-  team_zero(team, b.slot_cnt, 4ull * b.cnt_stride * sizeof(uint32_t));
-  team_zero(team, b.last_edges, (unsigned long long)b.lay * sizeof(unsigned long long));
-  if (team.rank == 0 && threadIdx.x == 0) {
+  grid_zero(b.r, cells * sizeof(double));
+  grid_zero(b.res, cells * sizeof(double));
+  grid_zero(b.hotr, (unsigned long long)b.hot_copies * b.lgrp * g.nhot * b.gw * sizeof(double));
+  grid_zero(b.dirty, ((unsigned long long)b.lgrp * b.tiles + 31) / 32 * 4);
+  grid_zero(b.slot_cnt, 4ull * b.cnt_stride * sizeof(uint32_t));
+  grid_zero(b.last_edges, (unsigned long long)b.lay * sizeof(unsigned long long));
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
     b.work[0] = b.work[16] = 0;
     b.ctl->nheavy = b.ctl->nlist = 0;
   }
 }
 
-// A block's place in a launch, in shared memory (thread 0 writes it).
-struct TeamState {
-  Team team;
-  uint32_t arrivals;  // of the team up to the last meeting
+// What a block keeps in shared memory of the launch's meetings (thread 0 writes it).
+struct MeetState {
+  uint32_t arrivals;  // up to the last meeting
   uint32_t value;
   uint32_t begin;     // kBeginTake or kBeginSpread, with the round's parity
 };
 constexpr uint32_t kBeginTake = 0u, kBeginSpread = 2u;
 
-// The word of the last meeting with work: its arrivals, the size of the team after it and whether
-// the launch goes on.  Blocks whose rank is not below the size wait for a later word.
+// The word of the last meeting with work: the arrivals up to it + 1 (0: none yet), and whether the
+// launch goes on.
 __device__ __forceinline__ unsigned long long meet_word(const BatchDev& b) {
   return *(volatile unsigned long long*)(b.meet + kMeetWord);
 }
-__device__ __forceinline__ void write_meet_word(const BatchDev& b, uint32_t arrivals, uint32_t size,
-                                                bool go) {
+__device__ __forceinline__ void write_meet_word(const BatchDev& b, uint32_t arrivals, bool go) {
   *(volatile unsigned long long*)(b.meet + kMeetWord) =
-      (unsigned long long)arrivals << 32 | size << 1 | (go ? 1u : 0u);
+      ((unsigned long long)arrivals + 1ull) << 1 | (go ? 1ull : 0ull);
 }
-constexpr uint32_t kEveryone = 0x7FFFFFFFu;
 constexpr unsigned long long kClocksPerUs = 2000;  // about (2070 MHz at most)
+constexpr uint32_t kClosed = 0x80000000u;  // in kMeetEntered: the launch leaves, blocks are missing
+constexpr uint32_t kNotBegun = 2u;  // PushState::go where not even the start was done
+constexpr long long kPatience = 100 * (long long)kClocksPerUs;
 
-__device__ __forceinline__ unsigned long long now_ns() {
-  unsigned long long t;
-  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-  return t;
-}
-
-constexpr uint32_t kClosed = 0x80000000u;  // in kMeetEntered: the push began without the later blocks
-
-// The number of blocks that have entered.  While some have not (where other kernels hold their
-// places, which they may leave any time), waits `least` microseconds for them, and a quarter of
-// what their help would save in work of `us` microseconds of all blocks: a block that comes later
-// has to wait for the next round.  (Without this, batches of 256 sources in two parts on two
-// streams took 1.8 s, not 0.23: a few blocks began heavy rounds beside the other part's walks.)
-__device__ uint32_t await_blocks(const BatchDev& b, float us, float least) {
-  volatile uint32_t* entered = b.meet + kMeetEntered;
-  uint32_t size = *entered & ~kClosed;
-  if (size >= gridDim.x) return size;
-  const unsigned long long t0 = now_ns();
-  for (uint32_t polls = 0; polls < kMaxPolls && size < gridDim.x; ++polls) {
-    const float waited = (float)(now_ns() - t0) * 1e-3f;
-    if (waited >= least && 4.0f * waited * (float)size >= us * (float)(gridDim.x - size)) break;
-    size = *entered & ~kClosed;
-  }
-  return size;
-}
-
-// Enters the launch.  The first block to do so waits a little for the others, which all start
-// within a microsecond on an idle device, and lets those begin that are there.  A block's rank is
-// its index where that is all of them (neighbouring ranks are then on different SMs, among which
-// light rounds spread their work), else the order of entry; the block of rank 0 leads the launch.
-// At the start of a push a block clears its share of the state as it enters (no block does once the
-// first has closed the start), and if all are there the first block sets the sources' residues.
-// Returns 0 where the launch has ended already, 1 at its start, 2 before the spread of a later round.
+// Enters the launch; true if all its blocks have, within kPatience of the first (they do within a
+// microsecond on an idle device), or however long it takes where the launch guarantees it
+// (`sure`).  At the start of a push (`fresh`) a block clears its share of the state as it enters,
+// and when all have the first block sets the sources' residues.  A block that comes after the first
+// has given up leaves at once and clears nothing.
 template <int G>
-__device__ uint32_t team_enter(const GraphDev& g, const BatchDev& b, bool fresh, float us,
-                               TeamState& ts) {
+__device__ bool all_enter(const GraphDev& g, const BatchDev& b, bool fresh, bool sure,
+                          MeetState& ms) {
   if (threadIdx.x == 0) {
     const uint32_t old = atomicAdd(b.meet + kMeetEntered, 1u);
-    ts.team.rank = old & ~kClosed;
-    ts.value = fresh && !(old & kClosed) ? 1u : 0u;
+    ms.value = old & kClosed ? 0u : 1u;
+    ms.arrivals = old;
   }
   __syncthreads();
-  const uint32_t rank = ts.team.rank;
-  const bool clears = ts.value != 0;
-  __syncthreads();  // ts free
-  if (clears) {
-    zero_phase(g, b, Team{blockIdx.x, gridDim.x});
+  const bool in = ms.value != 0, first = ms.arrivals == 0;
+  __syncthreads();  // ms free
+  if (!in) return false;
+  if (fresh) {
+    zero_phase(g, b);
     __syncthreads();
     if (threadIdx.x == 0) {
       __threadfence();
       atomicAdd(b.meet + kMeetReady, 1u);
     }
   }
-  if (rank == 0) {
+  if (first) {  // block-uniform
     if (threadIdx.x == 0) {
-      uint32_t size = await_blocks(b, us, 20.0f), polls = 0;
-      if (fresh) {  // those that are there have cleared their shares, and no other will
-        volatile uint32_t* ready = b.meet + kMeetReady;
-        for (;; size = await_blocks(b, 0.0f, 0.0f)) {
-          while (*ready < size && ++polls <= kMaxPolls)
-            if (polls > 64) __nanosleep(100);
-          if (polls > kMaxPolls || size == gridDim.x ||
-              atomicCAS(b.meet + kMeetEntered, size, size | kClosed) == size)
-            break;
-        }
-        __threadfence();
+      volatile uint32_t* entered = b.meet + kMeetEntered;
+      volatile uint32_t* ready = b.meet + kMeetReady;
+      const long long t0 = clock64();
+      uint32_t n = *entered, polls = 0;
+      bool all;
+      for (;;) {
+        all = n == gridDim.x && (!fresh || *ready == n);
+        if (all || ++polls > kMaxPolls) break;
+        // blocks that have entered a fresh push finish clearing before the launch gives up
+        if (!sure && n < gridDim.x && clock64() - t0 > kPatience && (!fresh || *ready == n) &&
+            atomicCAS(b.meet + kMeetEntered, n, n | kClosed) == n)
+          break;
+        n = *entered;
       }
       if (polls > kMaxPolls) atomicOr(b.err, kErrBarrier);
-      ts.team.size = size;
-      ts.value = polls <= kMaxPolls ? 1u : 0u;
+      __threadfence();
+      ms.value = all ? 1u : 0u;
     }
     __syncthreads();
-    const bool go = ts.value != 0;
-    if (go && fresh && ts.team.size == gridDim.x) seed_phase<G>(g, b);  // block-uniform
+    const bool all = ms.value != 0;
+    if (all && fresh) seed_phase<G>(g, b);
+    if (!all && fresh && threadIdx.x == 0) b.ps->go = kNotBegun;
     __syncthreads();
     if (threadIdx.x == 0) {
       __threadfence();
-      write_meet_word(b, 0u, go ? ts.team.size : kEveryone, go);
+      write_meet_word(b, 0u, all);
     }
   }
   if (threadIdx.x == 0) {
     unsigned long long w;
-    uint32_t polls = 0, size;
-    while ((size = (uint32_t)(w = meet_word(b)) >> 1) <= rank && ++polls <= kMaxPolls)
+    uint32_t polls = 0;
+    while ((w = meet_word(b)) == 0 && ++polls <= kMaxPolls)
       if (polls > 64) __nanosleep(100);
-    const uint32_t arrivals = (uint32_t)(w >> 32);
-    const uint32_t how = polls > kMaxPolls || !(w & 1ull) ? 0u : arrivals == 0 ? 1u : 2u;
     if (polls > kMaxPolls) atomicOr(b.err, kErrBarrier);
     __threadfence();
-    if (how == 1 && size == gridDim.x) ts.team.rank = blockIdx.x;
-    ts.team.size = size;
-    ts.arrivals = arrivals;
-    ts.value = how;
+    ms.arrivals = 0;
+    ms.value = (uint32_t)w & 1u;
   }
   __syncthreads();
-  const uint32_t how = ts.value;
+  const bool go = ms.value != 0;
   __syncthreads();
-  return how;
+  return go;
 }
 
-// Meeting point of the team.  With `work`, the leader (always the same block: its instructions stay
-// in that SM's cache; run by whichever block came last they cost 10 us of fetches a round) runs it
-// when all have arrived and lets the others go on, with the blocks that have entered meanwhile when
-// `admit`; the value that its thread 0 returned comes back to every thread.  The waits are
-// bounded: a block that gives up reports kErrBarrier and gets 0, as then do the others.
+// Meeting point of all blocks.  With `work`, block 0 (always the same: its instructions stay in that
+// SM's cache; run by whichever block came last they cost 10 us of fetches a round) runs it when all
+// have arrived and lets the others go on, and the value that its thread 0 returned comes back to
+// every thread.  The waits are bounded: a block that gives up reports kErrBarrier and gets 0, as
+// then do the others.
 template <typename F>
-__device__ bool team_meet(const BatchDev& b, TeamState& ts, bool work, bool admit, F f) {
+__device__ bool grid_meet(const BatchDev& b, MeetState& ms, bool work, F f) {
   __syncthreads();
   if (threadIdx.x == 0) {
     __threadfence();
     atomicAdd(b.meet + kMeetArrived, 1u);
-    const uint32_t all = ts.arrivals + ts.team.size;
+    const uint32_t all = ms.arrivals + gridDim.x;
     uint32_t polls = 0, v = 1;
-    if (work && ts.team.rank != 0) {
+    if (work && blockIdx.x != 0) {
       unsigned long long w;
-      while ((int32_t)((uint32_t)((w = meet_word(b)) >> 32) - all) < 0 && ++polls <= kMaxPolls)
+      while ((uint32_t)((w = meet_word(b)) >> 1) <= all && ++polls <= kMaxPolls)
         if (polls > 64) __nanosleep(100);
       v = (uint32_t)w & 1u;
-      if (v) ts.team.size = (uint32_t)w >> 1;
     } else {
       volatile uint32_t* arrived = b.meet + kMeetArrived;
-      while ((int32_t)(*arrived - all) < 0 && ++polls <= kMaxPolls)
+      while (*arrived < all && ++polls <= kMaxPolls)
         if (polls > 64) __nanosleep(100);
     }
     if (polls > kMaxPolls) {
       atomicOr(b.err, kErrBarrier);
       v = 0;
     }
-    ts.arrivals = all;
-    ts.value = v;
+    ms.arrivals = all;
+    ms.value = v;
     __threadfence();
   }
   __syncthreads();
-  bool v = ts.value != 0;
-  if (work && ts.team.rank == 0) {
-    if (v) v = f();
+  bool v = ms.value != 0;
+  if (work && blockIdx.x == 0 && v) {
+    v = f();
     __syncthreads();
     if (threadIdx.x == 0) {
       __threadfence();
-      if (v && admit && ts.team.size < gridDim.x) ts.team.size = await_blocks(b, b.ps->us, 0.0f);
-      write_meet_word(b, ts.arrivals, v ? ts.team.size : kEveryone, v);
-      ts.value = v ? 1u : 0u;
+      write_meet_word(b, ms.arrivals, v);
+      ms.value = v ? 1u : 0u;
     }
     __syncthreads();
-    v = ts.value != 0;
+    v = ms.value != 0;
   }
   __syncthreads();
   return v;
@@ -1334,75 +1299,83 @@ __global__ void __launch_bounds__(kPushThreads, kPushBlocks)
     k_push(const __grid_constant__ GraphDev g, const __grid_constant__ BatchDev b,
            const __grid_constant__ PushPart part) {
   __shared__ PushShared<G> sh;
-  __shared__ TeamState ts;
+  __shared__ MeetState ms;
   __shared__ long long s_started;
   const PushState* ps = b.ps;
   const PushCtl* ctl = b.ctl;
   const uint32_t wid = threadIdx.x >> 5;
-  if (kParts && part.resume && !__ldcg(&ps->go)) return;  // the push is through
   const bool fresh = !(kParts && part.resume);
-  const uint32_t how = team_enter<G>(g, b, fresh, fresh ? 0.0f : __ldcg(&ps->us), ts);
-  if (how == 0) return;
-  if (kParts && ts.team.rank == 0 && threadIdx.x == 0) {
-    s_started = clock64();
+  const bool leads = blockIdx.x == 0 && threadIdx.x == 0;
+  if (kParts && leads) {
     uint32_t* other = part.turn ? b.meet - kMeetWords : b.meet + kMeetWords;  // the next launch's
     other[kMeetArrived] = other[kMeetEntered] = other[kMeetReady] = 0;
     *(unsigned long long*)(other + kMeetWord) = 0;
   }
-  bool go = true;
-  if (how == 1 && fresh && ts.team.size < gridDim.x) {  // without the shares of the others
-    zero_phase(g, b, ts.team);
-    go = team_meet(b, ts, true, false, [&] {
-      seed_phase<G>(g, b);
-      return true;
-    });
+  if (!fresh) {
+    const uint32_t state = __ldcg(&ps->go);
+    if (state != 1u) {  // through, or not begun
+      if (part.host && leads)
+        *(volatile uint32_t*)&part.host->go[part.turn] = state ? kPushMissing : kPushDone;
+      return;
+    }
   }
+  if (!all_enter<G>(g, b, fresh, part.sure != 0, ms)) {
+    if (leads) {
+      if (part.host)
+        *(volatile uint32_t*)&part.host->go[part.turn] = kPushMissing;
+      else
+        atomicOr(b.err, kErrMissing);
+    }
+    return;
+  }
+  if (kParts && leads) s_started = clock64();
+  bool go = true;
   // Where the first round begins is kept in shared memory: seen by the compiler it makes a copy of
   // the loop, whose fetches cost a small push a microsecond a round.
-  if (threadIdx.x == 0) {
-    uint32_t begin = kBeginTake;
-    if (how == 2 || !fresh) {
-      begin = (uint32_t)__ldcg(&ps->cur);
-      if (kParts && how == 1 && __ldcg(&ctl->cut))
-        begin ^= 1u;
-      else
-        begin |= kBeginSpread;
+  if (kParts) {
+    if (threadIdx.x == 0) {
+      uint32_t begin = kBeginTake;
+      if (!fresh) {
+        begin = (uint32_t)__ldcg(&ps->cur);
+        if (__ldcg(&ctl->cut))
+          begin ^= 1u;
+        else
+          begin |= kBeginSpread;
+      }
+      ms.begin = begin;
     }
-    ts.begin = begin;
+    __syncthreads();
   }
-  __syncthreads();
-  for (int nx = (int)(ts.begin & 1u); go; nx ^= 1) {
-    if (!(ts.begin & kBeginSpread)) {
-      take_phase<G, L, kFar>(g, b, ts.team, nx, __ldcg(&ctl->nheavy), __ldcg(&ctl->nlist),
-                             sh.take[wid]);
-      go = team_meet(b, ts, true, true, [&] {
+  for (int nx = kParts ? (int)(ms.begin & 1u) : 0; go; nx ^= 1) {
+    if (!kParts || !(ms.begin & kBeginSpread)) {
+      take_phase<G, L, kFar>(g, b, nx, __ldcg(&ctl->nheavy), __ldcg(&ctl->nlist), sh.take[wid]);
+      go = grid_meet(b, ms, true, [&] {
         bool stop = false;
         if (kParts && threadIdx.x == 0) {
           stop = part.slice != kNoSlice &&
                  (unsigned long long)(clock64() - s_started) >= kClocksPerUs * part.slice;
           if (part.stops) stop |= *(volatile uint32_t*)&part.host->stop != 0;
         }
-        const bool on = advance_phase<G>(g, b, nx, ts.team.size * kPushWarps) && !stop;
+        const bool on = advance_phase<G>(g, b, nx, gridDim.x * kPushWarps) && !stop;
         if (kParts && threadIdx.x == 0)
           b.ctl->cut = on && part.slice != kNoSlice && b.ps->us >= (float)part.slice ? 1u : 0u;
         return on;
       });
       if (!go) break;
     }
-    spread_phase<G, G == 1 && L == 8>(g, b, ts.team, nx, __ldcg(&ps->nhub), __ldcg(&ps->ngroups), __ldcg(&ctl->span),
-                    sh.spread[wid]);
-    if (threadIdx.x == 0) ts.begin = kBeginTake;
-    if (kParts && __ldcg(&ctl->cut)) break;
-    go = team_meet(b, ts, false, false, [] { return true; });
+    spread_phase<G, G == 1 && L == 8>(g, b, nx, __ldcg(&ps->nhub), __ldcg(&ps->ngroups),
+                                      __ldcg(&ctl->span), sh.spread[wid]);
+    if (kParts) {
+      if (threadIdx.x == 0) ms.begin = kBeginTake;
+      if (__ldcg(&ctl->cut)) break;
+    }
+    go = grid_meet(b, ms, false, [] { return true; });
   }
   const bool left = kParts && __ldcg(&ps->go);
-  if (!left) finish_phase<G>(g, b, ts.team);
-  if (kParts && ts.team.rank == 0 && threadIdx.x == 0) {
-    write_meet_word(b, ts.arrivals, kEveryone, false);  // after a cut round too
-    if (part.host)
-      *(volatile uint32_t*)&part.host->go[part.turn] =
-          left && !(*(volatile uint32_t*)b.err & kErrBarrier) ? 1u : 0u;
-  }
+  if (!left) finish_phase<G>(g, b);
+  if (kParts && part.host && leads)
+    *(volatile uint32_t*)&part.host->go[part.turn] =
+        left && !(*(volatile uint32_t*)b.err & kErrBarrier) ? kPushLeft : kPushDone;
 }
 
 // The phases on their own.
@@ -1413,20 +1386,21 @@ __global__ void __launch_bounds__(kPushThreads) k_push_seed(const __grid_constan
 }
 __global__ void __launch_bounds__(kPushThreads) k_push_zero(const __grid_constant__ GraphDev g,
                                                             const __grid_constant__ BatchDev b) {
-  zero_phase(g, b, Team{blockIdx.x, gridDim.x});
+  zero_phase(g, b);
 }
 template <int G>
 __global__ void __launch_bounds__(kPushThreads, kPushBlocks)
     k_push_spread(const __grid_constant__ GraphDev g, const __grid_constant__ BatchDev b) {
   __shared__ SpreadStage<G> stage[kPushWarps];
-  spread_phase<G, G == 1>(g, b, Team{blockIdx.x, gridDim.x}, b.ps->cur, b.ps->nhub, b.ps->ngroups,
+  if (b.ctl->cut) return;  // done by the launch before
+  spread_phase<G, G == 1>(g, b, b.ps->cur, b.ps->nhub, b.ps->ngroups,
                   b.ctl->span, stage[threadIdx.x >> 5]);
 }
 template <int G>
 __global__ void __launch_bounds__(kPushThreads, kPushBlocks)
     k_push_take(const __grid_constant__ GraphDev g, const __grid_constant__ BatchDev b) {
   __shared__ TakeStage<G> stage[kPushWarps];
-  take_phase<G, 8, false>(g, b, Team{blockIdx.x, gridDim.x}, b.ps->cur ^ 1, b.ctl->nheavy,
+  take_phase<G, 8, false>(g, b, b.ps->cur ^ 1, b.ctl->nheavy,
                           b.ctl->nlist, stage[threadIdx.x >> 5]);
 }
 template <int G>
@@ -1435,11 +1409,12 @@ __global__ void __launch_bounds__(kPushThreads) k_push_advance(const __grid_cons
   const int nx = b.ps->cur ^ 1;
   __syncthreads();
   advance_phase<G>(g, b, nx, 0u);
+  if (threadIdx.x == 0) b.ctl->cut = 0;
 }
 template <int G>
 __global__ void __launch_bounds__(kPushThreads) k_push_finish(const __grid_constant__ GraphDev g,
                                                               const __grid_constant__ BatchDev b) {
-  finish_phase<G>(g, b, Team{blockIdx.x, gridDim.x});
+  finish_phase<G>(g, b);
 }
 
 // Sources joining a batch between two push rounds (serving): slots [first, first + k) (their
@@ -1514,8 +1489,12 @@ cudaError_t push_t(const GraphDev& g, const BatchDev& b, int num_sms, const Push
   while (blocks < want && blocks < (unsigned)(num_sms * per_sm)) blocks += (unsigned)num_sms;
   BatchDev bd = b;
   bd.meet += part.turn * kMeetWords;
-  k_push<G, L, kParts, kFar><<<blocks, kPushThreads, 0, st>>>(g, bd, part);
-  return cudaGetLastError();
+  const void* kernel = (const void*)k_push<G, L, kParts, kFar>;
+  GraphDev gd = g;
+  PushPart pt = part;
+  void* args[] = {&gd, &bd, &pt};
+  if (part.sure) return cudaLaunchCooperativeKernel(kernel, dim3(blocks), dim3(kPushThreads), args, 0, st);
+  return cudaLaunchKernel(kernel, dim3(blocks), dim3(kPushThreads), args, 0, st);
 }
 
 template <int G>
@@ -1524,11 +1503,9 @@ cudaError_t push_any(const GraphDev& g, const BatchDev& b, int num_sms, const Pu
   // a small batch's full scan has few units: a warp reads a quarter of one, which shortens a round
   const unsigned long long units = (unsigned long long)b.ngrp * b.tiles;
   const bool small = units < kSmallUnits * (unsigned)num_sms;
-  if (!part) {
-    const PushPart whole{0, 0, kNoSlice, 0, nullptr};
-    return small ? push_t<G, 2, false>(g, b, num_sms, whole, st)
-                 : push_t<G, 8, false>(g, b, num_sms, whole, st);
-  }
+  if (part->slice == kNoSlice && !part->resume)
+    return small ? push_t<G, 2, false>(g, b, num_sms, *part, st)
+                 : push_t<G, 8, false>(g, b, num_sms, *part, st);
   if (small) return push_t<G, 2, true>(g, b, num_sms, *part, st);
   if (G == 1 && units >= kFarUnits * (unsigned)num_sms * kPushBlocks * kPushWarps)
     return push_t<G, 8, true, G == 1>(g, b, num_sms, *part, st);
@@ -1562,6 +1539,25 @@ cudaError_t launch_threshold_table(const double* r, const double* rm, const uint
 cudaError_t launch_push(const GraphDev& g, const BatchDev& b, int num_sms, const PushPart* part,
                         cudaStream_t st) {
   return b.gw == 1 ? push_any<1>(g, b, num_sms, part, st) : push_any<4>(g, b, num_sms, part, st);
+}
+
+template <int G>
+cudaError_t load_phases() {
+  cudaFuncAttributes a;
+  for (const void* k : {(const void*)k_push_seed<G>, (const void*)k_push_spread<G>,
+                        (const void*)k_push_take<G>, (const void*)k_push_advance<G>,
+                        (const void*)k_push_finish<G>, (const void*)k_push_join<G>}) {
+    const cudaError_t e = cudaFuncGetAttributes(&a, k);
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
+}
+
+cudaError_t load_push_phases() {
+  cudaFuncAttributes a;
+  cudaError_t e = cudaFuncGetAttributes(&a, (const void*)k_push_zero);
+  if (e == cudaSuccess) e = load_phases<1>();
+  return e == cudaSuccess ? load_phases<4>() : e;
 }
 
 cudaError_t launch_push_start(const GraphDev& g, const BatchDev& b, int num_sms, cudaStream_t st) {

@@ -3,6 +3,7 @@
 
 #include <cuda_runtime.h>
 
+#include <atomic>
 #include <condition_variable>
 #include <functional>
 #include <mutex>
@@ -25,7 +26,7 @@ struct WorkspaceSizes {
          slot_cnt = 0, pre = 0, ps = 0, err = 0, sources = 0, rmax = 0, stats = 0, stopped = 0,
          light = 0, tile_dirty = 0, last_edges = 0, blk = 0,
          topk = 0, feat = 0, pred = 0, rmax_learned = 0, out_ids = 0, out_vals = 0;
-  size_t total() const;  // q and hub count twice (two parities)
+  size_t total() const;  // q and hub count twice (Workspace::q, Workspace::hub)
 };
 WorkspaceSizes workspace_sizes(int64_t n, uint64_t hub_chunks, int nsrc);
 
@@ -45,21 +46,23 @@ struct Workspace {
   double* res = nullptr;
   // walk ends of every source (BatchDev::acc), then the walk counts of a debug call
   unsigned long long* tally = nullptr;
+  // q[0]: the frontier, then the residual entries; q[1]: the take's list of units and the copies
+  // of the hot nodes' residues, then the walk offsets.  hub[0]: hub items, hub[1]: their lengths.
   unsigned long long* q[2] = {nullptr, nullptr};
   unsigned long long* hub[2] = {nullptr, nullptr};
-  double* fa = nullptr;
-  unsigned long long* small = nullptr;  // counters[4] totals[2]
-  unsigned long long* work = nullptr;
-  uint32_t* alist = nullptr;      // [nsrc] sources with a non-empty frontier
-  uint32_t* slot_cnt = nullptr;   // [4][nsrc] per-source frontier entries and hub items
-  unsigned long long* pre = nullptr;  // [2][nsrc + 1] group and hub-item prefixes
+  double* fa = nullptr;  // increments, then walk weights, then estimates
+  unsigned long long* small = nullptr;  // PushCtl, totals[2] (from 4 on), walk_next (6)
+  unsigned long long* work = nullptr;   // work counters of the spread, meeting points of the push
+  uint32_t* alist = nullptr;      // groups of sources that the next take scans whole
+  uint32_t* slot_cnt = nullptr;   // [4][nsrc] frontier entries and hub items of each group
+  unsigned long long* pre = nullptr;  // [2][nsrc + 1] prefixes of the groups' items and hub items
   uint32_t* err = nullptr;
   int32_t* sources = nullptr;
   double* rmax = nullptr;
   SlotStats* stats = nullptr;
   uint32_t* stopped = nullptr;        // [nsrc] balanced push: the cost rule stopped the source
-  uint8_t* light = nullptr;           // [nsrc] light-round flags of the push take
-  uint8_t* tile_dirty = nullptr;      // tiles a light round's spread touched
+  uint8_t* light = nullptr;           // state of each group in the push (BatchDev::light)
+  uint8_t* tile_dirty = nullptr;      // bits of the units a light round's spread touched
   unsigned long long* last_edges = nullptr;  // [nsrc]
   unsigned long long* blk = nullptr;  // [2][kUnitPairs]
   void* topk_scratch = nullptr;
@@ -198,6 +201,7 @@ struct fora_graph {
   int num_sms = 0;
   fora::Tuning tune;
   std::mutex mu;              // guards `tune`
+  std::atomic<long long> push_launches{0};  // of k_push, of all calls so far
   fora::Workspace ws;         // the graph's own entry points
   // parts of a pipelined batch: a workspace and a stream each
   fora::Workspace pipe_ws[fora::kMaxPipeline];

@@ -104,6 +104,63 @@ def test_a_kernel_that_holds_an_SM_does_not_hold_a_query():
     g.close()
 
 
+@pytest.mark.parametrize("nsrc,balanced", [(2, False), (64, False), (40, True)])
+def test_pushes_beside_a_kernel_that_holds_an_SM(nsrc, balanced):
+    """Whole and cut pushes whose blocks do not all find room: rounds as kernels of their own."""
+    g = fora.Graph(*inputs.rmat_csr(18, 16, 2))
+    g.tune("push_slice", 300)
+    p = fora.Params.make(k=50)
+    sources = inputs.uniform_sources(g.n, nsrc, 5)
+    mine, other = torch.cuda.Stream(), torch.cuda.Stream()
+
+    def run():
+        if balanced:
+            return g.ssppr_batch_balanced(sources, p, COSTS, stream=mine)
+        return g.ssppr_batch(sources, p, stream=mine)
+
+    _, alone, st0 = run()
+    torch.cuda.synchronize()
+    done = torch.cuda.Event()
+    with torch.cuda.stream(other):
+        torch.cuda._sleep(800_000_000)  # about 0.4 s
+        done.record()
+    _, vals, st1 = run()
+    held = not done.query()
+    torch.cuda.synchronize()
+    np.testing.assert_allclose(vals, alone, rtol=0, atol=ATOL_PUSH)
+    for a, b in zip(st0, st1):
+        assert (a.pushes, a.edge_pushes, a.walks) == (b.pushes, b.edge_pushes, b.walks)
+        assert a.push_rounds == b.push_rounds
+    assert held
+    g.close()
+
+
+def test_requests_beside_a_kernel_that_holds_an_SM():
+    g = fora.Graph(*inputs.rmat_csr(18, 16, 2))
+    server = fora.Server([g], lanes_per_graph=1, max_batch=32, memory_budget_bytes=4 << 30,
+                         batch_window_ms=0.0, admit_during_push=True)
+    try:
+        p = fora.Params.make(k=50, seed=21)
+        src = inputs.uniform_sources(g.n, 40, 2024)
+        server.wait(server.submit(0, int(src[0]), p), 50)
+        other = torch.cuda.Stream()
+        with torch.cuda.stream(other):
+            torch.cuda._sleep(800_000_000)
+        tickets = []
+        for s in src:
+            tickets.append(server.submit(0, int(s), p))
+            time.sleep(0.0002)
+        results = [server.wait(t, 50) for t in tickets]
+        torch.cuda.synchronize()
+        for s, (ids, vals, info) in zip(src, results):
+            _, vals1, st1 = g.ssppr(int(s), p)
+            np.testing.assert_allclose(vals, vals1, rtol=0, atol=ATOL_PUSH)
+            assert info.stats.walks == st1.walks and info.stats.pushes == st1.pushes
+    finally:
+        server.close()
+        g.close()
+
+
 def test_a_long_push_does_not_hold_queries_of_another_thread():
     """Single queries beside balanced batches, whose push is most of the call: they wait for a
     slice of it at a time, not for the whole push."""
