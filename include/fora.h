@@ -444,8 +444,8 @@ int fora_threshold_debug(const double *r, const double *rmax, const uint32_t *d,
  * "push_host_loop" (0 or 1, default 0): 1 launches the push rounds from a host loop with
  * one device-to-host read per round, instead of a launch that runs many of them
  * on the device; the steps are the same (a profiler sees each of them on its own).
- * "push_slice" (0..1000000, default 1000): a push that is expected to take longer than twice
- * this many microseconds is a sequence of launches that end after the round in which they have
+ * "push_slice" (0..1000000, default 1000): a push that is expected to take longer than eight
+ * times this many microseconds is a sequence of launches that end after the round in which they have
  * run so long (0: one round each), and after the spread of a longer round, so that work of other
  * streams and calls starts in between; the host thread of a synchronous call enqueues them as the
  * push goes on.  Results do not depend on it.  "pipeline" (1..4, default 1): a batched

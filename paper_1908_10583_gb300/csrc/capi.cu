@@ -335,8 +335,12 @@ cudaError_t push_round_apart(const GraphDev& gd, const BatchDev& b, const fora_g
   return e == cudaSuccess ? launch_push_round(gd, b, g->num_sms, stream) : e;
 }
 
-// A push that is expected to take longer than two slices, as a sequence of launches of about a
-// slice each, so that work of other streams starts between them.  The host keeps one launch
+// Slices that a push which is not cut may take: the launches of a cut one cost 2 to 4% of a push of
+// 5 to 10 ms (100 sources of 200003 nodes 6.25 -> 6.53 ms, 32 of 2^18 balanced 12.4 -> 12.8) and 1%
+// of longer ones, and who waits behind it waits as long behind a walk kernel.
+constexpr double kWholeSlices = 8.0;
+
+// A push that is expected to take longer, as a sequence of launches of about a slice each, so that work of other streams starts between them.  The host keeps one launch
 // ahead of the one that is running (the last does nothing), so the device does not wait for it.
 // An asynchronous call enqueues as many as the estimate tells, and one without a limit.
 cudaError_t push_in_parts(const GraphDev& gd, const BatchDev& b, fora_graph* g, Workspace* w,
@@ -653,7 +657,7 @@ int try_batch(fora_graph* g, Workspace* w, const fora_params* p, const int32_t* 
       const double us = push_estimate(guess.empty() ? w->h_rmax : guess.data(), nsrc, g->n);
       // (a part of a pipelined batch is not cut: its own walks of the part before would start in
       // between, and beside each other both are slower, 248 ms for 256 sources of 2^20, not 234)
-      if (us > 2.0 * slice && !hook) {
+      if (us > kWholeSlices * slice && !hook) {
         CUDA_TRY(push_in_parts(gd, b, g, w, slice, us, async, stream));
       } else {
         // nobody could take up an asynchronous call's push, and a part's waits for its walks

@@ -86,7 +86,7 @@ struct PushState {
   int cur;
   uint32_t round;
   uint32_t go;      // the loop condition of the last round
-  float us;         // about how long the rest of the round takes with every block, microseconds
+  uint32_t pad;
   unsigned long long ngroups;  // items of `span` entries of the current frontier, over all groups
   unsigned long long nhub;     // hub items of the current frontier, over all groups
 };

@@ -192,7 +192,6 @@ __device__ void seed_phase(const GraphDev& g, const BatchDev& b) {
     ps->cur = 1;
     ps->round = 0;
     ps->go = 1;
-    ps->us = 0.0f;
     ps->ngroups = 0;
     ps->nhub = 0;
     b.ctl->span = kSpan;
@@ -1015,10 +1014,12 @@ __device__ __forceinline__ void advance_group(const BatchDev& b, int gr, bool* l
 
 // End of a round (one block; up to 32 groups: its first warp): the new frontier's per-group item
 // prefixes, the list of groups that still push, zeroed counters for the round after, and the
-// loop condition (at most b.max_rounds push rounds), which thread 0 returns.  Items of the spread
+// loop condition (at most b.max_rounds push rounds), which thread 0 returns, with about how long the
+// round takes (its spread and its full scans) in *us.  Items of the spread
 // are 32 entries, fewer where 32 would leave some of nwarps warps without one.
 template <int G>
-__device__ bool advance_phase(const GraphDev& g, const BatchDev& b, int nx, uint32_t nwarps) {
+__device__ bool advance_phase(const GraphDev& g, const BatchDev& b, int nx, uint32_t nwarps,
+                              float* us) {
   PushState* ps = b.ps;
   const size_t cs = (size_t)b.cnt_stride;
   const uint32_t* cnt_nx = b.slot_cnt + (size_t)nx * cs;
@@ -1083,8 +1084,8 @@ __device__ bool advance_phase(const GraphDev& g, const BatchDev& b, int nx, uint
     ps->ngroups = carry_g;
     ps->nhub = carry_h;
     // edge pushes at 2.5e11 a second, scanned residues at 6 TB/s
-    ps->us = G * (float)(carry_g * span * ((float)g.m / (float)g.n) + carry_h * kHubChunk) * 4e-6f +
-             (float)carry_heavy * (float)b.tiles * (kUnit * 8 / 6e6f);
+    *us = G * (float)(carry_g * span * ((float)g.m / (float)g.n) + carry_h * kHubChunk) * 4e-6f +
+          (float)carry_heavy * (float)b.tiles * (kUnit * 8 / 6e6f);
     b.ctl->nheavy = (uint32_t)carry_heavy;
     b.ctl->nlist = 0;
     b.ctl->span = span;
@@ -1146,14 +1147,15 @@ struct MeetState {
 };
 constexpr uint32_t kBeginTake = 0u, kBeginSpread = 2u;
 
-// The word of the last meeting with work: the arrivals up to it + 1 (0: none yet), and whether the
-// launch goes on.
+// The word of the last meeting with work: the arrivals up to it + 1 (0: none yet), and what follows.
+constexpr uint32_t kStop = 0u, kGo = 1u, kGoCut = 3u;  // kGoCut: as far as the end of the spread
 __device__ __forceinline__ unsigned long long meet_word(const BatchDev& b) {
   return *(volatile unsigned long long*)(b.meet + kMeetWord);
 }
-__device__ __forceinline__ void write_meet_word(const BatchDev& b, uint32_t arrivals, bool go) {
+__device__ __forceinline__ void write_meet_word(const BatchDev& b, uint32_t arrivals,
+                                                uint32_t next) {
   *(volatile unsigned long long*)(b.meet + kMeetWord) =
-      ((unsigned long long)arrivals + 1ull) << 1 | (go ? 1ull : 0ull);
+      ((unsigned long long)arrivals + 1ull) << 2 | next;
 }
 constexpr unsigned long long kClocksPerUs = 2000;  // about (2070 MHz at most)
 constexpr uint32_t kClosed = 0x80000000u;  // in kMeetEntered: the launch leaves, blocks are missing
@@ -1212,7 +1214,7 @@ __device__ bool all_enter(const GraphDev& g, const BatchDev& b, bool fresh, bool
     __syncthreads();
     if (threadIdx.x == 0) {
       __threadfence();
-      write_meet_word(b, 0u, all);
+      write_meet_word(b, 0u, all ? kGo : kStop);
     }
   }
   if (threadIdx.x == 0) {
@@ -1233,22 +1235,22 @@ __device__ bool all_enter(const GraphDev& g, const BatchDev& b, bool fresh, bool
 
 // Meeting point of all blocks.  With `work`, block 0 (always the same: its instructions stay in that
 // SM's cache; run by whichever block came last they cost 10 us of fetches a round) runs it when all
-// have arrived and lets the others go on, and the value that its thread 0 returned comes back to
-// every thread.  The waits are bounded: a block that gives up reports kErrBarrier and gets 0, as
+// have arrived and lets the others go on, and the value (kStop, kGo, kGoCut) that its thread 0
+// returned comes back to every thread.  The waits are bounded: a block that gives up reports kErrBarrier and gets 0, as
 // then do the others.
 template <typename F>
-__device__ bool grid_meet(const BatchDev& b, MeetState& ms, bool work, F f) {
+__device__ uint32_t grid_meet(const BatchDev& b, MeetState& ms, bool work, F f) {
   __syncthreads();
   if (threadIdx.x == 0) {
     __threadfence();
     atomicAdd(b.meet + kMeetArrived, 1u);
     const uint32_t all = ms.arrivals + gridDim.x;
-    uint32_t polls = 0, v = 1;
+    uint32_t polls = 0, v = kGo;
     if (work && blockIdx.x != 0) {
       unsigned long long w;
-      while ((uint32_t)((w = meet_word(b)) >> 1) <= all && ++polls <= kMaxPolls)
+      while ((uint32_t)((w = meet_word(b)) >> 2) <= all && ++polls <= kMaxPolls)
         if (polls > 64) __nanosleep(100);
-      v = (uint32_t)w & 1u;
+      v = (uint32_t)w & 3u;
     } else {
       volatile uint32_t* arrived = b.meet + kMeetArrived;
       while (*arrived < all && ++polls <= kMaxPolls)
@@ -1256,24 +1258,24 @@ __device__ bool grid_meet(const BatchDev& b, MeetState& ms, bool work, F f) {
     }
     if (polls > kMaxPolls) {
       atomicOr(b.err, kErrBarrier);
-      v = 0;
+      v = kStop;
     }
     ms.arrivals = all;
     ms.value = v;
     __threadfence();
   }
   __syncthreads();
-  bool v = ms.value != 0;
-  if (work && blockIdx.x == 0 && v) {
+  uint32_t v = ms.value;
+  if (work && blockIdx.x == 0 && v != kStop) {
     v = f();
     __syncthreads();
     if (threadIdx.x == 0) {
       __threadfence();
       write_meet_word(b, ms.arrivals, v);
-      ms.value = v ? 1u : 0u;
+      ms.value = v;
     }
     __syncthreads();
-    v = ms.value != 0;
+    v = ms.value;
   }
   __syncthreads();
   return v;
@@ -1329,7 +1331,7 @@ __global__ void __launch_bounds__(kPushThreads, kPushBlocks)
     return;
   }
   if (kParts && leads) s_started = clock64();
-  bool go = true;
+  uint32_t go = kGo;
   // Where the first round begins is kept in shared memory: seen by the compiler it makes a copy of
   // the loop, whose fetches cost a small push a microsecond a round.
   if (kParts) {
@@ -1346,7 +1348,7 @@ __global__ void __launch_bounds__(kPushThreads, kPushBlocks)
     }
     __syncthreads();
   }
-  for (int nx = kParts ? (int)(ms.begin & 1u) : 0; go; nx ^= 1) {
+  for (int nx = kParts ? (int)(ms.begin & 1u) : 0; go != kStop; nx ^= 1) {
     if (!kParts || !(ms.begin & kBeginSpread)) {
       take_phase<G, L, kFar>(g, b, nx, __ldcg(&ctl->nheavy), __ldcg(&ctl->nlist), sh.take[wid]);
       go = grid_meet(b, ms, true, [&] {
@@ -1356,20 +1358,21 @@ __global__ void __launch_bounds__(kPushThreads, kPushBlocks)
                  (unsigned long long)(clock64() - s_started) >= kClocksPerUs * part.slice;
           if (part.stops) stop |= *(volatile uint32_t*)&part.host->stop != 0;
         }
-        const bool on = advance_phase<G>(g, b, nx, gridDim.x * kPushWarps) && !stop;
-        if (kParts && threadIdx.x == 0)
-          b.ctl->cut = on && part.slice != kNoSlice && b.ps->us >= (float)part.slice ? 1u : 0u;
-        return on;
+        float us = 0.0f;
+        const bool on = advance_phase<G>(g, b, nx, gridDim.x * kPushWarps, &us) && !stop;
+        const bool cut = kParts && on && part.slice != kNoSlice && us >= (float)part.slice;
+        if (kParts && threadIdx.x == 0) b.ctl->cut = cut ? 1u : 0u;
+        return cut ? kGoCut : on ? kGo : kStop;
       });
-      if (!go) break;
+      if (go == kStop) break;
     }
     spread_phase<G, G == 1 && L == 8>(g, b, nx, __ldcg(&ps->nhub), __ldcg(&ps->ngroups),
                                       __ldcg(&ctl->span), sh.spread[wid]);
     if (kParts) {
       if (threadIdx.x == 0) ms.begin = kBeginTake;
-      if (__ldcg(&ctl->cut)) break;
+      if (go == kGoCut) break;
     }
-    go = grid_meet(b, ms, false, [] { return true; });
+    go = grid_meet(b, ms, false, [] { return kGo; });
   }
   const bool left = kParts && __ldcg(&ps->go);
   if (!left) finish_phase<G>(g, b);
@@ -1408,7 +1411,8 @@ __global__ void __launch_bounds__(kPushThreads) k_push_advance(const __grid_cons
                                                                const __grid_constant__ BatchDev b) {
   const int nx = b.ps->cur ^ 1;
   __syncthreads();
-  advance_phase<G>(g, b, nx, 0u);
+  float us;
+  advance_phase<G>(g, b, nx, 0u, &us);
   if (threadIdx.x == 0) b.ctl->cut = 0;
 }
 template <int G>
