@@ -656,7 +656,7 @@ int try_batch(fora_graph* g, Workspace* w, const fora_params* p, const int32_t* 
       if (bal || rsrc.device) guess.assign(nsrc, rp.rmax / 3);
       const double us = push_estimate(guess.empty() ? w->h_rmax : guess.data(), nsrc, g->n);
       // (a part of a pipelined batch is not cut: its own walks of the part before would start in
-      // between, and beside each other both are slower, 248 ms for 256 sources of 2^20, not 234)
+      // between, and beside each other both are slower, 248 ms for 256 sources of 2^20, not 237)
       if (us > kWholeSlices * slice && !hook) {
         CUDA_TRY(push_in_parts(gd, b, g, w, slice, us, async, stream));
       } else {
@@ -768,8 +768,8 @@ namespace {
 // A batch in `parts` parts, each on its own workspace and stream, driven by its own host
 // thread; part k's push waits for part k-1's push to finish, and part k-1's walks start as the
 // blocks of part k's push leave their SMs.  (Both are bound by L2 now, so little is gained: 256
-// sources of 2^20, rule's r_max, 231.6 ms in one part, 233.6 in two, 261 in four; 64 of 2^25 8.71 s
-// in one or two.)  The caller's stream waits for every part, so work queued on it afterwards sees
+// sources of 2^20, rule's r_max, 233.9 ms in one part, 236.9 in two, 240.5 in four; 64 of 2^25
+// 8.71 s in one or two.)  The caller's stream waits for every part, so work queued on it afterwards sees
 // the results.
 constexpr int kMinPartSources = 32;
 
